@@ -57,7 +57,8 @@ _SIGS = {
     "moe_permute": (C.c_int, [_P, _P, C.c_int32, _P, _P, _P, _P]),
     "moe_expert_ffn": (C.c_int, [_P, _P, C.c_int32, C.POINTER(moe_weights), _P, _P, _P, _P, C.c_size_t, _P]),
     "moe_combine": (C.c_int, [_P, _P, _P, _P, C.c_int32, _P, _P]),
-    "moe_layer_forward": (C.c_int, [_P, _P, C.c_int32, C.POINTER(moe_weights), _P, _P, _P, _P, C.c_size_t, _P]),
+    # (weights as a plain address: the call a decode step makes per layer, and converting an int is the cheapest)
+    "moe_layer_forward": (C.c_int, [_P, _P, C.c_int32, _P, _P, _P, _P, _P, C.c_size_t, _P]),
     "moe_layer_forward_static": (C.c_int, [C.POINTER(moe_config), _P, C.c_int32, C.POINTER(moe_weights), _P, _P, _P, _P]),
     "moe_offload_create": (C.c_int, [C.POINTER(moe_config), C.c_int32, C.c_int32, C.POINTER(_P), _P, C.c_size_t,
                                      C.POINTER(_P)]),
@@ -94,6 +95,10 @@ def _lib():
     return _LIB
 
 
+# the current stream's handle, without the Stream object that torch.cuda.current_stream() builds on every call
+_current_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _ptr(t) -> int | None:
     if t is None:
         return None
@@ -106,7 +111,7 @@ def _ptr(t) -> int | None:
 
 def _stream(stream=None) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return _current_raw_stream(_current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -196,8 +201,12 @@ def moe_combine(ctx, out_slots, topk_w, inv, T, y, stream=None):
 
 
 def moe_layer_forward(ctx, x, T, w: moe_weights, y, topk_idx=None, topk_w=None, ws=None, stream=None):
-    _ok(_lib().moe_layer_forward(ctx, _ptr(x), T, C.byref(w), _ptr(y), _ptr(topk_idx), _ptr(topk_w), _ptr(ws),
-                                 ws.numel() * ws.element_size(), _stream(stream)), "moe_layer_forward")
+    rc = (_LIB or _lib()).moe_layer_forward(
+        ctx, _ptr(x), T, C.addressof(w), _ptr(y), None if topk_idx is None else _ptr(topk_idx),
+        None if topk_w is None else _ptr(topk_w), _ptr(ws), ws.nbytes,
+        _current_raw_stream(_current_device()) if stream is None else _stream(stream))
+    if rc:
+        raise MoeError(rc, "moe_layer_forward")
 
 
 def moe_layer_forward_static(cfg: moe_config, x, T, w: moe_weights, y, topk_idx=None, topk_w=None, stream=None) -> int:

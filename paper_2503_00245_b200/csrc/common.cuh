@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/cosmoe.h"
 
 namespace cosmoe {
@@ -61,6 +63,22 @@ struct moe_ctx {
 };
 
 namespace cosmoe {
+
+// Lets `Kernel` use all the dynamic shared memory the device offers a CTA: once per kernel and device instead of a
+// driver call in front of every launch.  (The limit only permits; a launch still takes what it asks for.)
+constexpr int kMaxDevices = 64;
+template <auto Kernel>
+int allow_full_smem(const moe_ctx* ctx) {
+  static std::atomic<bool> done[kMaxDevices];
+  const bool tracked = ctx->device >= 0 && ctx->device < kMaxDevices;
+  if (tracked && done[ctx->device].load(std::memory_order_acquire)) return MOE_OK;
+  cudaFuncAttributes fa{};
+  MOE_CUDA_TRY(cudaFuncGetAttributes(&fa, Kernel));
+  MOE_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    ctx->max_smem_optin - (int)fa.sharedSizeBytes));
+  if (tracked) done[ctx->device].store(true, std::memory_order_release);
+  return MOE_OK;
+}
 
 // Offsets (bytes) of the pieces of the caller's scratch buffer.
 struct WsLayout {
@@ -147,6 +165,12 @@ __device__ __forceinline__ void flag_error(DeviceState* st, unsigned code, unsig
 // predecessor has completed and its writes are visible.  (Without the launch attribute both are no-ops.)
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+#define MOE_TRY(expr)              \
+  do {                             \
+    const int _rc = (expr);        \
+    if (_rc != MOE_OK) return _rc; \
+  } while (0)
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {

@@ -1454,8 +1454,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
 }
 
 template <int V>
-int launch_variant(const DenseParams& P, int grid, size_t smem, cudaStream_t s) {
-  MOE_CUDA_TRY(cudaFuncSetAttribute(dense_stream_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+int launch_variant(const moe_ctx* ctx, const DenseParams& P, int grid, size_t smem, cudaStream_t s) {
+  MOE_TRY(allow_full_smem<dense_stream_kernel<V>>(ctx));
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(grid), lc.blockDim = dim3(kThreads), lc.dynamicSmemBytes = smem, lc.stream = s;
   cudaLaunchAttribute attr[1];
@@ -1545,12 +1545,12 @@ int launch_dense_stream(moe_ctx* ctx, int mode, const void* x, int T, const moe_
                   : 0;
   int rc;
   switch (v) {
-    case V_T1: rc = launch_variant<V_T1>(P, G, smem, s); break;
-    case V_COLS: rc = launch_variant<V_COLS>(P, G, smem, s); break;
-    case V_MMA_BF16_S: rc = launch_variant<V_MMA_BF16_S>(P, G, smem, s); break;
-    case V_MMA_F32_S: rc = launch_variant<V_MMA_F32_S>(P, G, smem, s); break;
-    case V_MMA_BF16_L: rc = launch_variant<V_MMA_BF16_L>(P, G, smem, s); break;
-    default: rc = launch_variant<V_MMA_F32_L>(P, G, smem, s); break;
+    case V_T1: rc = launch_variant<V_T1>(ctx, P, G, smem, s); break;
+    case V_COLS: rc = launch_variant<V_COLS>(ctx, P, G, smem, s); break;
+    case V_MMA_BF16_S: rc = launch_variant<V_MMA_BF16_S>(ctx, P, G, smem, s); break;
+    case V_MMA_F32_S: rc = launch_variant<V_MMA_F32_S>(ctx, P, G, smem, s); break;
+    case V_MMA_BF16_L: rc = launch_variant<V_MMA_BF16_L>(ctx, P, G, smem, s); break;
+    default: rc = launch_variant<V_MMA_F32_L>(ctx, P, G, smem, s); break;
   }
   if (rc != MOE_OK) return rc;
   ctx->launches++;
@@ -1580,7 +1580,6 @@ constexpr size_t kStaticBytes = kStaticStateBytes + kStaticAccBytes;
 // handle for cudaGetSymbolAddress; it is not a device address and is never passed to a kernel.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
-constexpr int kMaxDevices = 64;
 struct StaticDevice {
   std::once_flag once;
   int rc;               // outcome of the one-off set-up

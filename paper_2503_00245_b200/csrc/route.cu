@@ -205,7 +205,7 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
   const uint16_t* wr = (const uint16_t*)w->w_router;
   const size_t staged = 18 * (size_t)c.d_model;  // bytes of the shifted copy of W_r (8 experts)
   if (!few && c.n_experts == 8 && staged <= 96 * 1024) {
-    MOE_CUDA_TRY(cudaFuncSetAttribute(route_smem_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged));
+    MOE_TRY(allow_full_smem<route_smem_kernel<XT>>(ctx));
     const int ctas = (T + kRouteWarps - 1) / kRouteWarps;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(ctas < 2 * ctx->sm_count ? ctas : 2 * ctx->sm_count), lc.blockDim = block;

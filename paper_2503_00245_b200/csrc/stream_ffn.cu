@@ -765,7 +765,7 @@ int launch_stream_ffn(moe_ctx* ctx, int mode, const void* x, int T, const moe_we
     while ((1 << ph.seg_shift) < S) ph.seg_shift++;
   }
   const size_t smem = (size_t)P.n_stages * P.stage_bytes + fixed;
-  MOE_CUDA_TRY(cudaFuncSetAttribute(stream_ffn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MOE_TRY(allow_full_smem<stream_ffn_kernel>(ctx));
   void* args[] = {(void*)&P};
   MOE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)stream_ffn_kernel, dim3(G), dim3(kThreads), args, smem, s));
   ctx->launches++;

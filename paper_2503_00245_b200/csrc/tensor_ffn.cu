@@ -538,7 +538,6 @@ int make_map_b(CUtensorMap* m, const void* base, long long inner, int nsub, long
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
 
-// Pairs of CTAs the device can hold at once (one CTA per SM; a pair sits on two SMs of one cluster).
 void pair_launch_config(cudaLaunchConfig_t& lc, cudaLaunchAttribute* attr, int ctas, size_t smem, cudaStream_t s) {
   lc = cudaLaunchConfig_t{};
   lc.gridDim = dim3(ctas), lc.blockDim = dim3(kThreadsGG), lc.dynamicSmemBytes = smem, lc.stream = s;
@@ -550,7 +549,13 @@ void pair_launch_config(cudaLaunchConfig_t& lc, cudaLaunchAttribute* attr, int c
 }
 
 // Pairs of CTAs the device can hold at once (one CTA per SM; a pair sits on two SMs of one cluster).
-int max_pairs(moe_ctx* ctx, size_t smem) {
+// Every launch of the kernel takes more than half of an SM's shared memory, so the number does not depend on the
+// launch: the driver is asked once per device (the query costs more than a launch).
+int max_pairs(const moe_ctx* ctx, size_t smem) {
+  static std::atomic<int> known[kMaxDevices];
+  const bool tracked = ctx->device >= 0 && ctx->device < kMaxDevices;
+  if (tracked && known[ctx->device].load(std::memory_order_relaxed) > 0)
+    return known[ctx->device].load(std::memory_order_relaxed);
   cudaLaunchConfig_t lc;
   cudaLaunchAttribute attr[2];
   pair_launch_config(lc, attr, ctx->sm_count & ~1, smem, nullptr);
@@ -560,7 +565,9 @@ int max_pairs(moe_ctx* ctx, size_t smem) {
     (void)cudaGetLastError();
     n = ctx->sm_count / 2;
   }
-  return std::max(1, std::min(n, ctx->sm_count / 2));
+  n = std::max(1, std::min(n, ctx->sm_count / 2));
+  if (tracked) known[ctx->device].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b, GGParams P,
@@ -575,7 +582,7 @@ int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const 
   P.n_stages = P.bmode == B_DUAL ? 4 : kMaxStagesGG;
   const size_t smem = P.n_stages * stage_bytes + sizeof(SmemGG) + 1024 + 128;
   if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
-  MOE_CUDA_TRY(cudaFuncSetAttribute(grouped_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MOE_TRY(allow_full_smem<grouped_gemm_kernel>(ctx));
   const long long m_tiles = (n_slots + kPairRows - 1) / kPairRows + c.n_experts;  // upper bound
   const int pairs = (int)std::min<long long>(m_tiles * n_tiles * P.ksplit, max_pairs(ctx, smem));
   cudaLaunchConfig_t lc;

@@ -798,17 +798,14 @@ int launch_wd_decode(moe_ctx* ctx, const void* x, const moe_weights* w, int32_t*
   if (!wd_small(c)) {
     const size_t smem = wd_stream_smem(c);
     if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
-    MOE_CUDA_TRY(cudaFuncSetAttribute(wd_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MOE_TRY(allow_full_smem<wd_stream_kernel>(ctx));
     P.split = kWsSeg;
     MOE_CUDA_TRY(launch_pdl(wd_stream_kernel, dim3(grid), dim3(kWsThreads), smem, s, P));
     ctx->launches++;
     return MOE_OK;
   }
   const size_t smem = sizeof(WdSmem);
-  MOE_CUDA_TRY(cudaFuncSetAttribute(wd_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 0;
-  MOE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wd_decode_kernel, kWdThreads, smem));
-  if (per_sm < 1) return MOE_ERR_UNSUPPORTED;
+  MOE_TRY(allow_full_smem<wd_decode_kernel>(ctx));
   const int n_warps = grid * kWdWarps;
   int split = n_warps / (c.top_k * c.wd_rank);
   P.split = split < 1 ? 1 : (split > kWdMaxSplit ? kWdMaxSplit : split);

@@ -97,10 +97,16 @@ class MoELayer:
 
     # ---- the whole layer ------------------------------------------------------------------
     def forward(self, x, y=None, topk_idx=None, topk_w=None):
-        T = x.shape[0]
-        self._need(T)
+        shape = x.shape
+        T = shape[0]
+        if T > self.max_tokens:
+            self._need(T)
         if y is None:
-            y = torch.empty((T, self.d), dtype=self.x_dtype, device=self.device)
+            # one token's layer takes about as long as a few calls into PyTorch: y is allocated the cheapest way
+            if x.is_cuda and len(shape) == 2 and shape[1] == self.d and x.dtype == self.x_dtype:
+                y = torch.empty_like(x)
+            else:
+                y = torch.empty((T, self.d), dtype=self.x_dtype, device=self.device)
         B.moe_layer_forward(self.ctx, x, T, self.weights, y, topk_idx, topk_w, self.ws)
         return y
 
