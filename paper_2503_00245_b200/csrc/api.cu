@@ -37,9 +37,12 @@ WsLayout ws_layout(const moe_config& c, int T) {
   L.inv = take(n * 4);
   const bool stream_ok = T <= MOE_STREAM_MAX_TOKENS;
   const bool tensor_ok = true;
-  L.vec_a = take(stream_ok ? n * 2 * (size_t)c.wd_rank * 4 : 0);
-  L.vec_b = take(stream_ok ? n * (size_t)c.d_ff * 4 : 0);
-  L.vec_c = take(stream_ok ? n * (size_t)c.wd_rank * 8 * 4 : 0);  // v, in up to 8 segments per value
+  // one token: fp32 vectors, v in up to 8 segments per value; several: three bf16 terms per value (t is a pair)
+  const bool wd_stream = stream_ok && c.wd_rank > 0;
+  L.vec_x = take(wd_stream && c.x_dtype == MOE_F32 ? (size_t)T * c.d_model * 6 : 0);
+  L.vec_a = take(wd_stream ? n * 2 * (size_t)c.wd_rank * 6 : 0);
+  L.vec_b = take(wd_stream ? n * (size_t)c.d_ff * 6 : 0);
+  L.vec_c = take(wd_stream ? n * (size_t)c.wd_rank * 8 * 4 : 0);
   L.xperm = take(tensor_ok ? n * (size_t)c.d_model * 2 : 0);
   L.hidden = take(tensor_ok ? n * (size_t)c.d_ff * 2 : 0);
   const size_t rp = ((size_t)c.wd_rank + 63) / 64 * 64;            // the rank rounded up to the tensor path's K step
@@ -248,7 +251,7 @@ int moe_expert_ffn(moe_ctx* ctx, const void* x, int32_t T, const moe_weights* w,
     if (T > MOE_STREAM_MAX_TOKENS) return MOE_ERR_UNSUPPORTED;
     if (ctx->cfg.wd_rank == 0)
       return launch_dense_stream(ctx, 1, x, T, w, nullptr, nullptr, expert_offsets, perm, nullptr, out_slots, s);
-    return launch_stream_ffn(ctx, 1, x, T, w, nullptr, nullptr, expert_offsets, perm, nullptr, out_slots, (char*)ws, L,
+    return launch_wd_tokens(ctx, 1, x, T, w, nullptr, nullptr, expert_offsets, perm, nullptr, out_slots, (char*)ws, L,
                              s);
   }
   return launch_tensor_ffn(ctx, x, T, w, expert_offsets, perm, (char*)ws, L, out_slots, nullptr, s);
@@ -286,7 +289,7 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   if (rc != MOE_OK) return rc;
   if (path == MOE_PATH_STREAM) {
     if (ctx->cfg.wd_rank == 0) return launch_dense_stream(ctx, 0, x, T, w, idx, wt, nullptr, nullptr, y, nullptr, s);
-    return launch_stream_ffn(ctx, 0, x, T, w, idx, wt, nullptr, nullptr, y, nullptr, wsb, L, s);
+    return launch_wd_tokens(ctx, 0, x, T, w, idx, wt, nullptr, nullptr, y, nullptr, wsb, L, s);
   }
   int32_t* offsets = (int32_t*)(wsb + L.offsets);
   int32_t* perm = (int32_t*)(wsb + L.perm);

@@ -24,19 +24,15 @@ extern thread_local int g_last_cuda_error;
     }                                        \
   } while (0)
 
-// Device-resident state of a ctx: status word written by kernels, grid barrier.
+// Device-resident state of a ctx: status word and arrival counters written by kernels.
 struct DeviceState {
   unsigned int status;  // 0 ok, else moe_status
   unsigned int detail;  // where it happened (kernel-specific code)
   unsigned int pad0[30];
-  unsigned int bar_count;  // arrivals at the current grid barrier (own 128-byte line: it takes the atomics)
-  unsigned int pad1[31];
-  unsigned int bar_gen;  // generation, bumped by the last arriver (own line: it takes the polling)
-  unsigned int pad2[31];
   // dense streaming path: CTAs that have added their partial outputs, over all launches since the state was last
   // cleared (never reset by the kernels: a launch's arrivals are numbered by the remainder modulo its grid size)
   unsigned long long done_total;
-  // weight-decomposed decode kernel: arrivals at its meetings between the products, counted the same way
+  // weight-decomposed decode kernels: arrivals at its meetings between the products, counted the same way
   unsigned long long phase_total;
   // dense streaming kernel, one token: next stage (4 hidden units) of each active expert that no CTA has taken yet;
   // the finalisers leave zeros
@@ -83,7 +79,7 @@ int allow_full_smem(const moe_ctx* ctx) {
 // Offsets (bytes) of the pieces of the caller's scratch buffer.
 struct WsLayout {
   size_t topk_idx, topk_w, offsets, perm, inv;  // routing products when the caller does not ask for them
-  size_t vec_a, vec_b, vec_c;                   // fp32 inter-phase vectors of the streaming path
+  size_t vec_x, vec_a, vec_b, vec_c;            // vectors between the products of the weight-decomposed streaming path
   size_t xperm, hidden, mid_a, mid_b;           // bf16 operands of the tensor path
   size_t out_slots;                             // fp32 [T*k][d]
   size_t total;
@@ -112,7 +108,7 @@ int launch_gather_rows(moe_ctx* ctx, const void* x, const int32_t* perm, int n_s
 bool wd_decode_applies(const moe_config& c, int T);
 int launch_wd_decode(moe_ctx* ctx, const void* x, const moe_weights* w, int32_t* topk_idx, float* topk_w, void* y,
                      float* t, float* h, float* vpart, cudaStream_t s);
-int launch_stream_ffn(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
+int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
                       const float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots,
                       char* ws, const WsLayout& L, cudaStream_t s);
 // Dense experts, streaming path, one kernel (router fused when T == 1 and mode == 0; mode 2 = mode 0 with the
@@ -306,36 +302,6 @@ __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
   unsigned old;
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
   return old;
-}
-
-// Barrier over all CTAs of a co-resident (cooperative) grid.  Thread 0 of each CTA arrives; the
-// wait is bounded.  Returns false (for the whole CTA) when the budget ran out.
-__device__ __forceinline__ bool grid_barrier(DeviceState* st, unsigned n_ctas, int* smem_flag) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    const unsigned gen = ld_acquire(&st->bar_gen);
-    __threadfence();
-    const unsigned old = atom_add_acq_rel(&st->bar_count, 1u);
-    if (old == n_ctas - 1u) {
-      st->bar_count = 0u;
-      __threadfence();
-      st_release(&st->bar_gen, gen + 1u);
-    } else {
-      const long long t0 = clock64();
-      unsigned spins = 0;
-      while (ld_acquire(&st->bar_gen) == gen) {
-        if ((++spins & 255u) == 0u && clock64() - t0 > kWaitBudgetCycles) {
-          ok = 0;
-          break;
-        }
-      }
-    }
-    __threadfence();
-    *smem_flag = ok;
-  }
-  __syncthreads();
-  return *smem_flag != 0;
 }
 
 // ---- bf16 helpers ---------------------------------------------------------------------

@@ -76,6 +76,8 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
   __shared__ float s_logit[kRouteWarps][EMAX];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int t = blockIdx.x * kRouteWarps + wib;
+  pdl_launch_dependents();
+  pdl_wait();
   if (t >= T) return;
   float acc[EMAX];
 #pragma unroll
@@ -166,6 +168,8 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
                        float* __restrict__ topk_w, float* __restrict__ probs) {
   __shared__ float s_part[kRouteWarps][EMAX];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  pdl_launch_dependents();
+  pdl_wait();
   const int t = blockIdx.x;
   float acc[EMAX];
 #pragma unroll
@@ -219,15 +223,9 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
     ctx->launches++;
     return MOE_OK;
   }
-#define ROUTE_CASE(EM)                                                                                              \
-  do {                                                                                                              \
-    if (few)                                                                                                        \
-      route_block_kernel<XT, EM><<<grid, block, 0, s>>>(xp, wr, w->b_router, T, c.d_model, c.n_experts, c.top_k,    \
-                                                        c.renorm, idx, wt, probs);                                  \
-    else                                                                                                            \
-      route_kernel<XT, EM><<<grid, block, 0, s>>>(xp, wr, w->b_router, T, c.d_model, c.n_experts, c.top_k, c.renorm, \
-                                                  idx, wt, probs);                                                  \
-  } while (0)
+#define ROUTE_CASE(EM)                                                                                                \
+  MOE_CUDA_TRY(launch_pdl(few ? route_block_kernel<XT, EM> : route_kernel<XT, EM>, grid, block, 0, s, xp, wr, w->b_router, \
+                          T, c.d_model, c.n_experts, c.top_k, c.renorm, idx, wt, probs))
   if (c.n_experts <= 8)
     ROUTE_CASE(8);
   else if (c.n_experts <= 16)
@@ -237,7 +235,6 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
   else
     ROUTE_CASE(64);
 #undef ROUTE_CASE
-  MOE_CUDA_TRY(cudaGetLastError());
   ctx->launches++;
   return MOE_OK;
 }

@@ -1,0 +1,666 @@
+// Decode of a layer with weight-decomposed experts (Eq. 1) for several tokens (T <= 16), and the per-slot expert FFN
+// of the streaming path: ONE launch that streams every selected expert's factors once and does the arithmetic on
+// the tensor cores.
+//
+//   product 0   t = x [gL | uL]                           rows (j, gate|up) of d values   wd_a [S][r][2][d]
+//   product 1   h_c = silu(t_g . gR_c) * (t_u . uR_c)     pairs of rows of r values       wd_b [S][f][2][r]
+//   product 2   v = h dL                                  rows of f values                wd_c [S][r][f]
+//   product 3   y = sum_a w_a (v_a dR_a)                  rows of r values                wd_d [S][d][r]
+//
+// Every product is a skinny GEMM per active expert: out[slot][row] = W[row][:] . in[slot][:], at most 8 tokens at a
+// time.  It is bound by the bytes of the factors, so the weights go through a ring of shared-memory stages filled
+// with bulk asynchronous copies, and the arithmetic goes to mma.sync m16n8k16 (16 weight rows x 8 tokens): the
+// instruction count does not grow with the tokens of an expert.  (N = 8 tokens is far below a tcgen05 tile; the MMA
+// only has to keep out of the way of the stream.)  The input vectors are kept as THREE bf16 terms whose sum is the
+// fp32 value (8 + 8 + 8 significand bits), each with accumulators of its own, so t, h and v carry fp32 precision as
+// in the one-token kernels; bf16 token rows are one exact term.
+//
+// Rows of (active expert x product) are dealt to the CTAs (one per SM) evenly, row by row; in product 3 the CTAs split
+// the output columns instead, each summing all experts itself, so every value has one writer and a fixed order of
+// summation: no atomics, results bit-identical from call to call.  Between the products the CTAs meet at an arrival
+// counter that runs over launches, with a bounded wait.
+//
+// A CTA's rows of a product are walked in groups of up to 4 tiles of 16 rows; a group goes through the contraction
+// in slices of at most 512 values.  Roles, talking through mbarriers only (all waits bounded):
+//   weight producer warp   a stage = one tile's slice: 16 copies of <= 1 KB, one per lane.  The weights depend on
+//                          nothing but the routing, so it runs ahead across the meetings as far as the ring allows;
+//   vector producer warp   meets the other CTAs, then brings the slices of the input vectors (terms x tokens rows);
+//   8 consumer warps       split a slice's 16-value steps; a step's input fragments stay in registers for all tiles
+//                          of the group; rows in shared memory lie 16 bytes beyond a multiple of 128 apart, so that
+//                          ldmatrix meets no bank conflict;
+//   2 epilogue warps       add the 8 warps' partial sums in order, SiLU * mul, split into terms, store.
+// Measured on B200 (d 1600, f 4352, r 800, T = 5, 8 experts): see the launch function.
+#include "common.cuh"
+
+namespace cosmoe {
+
+namespace {
+
+constexpr int kConsWarps = 8;
+constexpr int kEpiWarp0 = kConsWarps;
+constexpr int kEpiWarps = 2;  // (12 warps in all: three per SM sub-partition, 168 registers each)
+constexpr int kWeightWarp = kEpiWarp0 + kEpiWarps;
+constexpr int kVectorWarp = kWeightWarp + 1;
+constexpr int kThreads = (kVectorWarp + 1) * 32;
+constexpr int kTileRows = 16;
+constexpr int kTok = 8;                          // tokens of one expert per pass (N of the MMA)
+constexpr int kTerms = 3;                        // bf16 terms of an fp32 value
+constexpr int kSlice = 512;                      // contraction values per stage: 4 steps of 16 for each consumer warp
+constexpr int kSteps = kSlice / 16 / kConsWarps;
+constexpr int kRowBytes = kSlice * 2 + 16;       // row distance in shared memory
+constexpr int kStageBytes = kTileRows * kRowBytes;
+constexpr int kStages = 6;                       // 98 KB of weights in flight per SM
+constexpr int kVecBytes = kTerms * kTok * kRowBytes;
+constexpr int kVecSlots = 3;
+constexpr int kGroupTiles = 4;                   // tiles of 16 rows a group holds accumulators for
+constexpr int kPartTok = 20;                     // floats between two tokens' partial sums (16 rows + padding: no bank conflicts)
+constexpr int kPartTile = kTok * kPartTok;
+constexpr int kPartBytes = kGroupTiles * kConsWarps * kPartTile * 4;  // one of two buffers
+constexpr int kMaxSlots = MOE_STREAM_MAX_TOKENS * MOE_MAX_TOPK;
+constexpr int kProducts = 4;
+
+struct Product {
+  const uint16_t* w;          // packed matrix of expert slot 0
+  unsigned long long stride;  // values between expert slots
+  int rows;                   // outputs per expert
+  int K;                      // contraction length
+  int nsub;                   // 2: an output is made from a (gate, up) pair of rows, each with an input vector of its own
+  int n_slices, slice;        // slices of the contraction and their width (a multiple of 16)
+};
+
+struct WtParams {
+  int T, k, E, d, r, f, mode, x_is_bf16, y_rows;
+  const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][3][d]
+  const int32_t* topk_idx;
+  const float* topk_w;
+  const int32_t* offsets;
+  const int32_t* perm;
+  const int32_t* expert_slot;
+  uint16_t *t, *h, *v;  // terms of the intermediates: [slot][2][3][r], [slot][3][f], [slot][3][r]
+  void* y;
+  float* out_slots;
+  DeviceState* st;
+  Product pr[kProducts];
+};
+
+struct WtSmem {
+  uint64_t full[kStages], freeb[kStages];
+  uint64_t vfull[kVecSlots], vfree[kVecSlots];
+  uint64_t pfull[2], pfree[2];
+  uint64_t product_done[kProducts];    // this CTA's outputs of the product are stored (one each: a CTA may have no rows of some)
+  int act_e[MOE_MAX_EXPERTS];
+  int act_slot[MOE_MAX_EXPERTS];       // packed-array slot of the active expert
+  int act_off[MOE_MAX_EXPERTS + 1];    // slot ranges, expert-ascending (same numbering as moe_permute)
+  int slot_tok[kMaxSlots];
+  float slot_w[kMaxSlots];
+  int stage_e[kMaxSlots];              // the routing as read from global memory
+  int cursor[MOE_MAX_EXPERTS];
+  int n_act;
+  volatile int abort;
+};
+constexpr int kHeaderBytes = (sizeof(WtSmem) + 127) / 128 * 128;
+
+struct Ring {
+  int slot;
+  unsigned par;
+  int n;
+  __device__ __forceinline__ void advance(int slots) {
+    ++n;
+    if (++slot == slots) slot = 0, par ^= 1u;
+  }
+};
+
+// One group: rows [row0, row0 + rows) of active expert a for the tokens of its slots slot0 .. slot0 + ns - 1.
+struct Group {
+  int a, slot0, ns, row0, rows;
+  bool last_use;  // no further token group reads these rows
+};
+
+// Every role walks this list of groups: a pure function of (routing, product, CTA).
+template <class F>
+__device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph, F&& body) {
+  const int N = P.pr[ph].rows, na = sm.n_act;
+  const long long b = blockIdx.x, G = gridDim.x;
+  const bool split_out = ph == kProducts - 1;
+  const long long tot = split_out ? N : (long long)na * N;
+  const int g0 = (int)(tot * b / G), g1 = (int)(tot * (b + 1) / G);
+  if (g0 >= g1) return true;
+  const int per = kGroupTiles / P.pr[ph].nsub * kTileRows;
+  for (int a = split_out ? 0 : g0 / N; a < na; ++a) {
+    const int lo = split_out ? g0 : max(g0 - a * N, 0), hi = split_out ? g1 : min(g1 - a * N, N);
+    if (hi <= lo) break;
+    const int groups = (hi - lo + per - 1) / per;
+    const int step = ((hi - lo + groups - 1) / groups + kTileRows - 1) / kTileRows * kTileRows;
+    const int s_lo = sm.act_off[a], s_hi = sm.act_off[a + 1];
+    for (int r0 = lo; r0 < hi; r0 += step)
+      for (int s0 = s_lo; s0 < s_hi; s0 += kTok)
+        if (!body(Group{a, s0, min(kTok, s_hi - s0), r0, min(step, hi - r0), s0 + kTok >= s_hi})) return false;
+  }
+  return true;
+}
+
+__device__ __forceinline__ void give_up(const WtParams& P, WtSmem& sm, unsigned detail) {
+  sm.abort = 1;
+  flag_error(P.st, MOE_ERR_TIMEOUT, detail);
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t* v) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t addr, uint32_t* v) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16(float* c, const uint32_t* a, const uint32_t* b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// fp32 -> three bf16 terms, the largest first: each remainder is exact in fp32
+__device__ __forceinline__ void split3(float v, uint16_t* out) {
+#pragma unroll
+  for (int i = 0; i < kTerms; ++i) {
+    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+    out[i] = __bfloat16_as_ushort(b);
+    v -= __bfloat162float(b);
+  }
+}
+
+// All groups of one product by one consumer warp.  NSUB sub-rows per output, NT terms per input value.
+template <int NSUB, int NT>
+__device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, uint32_t stages, uint32_t vecs, float* parts,
+                                        Ring& rs, Ring& rv, Ring& rp, int warp, int lane) {
+  constexpr int kUnits = kGroupTiles / NSUB;
+  const int K = P.pr[ph].K, slice = P.pr[ph].slice, n_slices = P.pr[ph].n_slices;
+  // ldmatrix lane addresses inside a stage / a vector slot (the token row is clamped per group)
+  const uint32_t a_lane = (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * kRowBytes + (lane >> 4) * 16 + warp * 32;
+  return walk(P, sm, ph, [&](const Group& g) -> bool {
+    float acc[kGroupTiles][4];
+#pragma unroll
+    for (int i = 0; i < kGroupTiles; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+    const int tok = min(lane & 7, g.ns - 1);
+    const uint32_t b_lane4 = (uint32_t)((lane >> 4) * kTok + tok) * kRowBytes + ((lane >> 3) & 1) * 16 + warp * 32;
+    const uint32_t b_lane2 = (uint32_t)(tok)*kRowBytes + ((lane >> 3) & 1) * 16 + warp * 32;
+    const int units = (g.rows + kTileRows - 1) / kTileRows;
+    for (int ks = 0; ks < n_slices; ++ks) {
+      const int width = min(slice, K - ks * slice);
+#pragma unroll
+      for (int sub = 0; sub < NSUB; ++sub) {
+        uint32_t b[kSteps][NT][2];
+        if (!mbar_wait(&sm.vfull[rv.slot], rv.par)) {
+          if (lane == 0) give_up(P, sm, 0x610u);
+          return false;
+        }
+        const uint32_t vec = vecs + (uint32_t)rv.slot * kVecBytes;
+#pragma unroll
+        for (int j = 0; j < kSteps; ++j) {
+          const int k0 = (warp + kConsWarps * j) * 16;
+          if (k0 < width) {
+            if (NT == 1) {
+              ldsm2(vec + b_lane2 + j * (kConsWarps * 32), b[j][0]);
+            } else {
+              uint32_t v4[4];
+              ldsm4(vec + b_lane4 + j * (kConsWarps * 32), v4);
+              b[j][0][0] = v4[0], b[j][0][1] = v4[1], b[j][NT > 1 ? 1 : 0][0] = v4[2], b[j][NT > 1 ? 1 : 0][1] = v4[3];
+              ldsm2(vec + 2 * kTok * kRowBytes + b_lane2 + j * (kConsWarps * 32), b[j][NT - 1]);
+            }
+            if (k0 + 8 >= width) {  // a step of 8 values only: what lies beyond is not part of the row
+#pragma unroll
+              for (int t = 0; t < NT; ++t) b[j][t][1] = 0u;
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.vfree[rv.slot]);
+        rv.advance(kVecSlots);
+#pragma unroll
+        for (int u = 0; u < kUnits; ++u) {
+          if (u < units) {
+            if (!mbar_wait(&sm.full[rs.slot], rs.par)) {
+              if (lane == 0) give_up(P, sm, 0x611u);
+              return false;
+            }
+            const uint32_t st = stages + (uint32_t)rs.slot * kStageBytes + a_lane;
+            // A slice is summed by the MMAs in accumulators of its own, one set per term, and added to the tile's sum in
+            // fp32: at most 4 MMAs deep, because their sums are cut, not rounded (one accumulator over the whole
+            // contraction: 1.2e-6 relative error at K = 4352 against 2.6e-7 of fp32 multiply-adds).
+            float m[NT][4];
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) m[t][q] = 0.f;
+            uint32_t a[kSteps][4];
+#pragma unroll
+            for (int j = 0; j < kSteps; ++j)
+              if ((warp + kConsWarps * j) * 16 < width) ldsm4(st + j * (kConsWarps * 32), a[j]);
+#pragma unroll
+            for (int j = 0; j < kSteps; ++j) {
+              const int k0 = (warp + kConsWarps * j) * 16;
+              if (k0 < width) {
+                if (k0 + 8 >= width) a[j][2] = a[j][3] = 0u;  // (stale bytes there could be NaNs)
+#pragma unroll
+                for (int t = 0; t < NT; ++t) mma16(m[t], a[j], b[j][t]);
+              }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.freeb[rs.slot]);
+            rs.advance(kStages);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              float v = m[NT - 1][q];  // the smallest terms first
+#pragma unroll
+              for (int t = NT - 2; t >= 0; --t) v += m[t][q];
+              acc[u * NSUB + sub][q] += v;
+            }
+          }
+        }
+      }
+    }
+    if (rp.n >= 2 && !mbar_wait(&sm.pfree[rp.slot], rp.par ^ 1u)) {
+      if (lane == 0) give_up(P, sm, 0x612u);
+      return false;
+    }
+    float* part = parts + (size_t)rp.slot * (kPartBytes / 4) + warp * kPartTile;
+#pragma unroll
+    for (int i = 0; i < kGroupTiles; ++i) {
+      if (i < units * NSUB) {
+        const float* s = acc[i];
+        float* dst = part + (size_t)i * kConsWarps * kPartTile + (2 * (lane & 3)) * kPartTok + (lane >> 2);
+        dst[0] = s[0], dst[kPartTok] = s[1], dst[8] = s[2], dst[kPartTok + 8] = s[3];
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sm.pfull[rp.slot]);
+    rp.advance(2);
+    return true;
+  });
+}
+
+__global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_constant__ WtParams P) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  WtSmem& sm = *reinterpret_cast<WtSmem*>(smem_raw);
+  unsigned char* const stages = smem_raw + kHeaderBytes;
+  unsigned char* const vecs = stages + kStages * kStageBytes;
+  float* const parts = reinterpret_cast<float*>(vecs + kVecSlots * kVecBytes);
+  float* const yacc = parts + 2 * (kPartBytes / 4);  // [T][y_rows]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  DeviceState* const st = P.st;
+
+  pdl_launch_dependents();
+  if (tid == kWeightWarp * 32) {
+    for (int i = 0; i < kStages; ++i) mbar_init(&sm.full[i], 1), mbar_init(&sm.freeb[i], kConsWarps);
+    for (int i = 0; i < kVecSlots; ++i) mbar_init(&sm.vfull[i], 1), mbar_init(&sm.vfree[i], kConsWarps);
+    for (int i = 0; i < 2; ++i) mbar_init(&sm.pfull[i], kConsWarps), mbar_init(&sm.pfree[i], kEpiWarps);
+    for (int i = 0; i < kProducts; ++i) mbar_init(&sm.product_done[i], kEpiWarps);
+    fence_mbar_init();
+    fence_proxy_async_smem();
+    sm.abort = 0;
+  }
+  if (P.mode == 0)
+    for (int i = tid; i < P.T * P.y_rows; i += kThreads) yacc[i] = 0.f;
+  pdl_wait();
+
+  // ---------------------------------------------------------------- routing -> active experts and their slots
+  const int n = P.T * P.k;
+  if (warp == 0 && P.mode == 0) {
+    const unsigned below = (1u << lane) - 1u;
+    int bad = 0;
+    sm.cursor[lane] = 0, sm.cursor[lane + 32] = 0;
+    for (int p = lane; p < n; p += 32) sm.stage_e[p] = P.topk_idx[p];
+    __syncwarp();
+    for (int p0 = 0; p0 < n; p0 += 32) {  // counts: the first lane of each group of equal experts adds the group
+      const int p = p0 + lane;
+      int e = p < n ? sm.stage_e[p] : -1;
+      if (p < n && (e < 0 || e >= P.E)) bad = 1, e = -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, e);
+      if (e >= 0 && (peers & below) == 0u) sm.cursor[e] += __popc(peers);
+      __syncwarp();
+    }
+    const int c[2] = {sm.cursor[lane], sm.cursor[lane + 32]};
+    int run = 0, na = 0;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      int s = c[half];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += u;
+      }
+      const int off = run + s - c[half], e = lane + 32 * half;
+      run += __shfl_sync(0xffffffffu, s, 31);
+      const unsigned m = __ballot_sync(0xffffffffu, c[half] > 0);
+      sm.cursor[e] = off;  // next free slot of every expert
+      if (c[half] > 0) {
+        const int a = na + __popc(m & below);
+        const int sl = P.expert_slot ? P.expert_slot[e] : e;
+        bad |= sl < 0;
+        sm.act_e[a] = e, sm.act_off[a] = off, sm.act_slot[a] = sl < 0 ? 0 : sl;
+      }
+      na += __popc(m);
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    __syncwarp();
+    for (int p0 = 0; p0 < n && !bad; p0 += 32) {
+      const int p = p0 + lane;
+      const int e = p < n ? sm.stage_e[p] : -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, e);
+      const int base = e >= 0 ? sm.cursor[e] : 0;
+      __syncwarp();
+      if (e >= 0) {
+        const int s = base + __popc(peers & below);  // pairs of one expert keep their order
+        sm.slot_tok[s] = p / P.k;
+        sm.slot_w[s] = P.topk_w[p];
+        if ((peers & below) == 0u) sm.cursor[e] = base + __popc(peers);
+      }
+      __syncwarp();
+    }
+    if (lane == 0) {
+      sm.act_off[bad ? 0 : na] = bad ? 0 : n;
+      sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: nobody streams anything
+      if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
+    }
+  } else if (tid == 0) {
+    // the caller's grouping (moe_permute's products)
+    int na = 0, bad = 0;
+    sm.act_off[0] = 0;
+    for (int e = 0; e < P.E && !bad; ++e) {
+      const int lo = P.offsets[e], hi = P.offsets[e + 1];
+      if (lo < 0 || hi < lo || hi > n || (hi > lo && lo != sm.act_off[na])) {
+        bad = 1;
+        break;
+      }
+      if (hi == lo) continue;
+      for (int s = lo; s < hi; ++s) {
+        const int p = P.perm[s];
+        if (p < 0 || p >= n) {
+          bad = 1;
+          break;
+        }
+        sm.slot_tok[s] = p / P.k;
+        sm.slot_w[s] = 1.0f;
+      }
+      const int sl = P.expert_slot ? P.expert_slot[e] : e;
+      bad |= sl < 0;
+      sm.act_e[na] = e, sm.act_slot[na] = sl < 0 ? 0 : sl;
+      sm.act_off[++na] = hi;
+    }
+    if (!bad && sm.act_off[na] != n) bad = 1;
+    if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
+    sm.n_act = bad ? 0 : na;
+  }
+  __syncthreads();
+  // From here on the roles meet at mbarriers only; every wait is bounded.
+  const int last = sm.n_act > 0 ? kProducts : 0;  // (nothing to do: no products, no meetings, zeros out)
+
+  if (warp == kWeightWarp) {
+    // ================================================================= weight producer
+    const uint64_t once = l2_policy_evict_first();
+    Ring rs{0, 0u, 0};
+    bool ok = true;
+    for (int ph = 0; ph < last && ok; ++ph) {
+      const Product& pr = P.pr[ph];
+      const int K = pr.K, nsub = pr.nsub;
+      ok = walk(P, sm, ph, [&](const Group& g) -> bool {
+        const uint16_t* base = pr.w + (size_t)sm.act_slot[g.a] * pr.stride + (size_t)g.row0 * nsub * K;
+        for (int ks = 0; ks < pr.n_slices; ++ks) {
+          const int k0 = ks * pr.slice;
+          const uint32_t bytes = (uint32_t)min(pr.slice, K - k0) * 2u;
+          for (int sub = 0; sub < nsub; ++sub)
+            for (int u = 0; u < g.rows; u += kTileRows) {
+              const int rows = min(kTileRows, g.rows - u);
+              if (!__all_sync(0xffffffffu, (rs.n < kStages || mbar_wait(&sm.freeb[rs.slot], rs.par ^ 1u)) && !sm.abort)) {
+                if (lane == 0) give_up(P, sm, 0x620u);
+                return false;
+              }
+              fence_proxy_async_smem();
+              if (lane == 0) mbar_arrive_expect_tx(&sm.full[rs.slot], bytes * (uint32_t)rows);
+              __syncwarp();
+              if (lane < rows) {
+                const void* src = base + ((size_t)(u + lane) * nsub + sub) * K + k0;
+                unsigned char* dst = stages + (size_t)rs.slot * kStageBytes + lane * kRowBytes;
+                if (g.last_use)
+                  bulk_g2s_hint(dst, src, bytes, &sm.full[rs.slot], once);
+                else
+                  bulk_g2s(dst, src, bytes, &sm.full[rs.slot]);
+              }
+              rs.advance(kStages);
+            }
+        }
+        return true;
+      });
+    }
+    if (!ok)  // copies in flight must land before this CTA's shared memory goes away
+      for (int j = max(0, rs.n - kStages); j < rs.n; ++j) (void)mbar_wait(&sm.full[j % kStages], (unsigned)(j / kStages) & 1u);
+    return;
+  }
+
+  if (warp == kVectorWarp) {
+    // ================================================================= vector producer, meetings
+    Ring rv{0, 0u, 0};
+    bool ok = true;
+    for (int ph = 0; ph < last && ok; ++ph) {
+      if (ph > 0) {  // every CTA has stored its outputs of the product before
+        int met = 1;
+        if (lane == 0) {
+          met = mbar_wait(&sm.product_done[ph - 1], 0u);
+          if (met) {
+            // (release: the epilogue warps' stores, ordered before this thread by the barrier; acquire: the others')
+            const unsigned G = gridDim.x;
+            const unsigned long long old = atom_add_acq_rel64(&st->phase_total, 1ull);
+            const unsigned long long target = old - old % G + G;
+            const long long t0 = clock64();
+            while (ld_acquire64(&st->phase_total) < target)
+              if (clock64() - t0 > kWaitBudgetCycles || sm.abort) {
+                met = 0;
+                break;
+              }
+          }
+          if (!met) give_up(P, sm, 0x630u);
+        }
+        ok = __shfl_sync(0xffffffffu, met, 0) != 0;
+        if (!ok) break;
+        fence_proxy_async_all();  // the vectors were stored through the generic proxy, the copies below read them
+      }
+      const Product& pr = P.pr[ph];
+      const int K = pr.K, nt = ph == 0 && P.x_is_bf16 ? 1 : kTerms;
+      ok = walk(P, sm, ph, [&](const Group& g) -> bool {
+        // lane = (term, token): the row it brings
+        const int term = lane >> 3, tok = lane & 7;
+        const bool mine = term < nt && tok < g.ns;
+        const int s = g.slot0 + min(tok, g.ns - 1);
+        const uint16_t* row;
+        size_t sub_stride = 0;
+        if (ph == 0)
+          row = P.x + ((size_t)sm.slot_tok[s] * nt + term) * K;
+        else if (ph == 1)
+          row = P.t + ((size_t)s * 2 * kTerms + term) * K, sub_stride = (size_t)kTerms * K;
+        else
+          row = (ph == 2 ? P.h : P.v) + ((size_t)s * kTerms + term) * K;
+        for (int ks = 0; ks < pr.n_slices; ++ks) {
+          const int k0 = ks * pr.slice;
+          const uint32_t bytes = (uint32_t)min(pr.slice, K - k0) * 2u;
+          for (int sub = 0; sub < pr.nsub; ++sub) {
+            if (!__all_sync(0xffffffffu, (rv.n < kVecSlots || mbar_wait(&sm.vfree[rv.slot], rv.par ^ 1u)) && !sm.abort)) {
+              if (lane == 0) give_up(P, sm, 0x631u);
+              return false;
+            }
+            fence_proxy_async_smem();
+            if (lane == 0) mbar_arrive_expect_tx(&sm.vfull[rv.slot], bytes * (uint32_t)(nt * g.ns));
+            __syncwarp();
+            if (mine)
+              bulk_g2s(vecs + (size_t)rv.slot * kVecBytes + (size_t)(term * kTok + tok) * kRowBytes, row + sub * sub_stride + k0,
+                       bytes, &sm.vfull[rv.slot]);
+            rv.advance(kVecSlots);
+          }
+        }
+        return true;
+      });
+    }
+    if (!ok)
+      for (int j = max(0, rv.n - kVecSlots); j < rv.n; ++j)
+        (void)mbar_wait(&sm.vfull[j % kVecSlots], (unsigned)(j / kVecSlots) & 1u);
+    return;
+  }
+
+  if (warp >= kEpiWarp0) {
+    // ================================================================= epilogue
+    // Warp ew takes rows 8 ew .. 8 ew + 7 of every tile (four at a time) for all 8 tokens: in product 3 all experts'
+    // contributions to an output meet in one warp, in expert order.
+    const int rq0 = 8 * (warp - kEpiWarp0) + (lane & 3), tok = lane >> 2;
+    const int y0 = (int)((long long)P.d * blockIdx.x / gridDim.x);
+    Ring rp{0, 0u, 0};
+    bool ok = true;
+    for (int ph = 0; ph < last && ok; ++ph) {
+      const Product& pr = P.pr[ph];
+      ok = walk(P, sm, ph, [&](const Group& g) -> bool {
+        if (!mbar_wait(&sm.pfull[rp.slot], rp.par)) {
+          if (lane == 0) give_up(P, sm, 0x640u);
+          return false;
+        }
+        const int s = g.slot0 + tok;
+        for (int q = 0; (q >> 1) * kTileRows < g.rows; ++q) {
+          const int u = q >> 1, rq = rq0 + 4 * (q & 1);
+          const float* part = parts + (size_t)rp.slot * (kPartBytes / 4) + tok * kPartTok + rq;
+          auto total = [&](int tile) {
+            const float* p = part + (size_t)tile * kConsWarps * kPartTile;
+            float v = 0.f;
+#pragma unroll
+            for (int w = 0; w < kConsWarps; ++w) v += p[w * kPartTile];
+            return v;
+          };
+          const int rl = u * kTileRows + rq, row = g.row0 + rl;
+          float v;
+          if (pr.nsub == 2) {
+            const float gt = total(2 * u), up = total(2 * u + 1);
+            v = gt / (1.0f + expf(-gt)) * up;
+          } else {
+            v = total(u);
+          }
+          if (rl >= g.rows || tok >= g.ns) continue;
+          if (ph == kProducts - 1) {
+            if (P.mode == 1)
+              P.out_slots[(size_t)s * P.d + row] = v;
+            else
+              yacc[sm.slot_tok[s] * P.y_rows + (row - y0)] += sm.slot_w[s] * v;
+          } else {
+            uint16_t tm[kTerms];
+            split3(v, tm);
+            const int K = ph == 1 ? P.f : P.r;
+            uint16_t* dst = ph == 0 ? P.t + ((size_t)(s * 2 + (row & 1)) * kTerms) * K + (row >> 1)
+                                    : (ph == 1 ? P.h : P.v) + (size_t)s * kTerms * K + row;
+#pragma unroll
+            for (int i = 0; i < kTerms; ++i) dst[(size_t)i * K] = tm[i];
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.pfree[rp.slot]);
+        rp.advance(2);
+        return true;
+      });
+      ok = __all_sync(0xffffffffu, ok);
+      __syncwarp();
+      if (ok && lane == 0) mbar_arrive(&sm.product_done[ph]);
+    }
+    if (ok && P.mode == 0) {
+      const int y1 = (int)((long long)P.d * (blockIdx.x + 1) / gridDim.x);
+      for (int q = 0; (q >> 1) * kTileRows < y1 - y0; ++q)
+        for (int t = tok; t < P.T; t += kTok) {
+          const int rl = (q >> 1) * kTileRows + rq0 + 4 * (q & 1);
+          if (rl >= y1 - y0) continue;
+          const float v = yacc[t * P.y_rows + rl];
+          if (P.x_is_bf16)
+            ((__nv_bfloat16*)P.y)[(size_t)t * P.d + y0 + rl] = __float2bfloat16_rn(v);
+          else
+            ((float*)P.y)[(size_t)t * P.d + y0 + rl] = v;
+        }
+    }
+    return;
+  }
+
+  // ===================================================================== consumers
+  Ring rs{0, 0u, 0}, rv{0, 0u, 0}, rp{0, 0u, 0};
+  const uint32_t sa = smem_u32(stages), va = smem_u32(vecs);
+  bool ok = true;
+  for (int ph = 0; ph < last && ok; ++ph) {
+    if (ph == 0 && P.x_is_bf16)
+      ok = consume<1, 1>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
+    else if (ph == 1)
+      ok = consume<2, kTerms>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
+    else
+      ok = consume<1, kTerms>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
+  }
+}
+
+// fp32 token rows -> their bf16 terms [T][3][d]
+__global__ void split_rows_kernel(const float* __restrict__ x, int d, uint16_t* __restrict__ out) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const float* row = x + (size_t)blockIdx.x * d;
+  uint16_t* dst = out + (size_t)blockIdx.x * kTerms * d;
+  for (int i = threadIdx.x; i < d; i += blockDim.x) {
+    uint16_t tm[kTerms];
+    split3(row[i], tm);
+#pragma unroll
+    for (int j = 0; j < kTerms; ++j) dst[(size_t)j * d + i] = tm[j];
+  }
+}
+
+}  // namespace
+
+int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
+                     const float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots, char* ws,
+                     const WsLayout& L, cudaStream_t s) {
+  const moe_config& c = ctx->cfg;
+  if (c.wd_rank == 0) return MOE_ERR_UNSUPPORTED;  // dense experts stream through launch_dense_stream
+  const int d = c.d_model, f = c.d_ff, r = c.wd_rank, G = ctx->sm_count;
+  WtParams P{};
+  P.T = T, P.k = c.top_k, P.E = c.n_experts, P.d = d, P.r = r, P.f = f, P.mode = mode;
+  P.x_is_bf16 = c.x_dtype == MOE_BF16;
+  P.topk_idx = topk_idx, P.topk_w = topk_w, P.offsets = offsets, P.perm = perm, P.expert_slot = w->expert_slot;
+  P.t = (uint16_t*)(ws + L.vec_a), P.h = (uint16_t*)(ws + L.vec_b), P.v = (uint16_t*)(ws + L.vec_c);
+  P.y = y, P.out_slots = out_slots, P.st = ctx->d_state;
+  P.y_rows = (d + G - 1) / G + 1;
+  auto set = [&](int i, const void* mat, int rows, int K, int nsub) {
+    Product& p = P.pr[i];
+    p.w = (const uint16_t*)mat, p.rows = rows, p.K = K, p.nsub = nsub;
+    p.stride = (unsigned long long)rows * nsub * K;
+    p.n_slices = (K + kSlice - 1) / kSlice;
+    p.slice = ((K + p.n_slices - 1) / p.n_slices + 15) / 16 * 16;  // equal slices, whole steps of the MMA
+  };
+  set(0, w->wd_a, 2 * r, d, 1);
+  set(1, w->wd_b, f, r, 2);
+  set(2, w->wd_c, r, f, 1);
+  set(3, w->wd_d, d, r, 1);
+  const size_t smem = kHeaderBytes + (size_t)kStages * kStageBytes + (size_t)kVecSlots * kVecBytes + 2 * (size_t)kPartBytes +
+                      (mode == 0 ? (size_t)T * P.y_rows * 4 : 0);
+  if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
+  if (P.x_is_bf16) {
+    P.x = (const uint16_t*)x;
+  } else {
+    uint16_t* terms = (uint16_t*)(ws + L.vec_x);
+    MOE_CUDA_TRY(launch_pdl(split_rows_kernel, dim3(T), dim3(256), 0, s, (const float*)x, d, terms));
+    ctx->launches++;
+    P.x = terms;
+  }
+  MOE_TRY(allow_full_smem<wd_tokens_kernel>(ctx));
+  // The CTAs wait for one another, so the launch is cooperative: it starts only when all of them fit on the device.
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(G), lc.blockDim = dim3(kThreads), lc.dynamicSmemBytes = smem, lc.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr, lc.numAttrs = 2;
+  MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, wd_tokens_kernel, P));
+  ctx->launches++;
+  return MOE_OK;
+}
+
+}  // namespace cosmoe
