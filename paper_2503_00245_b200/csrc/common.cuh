@@ -1,6 +1,7 @@
 // Shared host/device helpers for the MoE layer kernels (sm_100a only).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -130,6 +131,10 @@ int launch_dense_stream(moe_ctx* ctx, int mode, const void* x, int T, const moe_
                         cudaStream_t s, const DenseExtra* ex = nullptr);
 // FP8 E4M3 codes with one fp32 scale per row of n values -> bf16 (csrc/fp8_store.cu).
 int launch_fp8_dequant(const void* codes, const float* scales, long long rows, int n, void* w, cudaStream_t s);
+// Tensor map over an interleaved matrix [slots][rows][nsub][inner] of bf16: coordinates (inner, sub-row, row, slot), boxes
+// of box_inner x box_rows of one sub-row, rows box_inner values apart in shared memory (csrc/tensor_ffn.cu).
+int make_map_rows(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
+                  int box_rows);
 // Tensor-core (prefill) path: out_slots from x gathered by perm.
 int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, const int32_t* offsets,
                       const int32_t* perm, char* ws, const WsLayout& L, float* out_slots, int* out_planes,

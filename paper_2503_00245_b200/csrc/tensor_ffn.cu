@@ -524,7 +524,7 @@ int make_map_a(CUtensorMap* m, const void* base, long long rows, long long cols,
 }
 // rank-4 map over an interleaved matrix [S][rows][nsub][inner]: coordinates (inner, sub, row, slot)
 int make_map_b(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
-               int box_rows) {
+               int box_rows, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return MOE_ERR_CUDA;
   const cuuint64_t dims[4] = {(cuuint64_t)inner, (cuuint64_t)nsub, (cuuint64_t)rows, (cuuint64_t)slots};
@@ -533,7 +533,7 @@ int make_map_b(CUtensorMap* m, const void* base, long long inner, int nsub, long
   const cuuint32_t box[4] = {(cuuint32_t)box_inner, 1, (cuuint32_t)box_rows, 1};
   const cuuint32_t es[4] = {1, 1, 1, 1};
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
@@ -601,6 +601,11 @@ int pick_bn(int n_total, int cap, int floor_bn = 64) {
 }
 
 }  // namespace
+
+int make_map_rows(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
+                  int box_rows) {
+  return make_map_b(m, base, inner, nsub, rows, slots, box_inner, box_rows, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
 
 int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, const int32_t* offsets,
                       const int32_t* perm, char* ws, const WsLayout& L, float* out_slots, int* out_planes,

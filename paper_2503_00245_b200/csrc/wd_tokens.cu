@@ -22,14 +22,19 @@
 //
 // A CTA's rows of a product are walked in groups of up to 4 tiles of 16 rows; a group goes through the contraction
 // in slices of at most 512 values.  Roles, talking through mbarriers only (all waits bounded):
-//   weight producer warp   a stage = one tile's slice: 16 copies of <= 1 KB, one per lane.  The weights depend on
-//                          nothing but the routing, so it runs ahead across the meetings as far as the ring allows;
-//   vector producer warp   meets the other CTAs, then brings the slices of the input vectors (terms x tokens rows);
-//   8 consumer warps       split a slice's 16-value steps; a step's input fragments stay in registers for all tiles
-//                          of the group; rows in shared memory lie 16 bytes beyond a multiple of 128 apart, so that
-//                          ldmatrix meets no bank conflict;
+//   weight producer thread a stage = one tile's slice, in at most 4 tiled TMA loads of 8 rows x 256 values (a copy per
+//                          row costs its issuing thread 110 cycles per KB: 126 us per layer instead of FIXME).  The
+//                          weights depend on nothing but the routing, so it runs ahead across the meetings as far as
+//                          the ring allows;
+//   vector producer warp   meets the other CTAs, then brings the slices of the input vectors, one copy per token;
+//   8 consumer warps       split a slice's 32-value units; a unit's input fragments stay in registers for all tiles
+//                          of the group.  A lane fetches 8 consecutive values of a row at a time (16 bytes) and the two
+//                          MMA steps of a unit take them in that order, weights and vectors alike: the order of the
+//                          contraction inside a unit is free;
 //   2 epilogue warps       add the 8 warps' partial sums in order, SiLU * mul, split into terms, store.
 // Measured on B200 (d 1600, f 4352, r 800, T = 5, 8 experts): see the launch function.
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace cosmoe {
@@ -45,12 +50,16 @@ constexpr int kThreads = (kVectorWarp + 1) * 32;
 constexpr int kTileRows = 16;
 constexpr int kTok = 8;                          // tokens of one expert per pass (N of the MMA)
 constexpr int kTerms = 3;                        // bf16 terms of an fp32 value
-constexpr int kSlice = 512;                      // contraction values per stage: 4 steps of 16 for each consumer warp
-constexpr int kSteps = kSlice / 16 / kConsWarps;
-constexpr int kRowBytes = kSlice * 2 + 16;       // row distance in shared memory
-constexpr int kStageBytes = kTileRows * kRowBytes;
-constexpr int kStages = 6;                       // 98 KB of weights in flight per SM
-constexpr int kVecBytes = kTerms * kTok * kRowBytes;
+constexpr int kSlice = 512;                      // contraction values per stage: 2 units of 32 for each consumer warp
+constexpr int kUnit = 32;                        // contraction values of two MMA steps
+constexpr int kUnits = kSlice / kUnit / kConsWarps;
+constexpr int kBoxK = 256, kBoxRows = 8;         // one TMA load
+constexpr int kBoxBytes = kBoxK * kBoxRows * 2;
+constexpr int kStageBytes = kTileRows * kSlice * 2;  // [column half][row half][8 rows][256 values]
+constexpr int kStages = 6;                       // 96 KB of weights in flight per SM
+constexpr int kVecRun = kTerms * kSlice;         // values of one token's slice in memory: [term][512]
+constexpr int kTokBytes = kVecRun * 2 + 64;      // distance in shared memory (64 bytes: no bank conflict between two tokens)
+constexpr int kVecBytes = kTok * kTokBytes;
 constexpr int kVecSlots = 3;
 constexpr int kGroupTiles = 4;                   // tiles of 16 rows a group holds accumulators for
 constexpr int kPartTok = 20;                     // floats between two tokens' partial sums (16 rows + padding: no bank conflicts)
@@ -60,27 +69,28 @@ constexpr int kMaxSlots = MOE_STREAM_MAX_TOKENS * MOE_MAX_TOPK;
 constexpr int kProducts = 4;
 
 struct Product {
-  const uint16_t* w;          // packed matrix of expert slot 0
-  unsigned long long stride;  // values between expert slots
-  int rows;                   // outputs per expert
-  int K;                      // contraction length
-  int nsub;                   // 2: an output is made from a (gate, up) pair of rows, each with an input vector of its own
-  int n_slices, slice;        // slices of the contraction and their width (a multiple of 16)
+  int rows;      // outputs per expert
+  int K;         // contraction length
+  int nsub;      // 2: an output is made from a (gate, up) pair of rows, each with an input vector of its own
+  int n_slices;  // slices of the contraction
 };
 
 struct WtParams {
-  int T, k, E, d, r, f, mode, x_is_bf16, y_rows;
-  const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][3][d]
+  int T, k, E, d, mode, x_is_bf16, y_rows;
+  const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][slice][3][512]
   const int32_t* topk_idx;
   const float* topk_w;
   const int32_t* offsets;
   const int32_t* perm;
   const int32_t* expert_slot;
-  uint16_t *t, *h, *v;  // terms of the intermediates: [slot][2][3][r], [slot][3][f], [slot][3][r]
+  uint16_t *t, *h, *v;  // terms of the intermediates: [slot][2][slice][3][512], [slot][slice][3][512] twice
   void* y;
   float* out_slots;
   DeviceState* st;
   Product pr[kProducts];
+};
+struct WtMaps {
+  CUtensorMap m[kProducts];  // [slot][row][sub-row][value] of every product's matrix, boxes of 8 rows x 256 values
 };
 
 struct WtSmem {
@@ -144,20 +154,31 @@ __device__ __forceinline__ void give_up(const WtParams& P, WtSmem& sm, unsigned 
   flag_error(P.st, MOE_ERR_TIMEOUT, detail);
 }
 
-__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t* v) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(addr)
-               : "memory");
+__device__ __forceinline__ void tma_rows(void* dst, const CUtensorMap* map, int k, int sub, int row, int slot, uint64_t* bar,
+                                         uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, "
+      "%4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
+      "l"(map), "r"(k), "r"(sub), "r"(row), "r"(slot), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
 }
-__device__ __forceinline__ void ldsm2(uint32_t addr, uint32_t* v) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr) : "memory");
+__device__ __forceinline__ uint64_t l2_policy_normal() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
 }
-__device__ __forceinline__ void mma16(float* c, const uint32_t* a, const uint32_t* b) {
+__device__ __forceinline__ uint4 lds16(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  return v;
+}
+// 16 rows x 16 values times 16 values x 8 tokens; a row's (a token's) two registers hold 4 of its values per lane
+__device__ __forceinline__ void mma16(float* c, uint32_t a_lo0, uint32_t a_hi0, uint32_t a_lo1, uint32_t a_hi1, uint32_t b0,
+                                      uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+      : "r"(a_lo0), "r"(a_hi0), "r"(a_lo1), "r"(a_hi1), "r"(b0), "r"(b1));
 }
 
 // fp32 -> three bf16 terms, the largest first: each remainder is exact in fp32
@@ -174,54 +195,43 @@ __device__ __forceinline__ void split3(float v, uint16_t* out) {
 template <int NSUB, int NT>
 __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, uint32_t stages, uint32_t vecs, float* parts,
                                         Ring& rs, Ring& rv, Ring& rp, int warp, int lane) {
-  constexpr int kUnits = kGroupTiles / NSUB;
-  const int K = P.pr[ph].K, slice = P.pr[ph].slice, n_slices = P.pr[ph].n_slices;
-  // ldmatrix lane addresses inside a stage / a vector slot (the token row is clamped per group)
-  const uint32_t a_lane = (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * kRowBytes + (lane >> 4) * 16 + warp * 32;
+  constexpr int kTilesPerSub = kGroupTiles / NSUB;
+  const int K = P.pr[ph].K, n_slices = P.pr[ph].n_slices;
+  // lane (g, q) = (lane / 4, lane % 4) fetches values 8 q .. 8 q + 7 of a unit, of rows g and g + 8 / of token g; this
+  // warp's units are number `warp` of either column half of the slice
+  const uint32_t a_lane = (uint32_t)(lane >> 2) * (kBoxK * 2) + (lane & 3) * 16 + warp * (kUnit * 2);
+  const int col = warp * kUnit + (lane & 3) * 8;
   return walk(P, sm, ph, [&](const Group& g) -> bool {
     float acc[kGroupTiles][4];
 #pragma unroll
     for (int i = 0; i < kGroupTiles; ++i)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
-    const int tok = min(lane & 7, g.ns - 1);
-    const uint32_t b_lane4 = (uint32_t)((lane >> 4) * kTok + tok) * kRowBytes + ((lane >> 3) & 1) * 16 + warp * 32;
-    const uint32_t b_lane2 = (uint32_t)(tok)*kRowBytes + ((lane >> 3) & 1) * 16 + warp * 32;
-    const int units = (g.rows + kTileRows - 1) / kTileRows;
+    const uint32_t b_lane = (uint32_t)min(lane >> 2, g.ns - 1) * kTokBytes + col * 2;
+    const int tiles = (g.rows + kTileRows - 1) / kTileRows;
     for (int ks = 0; ks < n_slices; ++ks) {
-      const int width = min(slice, K - ks * slice);
+      const int width = min(kSlice, K - ks * kSlice);
 #pragma unroll
       for (int sub = 0; sub < NSUB; ++sub) {
-        uint32_t b[kSteps][NT][2];
+        uint4 b[kUnits][NT];
         if (!mbar_wait(&sm.vfull[rv.slot], rv.par)) {
           if (lane == 0) give_up(P, sm, 0x610u);
           return false;
         }
-        const uint32_t vec = vecs + (uint32_t)rv.slot * kVecBytes;
+        const uint32_t vec = vecs + (uint32_t)rv.slot * kVecBytes + b_lane;
 #pragma unroll
-        for (int j = 0; j < kSteps; ++j) {
-          const int k0 = (warp + kConsWarps * j) * 16;
-          if (k0 < width) {
-            if (NT == 1) {
-              ldsm2(vec + b_lane2 + j * (kConsWarps * 32), b[j][0]);
-            } else {
-              uint32_t v4[4];
-              ldsm4(vec + b_lane4 + j * (kConsWarps * 32), v4);
-              b[j][0][0] = v4[0], b[j][0][1] = v4[1], b[j][NT > 1 ? 1 : 0][0] = v4[2], b[j][NT > 1 ? 1 : 0][1] = v4[3];
-              ldsm2(vec + 2 * kTok * kRowBytes + b_lane2 + j * (kConsWarps * 32), b[j][NT - 1]);
-            }
-            if (k0 + 8 >= width) {  // a step of 8 values only: what lies beyond is not part of the row
+        for (int j = 0; j < kUnits; ++j)
 #pragma unroll
-              for (int t = 0; t < NT; ++t) b[j][t][1] = 0u;
-            }
+          for (int t = 0; t < NT; ++t) {
+            b[j][t] = lds16(vec + t * (kSlice * 2) + j * (kBoxK * 2));
+            if (col + j * kBoxK >= width) b[j][t] = make_uint4(0u, 0u, 0u, 0u);  // past the vector's end (the weights are zeros there)
           }
-        }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.vfree[rv.slot]);
         rv.advance(kVecSlots);
 #pragma unroll
-        for (int u = 0; u < kUnits; ++u) {
-          if (u < units) {
+        for (int u = 0; u < kTilesPerSub; ++u) {
+          if (u < tiles) {
             if (!mbar_wait(&sm.full[rs.slot], rs.par)) {
               if (lane == 0) give_up(P, sm, 0x611u);
               return false;
@@ -235,19 +245,21 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, u
             for (int t = 0; t < NT; ++t)
 #pragma unroll
               for (int q = 0; q < 4; ++q) m[t][q] = 0.f;
-            uint32_t a[kSteps][4];
+            uint4 lo[kUnits], hi[kUnits];  // rows g and g + 8
 #pragma unroll
-            for (int j = 0; j < kSteps; ++j)
-              if ((warp + kConsWarps * j) * 16 < width) ldsm4(st + j * (kConsWarps * 32), a[j]);
-#pragma unroll
-            for (int j = 0; j < kSteps; ++j) {
-              const int k0 = (warp + kConsWarps * j) * 16;
-              if (k0 < width) {
-                if (k0 + 8 >= width) a[j][2] = a[j][3] = 0u;  // (stale bytes there could be NaNs)
-#pragma unroll
-                for (int t = 0; t < NT; ++t) mma16(m[t], a[j], b[j][t]);
+            for (int j = 0; j < kUnits; ++j)
+              if (warp * kUnit + j * kBoxK < width) {
+                lo[j] = lds16(st + j * (2 * kBoxBytes));
+                hi[j] = lds16(st + j * (2 * kBoxBytes) + kBoxBytes);
               }
-            }
+#pragma unroll
+            for (int j = 0; j < kUnits; ++j)
+              if (warp * kUnit + j * kBoxK < width) {
+#pragma unroll
+                for (int t = 0; t < NT; ++t) mma16(m[t], lo[j].x, hi[j].x, lo[j].y, hi[j].y, b[j][t].x, b[j][t].y);
+#pragma unroll
+                for (int t = 0; t < NT; ++t) mma16(m[t], lo[j].z, hi[j].z, lo[j].w, hi[j].w, b[j][t].z, b[j][t].w);
+              }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.freeb[rs.slot]);
             rs.advance(kStages);
@@ -269,7 +281,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, u
     float* part = parts + (size_t)rp.slot * (kPartBytes / 4) + warp * kPartTile;
 #pragma unroll
     for (int i = 0; i < kGroupTiles; ++i) {
-      if (i < units * NSUB) {
+      if (i < tiles * NSUB) {
         const float* s = acc[i];
         float* dst = part + (size_t)i * kConsWarps * kPartTile + (2 * (lane & 3)) * kPartTok + (lane >> 2);
         dst[0] = s[0], dst[kPartTok] = s[1], dst[8] = s[2], dst[kPartTok + 8] = s[3];
@@ -282,7 +294,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, u
   });
 }
 
-__global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_constant__ WtParams P) {
+__global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_constant__ WtParams P, const __grid_constant__ WtMaps M) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WtSmem& sm = *reinterpret_cast<WtSmem*>(smem_raw);
   unsigned char* const stages = smem_raw + kHeaderBytes;
@@ -294,6 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
 
   pdl_launch_dependents();
   if (tid == kWeightWarp * 32) {
+    for (int i = 0; i < kProducts; ++i) asm volatile("prefetch.tensormap [%0];" ::"l"(&M.m[i]) : "memory");
     for (int i = 0; i < kStages; ++i) mbar_init(&sm.full[i], 1), mbar_init(&sm.freeb[i], kConsWarps);
     for (int i = 0; i < kVecSlots; ++i) mbar_init(&sm.vfull[i], 1), mbar_init(&sm.vfree[i], kConsWarps);
     for (int i = 0; i < 2; ++i) mbar_init(&sm.pfull[i], kConsWarps), mbar_init(&sm.pfree[i], kEpiWarps);
@@ -400,35 +413,34 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
 
   if (warp == kWeightWarp) {
     // ================================================================= weight producer
-    const uint64_t once = l2_policy_evict_first();
+    if (lane != 0) return;
+    const uint64_t once = l2_policy_evict_first(), keep = l2_policy_normal();
     Ring rs{0, 0u, 0};
     bool ok = true;
     for (int ph = 0; ph < last && ok; ++ph) {
       const Product& pr = P.pr[ph];
+      const CUtensorMap* map = &M.m[ph];
       const int K = pr.K, nsub = pr.nsub;
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
-        const uint16_t* base = pr.w + (size_t)sm.act_slot[g.a] * pr.stride + (size_t)g.row0 * nsub * K;
-        for (int ks = 0; ks < pr.n_slices; ++ks) {
-          const int k0 = ks * pr.slice;
-          const uint32_t bytes = (uint32_t)min(pr.slice, K - k0) * 2u;
+        const int e = sm.act_slot[g.a];
+        for (int k0 = 0; k0 < K; k0 += kSlice) {
+          const int halves = K - k0 > kBoxK ? 2 : 1;
           for (int sub = 0; sub < nsub; ++sub)
             for (int u = 0; u < g.rows; u += kTileRows) {
-              const int rows = min(kTileRows, g.rows - u);
-              if (!__all_sync(0xffffffffu, (rs.n < kStages || mbar_wait(&sm.freeb[rs.slot], rs.par ^ 1u)) && !sm.abort)) {
-                if (lane == 0) give_up(P, sm, 0x620u);
+              const int row = g.row0 + u, boxes = g.rows - u > kBoxRows ? 2 : 1;
+              // rows another CTA or another token group reads as well stay in L2
+              const uint64_t pol = g.last_use && g.rows - u >= kTileRows ? once : keep;
+              if ((rs.n >= kStages && !mbar_wait(&sm.freeb[rs.slot], rs.par ^ 1u)) || sm.abort) {
+                give_up(P, sm, 0x620u);
                 return false;
               }
               fence_proxy_async_smem();
-              if (lane == 0) mbar_arrive_expect_tx(&sm.full[rs.slot], bytes * (uint32_t)rows);
-              __syncwarp();
-              if (lane < rows) {
-                const void* src = base + ((size_t)(u + lane) * nsub + sub) * K + k0;
-                unsigned char* dst = stages + (size_t)rs.slot * kStageBytes + lane * kRowBytes;
-                if (g.last_use)
-                  bulk_g2s_hint(dst, src, bytes, &sm.full[rs.slot], once);
-                else
-                  bulk_g2s(dst, src, bytes, &sm.full[rs.slot]);
-              }
+              mbar_arrive_expect_tx(&sm.full[rs.slot], (uint32_t)(halves * boxes * kBoxBytes));
+              unsigned char* dst = stages + (size_t)rs.slot * kStageBytes;
+              for (int hf = 0; hf < halves; ++hf)
+                for (int bx = 0; bx < boxes; ++bx)
+                  tma_rows(dst + hf * (2 * kBoxBytes) + bx * kBoxBytes, map, k0 + hf * kBoxK, sub, row + bx * kBoxRows, e,
+                           &sm.full[rs.slot], pol);
               rs.advance(kStages);
             }
         }
@@ -468,34 +480,30 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
         fence_proxy_async_all();  // the vectors were stored through the generic proxy, the copies below read them
       }
       const Product& pr = P.pr[ph];
-      const int K = pr.K, nt = ph == 0 && P.x_is_bf16 ? 1 : kTerms;
+      const int K = pr.K;
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
-        // lane = (term, token): the row it brings
-        const int term = lane >> 3, tok = lane & 7;
-        const bool mine = term < nt && tok < g.ns;
-        const int s = g.slot0 + min(tok, g.ns - 1);
-        const uint16_t* row;
-        size_t sub_stride = 0;
-        if (ph == 0)
-          row = P.x + ((size_t)sm.slot_tok[s] * nt + term) * K;
-        else if (ph == 1)
-          row = P.t + ((size_t)s * 2 * kTerms + term) * K, sub_stride = (size_t)kTerms * K;
-        else
-          row = (ph == 2 ? P.h : P.v) + ((size_t)s * kTerms + term) * K;
+        // lane = the token whose slices it brings
+        const bool mine = lane < g.ns;
+        const int s = g.slot0 + min(lane, g.ns - 1);
+        const bool plain = ph == 0 && P.x_is_bf16;  // rows of x themselves
+        const size_t run = (size_t)pr.n_slices * kVecRun;
+        const uint16_t* src = plain     ? P.x + (size_t)sm.slot_tok[s] * K
+                              : ph == 0 ? P.x + (size_t)sm.slot_tok[s] * run
+                              : ph == 1 ? P.t + (size_t)s * 2 * run
+                                        : (ph == 2 ? P.h : P.v) + (size_t)s * run;
         for (int ks = 0; ks < pr.n_slices; ++ks) {
-          const int k0 = ks * pr.slice;
-          const uint32_t bytes = (uint32_t)min(pr.slice, K - k0) * 2u;
+          const uint32_t bytes = plain ? (uint32_t)min(kSlice, K - ks * kSlice) * 2u : (uint32_t)kVecRun * 2u;
           for (int sub = 0; sub < pr.nsub; ++sub) {
             if (!__all_sync(0xffffffffu, (rv.n < kVecSlots || mbar_wait(&sm.vfree[rv.slot], rv.par ^ 1u)) && !sm.abort)) {
               if (lane == 0) give_up(P, sm, 0x631u);
               return false;
             }
             fence_proxy_async_smem();
-            if (lane == 0) mbar_arrive_expect_tx(&sm.vfull[rv.slot], bytes * (uint32_t)(nt * g.ns));
+            if (lane == 0) mbar_arrive_expect_tx(&sm.vfull[rv.slot], bytes * (uint32_t)g.ns);
             __syncwarp();
             if (mine)
-              bulk_g2s(vecs + (size_t)rv.slot * kVecBytes + (size_t)(term * kTok + tok) * kRowBytes, row + sub * sub_stride + k0,
-                       bytes, &sm.vfull[rv.slot]);
+              bulk_g2s(vecs + (size_t)rv.slot * kVecBytes + (size_t)lane * kTokBytes,
+                       src + sub * run + (size_t)ks * (plain ? kSlice : kVecRun), bytes, &sm.vfull[rv.slot]);
             rv.advance(kVecSlots);
           }
         }
@@ -551,11 +559,12 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
           } else {
             uint16_t tm[kTerms];
             split3(v, tm);
-            const int K = ph == 1 ? P.f : P.r;
-            uint16_t* dst = ph == 0 ? P.t + ((size_t)(s * 2 + (row & 1)) * kTerms) * K + (row >> 1)
-                                    : (ph == 1 ? P.h : P.v) + (size_t)s * kTerms * K + row;
+            // (product 0's rows are (j, gate | up) pairs)
+            const int c = ph == 0 ? row >> 1 : row, sl = ph == 0 ? 2 * s + (row & 1) : s;
+            uint16_t* dst = (ph == 0 ? P.t : ph == 1 ? P.h : P.v) +
+                            ((size_t)sl * P.pr[ph + 1].n_slices + c / kSlice) * kVecRun + c % kSlice;
 #pragma unroll
-            for (int i = 0; i < kTerms; ++i) dst[(size_t)i * K] = tm[i];
+            for (int i = 0; i < kTerms; ++i) dst[i * kSlice] = tm[i];
           }
         }
         __syncwarp();
@@ -597,17 +606,17 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
   }
 }
 
-// fp32 token rows -> their bf16 terms [T][3][d]
+// fp32 token rows -> their bf16 terms [T][slice][3][512]
 __global__ void split_rows_kernel(const float* __restrict__ x, int d, uint16_t* __restrict__ out) {
   pdl_launch_dependents();
   pdl_wait();
   const float* row = x + (size_t)blockIdx.x * d;
-  uint16_t* dst = out + (size_t)blockIdx.x * kTerms * d;
+  uint16_t* dst = out + (size_t)blockIdx.x * ((d + kSlice - 1) / kSlice) * kVecRun;
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
     uint16_t tm[kTerms];
     split3(row[i], tm);
 #pragma unroll
-    for (int j = 0; j < kTerms; ++j) dst[(size_t)j * d + i] = tm[j];
+    for (int j = 0; j < kTerms; ++j) dst[(size_t)(i / kSlice) * kVecRun + j * kSlice + i % kSlice] = tm[j];
   }
 }
 
@@ -620,23 +629,24 @@ int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_wei
   if (c.wd_rank == 0) return MOE_ERR_UNSUPPORTED;  // dense experts stream through launch_dense_stream
   const int d = c.d_model, f = c.d_ff, r = c.wd_rank, G = ctx->sm_count;
   WtParams P{};
-  P.T = T, P.k = c.top_k, P.E = c.n_experts, P.d = d, P.r = r, P.f = f, P.mode = mode;
+  P.T = T, P.k = c.top_k, P.E = c.n_experts, P.d = d, P.mode = mode;
   P.x_is_bf16 = c.x_dtype == MOE_BF16;
   P.topk_idx = topk_idx, P.topk_w = topk_w, P.offsets = offsets, P.perm = perm, P.expert_slot = w->expert_slot;
   P.t = (uint16_t*)(ws + L.vec_a), P.h = (uint16_t*)(ws + L.vec_b), P.v = (uint16_t*)(ws + L.vec_c);
   P.y = y, P.out_slots = out_slots, P.st = ctx->d_state;
   P.y_rows = (d + G - 1) / G + 1;
+  WtMaps M;
+  int rc = MOE_OK;
   auto set = [&](int i, const void* mat, int rows, int K, int nsub) {
-    Product& p = P.pr[i];
-    p.w = (const uint16_t*)mat, p.rows = rows, p.K = K, p.nsub = nsub;
-    p.stride = (unsigned long long)rows * nsub * K;
-    p.n_slices = (K + kSlice - 1) / kSlice;
-    p.slice = ((K + p.n_slices - 1) / p.n_slices + 15) / 16 * 16;  // equal slices, whole steps of the MMA
+    P.pr[i] = Product{rows, K, nsub, (K + kSlice - 1) / kSlice};
+    // (the slot coordinate never leaves the array: its extent is not needed, only the rows' end inside a slot is)
+    if (rc == MOE_OK) rc = make_map_rows(&M.m[i], mat, K, nsub, rows, MOE_MAX_EXPERTS << 10, kBoxK, kBoxRows);
   };
   set(0, w->wd_a, 2 * r, d, 1);
   set(1, w->wd_b, f, r, 2);
   set(2, w->wd_c, r, f, 1);
   set(3, w->wd_d, d, r, 1);
+  if (rc != MOE_OK) return rc;
   const size_t smem = kHeaderBytes + (size_t)kStages * kStageBytes + (size_t)kVecSlots * kVecBytes + 2 * (size_t)kPartBytes +
                       (mode == 0 ? (size_t)T * P.y_rows * 4 : 0);
   if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
@@ -658,7 +668,7 @@ int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_wei
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr, lc.numAttrs = 2;
-  MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, wd_tokens_kernel, P));
+  MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, wd_tokens_kernel, P, M));
   ctx->launches++;
   return MOE_OK;
 }
