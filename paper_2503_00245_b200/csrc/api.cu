@@ -40,8 +40,9 @@ WsLayout ws_layout(const moe_config& c, int T) {
   const bool tensor_ok = true;
   // one token: fp32 vectors, v in up to 8 segments per value; several: three bf16 terms per value (t is a pair)
   const bool wd_stream = stream_ok && c.wd_rank > 0;
-  const size_t rs = ((size_t)c.wd_rank + 511) / 512 * 512, fs = ((size_t)c.d_ff + 511) / 512 * 512;  // whole slices
-  L.vec_x = take(wd_stream && c.x_dtype == MOE_F32 ? (size_t)T * (((size_t)c.d_model + 511) / 512 * 512) * 6 : 0);
+  const auto whole = [](int v) { return (size_t)(v + kWdSlice - 1) / kWdSlice * kWdTermRun; };
+  const size_t rs = whole(c.wd_rank), fs = whole(c.d_ff);
+  L.vec_x = take(wd_stream && c.x_dtype == MOE_F32 ? (size_t)T * whole(c.d_model) * 6 : 0);
   L.vec_a = take(wd_stream ? n * 2 * rs * 6 : 0);
   L.vec_b = take(wd_stream ? n * fs * 6 : 0);
   L.vec_c = take(wd_stream ? n * std::max(rs * 6, (size_t)c.wd_rank * 8 * 4) : 0);

@@ -109,6 +109,8 @@ int launch_gather_rows(moe_ctx* ctx, const void* x, const int32_t* perm, int n_s
 bool wd_decode_applies(const moe_config& c, int T);
 int launch_wd_decode(moe_ctx* ctx, const void* x, const moe_weights* w, int32_t* topk_idx, float* topk_w, void* y,
                      float* t, float* h, float* vpart, cudaStream_t s);
+constexpr int kWdSlice = 448;    // the vectors between its products are stored in slices of this many values,
+constexpr int kWdTermRun = 480;  // each as three runs (bf16 terms) this far apart
 int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
                       const float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots,
                       char* ws, const WsLayout& L, cudaStream_t s);

@@ -21,9 +21,9 @@
 // counter that runs over launches, with a bounded wait.
 //
 // A CTA's rows of a product are walked in groups of up to 4 tiles of 16 rows; a group goes through the contraction
-// in slices of at most 512 values.  Roles, talking through mbarriers only (all waits bounded):
-//   weight producer thread a stage = one tile's slice, in at most 4 tiled TMA loads of 8 rows x 256 values (a copy per
-//                          row costs its issuing thread 110 cycles per KB: 126 us per layer instead of FIXME).  The
+// in slices of at most 448 values.  Roles, talking through mbarriers only (all waits bounded):
+//   weight producer thread a stage = one tile's slice, in at most two tiled TMA loads of 16 rows x 224 values (one copy
+//                          per row: 100 cycles of the issuing thread per KB, a third of the copy bandwidth).  The
 //                          weights depend on nothing but the routing, so it runs ahead across the meetings as far as
 //                          the ring allows;
 //   vector producer warp   meets the other CTAs, then brings the slices of the input vectors, one copy per token;
@@ -42,6 +42,7 @@ namespace cosmoe {
 namespace {
 
 constexpr int kConsWarps = 8;
+constexpr int kTeams = 2, kTeamWarps = kConsWarps / kTeams;
 constexpr int kEpiWarp0 = kConsWarps;
 constexpr int kEpiWarps = 2;  // (12 warps in all: three per SM sub-partition, 168 registers each)
 constexpr int kWeightWarp = kEpiWarp0 + kEpiWarps;
@@ -50,19 +51,24 @@ constexpr int kThreads = (kVectorWarp + 1) * 32;
 constexpr int kTileRows = 16;
 constexpr int kTok = 8;                          // tokens of one expert per pass (N of the MMA)
 constexpr int kTerms = 3;                        // bf16 terms of an fp32 value
-constexpr int kSlice = 512;                      // contraction values per stage: 2 units of 32 for each consumer warp
 constexpr int kUnit = 32;                        // contraction values of two MMA steps
-constexpr int kUnits = kSlice / kUnit / kConsWarps;
-constexpr int kBoxK = 256, kBoxRows = 8;         // one TMA load
-constexpr int kBoxBytes = kBoxK * kBoxRows * 2;
-constexpr int kStageBytes = kTileRows * kSlice * 2;  // [column half][row half][8 rows][256 values]
-constexpr int kStages = 6;                       // 96 KB of weights in flight per SM
-constexpr int kVecRun = kTerms * kSlice;         // values of one token's slice in memory: [term][512]
-constexpr int kTokBytes = kVecRun * 2 + 64;      // distance in shared memory (64 bytes: no bank conflict between two tokens)
-constexpr int kVecBytes = kTok * kTokBytes;
-constexpr int kVecSlots = 3;
-constexpr int kGroupTiles = 4;                   // tiles of 16 rows a group holds accumulators for
-constexpr int kPartTok = 20;                     // floats between two tokens' partial sums (16 rows + padding: no bank conflicts)
+constexpr int kBoxK = 224;                       // one TMA load: a tile's rows x 7 units.  Not 256: rows 448 bytes apart
+                                                 // let lanes of two neighbouring rows fetch 16 bytes each without a bank
+                                                 // conflict (512 apart: two-way, shared memory was the bottleneck)
+constexpr int kBoxBytes = kBoxK * kTileRows * 2;
+constexpr int kSlice = 2 * kBoxK;                // contraction values per stage
+static_assert(kTeams == 2 && kTeamWarps == 4, "the epilogue adds two teams of four");
+static_assert(kSlice == kWdSlice, "the workspace is laid out in slices");
+constexpr int kStageBytes = 2 * kBoxBytes;       // [column half][16 rows][224 values]
+constexpr int kUnits = (kSlice / kUnit + kTeamWarps - 1) / kTeamWarps;  // units of a stage for each warp of a team
+constexpr int kTermRun = kWdTermRun;             // values between two terms of a slice: 64 bytes beyond a multiple of 128, so
+                                                 // that lanes of two terms meet no bank conflict
+constexpr int kVecRun = kTerms * kTermRun;       // values of one token's slice, in memory as in shared memory
+constexpr int kTokBytes = kVecRun * 2;
+constexpr int kMaxStages = 5;                    // of one team
+constexpr int kMaxVecs = 4;
+constexpr int kGroupTiles = 4;                   // tiles of 16 rows of a group
+constexpr int kPartTok = kTileRows;              // floats between two tokens' partial sums
 constexpr int kPartTile = kTok * kPartTok;
 constexpr int kPartBytes = kGroupTiles * kConsWarps * kPartTile * 4;  // one of two buffers
 constexpr int kMaxSlots = MOE_STREAM_MAX_TOKENS * MOE_MAX_TOPK;
@@ -77,25 +83,27 @@ struct Product {
 
 struct WtParams {
   int T, k, E, d, mode, x_is_bf16, y_rows;
-  const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][slice][3][512]
+  int n_stages;  // of a team's ring
+  const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][slice][3][480]
   const int32_t* topk_idx;
   const float* topk_w;
   const int32_t* offsets;
   const int32_t* perm;
   const int32_t* expert_slot;
-  uint16_t *t, *h, *v;  // terms of the intermediates: [slot][2][slice][3][512], [slot][slice][3][512] twice
+  uint16_t *t, *h, *v;  // terms of the intermediates: [slot][2][slice][3][480], [slot][slice][3][480] twice
   void* y;
   float* out_slots;
   DeviceState* st;
   Product pr[kProducts];
 };
 struct WtMaps {
-  CUtensorMap m[kProducts];  // [slot][row][sub-row][value] of every product's matrix, boxes of 8 rows x 256 values
+  CUtensorMap m[kProducts];  // [slot][row][sub-row][value] of every product's matrix, boxes of 16 rows x 224 values
 };
 
 struct WtSmem {
-  uint64_t full[kStages], freeb[kStages];
-  uint64_t vfull[kVecSlots], vfree[kVecSlots];
+  // Each team has rings of its own: a waiter must see every phase of a barrier it waits on.
+  uint64_t full[kTeams][kMaxStages], freeb[kTeams][kMaxStages];
+  uint64_t vfull[kTeams][kMaxVecs], vfree[kTeams][kMaxVecs];
   uint64_t pfull[2], pfree[2];
   uint64_t product_done[kProducts];    // this CTA's outputs of the product are stored (one each: a CTA may have no rows of some)
   int act_e[MOE_MAX_EXPERTS];
@@ -106,6 +114,7 @@ struct WtSmem {
   int stage_e[kMaxSlots];              // the routing as read from global memory
   int cursor[MOE_MAX_EXPERTS];
   int n_act;
+  int vec_toks, n_vecs;                // token slices of a vector buffer (the most tokens an expert has), buffers of a team
   volatile int abort;
 };
 constexpr int kHeaderBytes = (sizeof(WtSmem) + 127) / 128 * 128;
@@ -135,7 +144,7 @@ __device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph
   const long long tot = split_out ? N : (long long)na * N;
   const int g0 = (int)(tot * b / G), g1 = (int)(tot * (b + 1) / G);
   if (g0 >= g1) return true;
-  const int per = kGroupTiles / P.pr[ph].nsub * kTileRows;
+  constexpr int per = kGroupTiles * kTileRows;
   for (int a = split_out ? 0 : g0 / N; a < na; ++a) {
     const int lo = split_out ? g0 : max(g0 - a * N, 0), hi = split_out ? g1 : min(g1 - a * N, N);
     if (hi <= lo) break;
@@ -167,11 +176,6 @@ __device__ __forceinline__ uint64_t l2_policy_normal() {
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-__device__ __forceinline__ uint4 lds16(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
-}
 // 16 rows x 16 values times 16 values x 8 tokens; a row's (a token's) two registers hold 4 of its values per lane
 __device__ __forceinline__ void mma16(float* c, uint32_t a_lo0, uint32_t a_hi0, uint32_t a_lo1, uint32_t a_hi1, uint32_t b0,
                                       uint32_t b1) {
@@ -191,100 +195,107 @@ __device__ __forceinline__ void split3(float v, uint16_t* out) {
   }
 }
 
-// All groups of one product by one consumer warp.  NSUB sub-rows per output, NT terms per input value.
-template <int NSUB, int NT>
-__device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, uint32_t stages, uint32_t vecs, float* parts,
-                                        Ring& rs, Ring& rv, Ring& rp, int warp, int lane) {
-  constexpr int kTilesPerSub = kGroupTiles / NSUB;
-  const int K = P.pr[ph].K, n_slices = P.pr[ph].n_slices;
-  // lane (g, q) = (lane / 4, lane % 4) fetches values 8 q .. 8 q + 7 of a unit, of rows g and g + 8 / of token g; this
-  // warp's units are number `warp` of either column half of the slice
-  const uint32_t a_lane = (uint32_t)(lane >> 2) * (kBoxK * 2) + (lane & 3) * 16 + warp * (kUnit * 2);
-  const int col = warp * kUnit + (lane & 3) * 8;
+// All groups of one product by one consumer warp.  The loops stay rolled and serve all products (bf16 token rows meet
+// zeros as their second and third term): a launch runs each of them a few dozen times only, and code that is fetched
+// anew from L2 for every tile costs more than the idle columns.
+// The 8 columns of an MMA are two tokens with four columns each, their three terms and a zero: most experts have one or
+// two of the tokens, and one MMA then does what three (one per term) did; the columns of a token are added by its
+// two lanes.
+__device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, const unsigned char* stages,
+                                        const unsigned char* vecs, float* parts, Ring& rs, Ring& rv, unsigned& turn, Ring& rp,
+                                        int warp, int lane) {
+  const int K = P.pr[ph].K, nsub = P.pr[ph].nsub;
+  const int nt = ph == 0 && P.x_is_bf16 ? 1 : kTerms;
+  // The slices of the input vectors are taken by the two teams in turn: a stage is a chain of shared-memory loads, MMAs
+  // and additions, and two of them side by side keep up with the stream.
+  const unsigned team = warp / kTeamWarps;
+  const int tw = warp % kTeamWarps;
+  // lane (g, q) = (lane / 4, lane % 4) fetches values 8 q .. 8 q + 7 of a unit, of rows g and g + 8 / of column g; this
+  // warp's units are tw, tw + 4, tw + 8, tw + 12 (a column half of a stage holds 7)
+  const int g8 = lane >> 2, q4 = lane & 3;
+  const uint32_t a_lane = (uint32_t)g8 * (kBoxK * 2) + q4 * 16;
+  const int term = g8 & 3, col = tw * kUnit + q4 * 8;
+  constexpr int kUnitStep = kTeamWarps * kUnit;
+  const int n_vecs = sm.n_vecs;
   return walk(P, sm, ph, [&](const Group& g) -> bool {
-    float acc[kGroupTiles][4];
-#pragma unroll
-    for (int i = 0; i < kGroupTiles; ++i)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
-    const uint32_t b_lane = (uint32_t)min(lane >> 2, g.ns - 1) * kTokBytes + col * 2;
     const int tiles = (g.rows + kTileRows - 1) / kTileRows;
-    for (int ks = 0; ks < n_slices; ++ks) {
-      const int width = min(kSlice, K - ks * kSlice);
-#pragma unroll
-      for (int sub = 0; sub < NSUB; ++sub) {
-        uint4 b[kUnits][NT];
-        if (!mbar_wait(&sm.vfull[rv.slot], rv.par)) {
-          if (lane == 0) give_up(P, sm, 0x610u);
-          return false;
-        }
-        const uint32_t vec = vecs + (uint32_t)rv.slot * kVecBytes + b_lane;
-#pragma unroll
-        for (int j = 0; j < kUnits; ++j)
-#pragma unroll
-          for (int t = 0; t < NT; ++t) {
-            b[j][t] = lds16(vec + t * (kSlice * 2) + j * (kBoxK * 2));
-            if (col + j * kBoxK >= width) b[j][t] = make_uint4(0u, 0u, 0u, 0u);  // past the vector's end (the weights are zeros there)
-          }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.vfree[rv.slot]);
-        rv.advance(kVecSlots);
-#pragma unroll
-        for (int u = 0; u < kTilesPerSub; ++u) {
-          if (u < tiles) {
-            if (!mbar_wait(&sm.full[rs.slot], rs.par)) {
-              if (lane == 0) give_up(P, sm, 0x611u);
-              return false;
-            }
-            const uint32_t st = stages + (uint32_t)rs.slot * kStageBytes + a_lane;
-            // A slice is summed by the MMAs in accumulators of its own, one set per term, and added to the tile's sum in
-            // fp32: at most 4 MMAs deep, because their sums are cut, not rounded (one accumulator over the whole
-            // contraction: 1.2e-6 relative error at K = 4352 against 2.6e-7 of fp32 multiply-adds).
-            float m[NT][4];
-#pragma unroll
-            for (int t = 0; t < NT; ++t)
-#pragma unroll
-              for (int q = 0; q < 4; ++q) m[t][q] = 0.f;
-            uint4 lo[kUnits], hi[kUnits];  // rows g and g + 8
-#pragma unroll
-            for (int j = 0; j < kUnits; ++j)
-              if (warp * kUnit + j * kBoxK < width) {
-                lo[j] = lds16(st + j * (2 * kBoxBytes));
-                hi[j] = lds16(st + j * (2 * kBoxBytes) + kBoxBytes);
-              }
-#pragma unroll
-            for (int j = 0; j < kUnits; ++j)
-              if (warp * kUnit + j * kBoxK < width) {
-#pragma unroll
-                for (int t = 0; t < NT; ++t) mma16(m[t], lo[j].x, hi[j].x, lo[j].y, hi[j].y, b[j][t].x, b[j][t].y);
-#pragma unroll
-                for (int t = 0; t < NT; ++t) mma16(m[t], lo[j].z, hi[j].z, lo[j].w, hi[j].w, b[j][t].z, b[j][t].w);
-              }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.freeb[rs.slot]);
-            rs.advance(kStages);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float v = m[NT - 1][q];  // the smallest terms first
-#pragma unroll
-              for (int t = NT - 2; t >= 0; --t) v += m[t][q];
-              acc[u * NSUB + sub][q] += v;
-            }
-          }
-        }
-      }
-    }
     if (rp.n >= 2 && !mbar_wait(&sm.pfree[rp.slot], rp.par ^ 1u)) {
       if (lane == 0) give_up(P, sm, 0x612u);
       return false;
     }
-    float* part = parts + (size_t)rp.slot * (kPartBytes / 4) + warp * kPartTile;
+    // this lane's partial sums, [tile][warp][token][row]: row g8 (even lanes) or g8 + 8 of tokens q4 / 2 + 2 p.  A team's
+    // first slice stores, the others add.  Of a (gate, up) pair either team has one; a group with a single slice is
+    // one team's alone.
+    float* const part = parts + (size_t)rp.slot * (kPartBytes / 4) + warp * kPartTile + (q4 >> 1) * kPartTok + g8 + 8 * (q4 & 1);
+    bool first = true;
+#pragma unroll 1
+    for (int k0 = 0; k0 < K; k0 += kSlice) {
+      const int width = min(kSlice, K - k0);
+#pragma unroll 1
+      for (int sub = 0; sub < nsub; ++sub) {
+        if (turn++ % kTeams != team) continue;
+        if (!mbar_wait(&sm.vfull[team][rv.slot], rv.par)) {
+          if (lane == 0) give_up(P, sm, 0x610u);
+          return false;
+        }
+        const unsigned char* vec = vecs + (team * (uint32_t)kTok + (uint32_t)(rv.slot * sm.vec_toks)) * kTokBytes +
+                                   (term < nt ? term : 0) * (kTermRun * 2) + col * 2;
+        // (no branches below: what lies past the vector's end is fetched and dropped, and the weights that would meet it
+        // are those of unit 0, which are finite, or the zeros TMA puts past the end of a row)
+        uint32_t a_off[kUnits];
 #pragma unroll
-    for (int i = 0; i < kGroupTiles; ++i) {
-      if (i < tiles * NSUB) {
-        const float* s = acc[i];
-        float* dst = part + (size_t)i * kConsWarps * kPartTile + (2 * (lane & 3)) * kPartTok + (lane >> 2);
-        dst[0] = s[0], dst[kPartTok] = s[1], dst[8] = s[2], dst[kPartTok + 8] = s[3];
+        for (int j = 0; j < kUnits; ++j) {
+          const uint32_t n = tw + kTeamWarps * j, hf = n >= kBoxK / kUnit;
+          a_off[j] = a_lane + ((int)n * kUnit < width ? hf * kBoxBytes + (n - hf * (kBoxK / kUnit)) * (kUnit * 2) : 0u);
+        }
+#pragma unroll 1
+        for (int u = 0; u < tiles; ++u) {
+          if (!mbar_wait(&sm.full[team][rs.slot], rs.par)) {
+            if (lane == 0) give_up(P, sm, 0x611u);
+            return false;
+          }
+          const unsigned char* st = stages + (team * (uint32_t)P.n_stages + (uint32_t)rs.slot) * kStageBytes;
+          uint4 lo[kUnits], hi[kUnits];  // rows g8 and g8 + 8
+#pragma unroll
+          for (int j = 0; j < kUnits; ++j) {
+            lo[j] = *reinterpret_cast<const uint4*>(st + a_off[j]);
+            hi[j] = *reinterpret_cast<const uint4*>(st + a_off[j] + 8 * kBoxK * 2);
+          }
+          float* dst = part + u * (kConsWarps * kPartTile);
+#pragma unroll 1
+          for (int t0 = 0; t0 < g.ns; t0 += 2) {
+            const unsigned char* vt = vec + (uint32_t)min(t0 + (g8 >> 2), g.ns - 1) * kTokBytes;
+            uint4 b[kUnits];
+#pragma unroll
+            for (int j = 0; j < kUnits; ++j) {
+              b[j] = *reinterpret_cast<const uint4*>(vt + j * (kUnitStep * 2));
+              if (col + j * kUnitStep >= width || term >= nt) b[j] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            // Every unit has accumulators of its own, added up in fp32: the MMA's sums are cut, not rounded (one accumulator
+            // over the whole contraction: 1.2e-6 relative error at K = 4352 against 2.6e-7 of fp32 multiply-adds).
+            float m[kUnits][4];
+#pragma unroll
+            for (int j = 0; j < kUnits; ++j) {
+              m[j][0] = m[j][1] = m[j][2] = m[j][3] = 0.f;
+              mma16(m[j], lo[j].x, hi[j].x, lo[j].y, hi[j].y, b[j].x, b[j].y);
+            }
+#pragma unroll
+            for (int j = 0; j < kUnits; ++j) mma16(m[j], lo[j].z, hi[j].z, lo[j].w, hi[j].w, b[j].z, b[j].w);
+            float top = 0.f, bot = 0.f;  // rows g8 and g8 + 8: this lane's two columns
+#pragma unroll
+            for (int j = 0; j < kUnits; ++j) top += m[j][1] + m[j][0], bot += m[j][3] + m[j][2];
+            const float send = (q4 & 1) ? top : bot, keep = (q4 & 1) ? bot : top;
+            const float v = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+            dst[t0 * kPartTok] = first ? v : dst[t0 * kPartTok] + v;
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.freeb[team][rs.slot]);
+          rs.advance(P.n_stages);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.vfree[team][rv.slot]);
+        rv.advance(n_vecs);
+        first = false;
       }
     }
     __syncwarp();
@@ -298,8 +309,8 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WtSmem& sm = *reinterpret_cast<WtSmem*>(smem_raw);
   unsigned char* const stages = smem_raw + kHeaderBytes;
-  unsigned char* const vecs = stages + kStages * kStageBytes;
-  float* const parts = reinterpret_cast<float*>(vecs + kVecSlots * kVecBytes);
+  unsigned char* const vecs = stages + kTeams * P.n_stages * kStageBytes;
+  float* const parts = reinterpret_cast<float*>(vecs + kTeams * kTok * kTokBytes);
   float* const yacc = parts + 2 * (kPartBytes / 4);  // [T][y_rows]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   DeviceState* const st = P.st;
@@ -307,8 +318,10 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
   pdl_launch_dependents();
   if (tid == kWeightWarp * 32) {
     for (int i = 0; i < kProducts; ++i) asm volatile("prefetch.tensormap [%0];" ::"l"(&M.m[i]) : "memory");
-    for (int i = 0; i < kStages; ++i) mbar_init(&sm.full[i], 1), mbar_init(&sm.freeb[i], kConsWarps);
-    for (int i = 0; i < kVecSlots; ++i) mbar_init(&sm.vfull[i], 1), mbar_init(&sm.vfree[i], kConsWarps);
+    for (int t = 0; t < kTeams; ++t) {
+      for (int i = 0; i < P.n_stages; ++i) mbar_init(&sm.full[t][i], 1), mbar_init(&sm.freeb[t][i], kTeamWarps);
+      for (int i = 0; i < kMaxVecs; ++i) mbar_init(&sm.vfull[t][i], 1), mbar_init(&sm.vfree[t][i], kTeamWarps);
+    }
     for (int i = 0; i < 2; ++i) mbar_init(&sm.pfull[i], kConsWarps), mbar_init(&sm.pfree[i], kEpiWarps);
     for (int i = 0; i < kProducts; ++i) mbar_init(&sm.product_done[i], kEpiWarps);
     fence_mbar_init();
@@ -407,6 +420,14 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
     if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
     sm.n_act = bad ? 0 : na;
   }
+  if (warp == 0) {
+    // the vector buffers are cut to the tokens the busiest expert has: with few, more slices are on their way
+    __syncwarp();
+    int most = 1;
+    for (int a = lane; a < sm.n_act; a += 32) most = max(most, sm.act_off[a + 1] - sm.act_off[a]);
+    most = min(__reduce_max_sync(0xffffffffu, most), kTok);
+    if (lane == 0) sm.vec_toks = most, sm.n_vecs = min(kMaxVecs, kTok / most);
+  }
   __syncthreads();
   // From here on the roles meet at mbarriers only; every wait is bounded.
   const int last = sm.n_act > 0 ? kProducts : 0;  // (nothing to do: no products, no meetings, zeros out)
@@ -415,8 +436,10 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
     // ================================================================= weight producer
     if (lane != 0) return;
     const uint64_t once = l2_policy_evict_first(), keep = l2_policy_normal();
-    Ring rs{0, 0u, 0};
+    Ring rs{0, 0u, 0}, other{0, 0u, 0};  // the ring of the team whose turn it is, the other team's
+    int team = 0;
     bool ok = true;
+#pragma unroll 1
     for (int ph = 0; ph < last && ok; ++ph) {
       const Product& pr = P.pr[ph];
       const CUtensorMap* map = &M.m[ph];
@@ -425,37 +448,43 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
         const int e = sm.act_slot[g.a];
         for (int k0 = 0; k0 < K; k0 += kSlice) {
           const int halves = K - k0 > kBoxK ? 2 : 1;
-          for (int sub = 0; sub < nsub; ++sub)
+          for (int sub = 0; sub < nsub; ++sub) {
             for (int u = 0; u < g.rows; u += kTileRows) {
-              const int row = g.row0 + u, boxes = g.rows - u > kBoxRows ? 2 : 1;
+              const int row = g.row0 + u;
               // rows another CTA or another token group reads as well stay in L2
               const uint64_t pol = g.last_use && g.rows - u >= kTileRows ? once : keep;
-              if ((rs.n >= kStages && !mbar_wait(&sm.freeb[rs.slot], rs.par ^ 1u)) || sm.abort) {
+              uint64_t* bar = &sm.full[team][rs.slot];
+              if ((rs.n >= P.n_stages && !mbar_wait(&sm.freeb[team][rs.slot], rs.par ^ 1u)) || sm.abort) {
                 give_up(P, sm, 0x620u);
                 return false;
               }
-              fence_proxy_async_smem();
-              mbar_arrive_expect_tx(&sm.full[rs.slot], (uint32_t)(halves * boxes * kBoxBytes));
-              unsigned char* dst = stages + (size_t)rs.slot * kStageBytes;
-              for (int hf = 0; hf < halves; ++hf)
-                for (int bx = 0; bx < boxes; ++bx)
-                  tma_rows(dst + hf * (2 * kBoxBytes) + bx * kBoxBytes, map, k0 + hf * kBoxK, sub, row + bx * kBoxRows, e,
-                           &sm.full[rs.slot], pol);
-              rs.advance(kStages);
+              mbar_arrive_expect_tx(bar, (uint32_t)(halves * kBoxBytes));
+              unsigned char* dst = stages + (size_t)(team * P.n_stages + rs.slot) * kStageBytes;
+              tma_rows(dst, map, k0, sub, row, e, bar, pol);
+              if (halves == 2) tma_rows(dst + kBoxBytes, map, k0 + kBoxK, sub, row, e, bar, pol);
+              rs.advance(P.n_stages);
             }
+            const Ring t = rs;
+            rs = other, other = t, team ^= 1;
+          }
         }
         return true;
       });
     }
     if (!ok)  // copies in flight must land before this CTA's shared memory goes away
-      for (int j = max(0, rs.n - kStages); j < rs.n; ++j) (void)mbar_wait(&sm.full[j % kStages], (unsigned)(j / kStages) & 1u);
+      for (int t = 0; t < kTeams; ++t, rs = other, team ^= 1)
+        for (int j = max(0, rs.n - P.n_stages); j < rs.n; ++j)
+          (void)mbar_wait(&sm.full[team][j % P.n_stages], (unsigned)(j / P.n_stages) & 1u);
     return;
   }
 
   if (warp == kVectorWarp) {
     // ================================================================= vector producer, meetings
-    Ring rv{0, 0u, 0};
+    Ring rv{0, 0u, 0}, other{0, 0u, 0};  // the ring of the team whose turn it is, the other team's
+    int team = 0;
+    const int n_vecs = sm.n_vecs, vec_bytes = sm.vec_toks * kTokBytes;
     bool ok = true;
+#pragma unroll 1
     for (int ph = 0; ph < last && ok; ++ph) {
       if (ph > 0) {  // every CTA has stored its outputs of the product before
         int met = 1;
@@ -494,36 +523,39 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
         for (int ks = 0; ks < pr.n_slices; ++ks) {
           const uint32_t bytes = plain ? (uint32_t)min(kSlice, K - ks * kSlice) * 2u : (uint32_t)kVecRun * 2u;
           for (int sub = 0; sub < pr.nsub; ++sub) {
-            if (!__all_sync(0xffffffffu, (rv.n < kVecSlots || mbar_wait(&sm.vfree[rv.slot], rv.par ^ 1u)) && !sm.abort)) {
+            if (!__all_sync(0xffffffffu, (rv.n < n_vecs || mbar_wait(&sm.vfree[team][rv.slot], rv.par ^ 1u)) && !sm.abort)) {
               if (lane == 0) give_up(P, sm, 0x631u);
               return false;
             }
-            fence_proxy_async_smem();
-            if (lane == 0) mbar_arrive_expect_tx(&sm.vfull[rv.slot], bytes * (uint32_t)g.ns);
+            if (lane == 0) mbar_arrive_expect_tx(&sm.vfull[team][rv.slot], bytes * (uint32_t)g.ns);
             __syncwarp();
             if (mine)
-              bulk_g2s(vecs + (size_t)rv.slot * kVecBytes + (size_t)lane * kTokBytes,
-                       src + sub * run + (size_t)ks * (plain ? kSlice : kVecRun), bytes, &sm.vfull[rv.slot]);
-            rv.advance(kVecSlots);
+              bulk_g2s(vecs + (size_t)team * kTok * kTokBytes + (size_t)rv.slot * vec_bytes + (size_t)lane * kTokBytes,
+                       src + sub * run + (size_t)ks * (plain ? kSlice : kVecRun), bytes, &sm.vfull[team][rv.slot]);
+            rv.advance(n_vecs);
+            const Ring t = rv;
+            rv = other, other = t, team ^= 1;
           }
         }
         return true;
       });
     }
     if (!ok)
-      for (int j = max(0, rv.n - kVecSlots); j < rv.n; ++j)
-        (void)mbar_wait(&sm.vfull[j % kVecSlots], (unsigned)(j / kVecSlots) & 1u);
+      for (int t = 0; t < kTeams; ++t, rv = other, team ^= 1)
+        for (int j = max(0, rv.n - n_vecs); j < rv.n; ++j) (void)mbar_wait(&sm.vfull[team][j % n_vecs], (unsigned)(j / n_vecs) & 1u);
     return;
   }
 
   if (warp >= kEpiWarp0) {
     // ================================================================= epilogue
-    // Warp ew takes rows 8 ew .. 8 ew + 7 of every tile (four at a time) for all 8 tokens: in product 3 all experts'
-    // contributions to an output meet in one warp, in expert order.
-    const int rq0 = 8 * (warp - kEpiWarp0) + (lane & 3), tok = lane >> 2;
+    // Warp ew takes rows 8 ew .. 8 ew + 7 of every tile, a lane one (row, token) pair at a time: in product 3 all
+    // experts' contributions to an output meet in one warp, in expert order.
+    const int rq = 8 * (warp - kEpiWarp0) + (lane & 7), q0 = lane >> 3;
     const int y0 = (int)((long long)P.d * blockIdx.x / gridDim.x);
     Ring rp{0, 0u, 0};
+    unsigned turn = 0;  // as the consumers count their slices
     bool ok = true;
+#pragma unroll 1
     for (int ph = 0; ph < last && ok; ++ph) {
       const Product& pr = P.pr[ph];
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
@@ -531,26 +563,27 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
           if (lane == 0) give_up(P, sm, 0x640u);
           return false;
         }
-        const int s = g.slot0 + tok;
-        for (int q = 0; (q >> 1) * kTileRows < g.rows; ++q) {
-          const int u = q >> 1, rq = rq0 + 4 * (q & 1);
+        const int items = (g.rows + kTileRows - 1) / kTileRows * g.ns;
+        int u = 0, tok = q0;  // item (tile u, token tok) = number q of tiles x tokens
+        for (int q = q0; q < items; q += 4, tok += 4) {
+          while (tok >= g.ns) tok -= g.ns, ++u;
+          const int s = g.slot0 + tok;
           const float* part = parts + (size_t)rp.slot * (kPartBytes / 4) + tok * kPartTok + rq;
-          auto total = [&](int tile) {
-            const float* p = part + (size_t)tile * kConsWarps * kPartTile;
-            float v = 0.f;
+          const float* p = part + (size_t)u * kConsWarps * kPartTile;
+          float sum[kTeams];
 #pragma unroll
-            for (int w = 0; w < kConsWarps; ++w) v += p[w * kPartTile];
-            return v;
-          };
+          for (int t = 0; t < kTeams; ++t) {
+            const float* pt = p + t * kTeamWarps * kPartTile;
+            sum[t] = (pt[0] + pt[kPartTile]) + (pt[2 * kPartTile] + pt[3 * kPartTile]);
+          }
           const int rl = u * kTileRows + rq, row = g.row0 + rl;
           float v;
-          if (pr.nsub == 2) {
-            const float gt = total(2 * u), up = total(2 * u + 1);
-            v = gt / (1.0f + expf(-gt)) * up;
-          } else {
-            v = total(u);
-          }
-          if (rl >= g.rows || tok >= g.ns) continue;
+          const float mine = sum[turn % kTeams], theirs = sum[(turn + 1) % kTeams];  // the team of the first slice, the other
+          if (pr.nsub == 2)
+            v = mine / (1.0f + expf(-mine)) * theirs;
+          else
+            v = pr.n_slices > 1 ? sum[0] + sum[1] : mine;
+          if (rl >= g.rows) continue;
           if (ph == kProducts - 1) {
             if (P.mode == 1)
               P.out_slots[(size_t)s * P.d + row] = v;
@@ -564,12 +597,13 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
             uint16_t* dst = (ph == 0 ? P.t : ph == 1 ? P.h : P.v) +
                             ((size_t)sl * P.pr[ph + 1].n_slices + c / kSlice) * kVecRun + c % kSlice;
 #pragma unroll
-            for (int i = 0; i < kTerms; ++i) dst[i * kSlice] = tm[i];
+            for (int i = 0; i < kTerms; ++i) dst[i * kTermRun] = tm[i];
           }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.pfree[rp.slot]);
         rp.advance(2);
+        turn += (unsigned)(pr.n_slices * pr.nsub);
         return true;
       });
       ok = __all_sync(0xffffffffu, ok);
@@ -578,9 +612,9 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
     }
     if (ok && P.mode == 0) {
       const int y1 = (int)((long long)P.d * (blockIdx.x + 1) / gridDim.x);
-      for (int q = 0; (q >> 1) * kTileRows < y1 - y0; ++q)
-        for (int t = tok; t < P.T; t += kTok) {
-          const int rl = (q >> 1) * kTileRows + rq0 + 4 * (q & 1);
+      for (int r0 = 0; r0 < y1 - y0; r0 += kTileRows)
+        for (int t = q0; t < P.T; t += 4) {
+          const int rl = r0 + rq;
           if (rl >= y1 - y0) continue;
           const float v = yacc[t * P.y_rows + rl];
           if (P.x_is_bf16)
@@ -594,19 +628,13 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
 
   // ===================================================================== consumers
   Ring rs{0, 0u, 0}, rv{0, 0u, 0}, rp{0, 0u, 0};
-  const uint32_t sa = smem_u32(stages), va = smem_u32(vecs);
+  unsigned turn = 0;
   bool ok = true;
-  for (int ph = 0; ph < last && ok; ++ph) {
-    if (ph == 0 && P.x_is_bf16)
-      ok = consume<1, 1>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
-    else if (ph == 1)
-      ok = consume<2, kTerms>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
-    else
-      ok = consume<1, kTerms>(P, sm, ph, sa, va, parts, rs, rv, rp, warp, lane);
-  }
+#pragma unroll 1
+  for (int ph = 0; ph < last && ok; ++ph) ok = consume(P, sm, ph, stages, vecs, parts, rs, rv, turn, rp, warp, lane);
 }
 
-// fp32 token rows -> their bf16 terms [T][slice][3][512]
+// fp32 token rows -> their bf16 terms [T][slice][3][480]
 __global__ void split_rows_kernel(const float* __restrict__ x, int d, uint16_t* __restrict__ out) {
   pdl_launch_dependents();
   pdl_wait();
@@ -616,7 +644,7 @@ __global__ void split_rows_kernel(const float* __restrict__ x, int d, uint16_t* 
     uint16_t tm[kTerms];
     split3(row[i], tm);
 #pragma unroll
-    for (int j = 0; j < kTerms; ++j) dst[(size_t)(i / kSlice) * kVecRun + j * kSlice + i % kSlice] = tm[j];
+    for (int j = 0; j < kTerms; ++j) dst[(size_t)(i / kSlice) * kVecRun + j * kTermRun + i % kSlice] = tm[j];
   }
 }
 
@@ -640,16 +668,18 @@ int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_wei
   auto set = [&](int i, const void* mat, int rows, int K, int nsub) {
     P.pr[i] = Product{rows, K, nsub, (K + kSlice - 1) / kSlice};
     // (the slot coordinate never leaves the array: its extent is not needed, only the rows' end inside a slot is)
-    if (rc == MOE_OK) rc = make_map_rows(&M.m[i], mat, K, nsub, rows, MOE_MAX_EXPERTS << 10, kBoxK, kBoxRows);
+    if (rc == MOE_OK) rc = make_map_rows(&M.m[i], mat, K, nsub, rows, MOE_MAX_EXPERTS << 10, kBoxK, kTileRows);
   };
   set(0, w->wd_a, 2 * r, d, 1);
   set(1, w->wd_b, f, r, 2);
   set(2, w->wd_c, r, f, 1);
   set(3, w->wd_d, d, r, 1);
   if (rc != MOE_OK) return rc;
-  const size_t smem = kHeaderBytes + (size_t)kStages * kStageBytes + (size_t)kVecSlots * kVecBytes + 2 * (size_t)kPartBytes +
-                      (mode == 0 ? (size_t)T * P.y_rows * 4 : 0);
-  if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
+  const size_t fixed = kHeaderBytes + (size_t)kTeams * kTok * kTokBytes + 2 * (size_t)kPartBytes +
+                       (mode == 0 ? (size_t)T * P.y_rows * 4 : 0);
+  P.n_stages = (int)min((long long)kMaxStages, ((long long)ctx->max_smem_optin - (long long)fixed) / (kTeams * kStageBytes));
+  if (P.n_stages < 2) return MOE_ERR_UNSUPPORTED;
+  const size_t smem = fixed + (size_t)kTeams * P.n_stages * kStageBytes;
   if (P.x_is_bf16) {
     P.x = (const uint16_t*)x;
   } else {
