@@ -111,8 +111,10 @@ int launch_wd_decode(moe_ctx* ctx, const void* x, const moe_weights* w, int32_t*
                      float* t, float* h, float* vpart, cudaStream_t s);
 constexpr int kWdSlice = 448;    // the vectors between its products are stored in slices of this many values,
 constexpr int kWdTermRun = 480;  // each as three runs (bf16 terms) this far apart
-int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
-                      const float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots,
+// (mode 0 with 8 or 16 experts: routes the tokens itself)
+bool wd_tokens_fuses_route(const moe_config& c);
+int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, int32_t* topk_idx,
+                      float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots,
                       char* ws, const WsLayout& L, cudaStream_t s);
 // Dense experts, streaming path, one kernel (router fused when T == 1 and mode == 0; mode 2 = mode 0 with the
 // routing always taken from topk_idx / topk_w).

@@ -73,6 +73,10 @@ constexpr int kPartTile = kTok * kPartTok;
 constexpr int kPartBytes = kGroupTiles * kConsWarps * kPartTile * 4;  // one of two buffers
 constexpr int kMaxSlots = MOE_STREAM_MAX_TOKENS * MOE_MAX_TOPK;
 constexpr int kProducts = 4;
+// With this many CTAs per active expert or more a CTA's rows are all of one expert: the shares are then up to 1 / 8 uneven,
+// which costs less than the partly filled tiles on both sides of an expert boundary (at 6 experts the CTAs with a boundary
+// finished a product up to 9 % after the others).
+constexpr int kAlignCtas = 8;
 
 struct Product {
   int rows;      // outputs per expert
@@ -85,8 +89,12 @@ struct WtParams {
   int T, k, E, d, mode, x_is_bf16, y_rows;
   int n_stages;  // of a team's ring
   const uint16_t* x;  // bf16 rows [T][d], or fp32 rows as terms [T][slice][3][480]
-  const int32_t* topk_idx;
-  const float* topk_w;
+  const uint16_t* w_router;  // set: the router runs in the prologue, CTA 0 writes its products to topk_idx / topk_w
+  const float* b_router;
+  const void* x_rows;        // the token rows as the caller has them
+  int renorm;
+  int32_t* topk_idx;
+  float* topk_w;
   const int32_t* offsets;
   const int32_t* perm;
   const int32_t* expert_slot;
@@ -111,7 +119,8 @@ struct WtSmem {
   int act_off[MOE_MAX_EXPERTS + 1];    // slot ranges, expert-ascending (same numbering as moe_permute)
   int slot_tok[kMaxSlots];
   float slot_w[kMaxSlots];
-  int stage_e[kMaxSlots];              // the routing as read from global memory
+  int stage_e[kMaxSlots];              // the routing, before grouping
+  float stage_w[kMaxSlots];
   int cursor[MOE_MAX_EXPERTS];
   int n_act;
   int vec_toks, n_vecs;                // token slices of a vector buffer (the most tokens an expert has), buffers of a team
@@ -129,6 +138,11 @@ struct Ring {
   }
 };
 
+__device__ __forceinline__ void swap_rings(Ring& mine, Ring& other, int& team) {
+  const Ring t = mine;
+  mine = other, other = t, team ^= 1;
+}
+
 // One group: rows [row0, row0 + rows) of active expert a for the tokens of its slots slot0 .. slot0 + ns - 1.
 struct Group {
   int a, slot0, ns, row0, rows;
@@ -141,11 +155,23 @@ __device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph
   const int N = P.pr[ph].rows, na = sm.n_act;
   const long long b = blockIdx.x, G = gridDim.x;
   const bool split_out = ph == kProducts - 1;
-  const long long tot = split_out ? N : (long long)na * N;
-  const int g0 = (int)(tot * b / G), g1 = (int)(tot * (b + 1) / G);
-  if (g0 >= g1) return true;
   constexpr int per = kGroupTiles * kTileRows;
-  for (int a = split_out ? 0 : g0 / N; a < na; ++a) {
+  int g0, g1, a0 = 0;
+  if (split_out) {
+    g0 = (int)(N * b / G), g1 = (int)(N * (b + 1) / G);
+  } else if ((int)G >= kAlignCtas * na) {
+    // a CTA works for one expert: the first G mod na experts get one CTA more
+    const int c = (int)G / na, more = (int)G - c * na, big = more * (c + 1), bi = (int)b;
+    a0 = bi < big ? bi / (c + 1) : more + (bi - big) / c;
+    const int jn = bi < big ? bi - a0 * (c + 1) : bi - big - (a0 - more) * c, cn = bi < big ? c + 1 : c;
+    g0 = a0 * N + (int)((long long)N * jn / cn), g1 = a0 * N + (int)((long long)N * (jn + 1) / cn);
+  } else {
+    const long long tot = (long long)na * N;
+    g0 = (int)(tot * b / G), g1 = (int)(tot * (b + 1) / G);
+    a0 = g0 / N;
+  }
+  if (g0 >= g1) return true;
+  for (int a = a0; a < na; ++a) {
     const int lo = split_out ? g0 : max(g0 - a * N, 0), hi = split_out ? g1 : min(g1 - a * N, N);
     if (hi <= lo) break;
     const int groups = (hi - lo + per - 1) / per;
@@ -157,6 +183,10 @@ __device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph
   }
   return true;
 }
+
+// The two consumer teams take the slices of the contraction in turn; in product 3, whose groups are one short tile per
+// expert, the groups.
+__device__ __forceinline__ bool teams_by_group(int ph) { return ph == kProducts - 1; }
 
 __device__ __forceinline__ void give_up(const WtParams& P, WtSmem& sm, unsigned detail) {
   sm.abort = 1;
@@ -217,11 +247,17 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
   const int term = g8 & 3, col = tw * kUnit + q4 * 8;
   constexpr int kUnitStep = kTeamWarps * kUnit;
   const int n_vecs = sm.n_vecs;
+  const bool by_group = teams_by_group(ph);
   return walk(P, sm, ph, [&](const Group& g) -> bool {
     const int tiles = (g.rows + kTileRows - 1) / kTileRows;
     if (rp.n >= 2 && !mbar_wait(&sm.pfree[rp.slot], rp.par ^ 1u)) {
       if (lane == 0) give_up(P, sm, 0x612u);
       return false;
+    }
+    if (by_group && turn++ % kTeams != team) {
+      if (lane == 0) mbar_arrive(&sm.pfull[rp.slot]);
+      rp.advance(2);
+      return true;
     }
     // this lane's partial sums, [tile][warp][token][row]: row g8 (even lanes) or g8 + 8 of tokens q4 / 2 + 2 p.  A team's
     // first slice stores, the others add.  Of a (gate, up) pair either team has one; a group with a single slice is
@@ -233,7 +269,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
       const int width = min(kSlice, K - k0);
 #pragma unroll 1
       for (int sub = 0; sub < nsub; ++sub) {
-        if (turn++ % kTeams != team) continue;
+        if (!by_group && turn++ % kTeams != team) continue;
         if (!mbar_wait(&sm.vfull[team][rv.slot], rv.par)) {
           if (lane == 0) give_up(P, sm, 0x610u);
           return false;
@@ -305,6 +341,87 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
   });
 }
 
+// Router (Eq. 2, Eq. 3) of all T tokens by every CTA, E = 8 or 16.  A thread owns the input features tid, tid + 384, ...:
+// their rows of W_r are fetched once (wr0: the first eight experts', before the dependency wait) and serve every token.
+// part: [12 warps][16 tokens][16 experts].
+constexpr int kRouteQ = 6;  // features per thread and round: d <= 2304 in one
+__device__ __forceinline__ void route_fetch(const WtParams& P, int q0, int e8, int tid, uint4* wr) {
+#pragma unroll
+  for (int q = 0; q < kRouteQ; ++q)
+    wr[q] = __ldg(reinterpret_cast<const uint4*>(P.w_router + (size_t)min(tid + (q0 + q) * kThreads, P.d - 1) * P.E + e8));
+}
+__device__ __forceinline__ void route_tokens(const WtParams& P, WtSmem& sm, float* part, const uint4* wr0, int tid) {
+  const int lane = tid & 31, warp = tid >> 5, d = P.d;
+  for (int e8 = 0; e8 < P.E; e8 += 8) {
+    for (int q0 = 0; q0 * kThreads < d; q0 += kRouteQ) {
+      uint4 wr[kRouteQ];
+      if (e8 == 0 && q0 == 0) {
+#pragma unroll
+        for (int q = 0; q < kRouteQ; ++q) wr[q] = wr0[q];
+      } else {
+        route_fetch(P, q0, e8, tid, wr);
+      }
+#pragma unroll 1
+      for (int t0 = 0; t0 < P.T; t0 += 4) {
+        float xv[4][kRouteQ];  // four tokens' features in one round trip
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int q = 0; q < kRouteQ; ++q) {
+            const int i = tid + (q0 + q) * kThreads;
+            const size_t at = (size_t)min(t0 + t, P.T - 1) * d + min(i, d - 1);
+            xv[t][q] = P.x_is_bf16 ? bf16_to_float(__ldg((const uint16_t*)P.x_rows + at)) : __ldg((const float*)P.x_rows + at);
+            if (i >= d) xv[t][q] = 0.f;
+          }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          float a[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) a[e] = 0.f;
+#pragma unroll
+          for (int q = 0; q < kRouteQ; ++q) {
+            float w[8];
+            unpack8(wr[q], w);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) a[e] = fmaf(xv[t][q], w[e], a[e]);
+          }
+          // eight sums over the warp: each exchange halves the values a lane still carries
+#pragma unroll
+          for (int half = 4; half >= 1; half >>= 1) {
+            const bool up = lane & (half * 4);
+#pragma unroll
+            for (int e = 0; e < half; ++e) {
+              const float send = up ? a[e] : a[e + half], keep = up ? a[e + half] : a[e];
+              a[e] = keep + __shfl_xor_sync(0xffffffffu, send, half * 4);
+            }
+          }
+          a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+          a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+          if ((lane & 3) == 0 && t0 + t < P.T) {
+            float* dst = part + (warp * 16 + t0 + t) * 16 + e8 + (lane >> 2);
+            *dst = q0 == 0 ? a[0] : *dst + a[0];
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int t = warp; t < P.T; t += kThreads / 32) {
+    float l = 0.f;
+    if (lane < P.E) {
+      for (int w = 0; w < kThreads / 32; ++w) l += part[(w * 16 + t) * 16 + lane];
+      if (P.b_router) l += P.b_router[lane];
+    }
+    warp_route_finish(l, 0.f, P.E, P.k, P.renorm, lane, sm.stage_e + t * P.k, sm.stage_w + t * P.k, nullptr);
+    __syncwarp();
+    if (blockIdx.x == 0 && lane < P.k) {
+      P.topk_idx[t * P.k + lane] = sm.stage_e[t * P.k + lane];
+      P.topk_w[t * P.k + lane] = sm.stage_w[t * P.k + lane];
+    }
+  }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_constant__ WtParams P, const __grid_constant__ WtMaps M) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WtSmem& sm = *reinterpret_cast<WtSmem*>(smem_raw);
@@ -330,7 +447,10 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
   }
   if (P.mode == 0)
     for (int i = tid; i < P.T * P.y_rows; i += kThreads) yacc[i] = 0.f;
+  uint4 wr0[kRouteQ];  // constants: fetched before the dependency wait
+  if (P.w_router) route_fetch(P, 0, 0, tid, wr0);
   pdl_wait();
+  if (P.w_router) route_tokens(P, sm, parts, wr0, tid);
 
   // ---------------------------------------------------------------- routing -> active experts and their slots
   const int n = P.T * P.k;
@@ -338,7 +458,8 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
     const unsigned below = (1u << lane) - 1u;
     int bad = 0;
     sm.cursor[lane] = 0, sm.cursor[lane + 32] = 0;
-    for (int p = lane; p < n; p += 32) sm.stage_e[p] = P.topk_idx[p];
+    if (!P.w_router)
+      for (int p = lane; p < n; p += 32) sm.stage_e[p] = P.topk_idx[p], sm.stage_w[p] = P.topk_w[p];
     __syncwarp();
     for (int p0 = 0; p0 < n; p0 += 32) {  // counts: the first lane of each group of equal experts adds the group
       const int p = p0 + lane;
@@ -381,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       if (e >= 0) {
         const int s = base + __popc(peers & below);  // pairs of one expert keep their order
         sm.slot_tok[s] = p / P.k;
-        sm.slot_w[s] = P.topk_w[p];
+        sm.slot_w[s] = sm.stage_w[p];
         if ((peers & below) == 0u) sm.cursor[e] = base + __popc(peers);
       }
       __syncwarp();
@@ -444,6 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       const Product& pr = P.pr[ph];
       const CUtensorMap* map = &M.m[ph];
       const int K = pr.K, nsub = pr.nsub;
+      const bool by_group = teams_by_group(ph);
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
         const int e = sm.act_slot[g.a];
         for (int k0 = 0; k0 < K; k0 += kSlice) {
@@ -464,10 +586,10 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
               if (halves == 2) tma_rows(dst + kBoxBytes, map, k0 + kBoxK, sub, row, e, bar, pol);
               rs.advance(P.n_stages);
             }
-            const Ring t = rs;
-            rs = other, other = t, team ^= 1;
+            if (!by_group) swap_rings(rs, other, team);
           }
         }
+        if (by_group) swap_rings(rs, other, team);
         return true;
       });
     }
@@ -510,6 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       }
       const Product& pr = P.pr[ph];
       const int K = pr.K;
+      const bool by_group = teams_by_group(ph);
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
         // lane = the token whose slices it brings
         const bool mine = lane < g.ns;
@@ -533,10 +656,10 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
               bulk_g2s(vecs + (size_t)team * kTok * kTokBytes + (size_t)rv.slot * vec_bytes + (size_t)lane * kTokBytes,
                        src + sub * run + (size_t)ks * (plain ? kSlice : kVecRun), bytes, &sm.vfull[team][rv.slot]);
             rv.advance(n_vecs);
-            const Ring t = rv;
-            rv = other, other = t, team ^= 1;
+            if (!by_group) swap_rings(rv, other, team);
           }
         }
+        if (by_group) swap_rings(rv, other, team);
         return true;
       });
     }
@@ -558,6 +681,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
 #pragma unroll 1
     for (int ph = 0; ph < last && ok; ++ph) {
       const Product& pr = P.pr[ph];
+      const bool by_group = teams_by_group(ph);
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
         if (!mbar_wait(&sm.pfull[rp.slot], rp.par)) {
           if (lane == 0) give_up(P, sm, 0x640u);
@@ -582,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
           if (pr.nsub == 2)
             v = mine / (1.0f + expf(-mine)) * theirs;
           else
-            v = pr.n_slices > 1 ? sum[0] + sum[1] : mine;
+            v = pr.n_slices > 1 && !by_group ? sum[0] + sum[1] : mine;
           if (rl >= g.rows) continue;
           if (ph == kProducts - 1) {
             if (P.mode == 1)
@@ -603,7 +727,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.pfree[rp.slot]);
         rp.advance(2);
-        turn += (unsigned)(pr.n_slices * pr.nsub);
+        turn += by_group ? 1u : (unsigned)(pr.n_slices * pr.nsub);
         return true;
       });
       ok = __all_sync(0xffffffffu, ok);
@@ -650,8 +774,10 @@ __global__ void split_rows_kernel(const float* __restrict__ x, int d, uint16_t* 
 
 }  // namespace
 
-int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, const int32_t* topk_idx,
-                     const float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots, char* ws,
+bool wd_tokens_fuses_route(const moe_config& c) { return (c.n_experts & 7) == 0 && c.n_experts <= 16; }
+
+int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_weights* w, int32_t* topk_idx,
+                     float* topk_w, const int32_t* offsets, const int32_t* perm, void* y, float* out_slots, char* ws,
                      const WsLayout& L, cudaStream_t s) {
   const moe_config& c = ctx->cfg;
   if (c.wd_rank == 0) return MOE_ERR_UNSUPPORTED;  // dense experts stream through launch_dense_stream
@@ -661,6 +787,8 @@ int launch_wd_tokens(moe_ctx* ctx, int mode, const void* x, int T, const moe_wei
   P.x_is_bf16 = c.x_dtype == MOE_BF16;
   P.topk_idx = topk_idx, P.topk_w = topk_w, P.offsets = offsets, P.perm = perm, P.expert_slot = w->expert_slot;
   P.t = (uint16_t*)(ws + L.vec_a), P.h = (uint16_t*)(ws + L.vec_b), P.v = (uint16_t*)(ws + L.vec_c);
+  P.renorm = c.renorm, P.x_rows = x;
+  if (mode == 0 && wd_tokens_fuses_route(c)) P.w_router = (const uint16_t*)w->w_router, P.b_router = w->b_router;
   P.y = y, P.out_slots = out_slots, P.st = ctx->d_state;
   P.y_rows = (d + G - 1) / G + 1;
   WtMaps M;
