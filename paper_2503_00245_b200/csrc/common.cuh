@@ -100,6 +100,8 @@ constexpr int kKSplitMax = 4;          // planes the tensor path may ask for ...
 constexpr int kKSplitMaxSlots = 2048;  // ... when there are at most this many (token, choice) slots
 int launch_combine(moe_ctx* ctx, const float* out_slots, const float* wt, const int32_t* inv, int T, void* y,
                    int planes, cudaStream_t s);
+// out [n] = the sum of `planes` runs of n values, in order
+int launch_sum_planes(moe_ctx* ctx, const float* in, long long n, int planes, float* out, cudaStream_t s);
 int launch_gather_rows(moe_ctx* ctx, const void* x, const int32_t* perm, int n_slots, void* xperm, cudaStream_t s);
 
 // Streaming (decode) path.  mode 0: whole layer from topk (writes y); mode 1: FFN per slot from

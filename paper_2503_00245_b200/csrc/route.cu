@@ -406,6 +406,28 @@ int launch_combine(moe_ctx* ctx, const float* out_slots, const float* wt, const 
   return MOE_OK;
 }
 
+// out[i] = sum over the planes, in order (n a multiple of 4)
+__global__ void sum_planes_kernel(const float4* __restrict__ in, long long quads, int planes, float4* __restrict__ out) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < quads; i += (long long)gridDim.x * blockDim.x) {
+    float4 o = in[i];
+    for (int pl = 1; pl < planes; ++pl) {
+      const float4 o2 = in[i + pl * quads];
+      o.x += o2.x, o.y += o2.y, o.z += o2.z, o.w += o2.w;
+    }
+    out[i] = o;
+  }
+}
+
+int launch_sum_planes(moe_ctx* ctx, const float* in, long long n, int planes, float* out, cudaStream_t s) {
+  const long long quads = n / 4, want = (quads + 255) / 256;
+  const int grid = (int)(want < 16ll * ctx->sm_count ? want : 16ll * ctx->sm_count);
+  MOE_CUDA_TRY(launch_pdl(sum_planes_kernel, dim3(grid), dim3(256), 0, s, (const float4*)in, quads, planes, (float4*)out));
+  ctx->launches++;
+  return MOE_OK;
+}
+
 // ------------------------------------------------------------------------------------ packing
 // in [B][R][C] -> out[b][c][sub][r] with nsub interleaved row kinds: a tiled transpose.
 __global__ void pack_transpose_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, int R, int C,

@@ -42,6 +42,7 @@ constexpr int kThreadsGG = (2 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;  // two accumulator buffers of 256 columns
 constexpr int kAccCols = 256;
 constexpr int kMaxStagesGG = 6;
+constexpr int kEpiBuf = 2048;
 constexpr int kPairRows = 2 * kBM;  // rows of a pair's tile
 
 enum Epi { EPI_SWIGLU = 0, EPI_BF16_PAIR = 1, EPI_BF16 = 2, EPI_F32 = 3 };
@@ -203,6 +204,44 @@ __device__ __forceinline__ bool decode_tile(const GGParams& P, const SmemGG& sm,
 
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
 
+// 64 bytes of each of 32 rows from a warp's registers (lane = row) to memory, through 2 KB of shared memory: a store of
+// the accumulator layout as it is touches 32 lines with 16 bytes each; this one writes 8 rows' 64 bytes per instruction.
+// (16-byte pieces are swapped by row pair, so that neither side meets a bank conflict.)  rows: valid rows; pieces: valid
+// 16-byte pieces of a row.
+__device__ __forceinline__ void store_rows(unsigned char* buf, int lane, const uint32_t* v, void* dst, long long ld_bytes,
+                                           int rows, int pieces) {
+  __syncwarp();  // (the buffer's last contents have been read)
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<uint4*>(buf + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) =
+        make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  __syncwarp();
+  const int piece = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = (lane >> 2) + 8 * i;
+    if (r < rows && piece < pieces)
+      *reinterpret_cast<uint4*>((unsigned char*)dst + (long long)r * ld_bytes + piece * 16) =
+          *reinterpret_cast<const uint4*>(buf + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
+  }
+}
+// 32 fp32 columns rounded to bf16; lo_off > 0: the rounding remainders too, lo_off columns further on
+__device__ __forceinline__ void store_bf16(unsigned char* buf, int lane, const uint32_t* a, __nv_bfloat16* dst, long long ld_bytes,
+                                           int rows, int pieces, long long lo_off) {
+  uint32_t o[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) o[j] = pack_bf16x2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1]));
+  store_rows(buf, lane, o, dst, ld_bytes, rows, pieces);
+  if (lo_off > 0) {
+    uint32_t l[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      l[j] = pack_bf16x2(__uint_as_float(a[2 * j]) - __uint_as_float(o[j] << 16),
+                         __uint_as_float(a[2 * j + 1]) - __uint_as_float(o[j] & 0xffff0000u));
+    store_rows(buf, lane, l, dst + lo_off, ld_bytes, rows, pieces);
+  }
+}
+
 __global__ void __launch_bounds__(kThreadsGG, 1)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                         const __grid_constant__ CUtensorMap map_b, const GGParams P) {
@@ -215,7 +254,8 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   const uint32_t b_bytes = b_rows * kBK * 2;
   const uint32_t stage_bytes = n_a * a_bytes + 128u * kBK * 2u;
   unsigned char* stages = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  SmemGG& sm = *reinterpret_cast<SmemGG*>(stages + (size_t)P.n_stages * stage_bytes);
+  unsigned char* const epi_bufs = stages + (size_t)P.n_stages * stage_bytes;  // 2 KB per epilogue warp
+  SmemGG& sm = *reinterpret_cast<SmemGG*>(epi_bufs + kEpiWarps * kEpiBuf);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int NS = P.n_stages;
   const int num_kb = (P.K + kBK - 1) / kBK;
@@ -376,6 +416,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     const int q = warp & 3;  // TMEM lanes 32q .. 32q+31 are the only ones this warp may read
     const int cpar = (warp - 2) >> 2;  // which of the two warps of this quarter: it takes every other 32-column chunk
     const uint32_t acce_bar[2] = {map_to_rank(&sm.accum_empty[0], 0u), map_to_rank(&sm.accum_empty[1], 0u)};
+    unsigned char* const ebuf = epi_bufs + (warp - 2) * kEpiBuf;
     int tile_i = 0;
     for (int idx = pair; decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs, ++tile_i) {
       const int buf = tile_i & 1;
@@ -386,55 +427,27 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       tc_fence_after();
       const int ncols = min(P.bn, P.n_store - t.n0);  // columns of this tile to store (multiple of 8)
       const int row = t.m0 + (int)rank * kBM + 32 * q + lane;
-      const bool row_ok = row < t.m_end;
+      const int rows = t.m_end - (row - lane);  // rows of this warp's 32 that belong to the expert (<= 0: none)
       const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * kAccCols);
+      const size_t row0 = (size_t)(row - lane);
       if (P.epi == EPI_SWIGLU || P.epi == EPI_BF16_PAIR) {
-        __nv_bfloat16* out = (__nv_bfloat16*)P.out + (size_t)row * P.ld_out + t.n0;
+        __nv_bfloat16* out = (__nv_bfloat16*)P.out + row0 * P.ld_out + t.n0;
         for (int c = 32 * cpar; c < P.bn; c += 64) {
           uint32_t g[32], u[32];
           tc_ld32(tbase + c, g);
           tc_ld32(tbase + P.bn + c, u);
           tc_wait_ld();
-          if (!row_ok) continue;
+          const int pieces = (ncols - c) / 8;  // of 16 bytes
+          uint32_t o[16];
           if (P.epi == EPI_SWIGLU) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              if (c + 8 * v < ncols) {
-                uint32_t o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  o[j] = pack_bf16x2(silu_mul(__uint_as_float(g[8 * v + 2 * j]), __uint_as_float(u[8 * v + 2 * j])),
-                                     silu_mul(__uint_as_float(g[8 * v + 2 * j + 1]), __uint_as_float(u[8 * v + 2 * j + 1])));
-                *reinterpret_cast<uint4*>(out + c + 8 * v) = make_uint4(o[0], o[1], o[2], o[3]);
-              }
-            }
+            for (int j = 0; j < 16; ++j)
+              o[j] = pack_bf16x2(silu_mul(__uint_as_float(g[2 * j]), __uint_as_float(u[2 * j])),
+                                 silu_mul(__uint_as_float(g[2 * j + 1]), __uint_as_float(u[2 * j + 1])));
+            store_rows(ebuf, lane, o, out + c, P.ld_out * 2, rows, pieces);
           } else {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              if (c + 8 * v < ncols) {
-                uint32_t o[4], p[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  o[j] = pack_bf16x2(__uint_as_float(g[8 * v + 2 * j]), __uint_as_float(g[8 * v + 2 * j + 1]));
-                  p[j] = pack_bf16x2(__uint_as_float(u[8 * v + 2 * j]), __uint_as_float(u[8 * v + 2 * j + 1]));
-                }
-                *reinterpret_cast<uint4*>(out + c + 8 * v) = make_uint4(o[0], o[1], o[2], o[3]);
-                *reinterpret_cast<uint4*>(out + P.out_off2 + c + 8 * v) = make_uint4(p[0], p[1], p[2], p[3]);
-                if (P.split) {
-                  uint32_t ol[4], pl[4];
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    ol[j] = pack_bf16x2(__uint_as_float(g[8 * v + 2 * j]) - __uint_as_float(o[j] << 16),
-                                        __uint_as_float(g[8 * v + 2 * j + 1]) - __uint_as_float(o[j] & 0xffff0000u));
-                    pl[j] = pack_bf16x2(__uint_as_float(u[8 * v + 2 * j]) - __uint_as_float(p[j] << 16),
-                                        __uint_as_float(u[8 * v + 2 * j + 1]) - __uint_as_float(p[j] & 0xffff0000u));
-                  }
-                  *reinterpret_cast<uint4*>(out + P.out_off_lo + c + 8 * v) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
-                  *reinterpret_cast<uint4*>(out + P.out_off2 + P.out_off_lo + c + 8 * v) =
-                      make_uint4(pl[0], pl[1], pl[2], pl[3]);
-                }
-              }
-            }
+            store_bf16(ebuf, lane, g, out + c, P.ld_out * 2, rows, pieces, P.split ? P.out_off_lo : 0);
+            store_bf16(ebuf, lane, u, out + P.out_off2 + c, P.ld_out * 2, rows, pieces, P.split ? P.out_off_lo : 0);
           }
         }
       } else {
@@ -442,33 +455,13 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           uint32_t a[32];
           tc_ld32(tbase + c, a);
           tc_wait_ld();
-          if (!row_ok) continue;
           if (P.epi == EPI_F32) {
-            float* out = (float*)P.out + (size_t)t.ks * P.plane_elems + (size_t)row * P.ld_out + t.n0 + c;
-#pragma unroll
-            for (int v = 0; v < 8; ++v)
-              if (c + 4 * v < ncols)
-                *reinterpret_cast<uint4*>(out + 4 * v) = make_uint4(a[4 * v], a[4 * v + 1], a[4 * v + 2], a[4 * v + 3]);
+            float* out = (float*)P.out + (size_t)t.ks * P.plane_elems + row0 * P.ld_out + t.n0 + c;
+            store_rows(ebuf, lane, a, out, P.ld_out * 4, rows, (ncols - c) / 4);
+            store_rows(ebuf, lane, a + 16, out + 16, P.ld_out * 4, rows, (ncols - c - 16) / 4);
           } else {
-            __nv_bfloat16* out = (__nv_bfloat16*)P.out + (size_t)row * P.ld_out + t.n0 + c;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              if (c + 8 * v < ncols) {
-                uint32_t o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  o[j] = pack_bf16x2(__uint_as_float(a[8 * v + 2 * j]), __uint_as_float(a[8 * v + 2 * j + 1]));
-                *reinterpret_cast<uint4*>(out + 8 * v) = make_uint4(o[0], o[1], o[2], o[3]);
-                if (P.split) {
-                  uint32_t ol[4];
-#pragma unroll
-                  for (int j = 0; j < 4; ++j)
-                    ol[j] = pack_bf16x2(__uint_as_float(a[8 * v + 2 * j]) - __uint_as_float(o[j] << 16),
-                                        __uint_as_float(a[8 * v + 2 * j + 1]) - __uint_as_float(o[j] & 0xffff0000u));
-                  *reinterpret_cast<uint4*>(out + P.out_off_lo + 8 * v) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
-                }
-              }
-            }
+            store_bf16(ebuf, lane, a, (__nv_bfloat16*)P.out + row0 * P.ld_out + t.n0 + c, P.ld_out * 2, rows, (ncols - c) / 8,
+                       P.split ? P.out_off_lo : 0);
           }
         }
       }
@@ -580,7 +573,7 @@ int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const 
   const int n_tiles = (P.n_total + P.bn - 1) / P.bn;
   const size_t stage_bytes = (size_t)kBM * kBK * 2 * (P.bmode == B_DUAL ? 2 : 1) + 128 * kBK * 2;
   P.n_stages = P.bmode == B_DUAL ? 4 : kMaxStagesGG;
-  const size_t smem = P.n_stages * stage_bytes + sizeof(SmemGG) + 1024 + 128;
+  const size_t smem = P.n_stages * stage_bytes + kEpiWarps * kEpiBuf + sizeof(SmemGG) + 1024 + 128;
   if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
   MOE_TRY(allow_full_smem<grouped_gemm_kernel>(ctx));
   const long long m_tiles = (n_slots + kPairRows - 1) / kPairRows + c.n_experts;  // upper bound
@@ -634,15 +627,27 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
     if ((rc = make_map_b(&mb, w->gud, d, 3, f, E, 64, kBK)) != MOE_OK) return rc;
     P.K = f, P.n_total = d, P.bn = pick_bn(d, 256, 128), P.bmode = B_NMAJOR, P.b_sub = 2;
     P.epi = EPI_F32, P.out = out_slots, P.ld_out = d, P.out_off2 = 0;
-    if (out_planes && n_slots <= kKSplitMaxSlots) {
-      // short prefill: too few tiles for the SMs, and every tile streams a long run of weights.  The caller
-      // sums planes: cut the contraction so that every pair streams a part, each part into its own plane.
+    if (n_slots <= kKSplitMaxSlots) {
+      // short prefill: too few tiles for the SMs, and every tile streams a long run of weights.  Cut the contraction so
+      // that every pair streams a part, each part into its own plane; the caller sums the planes, or they are summed
+      // here (in the same order: the layer and its four calls give the same bits).
       const int m_est = std::max((n_slots + kPairRows - 1) / kPairRows, std::min(E, n_slots));
       const long long tiles = (long long)m_est * ((d + P.bn - 1) / P.bn);
-      int ks = (int)((ctx->sm_count / 2) / std::max<long long>(tiles, 1));
-      ks = std::min(std::min(ks, kKSplitMax), (f + kBK - 1) / kBK);
+      // Fewest rounds of k-steps over the pairs; a further plane has to save 1/8 (each is written and read once more).
+      const int num_kb = (f + kBK - 1) / kBK, pairs = ctx->sm_count / 2;
+      int ks = 1;
+      long long best = (tiles + pairs - 1) / pairs * num_kb;
+      for (int c = 2; c <= std::min(kKSplitMax, num_kb); ++c) {
+        const long long steps = (tiles * c + pairs - 1) / pairs * ((num_kb + c - 1) / c);
+        if (8 * steps <= 7 * best) best = steps, ks = c;
+      }
       if (ks > 1) {
         P.ksplit = ks, P.plane_elems = (long long)n_slots * d;
+        if (!out_planes) {
+          P.out = ws + L.out_slots;
+          if ((rc = launch_gg(ctx, ma, ma, mb, P, n_slots, s)) != MOE_OK) return rc;
+          return launch_sum_planes(ctx, (const float*)P.out, P.plane_elems, ks, out_slots, s);
+        }
         *out_planes = ks;
       }
     }
