@@ -288,11 +288,11 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   if (path == MOE_PATH_STREAM && wd_decode_applies(ctx->cfg, T))  // one launch, router included
     return launch_wd_decode(ctx, x, w, idx, wt, y, (float*)(wsb + L.vec_a), (float*)(wsb + L.vec_b),
                             (float*)(wsb + L.vec_c), s);
-  if (path != MOE_PATH_STREAM || ctx->cfg.wd_rank == 0 || !wd_tokens_fuses_route(ctx->cfg)) {
-    rc = launch_route(ctx, x, T, w, idx, wt, nullptr, s);
-    if (rc != MOE_OK) return rc;
-  }
   if (path == MOE_PATH_STREAM) {
+    if (ctx->cfg.wd_rank == 0 || !wd_tokens_fuses_route(ctx->cfg)) {
+      rc = launch_route(ctx, x, T, w, idx, wt, nullptr, s);
+      if (rc != MOE_OK) return rc;
+    }
     if (ctx->cfg.wd_rank == 0) return launch_dense_stream(ctx, 0, x, T, w, idx, wt, nullptr, nullptr, y, nullptr, s);
     return launch_wd_tokens(ctx, 0, x, T, w, idx, wt, nullptr, nullptr, y, nullptr, wsb, L, s);
   }
@@ -300,7 +300,8 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   int32_t* perm = (int32_t*)(wsb + L.perm);
   int32_t* inv = (int32_t*)(wsb + L.inv);
   float* out_slots = (float*)(wsb + L.out_slots);
-  rc = launch_permute(ctx, idx, T, offsets, perm, inv, s);
+  const Grouping grp{offsets, perm, inv};
+  rc = launch_route(ctx, x, T, w, idx, wt, nullptr, s, &grp);
   if (rc != MOE_OK) return rc;
   int planes = 1;
   rc = launch_tensor_ffn(ctx, x, T, w, offsets, perm, wsb, L, out_slots, &planes, s);

@@ -41,7 +41,9 @@ struct DeviceState {
   // dense streaming kernel, one token: added to the arrivals an accumulator word waits for (0; the diagnostics
   // hook sets 1, so that the wait runs out)
   unsigned int tail_bias;
-  unsigned int pad3[19];
+  // router of many tokens: CTAs that have stored their tokens' routing; the last one sets it back
+  unsigned int route_done;
+  unsigned int pad3[18];
 };
 
 }  // namespace cosmoe
@@ -90,8 +92,13 @@ WsLayout ws_layout(const moe_config& c, int T);
 int validate_config(const moe_config* c);
 
 // launchers implemented in the other translation units
+// Where the (token, choice) pairs go when they are grouped by expert (moe_permute's products).
+struct Grouping {
+  int32_t *offsets, *perm, *inv;
+};
+// With `grp` the pairs are grouped as well.
 int launch_route(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt, float* probs,
-                 cudaStream_t s);
+                 cudaStream_t s, const Grouping* grp = nullptr);
 int launch_permute(moe_ctx* ctx, const int32_t* idx, int T, int32_t* offsets, int32_t* perm, int32_t* inv,
                    cudaStream_t s);
 // out_slots may come as `planes` partial sums, one [T*k][d] plane after the other (summed in order).
@@ -331,6 +338,25 @@ __device__ __forceinline__ float bf16_to_float(uint16_t b) { return __uint_as_fl
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// 16 rows x 16 values times 16 values x 8 tokens; a row's (a token's) two registers hold 4 of its values per lane
+__device__ __forceinline__ void mma16(float* c, uint32_t a_lo0, uint32_t a_hi0, uint32_t a_lo1, uint32_t a_hi1, uint32_t b0,
+                                      uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a_lo0), "r"(a_hi0), "r"(a_lo1), "r"(a_hi1), "r"(b0), "r"(b1));
+}
+
+// fp32 -> three bf16 terms, the largest first: each remainder is exact in fp32
+__device__ __forceinline__ void split3(float v, uint16_t* out) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+    out[i] = __bfloat16_as_ushort(b);
+    v -= __bfloat162float(b);
+  }
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

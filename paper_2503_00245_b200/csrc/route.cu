@@ -98,65 +98,213 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
                     probs ? probs + (size_t)t * E : nullptr);
 }
 
-// Many tokens, 8 experts, a router matrix of at most 64 KB: every CTA first copies W_r into shared memory, its
-// 16-byte rows (one input feature each) shifted by 16 bytes per 8 rows so that lanes reading rows 8 apart fall
-// into different banks; then its warps walk the tokens, a lane taking 8 consecutive features per 16-byte load
-// of x.  (The kernel above reads W_r through L1 with 32 cache lines per warp instruction.)
+// Many tokens: the logits of 16 tokens per CTA on the tensor cores (mma.sync m16n8k16: 16 tokens x 8 experts; N is far
+// below a tcgen05 tile).  W_r lies transposed in shared memory, [expert][feature], the experts' rows 64 bytes beyond a
+// multiple of 128 apart; the 16 warps split the features in units of 32.  A lane takes 8 consecutive features of a row at a
+// time, of x straight from memory (all of a warp's loads of a round in flight together) and of W_r alike: the order of
+// the contraction inside a unit is free.  fp32 rows go in as three bf16 terms.  Sums stay short in the MMA's accumulators
+// (two units) and are added up in fp32.
+// The last CTA to finish groups the pairs by expert, a stable counting sort: every warp counts and then scatters a
+// contiguous run of them.  One launch instead of two, and no second walk over the routing by a lone CTA in rounds.
+// (2048 tokens, d 2048, 8 experts: FIXME)
+constexpr int kRtWarps = 16, kRtTokens = 16, kRtUnit = 32, kRtBatch = 4;
+struct RtShape {
+  int e8, row_bytes, part_off, smem;  // experts rounded up to 8; bytes between two experts' rows; partial logits; total
+};
+static __host__ __device__ inline RtShape rt_shape(int d, int E) {
+  RtShape r{};
+  r.e8 = (E + 7) / 8 * 8;
+  r.row_bytes = (d + kRtUnit - 1) / kRtUnit * kRtUnit * 2;
+  r.row_bytes += (r.row_bytes & 127) == 64 ? 0 : 64;
+  r.part_off = r.e8 * r.row_bytes;
+  const int part = kRtWarps * kRtTokens * r.e8 * 4, count = kRtWarps * MOE_MAX_EXPERTS * 4;
+  r.smem = r.part_off + (part > count ? part : count);
+  return r;
+}
+
 template <typename XT>
-__global__ void __launch_bounds__(kRouteWarps * 32)
-    route_smem_kernel(const XT* __restrict__ x, const uint16_t* __restrict__ w_router, const float* __restrict__ bias,
-                      int T, int d, int k, int renorm, int32_t* __restrict__ topk_idx, float* __restrict__ topk_w,
-                      float* __restrict__ probs) {
-  constexpr int E = 8;
-  extern __shared__ __align__(16) unsigned char s_w[];  // row r at byte 16 * (r + r / 8)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int r = threadIdx.x; r < d; r += blockDim.x)
-    *reinterpret_cast<uint4*>(s_w + 16 * (r + (r >> 3))) = __ldg(reinterpret_cast<const uint4*>(w_router) + r);
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // x may come from the kernel before
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int chunks = d >> 3;
-  const float b0 = (bias && lane < E) ? bias[lane] : 0.f;
-  for (int t = blockIdx.x * kRouteWarps + wib; t < T; t += gridDim.x * kRouteWarps) {
-    const XT* xr = x + (size_t)t * d;
-    float acc[E];
+__global__ void __launch_bounds__(kRtWarps * 32)
+    route_tile_kernel(const XT* __restrict__ x, const uint16_t* __restrict__ w_router, const float* __restrict__ bias, int T,
+                      int d, int E, int k, int renorm, int32_t* topk_idx, float* __restrict__ topk_w,
+                      float* __restrict__ probs, Grouping grp, DeviceState* st) {
+  constexpr int NT = sizeof(XT) == 4 ? 3 : 1;  // bf16 terms of a value
+  extern __shared__ __align__(128) unsigned char rt_smem[];
+  const RtShape sh = rt_shape(d, E);
+  float* const part = reinterpret_cast<float*>(rt_smem + sh.part_off);  // [warp][token][expert]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_launch_dependents();
+  const int units = (d + kRtUnit - 1) / kRtUnit;
+  for (int r = tid; r < units * kRtUnit; r += kRtWarps * 32) {
+    for (int e8 = 0; e8 < sh.e8; e8 += 8) {
+      uint16_t v[8];
+      if (r < d && (E & 7) == 0) {
+        *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(w_router + (size_t)r * E + e8));
+      } else {
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    for (int cb = lane; cb < chunks; cb += 32 * 8) {
-      float xv[8][8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = cb + 32 * u;
-        if (c < chunks) {
-          load_x8<XT>(xr + c * 8, xv[u]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) xv[u][i] = 0.f;
-        }
+        for (int e = 0; e < 8; ++e) v[e] = r < d && e8 + e < E ? __ldg(w_router + (size_t)r * E + e8 + e) : (uint16_t)0;
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = min(cb + 32 * u, chunks - 1);  // clamped rows meet zero inputs
-        const unsigned char* rows = s_w + 16 * (9 * c);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float wv[8];
-          unpack8(*reinterpret_cast<const uint4*>(rows + 16 * i), wv);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[j] = fmaf(xv[u][i], wv[j], acc[j]);
-        }
-      }
+      for (int e = 0; e < 8; ++e) *reinterpret_cast<uint16_t*>(rt_smem + (e8 + e) * sh.row_bytes + r * 2) = v[e];
     }
-    float l0 = 0.f;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const float v = warp_sum(acc[e]);
-      if (lane == e) l0 = v;
-    }
-    l0 += b0;
-    warp_route_finish(l0, 0.f, E, k, renorm, lane, topk_idx + (size_t)t * k, topk_w + (size_t)t * k,
-                      probs ? probs + (size_t)t * E : nullptr);
   }
+  pdl_wait();  // x may come from the kernel before
+  __syncthreads();
+  const int t0 = blockIdx.x * kRtTokens, g = lane >> 2, q = lane & 3;
+  const XT* const row0 = x + (size_t)min(t0 + g, T - 1) * d + q * 8;
+  const XT* const row1 = x + (size_t)min(t0 + g + 8, T - 1) * d + q * 8;
+  float* const mine = part + (warp * kRtTokens + g) * sh.e8 + 2 * q;
+  for (int u0 = warp; u0 < units || u0 == warp; u0 += kRtWarps * kRtBatch) {
+    uint4 a[kRtBatch][2][NT];
+#pragma unroll
+    for (int j = 0; j < kRtBatch; ++j)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = (u0 + j * kRtWarps) * kRtUnit;
+        const bool in = c + q * 8 < d;  // (what lies past the row: zeros)
+        const XT* src = (h ? row1 : row0) + (in ? c : 0);
+        if constexpr (NT == 1) {
+          a[j][h][0] = *reinterpret_cast<const uint4*>(src);
+          if (!in) a[j][h][0] = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+          float f[8];
+          load_x8<XT>(src, f);
+          uint16_t tm[8][3];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) split3(in ? f[i] : 0.f, tm[i]);
+#pragma unroll
+          for (int t = 0; t < NT; ++t)
+            a[j][h][t] = make_uint4(tm[0][t] | (uint32_t)tm[1][t] << 16, tm[2][t] | (uint32_t)tm[3][t] << 16,
+                                    tm[4][t] | (uint32_t)tm[5][t] << 16, tm[6][t] | (uint32_t)tm[7][t] << 16);
+        }
+      }
+    for (int e8 = 0; e8 < sh.e8; e8 += 8) {
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      const unsigned char* wrow = rt_smem + (e8 + g) * sh.row_bytes + q * 16;
+#pragma unroll
+      for (int j0 = 0; j0 < kRtBatch; j0 += 2) {
+        float m[NT][4];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) m[t][0] = m[t][1] = m[t][2] = m[t][3] = 0.f;
+#pragma unroll
+        for (int j = j0; j < j0 + 2; ++j) {
+          const int u = u0 + j * kRtWarps;
+          const uint4 b = *reinterpret_cast<const uint4*>(wrow + min(u, units - 1) * (kRtUnit * 2));
+#pragma unroll
+          for (int t = 0; t < NT; ++t) {
+            mma16(m[t], a[j][0][t].x, a[j][1][t].x, a[j][0][t].y, a[j][1][t].y, b.x, b.y);
+            mma16(m[t], a[j][0][t].z, a[j][1][t].z, a[j][0][t].w, a[j][1][t].w, b.z, b.w);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int t = NT - 1; t >= 0; --t) s[i] += m[t][i];
+      }
+      float* dst = mine + e8;  // D: tokens g and g + 8, experts 2q and 2q + 1
+      if (u0 == warp) {
+        dst[0] = s[0], dst[1] = s[1], dst[8 * sh.e8] = s[2], dst[8 * sh.e8 + 1] = s[3];
+      } else {
+        dst[0] += s[0], dst[1] += s[1], dst[8 * sh.e8] += s[2], dst[8 * sh.e8 + 1] += s[3];
+      }
+    }
+  }
+  __syncthreads();
+  {
+    const int t = t0 + warp;  // a warp finishes one token
+    if (t < T) {
+      float l0 = 0.f, l1 = 0.f;
+      const float* p = part + warp * sh.e8 + lane;
+      const int step = kRtTokens * sh.e8;
+      if (lane < E) {
+#pragma unroll
+        for (int w = 0; w < kRtWarps; ++w) l0 += p[w * step];
+        if (bias) l0 += bias[lane];
+      }
+      if (lane + 32 < E) {
+#pragma unroll
+        for (int w = 0; w < kRtWarps; ++w) l1 += p[w * step + 32];
+        if (bias) l1 += bias[lane + 32];
+      }
+      warp_route_finish(l0, l1, E, k, renorm, lane, topk_idx + (size_t)t * k, topk_w + (size_t)t * k,
+                        probs ? probs + (size_t)t * E : nullptr);
+    }
+  }
+  if (!grp.perm) return;
+  // ---- the last CTA groups the pairs
+  __shared__ int s_last, s_base[MOE_MAX_EXPERTS + 1];
+  __syncthreads();
+  if (tid == 0) {
+    // (release: the CTA's routing, ordered before this thread by the barrier; acquire: the other CTAs')
+    const unsigned old = atom_add_acq_rel(&st->route_done, 1u);
+    s_last = old == gridDim.x - 1u;
+    if (s_last) st->route_done = 0u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  int* const count = reinterpret_cast<int*>(part);  // [warp][expert]
+  for (int i = tid; i < kRtWarps * MOE_MAX_EXPERTS; i += kRtWarps * 32) count[i] = 0;
+  __syncthreads();
+  const int n = T * k, per = (n + kRtWarps * 32 - 1) / (kRtWarps * 32) * 32;
+  const int lo = warp * per, hi = min(n, lo + per);
+  int* const wc = count + warp * MOE_MAX_EXPERTS;
+  const unsigned below = (1u << lane) - 1u;
+  constexpr int kKeep = 8;  // pairs per lane kept in registers between the two walks
+  int keep[kKeep];
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    const int p = lo + i * 32 + lane;
+    keep[i] = p < hi ? __ldcg(topk_idx + p) : -1;
+  }
+  auto each = [&](auto&& body) {
+#pragma unroll
+    for (int i = 0; i < kKeep; ++i)
+      if (lo + i * 32 < hi) body(lo + i * 32 + lane, keep[i]);
+    for (int p0 = lo + kKeep * 32; p0 < hi; p0 += 32) body(p0 + lane, p0 + lane < hi ? __ldcg(topk_idx + p0 + lane) : -1);
+  };
+  each([&](int, int e) {
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    if (e >= 0 && (peers & below) == 0u) wc[e] += __popc(peers);
+    __syncwarp();
+  });
+  __syncthreads();
+  if (tid < MOE_MAX_EXPERTS) {
+    int run = 0;
+    for (int w = 0; w < kRtWarps; ++w) {
+      const int c = count[w * MOE_MAX_EXPERTS + tid];
+      count[w * MOE_MAX_EXPERTS + tid] = run;  // within the expert: where the warp's pairs start
+      run += c;
+    }
+    s_base[tid] = run;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int c0 = s_base[lane], c1 = s_base[lane + 32];
+    int a0 = c0, a1 = c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v0 = __shfl_up_sync(0xffffffffu, a0, o), v1 = __shfl_up_sync(0xffffffffu, a1, o);
+      if (lane >= o) a0 += v0, a1 += v1;
+    }
+    const int tot0 = __shfl_sync(0xffffffffu, a0, 31);
+    __syncwarp();
+    s_base[lane] = a0 - c0, s_base[lane + 32] = tot0 + a1 - c1;
+    if (lane < E) grp.offsets[lane] = a0 - c0;
+    if (lane + 32 < E) grp.offsets[lane + 32] = tot0 + a1 - c1;
+    if (lane == 0) grp.offsets[E] = n;
+  }
+  __syncthreads();
+  each([&](int p, int e) {
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    const int base = e >= 0 ? s_base[e] + wc[e] : 0;
+    __syncwarp();
+    if (e >= 0) {
+      const int slot = base + __popc(peers & below);
+      grp.perm[slot] = p;
+      grp.inv[p] = slot;
+      if ((peers & below) == 0u) wc[e] += __popc(peers);
+    }
+    __syncwarp();
+  });
 }
 
 // Few tokens (decode): one CTA per token, all 256 threads split the d axis so the weight rows are
@@ -200,29 +348,23 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
 
 template <typename XT>
 static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt,
-                          float* probs, cudaStream_t s) {
+                          float* probs, cudaStream_t s, const Grouping* grp) {
   const moe_config& c = ctx->cfg;
-  const dim3 block(kRouteWarps * 32);
-  const bool few = T <= 64;
-  const dim3 grid(few ? T : (T + kRouteWarps - 1) / kRouteWarps);
   const XT* xp = (const XT*)x;
   const uint16_t* wr = (const uint16_t*)w->w_router;
-  const size_t staged = 18 * (size_t)c.d_model;  // bytes of the shifted copy of W_r (8 experts)
-  if (!few && c.n_experts == 8 && staged <= 96 * 1024) {
-    MOE_TRY(allow_full_smem<route_smem_kernel<XT>>(ctx));
-    const int ctas = (T + kRouteWarps - 1) / kRouteWarps;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(ctas < 2 * ctx->sm_count ? ctas : 2 * ctx->sm_count), lc.blockDim = block;
-    lc.dynamicSmemBytes = staged, lc.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr, lc.numAttrs = 1;
-    MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, route_smem_kernel<XT>, xp, wr, (const float*)w->b_router, T, c.d_model, c.top_k,
-                                    c.renorm, idx, wt, probs));
+  const RtShape sh = rt_shape(c.d_model, c.n_experts);
+  // more than a decode step's tokens, and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 24 experts)
+  if (T > MOE_STREAM_MAX_TOKENS && sh.smem <= 112 * 1024) {
+    MOE_TRY(allow_full_smem<route_tile_kernel<XT>>(ctx));
+    MOE_CUDA_TRY(launch_pdl(route_tile_kernel<XT>, dim3((T + kRtTokens - 1) / kRtTokens), dim3(kRtWarps * 32), (size_t)sh.smem, s,
+                            xp, wr, w->b_router, T, c.d_model, c.n_experts, c.top_k, c.renorm, idx, wt, probs,
+                            grp ? *grp : Grouping{nullptr, nullptr, nullptr}, ctx->d_state));
     ctx->launches++;
     return MOE_OK;
   }
+  const dim3 block(kRouteWarps * 32);
+  const bool few = T <= 64;
+  const dim3 grid(few ? T : (T + kRouteWarps - 1) / kRouteWarps);
 #define ROUTE_CASE(EM)                                                                                                \
   MOE_CUDA_TRY(launch_pdl(few ? route_block_kernel<XT, EM> : route_kernel<XT, EM>, grid, block, 0, s, xp, wr, w->b_router, \
                           T, c.d_model, c.n_experts, c.top_k, c.renorm, idx, wt, probs))
@@ -236,13 +378,13 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
     ROUTE_CASE(64);
 #undef ROUTE_CASE
   ctx->launches++;
-  return MOE_OK;
+  return grp ? launch_permute(ctx, idx, T, grp->offsets, grp->perm, grp->inv, s) : MOE_OK;
 }
 
 int launch_route(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt, float* probs,
-                 cudaStream_t s) {
-  if (ctx->cfg.x_dtype == MOE_F32) return launch_route_t<float>(ctx, x, T, w, idx, wt, probs, s);
-  return launch_route_t<__nv_bfloat16>(ctx, x, T, w, idx, wt, probs, s);
+                 cudaStream_t s, const Grouping* grp) {
+  if (ctx->cfg.x_dtype == MOE_F32) return launch_route_t<float>(ctx, x, T, w, idx, wt, probs, s, grp);
+  return launch_route_t<__nv_bfloat16>(ctx, x, T, w, idx, wt, probs, s, grp);
 }
 
 // ------------------------------------------------------------------------------------ grouping

@@ -206,25 +206,6 @@ __device__ __forceinline__ uint64_t l2_policy_normal() {
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-// 16 rows x 16 values times 16 values x 8 tokens; a row's (a token's) two registers hold 4 of its values per lane
-__device__ __forceinline__ void mma16(float* c, uint32_t a_lo0, uint32_t a_hi0, uint32_t a_lo1, uint32_t a_hi1, uint32_t b0,
-                                      uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a_lo0), "r"(a_hi0), "r"(a_lo1), "r"(a_hi1), "r"(b0), "r"(b1));
-}
-
-// fp32 -> three bf16 terms, the largest first: each remainder is exact in fp32
-__device__ __forceinline__ void split3(float v, uint16_t* out) {
-#pragma unroll
-  for (int i = 0; i < kTerms; ++i) {
-    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-    out[i] = __bfloat16_as_ushort(b);
-    v -= __bfloat162float(b);
-  }
-}
-
 // All groups of one product by one consumer warp.  The loops stay rolled and serve all products (bf16 token rows meet
 // zeros as their second and third term): a launch runs each of them a few dozen times only, and code that is fetched
 // anew from L2 for every tile costs more than the idle columns.
