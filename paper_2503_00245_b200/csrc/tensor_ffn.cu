@@ -74,6 +74,7 @@ struct GGParams {
   int ksplit;             // the contraction is cut into this many parts, each a work item of its own ...
   long long plane_elems;  // ... writing its partial sums plane_elems further on in `out` (EPI_F32 only)
   int n_stages;
+  int resident;  // 1: A = [hi | lo] (2 K columns) resident in shared memory, K the contraction length of B
   DeviceState* st;
 };
 
@@ -106,8 +107,10 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t r
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(smem_ptr)), "r"(rank));
   return r;
 }
+// (Release at CTA scope: what the arrival hands over are tensor-memory columns, ordered by tcgen05.wait::ld and the tcgen05
+// fence.  A release at cluster scope also waits for the warp's stores to memory, about a microsecond per tile.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -174,6 +177,7 @@ __device__ __forceinline__ uint32_t instr_desc(int n, bool b_nmajor) {
 struct SmemGG {
   uint64_t full[kMaxStagesGG];   // leader's: both CTAs' operands of the stage have landed
   uint64_t empty[kMaxStagesGG];  // own: the MMAs have finished reading this CTA's stage
+  uint64_t a_full, a_empty;      // RES: leader's: both CTAs' A has landed; own: the MMAs have finished reading this CTA's A
   uint64_t accum_full[2];        // own: all MMAs of the tile in accumulator buffer b have completed
   uint64_t accum_empty[2];       // leader's: the epilogue warps of both CTAs have read buffer b out of TMEM
   uint32_t tmem_base;
@@ -242,6 +246,11 @@ __device__ __forceinline__ void store_bf16(unsigned char* buf, int lane, const u
   }
 }
 
+// RES: the whole A operand of a row tile -- [hi | lo] halves of a split operand, 2 P.K values per row -- stays in shared
+// memory while a pair walks a contiguous run of the tiles (columns of one row tile after the other), and a slice of B serves
+// both halves.  For short contractions over a split intermediate (rank <= 128 or 256), where the plain form brings A in
+// again for every column tile and B twice: 192 KB per CTA and tile instead of 32 KB.
+template <bool RES>
 __global__ void __launch_bounds__(kThreadsGG, 1)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                         const __grid_constant__ CUtensorMap map_b, const GGParams P) {
@@ -252,8 +261,10 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   const uint32_t n_a = P.bmode == B_DUAL ? 2u : 1u;
   const uint32_t b_rows = (P.bmode == B_PAIR || P.bmode == B_DUAL) ? (uint32_t)P.bn : (uint32_t)P.bn / 2u;  // per CTA
   const uint32_t b_bytes = b_rows * kBK * 2;
-  const uint32_t stage_bytes = n_a * a_bytes + 128u * kBK * 2u;
-  unsigned char* stages = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t stage_bytes = (RES ? 0u : n_a * a_bytes) + 128u * kBK * 2u;
+  unsigned char* const smem0 = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int res_kb = RES ? 2 * ((P.K + kBK - 1) / kBK) : 0;  // K slices of the resident A operand(s)
+  unsigned char* const stages = smem0 + (size_t)res_kb * n_a * a_bytes;
   unsigned char* const epi_bufs = stages + (size_t)P.n_stages * stage_bytes;  // 2 KB per epilogue warp
   SmemGG& sm = *reinterpret_cast<SmemGG*>(epi_bufs + kEpiWarps * kEpiBuf);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -273,6 +284,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       mbar_init(&sm.accum_full[b], 1);
       mbar_init(&sm.accum_empty[b], 2 * kEpiWarps);
     }
+    if (RES) mbar_init(&sm.a_full, 1), mbar_init(&sm.a_empty, 1);
     sm.abort = 0;
     fence_mbar_init();
     fence_proxy_async_smem();
@@ -302,6 +314,11 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   Tile t;
+  // this pair's tiles: dealt out in turn, or (RES) a contiguous run
+  const int n_work = RES ? sm.tile_prefix[P.E] * n_tiles * P.ksplit : 0x7fffffff;
+  const int idx0 = RES ? (int)((long long)n_work * pair / n_pairs) : pair;
+  const int idx1 = RES ? (int)((long long)n_work * (pair + 1) / n_pairs) : n_work;
+  const int idx_step = RES ? 1 : n_pairs;
 
   if (warp == 0) {
     // ================================================================= TMA producer (both CTAs)
@@ -309,14 +326,30 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       int it = 0;              // k-blocks issued so far, over all tiles
       uint32_t slot = 0, par = 1;  // ring position; parity of the `empty` phase the slot's next fill waits for
       bool ok = true;
-      const uint32_t tx_pair = 2u * (n_a * a_bytes + b_bytes);  // bytes both CTAs bring in per stage
+      const uint32_t tx_pair = 2u * ((RES ? 0u : n_a * a_bytes) + b_bytes);  // bytes both CTAs bring in per stage
+      int a_m0 = -1, a_n = 0;  // RES: the row tile whose A is resident, row tiles brought in so far
       const uint32_t full0 = map_to_rank(&sm.full[0], 0u);      // the leader's stage barriers, 8 bytes apart
       const int half_bn = P.bn / 2;
-      for (int idx = pair; ok && decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs) {
+      for (int idx = idx0; ok && idx < idx1 && decode_tile(P, sm, idx, n_tiles, t); idx += idx_step) {
         const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
         const int a_row = t.m0 + (int)rank * kBM;
         int k0 = kb0 * kBK;
         int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
+        if (RES && t.m0 != a_m0) {
+          if (a_n > 0 && !mbar_wait(&sm.a_empty, (a_n - 1) & 1)) {
+            flag_error(P.st, MOE_ERR_TIMEOUT, 0x404u);
+            sm.abort = 1;
+            ok = false;
+            break;
+          }
+          if (rank == 0) mbar_arrive_expect_tx(&sm.a_full, 2u * (uint32_t)res_kb * n_a * a_bytes);
+          const uint32_t abar = map_to_rank(&sm.a_full, 0u);
+          for (int i = 0; i < res_kb; ++i) {
+            tma_load_2d(smem0 + (size_t)i * a_bytes, &map_a0, i * kBK, a_row, abar);
+            if (P.bmode == B_DUAL) tma_load_2d(smem0 + (size_t)(res_kb + i) * a_bytes, &map_a1, i * kBK, a_row, abar);
+          }
+          a_m0 = t.m0, ++a_n;
+        }
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           if (it >= NS && !mbar_wait(&sm.empty[slot], par)) {
             flag_error(P.st, MOE_ERR_TIMEOUT, 0x400u);
@@ -325,15 +358,15 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
             break;
           }
           unsigned char* st_a0 = stages + (size_t)slot * stage_bytes;
-          unsigned char* st_b = st_a0 + n_a * a_bytes;
+          unsigned char* st_b = st_a0 + (RES ? 0u : n_a * a_bytes);
           const uint32_t bar = full0 + 8u * slot;
           if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], tx_pair);
-          tma_load_2d(st_a0, &map_a0, k0, a_row, bar);
+          if (!RES) tma_load_2d(st_a0, &map_a0, k0, a_row, bar);
           if (P.bmode == B_PAIR) {
             tma_load_4d(st_b, &map_b, kB, (int)rank, t.n0, t.e, bar);
           } else if (P.bmode == B_DUAL) {
             const int nr = t.n0 + (int)rank * half_bn;
-            tma_load_2d(st_a0 + a_bytes, &map_a1, k0, a_row, bar);
+            if (!RES) tma_load_2d(st_a0 + a_bytes, &map_a1, k0, a_row, bar);
             tma_load_4d(st_b, &map_b, kB, 0, nr, t.e, bar);
             tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, t.e, bar);
           } else if (P.bmode == B_SINGLE) {
@@ -350,6 +383,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       }
       if (!ok && rank == 0) {  // copies in flight (both CTAs' complete on these barriers) must land before the pair goes away
         for (int j = max(0, it - NS); j < it; ++j) (void)mbar_wait(&sm.full[j % NS], (j / NS) & 1);
+        if (RES && a_n > 0) (void)mbar_wait(&sm.a_full, (a_n - 1) & 1);
       }
     }
   } else if (warp == 1) {
@@ -365,12 +399,22 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       const uint32_t lo_b_lbo = (P.bmode == B_NMAJOR ? (uint32_t)(64 * kBK * 2 >> 4) : 1u) << 16;
       const uint32_t b_step = P.bmode == B_NMAJOR ? (2048u >> 4) : (32u >> 4);
       const uint32_t stage0 = smem_u32(stages) >> 4, stage_step = stage_bytes >> 4;
-      const uint32_t b_off = (n_a * a_bytes) >> 4, a1_off = a_bytes >> 4, b1_off = ((uint32_t)(P.bn / 2) * kBK * 2) >> 4;
+      const uint32_t b_off = RES ? 0u : (n_a * a_bytes) >> 4, a1_off = a_bytes >> 4, b1_off = ((uint32_t)(P.bn / 2) * kBK * 2) >> 4;
       uint32_t slot = 0, par = 0, st_lo = stage0;
       int tile_i = 0;
       bool ok = true;
-      for (int idx = pair; ok && decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs, ++tile_i) {
+      int a_m0 = -1, a_n = 0;
+      for (int idx = idx0; ok && idx < idx1 && decode_tile(P, sm, idx, n_tiles, t); idx += idx_step, ++tile_i) {
         const int buf = tile_i & 1;
+        if (RES && t.m0 != a_m0) {
+          if (a_n > 0) tc_commit_pair(&sm.a_empty);  // the MMAs of the row tile before are the last to read its A
+          if (!mbar_wait(&sm.a_full, a_n & 1)) {
+            flag_error(P.st, MOE_ERR_TIMEOUT, 0x405u);
+            sm.abort = 1;
+            break;
+          }
+          a_m0 = t.m0, ++a_n;
+        }
         if (tile_i >= 2) {  // the accumulators two tiles back must have left this buffer, in both CTAs
           if (!mbar_wait(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1)) {
             flag_error(P.st, MOE_ERR_TIMEOUT, 0x403u);
@@ -392,7 +436,23 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           tc_fence_after();
           const uint64_t da = hi_k | (uint64_t)(st_lo | (1u << 16));
           const uint64_t db = hi_b | (uint64_t)((st_lo + b_off) | lo_b_lbo);
-          if (P.bmode == B_DUAL) {
+          if (RES) {
+            const uint32_t a_slice = a_bytes >> 4, res0 = smem_u32(smem0) >> 4;
+            const uint64_t dh = hi_k | (uint64_t)((res0 + (uint32_t)kb * a_slice) | (1u << 16));
+            const uint64_t dl = dh + (uint32_t)(res_kb / 2) * a_slice;
+            const uint32_t a1 = (uint32_t)res_kb * a_slice;
+            const uint64_t db1 = db + b1_off;
+#pragma unroll
+            for (uint32_t kk = 0; kk < kBK / 16; ++kk) {
+              tc_mma_bf16(d_tmem, dh + 2u * kk, db + 2u * kk, idesc, acc | kk);
+              if (P.bmode == B_DUAL) tc_mma_bf16(d_tmem + (uint32_t)P.bn, dh + a1 + 2u * kk, db1 + 2u * kk, idesc, acc | kk);
+            }
+#pragma unroll
+            for (uint32_t kk = 0; kk < kBK / 16; ++kk) {
+              tc_mma_bf16(d_tmem, dl + 2u * kk, db + 2u * kk, idesc, 1u);
+              if (P.bmode == B_DUAL) tc_mma_bf16(d_tmem + (uint32_t)P.bn, dl + a1 + 2u * kk, db1 + 2u * kk, idesc, 1u);
+            }
+          } else if (P.bmode == B_DUAL) {
             const uint64_t da1 = da + a1_off, db1 = db + b1_off;
 #pragma unroll
             for (uint32_t kk = 0; kk < kBK / 16; ++kk) {
@@ -418,7 +478,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     const uint32_t acce_bar[2] = {map_to_rank(&sm.accum_empty[0], 0u), map_to_rank(&sm.accum_empty[1], 0u)};
     unsigned char* const ebuf = epi_bufs + (warp - 2) * kEpiBuf;
     int tile_i = 0;
-    for (int idx = pair; decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs, ++tile_i) {
+    for (int idx = idx0; idx < idx1 && decode_tile(P, sm, idx, n_tiles, t); idx += idx_step, ++tile_i) {
       const int buf = tile_i & 1;
       if (!mbar_wait(&sm.accum_full[buf], (tile_i >> 1) & 1)) {
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x402u);
@@ -554,7 +614,7 @@ int max_pairs(const moe_ctx* ctx, size_t smem) {
   pair_launch_config(lc, attr, ctx->sm_count & ~1, smem, nullptr);
   lc.numAttrs = 1;  // the cluster shape alone decides the occupancy
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, grouped_gemm_kernel, &lc) != cudaSuccess || n < 1) {
+  if (cudaOccupancyMaxActiveClusters(&n, grouped_gemm_kernel<false>, &lc) != cudaSuccess || n < 1) {
     (void)cudaGetLastError();
     n = ctx->sm_count / 2;
   }
@@ -571,17 +631,25 @@ int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const 
   if (P.n_store < P.n_total) P.n_store = P.n_total;
   if (P.ksplit < 1) P.ksplit = 1;
   const int n_tiles = (P.n_total + P.bn - 1) / P.bn;
-  const size_t stage_bytes = (size_t)kBM * kBK * 2 * (P.bmode == B_DUAL ? 2 : 1) + 128 * kBK * 2;
+  const int n_a = P.bmode == B_DUAL ? 2 : 1;
+  const size_t a_tile = (size_t)kBM * kBK * 2;
+  const size_t resident = P.resident ? 2 * (size_t)((P.K + kBK - 1) / kBK) * n_a * a_tile : 0;
+  const size_t stage_bytes = (P.resident ? 0 : n_a * a_tile) + 128 * kBK * 2;
   P.n_stages = P.bmode == B_DUAL ? 4 : kMaxStagesGG;
-  const size_t smem = P.n_stages * stage_bytes + kEpiWarps * kEpiBuf + sizeof(SmemGG) + 1024 + 128;
+  const size_t smem = resident + P.n_stages * stage_bytes + kEpiWarps * kEpiBuf + sizeof(SmemGG) + 1024 + 128;
   if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
-  MOE_TRY(allow_full_smem<grouped_gemm_kernel>(ctx));
   const long long m_tiles = (n_slots + kPairRows - 1) / kPairRows + c.n_experts;  // upper bound
   const int pairs = (int)std::min<long long>(m_tiles * n_tiles * P.ksplit, max_pairs(ctx, smem));
   cudaLaunchConfig_t lc;
   cudaLaunchAttribute attr[2];
   pair_launch_config(lc, attr, 2 * pairs, smem, s);
-  MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, grouped_gemm_kernel, a0, a1, b, P));
+  if (P.resident) {
+    MOE_TRY(allow_full_smem<grouped_gemm_kernel<true>>(ctx));
+    MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, grouped_gemm_kernel<true>, a0, a1, b, P));
+  } else {
+    MOE_TRY(allow_full_smem<grouped_gemm_kernel<false>>(ctx));
+    MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, grouped_gemm_kernel<false>, a0, a1, b, P));
+  }
   ctx->launches++;
   return MOE_OK;
 }
@@ -673,10 +741,13 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   if ((rc = make_map_a(&ma, mid_a, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
   if ((rc = make_map_a(&ma1, (const __nv_bfloat16*)mid_a + tw, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
   if ((rc = make_map_b(&mb, w->wd_b, r, 2, f, E, kBK, 64)) != MOE_OK) return rc;
-  P.K = tw, P.n_total = f, P.bn = 128, P.bmode = B_DUAL, P.b_sub = 0, P.epi = EPI_SWIGLU;
-  P.k_wrap = rp, P.split = 0, P.out = hidden, P.ld_out = f, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
+  // (A of both operands resident: 1 KB per value of the rank, beside 64 KB of B stages)
+  P.resident = rp <= 128;
+  P.K = P.resident ? rp : tw, P.n_total = f, P.bn = 128, P.bmode = B_DUAL, P.b_sub = 0, P.epi = EPI_SWIGLU;
+  P.k_wrap = P.resident ? 0 : rp, P.split = 0, P.out = hidden, P.ld_out = f, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
   if ((rc = launch_gg(ctx, ma, ma1, mb, P, n_slots, s)) != MOE_OK) return rc;
   // (3) V = hidden dL
+  P.resident = 0;
   if ((rc = make_map_a(&ma, hidden, n_slots, f, f)) != MOE_OK) return rc;
   P.bn = pick_bn(r, 256);
   if ((rc = make_map_b(&mb, w->wd_c, f, 1, r, E, kBK, P.bn / 2)) != MOE_OK) return rc;
@@ -687,8 +758,9 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   if ((rc = make_map_a(&ma, mid_b, n_slots, tw, tw)) != MOE_OK) return rc;
   P.bn = pick_bn(d, 256);
   if ((rc = make_map_b(&mb, w->wd_d, r, 1, d, E, kBK, P.bn / 2)) != MOE_OK) return rc;
-  P.K = tw, P.n_total = d, P.bmode = B_SINGLE, P.b_sub = 0, P.epi = EPI_F32;
-  P.k_wrap = rp, P.split = 0, P.out = out_slots, P.ld_out = d, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
+  P.resident = rp <= 128;
+  P.K = P.resident ? rp : tw, P.n_total = d, P.bmode = B_SINGLE, P.b_sub = 0, P.epi = EPI_F32;
+  P.k_wrap = P.resident ? 0 : rp, P.split = 0, P.out = out_slots, P.ld_out = d, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
   return launch_gg(ctx, ma, ma, mb, P, n_slots, s);
 }
 
