@@ -109,6 +109,8 @@ int launch_combine(moe_ctx* ctx, const float* out_slots, const float* wt, const 
                    int planes, cudaStream_t s);
 // out [n] = the sum of `planes` runs of n values, in order
 int launch_sum_planes(moe_ctx* ctx, const float* in, long long n, int planes, float* out, cudaStream_t s);
+// out [rows][hi n | lo n] bf16 = the sum of `planes` [rows][n] fp32, in order, as head and remainder
+int launch_split_planes(moe_ctx* ctx, const float* in, int rows, int n, int planes, void* out, cudaStream_t s);
 int launch_gather_rows(moe_ctx* ctx, const void* x, const int32_t* perm, int n_slots, void* xperm, cudaStream_t s);
 
 // Streaming (decode) path.  mode 0: whole layer from topk (writes y); mode 1: FFN per slot from

@@ -570,6 +570,35 @@ int launch_sum_planes(moe_ctx* ctx, const float* in, long long n, int planes, fl
   return MOE_OK;
 }
 
+// The planes of [rows][n] partial sums added in order and split into bf16 head and remainder: out [rows][hi n | lo n]
+__global__ void split_planes_kernel(const float4* __restrict__ in, int rows, int n, int planes, uint2* __restrict__ out) {
+  const int quads = n / 4;
+  const long long total = (long long)rows * quads;
+  pdl_launch_dependents();
+  pdl_wait();
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    float4 o = in[i];
+    for (int pl = 1; pl < planes; ++pl) {
+      const float4 o2 = in[i + pl * total];
+      o.x += o2.x, o.y += o2.y, o.z += o2.z, o.w += o2.w;
+    }
+    const uint2 hi = make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w));
+    const uint2 lo = make_uint2(pack_bf16x2(o.x - __uint_as_float(hi.x << 16), o.y - __uint_as_float(hi.x & 0xffff0000u)),
+                                pack_bf16x2(o.z - __uint_as_float(hi.y << 16), o.w - __uint_as_float(hi.y & 0xffff0000u)));
+    const long long r = i / quads;
+    out[r * quads + i] = hi;  // row r starts at 2 r quads
+    out[r * quads + i + quads] = lo;
+  }
+}
+
+int launch_split_planes(moe_ctx* ctx, const float* in, int rows, int n, int planes, void* out, cudaStream_t s) {
+  const long long want = ((long long)rows * (n / 4) + 255) / 256;
+  const int grid = (int)(want < 16ll * ctx->sm_count ? want : 16ll * ctx->sm_count);
+  MOE_CUDA_TRY(launch_pdl(split_planes_kernel, dim3(grid), dim3(256), 0, s, (const float4*)in, rows, n, planes, (uint2*)out));
+  ctx->launches++;
+  return MOE_OK;
+}
+
 // ------------------------------------------------------------------------------------ packing
 // in [B][R][C] -> out[b][c][sub][r] with nsub interleaved row kinds: a tiled transpose.
 __global__ void pack_transpose_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, int R, int C,
