@@ -95,6 +95,16 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
       "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar_cluster)
       : "memory");
 }
+// One lane of a converged warp.  The loops that issue loads and MMAs are run by the whole warp, with loop bounds and
+// coordinates taken from lane 0, and only the issuing itself is one lane's: the operands of these instructions live in
+// registers that a warp shares, and inside a branch that one lane takes every operand of every instruction has to be
+// moved there first -- about 100 cycles for each load and MMA.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ int lane0(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -181,6 +191,7 @@ struct SmemGG {
   uint32_t tmem_base;
   int abort;
   int tile_prefix[MOE_MAX_EXPERTS + 1];  // 256-row tiles per expert, exclusive scan
+  int offsets[MOE_MAX_EXPERTS + 1];      // slot ranges per expert
 };
 
 struct Tile {
@@ -189,19 +200,17 @@ struct Tile {
 
 // idx-th tile of this launch: row-tile major, column tile minor (pairs that run side by side share the A rows
 // and sweep the expert's B columns, which then sit in L2 for the expert's other row tiles).
-__device__ __forceinline__ bool decode_tile(const GGParams& P, const SmemGG& sm, int idx, int n_tiles, Tile& t) {
+__device__ __forceinline__ void decode_tile(const GGParams& P, const SmemGG& sm, int idx, int n_tiles, Tile& t) {
   const int per_row = n_tiles * P.ksplit;
   const int mt = idx / per_row, rem = idx - mt * per_row;
   const int nt = rem / P.ksplit;
   t.ks = rem - nt * P.ksplit;
-  if (mt >= sm.tile_prefix[P.E]) return false;
   int e = 0;
   while (sm.tile_prefix[e + 1] <= mt) ++e;
   t.e = e;
-  t.m0 = P.offsets[e] + (mt - sm.tile_prefix[e]) * kPairRows;
-  t.m_end = P.offsets[e + 1];
+  t.m0 = sm.offsets[e] + (mt - sm.tile_prefix[e]) * kPairRows;
+  t.m_end = sm.offsets[e + 1];
   t.n0 = nt * P.bn;
-  return true;
 }
 
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
@@ -258,11 +267,11 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   unsigned char* stages = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* const epi_bufs = stages + (size_t)P.n_stages * stage_bytes;  // 2 KB per epilogue warp
   SmemGG& sm = *reinterpret_cast<SmemGG*>(epi_bufs + kEpiWarps * kEpiBuf);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = lane0(tid >> 5);
   const int NS = P.n_stages;
   const int num_kb = (P.K + kBK - 1) / kBK;
   const int n_tiles = (P.n_total + P.bn - 1) / P.bn;
-  const uint32_t rank = cluster_ctarank();
+  const uint32_t rank = (uint32_t)lane0((int)cluster_ctarank());
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   pdl_launch_dependents();
@@ -276,6 +285,8 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       mbar_init(&sm.accum_empty[b], 2 * kEpiWarps);
     }
     sm.abort = 0;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a0) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
     fence_mbar_init();
     fence_proxy_async_smem();
   }
@@ -288,76 +299,91 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   // everything above touches only this CTA's shared memory and TMEM; the expert offsets and the operands may
   // come from the kernel before
   pdl_wait();
-  if (tid == 0) {
-    int run = 0;
-    for (int i = 0; i < P.E; ++i) {
-      sm.tile_prefix[i] = run;
-      const int rows = P.offsets[i + 1] - P.offsets[i];
-      run += rows > 0 ? (rows + kPairRows - 1) / kPairRows : 0;
+  if (warp == 0) {  // lane l: experts l and l + 32
+    const int o0 = lane <= P.E ? P.offsets[lane] : 0, o1 = lane + 32 <= P.E ? P.offsets[lane + 32] : 0;
+    const int o2 = lane == 0 && P.E == MOE_MAX_EXPERTS ? P.offsets[MOE_MAX_EXPERTS] : 0;
+    if (lane <= P.E) sm.offsets[lane] = o0;
+    if (lane + 32 <= P.E) sm.offsets[lane + 32] = o1;
+    if (lane == 0 && P.E == MOE_MAX_EXPERTS) sm.offsets[MOE_MAX_EXPERTS] = o2;
+    __syncwarp();
+    auto tiles_of = [&](int e) { return e < P.E ? (max(sm.offsets[e + 1] - sm.offsets[e], 0) + kPairRows - 1) / kPairRows : 0; };
+    const int c0 = tiles_of(lane), c1 = tiles_of(lane + 32);
+    int s0 = c0, s1 = c1;  // inclusive scans over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v0 = __shfl_up_sync(0xffffffffu, s0, o), v1 = __shfl_up_sync(0xffffffffu, s1, o);
+      if (lane >= o) s0 += v0, s1 += v1;
     }
-    sm.tile_prefix[P.E] = run;
+    const int tot0 = __shfl_sync(0xffffffffu, s0, 31);
+    sm.tile_prefix[lane + 1] = s0;
+    sm.tile_prefix[lane + 33] = tot0 + s1;
+    if (lane == 0) sm.tile_prefix[0] = 0;
   }
   tc_fence_before();
   __syncthreads();
   __syncwarp();
   cluster_sync_all();  // the other CTA's barriers are initialised before anything is counted on them
   tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
+  const uint32_t tmem = (uint32_t)lane0((int)sm.tmem_base);
+  const int n_work = lane0(sm.tile_prefix[P.E]) * n_tiles * P.ksplit;
   Tile t;
 
   if (warp == 0) {
     // ================================================================= TMA producer (both CTAs)
-    if (lane == 0) {
-      int it = 0;              // k-blocks issued so far, over all tiles
-      uint32_t slot = 0, par = 1;  // ring position; parity of the `empty` phase the slot's next fill waits for
-      bool ok = true;
-      const uint32_t tx_pair = 2u * (n_a * a_bytes + b_bytes);  // bytes both CTAs bring in per stage
-      const uint32_t full0 = map_to_rank(&sm.full[0], 0u);      // the leader's stage barriers, 8 bytes apart
-      const int half_bn = P.bn / 2;
-      for (int idx = pair; ok && decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs) {
-        const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
-        const int a_row = t.m0 + (int)rank * kBM;
-        int k0 = kb0 * kBK;
-        int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          if (it >= NS && !mbar_wait(&sm.empty[slot], par)) {
-            flag_error(P.st, MOE_ERR_TIMEOUT, 0x400u);
-            sm.abort = 1;
-            ok = false;
-            break;
-          }
-          unsigned char* st_a0 = stages + (size_t)slot * stage_bytes;
-          unsigned char* st_b = st_a0 + n_a * a_bytes;
-          const uint32_t bar = full0 + 8u * slot;
+    int it = 0;                  // k-blocks issued so far, over all tiles
+    uint32_t slot = 0, par = 1;  // ring position; parity of the `empty` phase the slot's next fill waits for
+    bool ok = true;
+    const uint32_t tx_pair = 2u * (n_a * a_bytes + b_bytes);  // bytes both CTAs bring in per stage
+    const uint32_t full0 = (uint32_t)lane0((int)map_to_rank(&sm.full[0], 0u));  // the leader's stage barriers, 8 bytes apart
+    const int half_bn = P.bn / 2;
+    for (int idx = pair; ok && idx < n_work; idx += n_pairs) {
+      decode_tile(P, sm, idx, n_tiles, t);
+      const int e = lane0(t.e), n0 = t.n0;
+      const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
+      const int a_row = lane0(t.m0) + (int)rank * kBM;
+      int k0 = kb0 * kBK;
+      int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
+      for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        if (it >= NS && !__all_sync(0xffffffffu, mbar_wait(&sm.empty[slot], par))) {
+          if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x400u);
+          sm.abort = 1;
+          ok = false;
+          break;
+        }
+        unsigned char* st_a0 = stages + (size_t)slot * stage_bytes;
+        unsigned char* st_b = st_a0 + n_a * a_bytes;
+        const uint32_t bar = full0 + 8u * slot;
+        if (elect_one()) {
           if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], tx_pair);
           tma_load_2d(st_a0, &map_a0, k0, a_row, bar);
           if (P.bmode == B_PAIR) {
-            tma_load_4d(st_b, &map_b, kB, (int)rank, t.n0, t.e, bar);
+            tma_load_4d(st_b, &map_b, kB, (int)rank, n0, e, bar);
           } else if (P.bmode == B_DUAL) {
-            const int nr = t.n0 + (int)rank * half_bn;
+            const int nr = n0 + (int)rank * half_bn;
             tma_load_2d(st_a0 + a_bytes, &map_a1, k0, a_row, bar);
-            tma_load_4d(st_b, &map_b, kB, 0, nr, t.e, bar);
-            tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, t.e, bar);
+            tma_load_4d(st_b, &map_b, kB, 0, nr, e, bar);
+            tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, e, bar);
           } else if (P.bmode == B_SINGLE) {
-            tma_load_4d(st_b, &map_b, kB, P.b_sub, t.n0 + (int)rank * half_bn, t.e, bar);
+            tma_load_4d(st_b, &map_b, kB, P.b_sub, n0 + (int)rank * half_bn, e, bar);
           } else {
-            const int nc = t.n0 + (int)rank * half_bn;
-            for (int j = 0; j < P.bn / 128; ++j)
-              tma_load_4d(st_b + (size_t)j * 64 * kBK * 2, &map_b, nc + 64 * j, P.b_sub, kB, t.e, bar);
+            const int nc = n0 + (int)rank * half_bn;
+            tma_load_4d(st_b, &map_b, nc, P.b_sub, kB, e, bar);
+            if (P.bn > 128) tma_load_4d(st_b + (size_t)64 * kBK * 2, &map_b, nc + 64, P.b_sub, kB, e, bar);
           }
-          k0 += kBK, kB += kBK;
-          if (P.k_wrap > 0 && kB >= P.k_wrap) kB -= P.k_wrap;
-          if (++slot == (uint32_t)NS) slot = 0, par ^= 1u;
         }
+        __syncwarp();
+        k0 += kBK, kB += kBK;
+        if (P.k_wrap > 0 && kB >= P.k_wrap) kB -= P.k_wrap;
+        if (++slot == (uint32_t)NS) slot = 0, par ^= 1u;
       }
-      if (!ok && rank == 0) {  // copies in flight (both CTAs' complete on these barriers) must land before the pair goes away
-        for (int j = max(0, it - NS); j < it; ++j) (void)mbar_wait(&sm.full[j % NS], (j / NS) & 1);
-      }
+    }
+    if (!ok && rank == 0) {  // copies in flight (both CTAs' complete on these barriers) must land before the pair goes away
+      for (int j = max(0, it - NS); j < it; ++j) (void)mbar_wait(&sm.full[j % NS], (j / NS) & 1);
     }
   } else if (warp == 1) {
     // ================================================================= MMA issuer (leader CTA only)
-    if (lane == 0 && rank == 0) {
-      // One thread feeds the tensor cores of both SMs, so its instruction stream is kept short: the ring position
+    if (rank == 0) {
+      // One warp feeds the tensor cores of both SMs, so its instruction stream is kept short: the ring position
       // is a counter, not a division, and the operand descriptors are a constant high word plus a low word that
       // steps through the stage (K-major operands: 32 bytes per 16 k-values; N-major: 16 k-rows of 128 bytes).
       const int n_mma = P.bmode == B_PAIR ? 2 * P.bn : P.bn;
@@ -366,27 +392,28 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       const uint64_t hi_b = (P.bmode == B_NMAJOR ? smem_desc(0, 64 * kBK * 2, 1024) : smem_desc(0, 16, 1024)) & 0xffffffff00000000ull;
       const uint32_t lo_b_lbo = (P.bmode == B_NMAJOR ? (uint32_t)(64 * kBK * 2 >> 4) : 1u) << 16;
       const uint32_t b_step = P.bmode == B_NMAJOR ? (2048u >> 4) : (32u >> 4);
-      const uint32_t stage0 = smem_u32(stages) >> 4, stage_step = stage_bytes >> 4;
+      const uint32_t stage0 = (uint32_t)lane0((int)(smem_u32(stages) >> 4)), stage_step = stage_bytes >> 4;
       const uint32_t b_off = (n_a * a_bytes) >> 4, a1_off = a_bytes >> 4, b1_off = ((uint32_t)(P.bn / 2) * kBK * 2) >> 4;
       uint32_t slot = 0, par = 0, st_lo = stage0;
       int tile_i = 0;
       bool ok = true;
-      for (int idx = pair; ok && decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs, ++tile_i) {
+      for (int idx = pair; ok && idx < n_work; idx += n_pairs, ++tile_i) {
         const int buf = tile_i & 1;
         if (tile_i >= 2) {  // the accumulators two tiles back must have left this buffer, in both CTAs
-          if (!mbar_wait(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1)) {
-            flag_error(P.st, MOE_ERR_TIMEOUT, 0x403u);
+          if (!__all_sync(0xffffffffu, mbar_wait(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1))) {
+            if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x403u);
             sm.abort = 1;
             break;
           }
           tc_fence_after();
         }
         const uint32_t d_tmem = tmem + (uint32_t)(buf * kAccCols);
-        const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
+        const int ks = idx % P.ksplit;
+        const int kb0 = ks * num_kb / P.ksplit, kb1 = (ks + 1) * num_kb / P.ksplit;
         uint32_t acc = 0;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&sm.full[slot], par)) {
-            flag_error(P.st, MOE_ERR_TIMEOUT, 0x401u);
+          if (!__all_sync(0xffffffffu, mbar_wait(&sm.full[slot], par))) {
+            if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x401u);
             sm.abort = 1;
             ok = false;
             break;
@@ -394,23 +421,26 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           tc_fence_after();
           const uint64_t da = hi_k | (uint64_t)(st_lo | (1u << 16));
           const uint64_t db = hi_b | (uint64_t)((st_lo + b_off) | lo_b_lbo);
-          if (P.bmode == B_DUAL) {
-            const uint64_t da1 = da + a1_off, db1 = db + b1_off;
+          if (elect_one()) {
+            if (P.bmode == B_DUAL) {
+              const uint64_t da1 = da + a1_off, db1 = db + b1_off;
 #pragma unroll
-            for (uint32_t kk = 0; kk < kBK / 16; ++kk) {
-              tc_mma_bf16(d_tmem, da + 2u * kk, db + 2u * kk, idesc, acc | kk);
-              tc_mma_bf16(d_tmem + (uint32_t)P.bn, da1 + 2u * kk, db1 + 2u * kk, idesc, acc | kk);
+              for (uint32_t kk = 0; kk < kBK / 16; ++kk) {
+                tc_mma_bf16(d_tmem, da + 2u * kk, db + 2u * kk, idesc, acc | kk);
+                tc_mma_bf16(d_tmem + (uint32_t)P.bn, da1 + 2u * kk, db1 + 2u * kk, idesc, acc | kk);
+              }
+            } else {
+#pragma unroll
+              for (uint32_t kk = 0; kk < kBK / 16; ++kk) tc_mma_bf16(d_tmem, da + 2u * kk, db + b_step * kk, idesc, acc | kk);
             }
-          } else {
-#pragma unroll
-            for (uint32_t kk = 0; kk < kBK / 16; ++kk) tc_mma_bf16(d_tmem, da + 2u * kk, db + b_step * kk, idesc, acc | kk);
+            tc_commit_pair(&sm.empty[slot]);  // both CTAs' producers may refill the stage once these MMAs have read it
+            if (kb + 1 == kb1) tc_commit_pair(&sm.accum_full[buf]);
           }
+          __syncwarp();
           acc = 1;
-          tc_commit_pair(&sm.empty[slot]);  // both CTAs' producers may refill the stage once these MMAs have read it
           st_lo += stage_step;
           if (++slot == (uint32_t)NS) slot = 0, par ^= 1u, st_lo = stage0;
         }
-        if (ok) tc_commit_pair(&sm.accum_full[buf]);
       }
     }
   } else {
@@ -420,7 +450,8 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     const uint32_t acce_bar[2] = {map_to_rank(&sm.accum_empty[0], 0u), map_to_rank(&sm.accum_empty[1], 0u)};
     unsigned char* const ebuf = epi_bufs + (warp - 2) * kEpiBuf;
     int tile_i = 0;
-    for (int idx = pair; decode_tile(P, sm, idx, n_tiles, t); idx += n_pairs, ++tile_i) {
+    for (int idx = pair; idx < n_work; idx += n_pairs, ++tile_i) {
+      decode_tile(P, sm, idx, n_tiles, t);
       const int buf = tile_i & 1;
       if (!mbar_wait(&sm.accum_full[buf], (tile_i >> 1) & 1)) {
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x402u);
