@@ -42,7 +42,7 @@ constexpr int kThreadsGG = (2 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;  // two accumulator buffers of 256 columns
 constexpr int kAccCols = 256;
 constexpr int kMaxStagesGG = 6;
-constexpr int kEpiBuf = 2048;
+constexpr int kEpiBuf = 4096;
 constexpr int kPairRows = 2 * kBM;  // rows of a pair's tile
 
 enum Epi { EPI_SWIGLU = 0, EPI_BF16_PAIR = 1, EPI_BF16 = 2, EPI_F32 = 3 };
@@ -190,27 +190,55 @@ struct SmemGG {
   uint64_t accum_empty[2];       // leader's: the epilogue warps of both CTAs have read buffer b out of TMEM
   uint32_t tmem_base;
   int abort;
-  int tile_prefix[MOE_MAX_EXPERTS + 1];  // 256-row tiles per expert, exclusive scan
-  int offsets[MOE_MAX_EXPERTS + 1];      // slot ranges per expert
 };
 
 struct Tile {
   int e, m0, m_end, n0, ks;
 };
 
+// The experts' slot ranges and tiles, spread over a warp's lanes (lane l: experts l and l + 32).  Every warp keeps its own:
+// nothing has to be published to the CTA between the dependency wait and the first load.
+struct TileMap {
+  int lo0, lo1, hi0, hi1;  // slots [lo, hi)
+  int p0, p1;              // 256-row tiles of the experts up to and including this one
+  int total;
+};
+__device__ __forceinline__ TileMap read_tile_map(const GGParams& P, int lane) {
+  TileMap m;
+  const int e0 = min(lane, P.E), e1 = min(lane + 32, P.E);
+  m.lo0 = P.offsets[e0], m.hi0 = P.offsets[min(e0 + 1, P.E)];
+  m.lo1 = P.offsets[e1], m.hi1 = P.offsets[min(e1 + 1, P.E)];
+  m.p0 = (max(m.hi0 - m.lo0, 0) + kPairRows - 1) / kPairRows;
+  m.p1 = (max(m.hi1 - m.lo1, 0) + kPairRows - 1) / kPairRows;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v0 = __shfl_up_sync(0xffffffffu, m.p0, o), v1 = __shfl_up_sync(0xffffffffu, m.p1, o);
+    if (lane >= o) m.p0 += v0, m.p1 += v1;
+  }
+  m.p1 += __shfl_sync(0xffffffffu, m.p0, 31);
+  m.total = __shfl_sync(0xffffffffu, m.p1, 31);
+  return m;
+}
+
 // idx-th tile of this launch: row-tile major, column tile minor (pairs that run side by side share the A rows
-// and sweep the expert's B columns, which then sit in L2 for the expert's other row tiles).
-__device__ __forceinline__ void decode_tile(const GGParams& P, const SmemGG& sm, int idx, int n_tiles, Tile& t) {
+// and sweep the expert's B columns, which then sit in L2 for the expert's other row tiles).  By a whole warp.
+__device__ __forceinline__ Tile decode_tile(const GGParams& P, const TileMap& m, int idx, int n_tiles) {
+  Tile t;
   const int per_row = n_tiles * P.ksplit;
   const int mt = idx / per_row, rem = idx - mt * per_row;
   const int nt = rem / P.ksplit;
   t.ks = rem - nt * P.ksplit;
-  int e = 0;
-  while (sm.tile_prefix[e + 1] <= mt) ++e;
-  t.e = e;
-  t.m0 = sm.offsets[e] + (mt - sm.tile_prefix[e]) * kPairRows;
-  t.m_end = sm.offsets[e + 1];
   t.n0 = nt * P.bn;
+  // the first expert whose tiles reach past mt (mt < total: there is one)
+  const int e = __popc(__ballot_sync(0xffffffffu, m.p0 <= mt)) + __popc(__ballot_sync(0xffffffffu, m.p1 <= mt));
+  const int before0 = __shfl_sync(0xffffffffu, m.p0, (e - 1) & 31), before1 = __shfl_sync(0xffffffffu, m.p1, (e - 1) & 31);
+  const int lo0 = __shfl_sync(0xffffffffu, m.lo0, e & 31), lo1 = __shfl_sync(0xffffffffu, m.lo1, e & 31);
+  const int hi0 = __shfl_sync(0xffffffffu, m.hi0, e & 31), hi1 = __shfl_sync(0xffffffffu, m.hi1, e & 31);
+  const int before = e == 0 ? 0 : e <= 32 ? before0 : before1;
+  t.e = e;
+  t.m0 = (e < 32 ? lo0 : lo1) + (mt - before) * kPairRows;
+  t.m_end = e < 32 ? hi0 : hi1;
+  return t;
 }
 
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
@@ -234,6 +262,24 @@ __device__ __forceinline__ void store_rows(unsigned char* buf, int lane, const u
     if (r < rows && piece < pieces)
       *reinterpret_cast<uint4*>((unsigned char*)dst + (long long)r * ld_bytes + piece * 16) =
           *reinterpret_cast<const uint4*>(buf + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
+  }
+}
+// The same for 128 bytes of each row: 4 whole lines per instruction.
+__device__ __forceinline__ void store_rows128(unsigned char* buf, int lane, const uint32_t* v, void* dst, long long ld_bytes,
+                                              int rows, int pieces) {
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<uint4*>(buf + lane * 128 + ((i ^ (lane & 7)) << 4)) =
+        make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  __syncwarp();
+  const int piece = lane & 7;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = (lane >> 3) + 4 * i;
+    if (r < rows && piece < pieces)
+      *reinterpret_cast<uint4*>((unsigned char*)dst + (long long)r * ld_bytes + piece * 16) =
+          *reinterpret_cast<const uint4*>(buf + r * 128 + ((piece ^ (r & 7)) << 4));
   }
 }
 // 32 fp32 columns rounded to bf16; lo_off > 0: the rounding remainders too, lo_off columns further on
@@ -296,37 +342,17 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  // everything above touches only this CTA's shared memory and TMEM; the expert offsets and the operands may
-  // come from the kernel before
-  pdl_wait();
-  if (warp == 0) {  // lane l: experts l and l + 32
-    const int o0 = lane <= P.E ? P.offsets[lane] : 0, o1 = lane + 32 <= P.E ? P.offsets[lane + 32] : 0;
-    const int o2 = lane == 0 && P.E == MOE_MAX_EXPERTS ? P.offsets[MOE_MAX_EXPERTS] : 0;
-    if (lane <= P.E) sm.offsets[lane] = o0;
-    if (lane + 32 <= P.E) sm.offsets[lane + 32] = o1;
-    if (lane == 0 && P.E == MOE_MAX_EXPERTS) sm.offsets[MOE_MAX_EXPERTS] = o2;
-    __syncwarp();
-    auto tiles_of = [&](int e) { return e < P.E ? (max(sm.offsets[e + 1] - sm.offsets[e], 0) + kPairRows - 1) / kPairRows : 0; };
-    const int c0 = tiles_of(lane), c1 = tiles_of(lane + 32);
-    int s0 = c0, s1 = c1;  // inclusive scans over the lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v0 = __shfl_up_sync(0xffffffffu, s0, o), v1 = __shfl_up_sync(0xffffffffu, s1, o);
-      if (lane >= o) s0 += v0, s1 += v1;
-    }
-    const int tot0 = __shfl_sync(0xffffffffu, s0, 31);
-    sm.tile_prefix[lane + 1] = s0;
-    sm.tile_prefix[lane + 33] = tot0 + s1;
-    if (lane == 0) sm.tile_prefix[0] = 0;
-  }
   tc_fence_before();
   __syncthreads();
   __syncwarp();
   cluster_sync_all();  // the other CTA's barriers are initialised before anything is counted on them
   tc_fence_after();
   const uint32_t tmem = (uint32_t)lane0((int)sm.tmem_base);
-  const int n_work = lane0(sm.tile_prefix[P.E]) * n_tiles * P.ksplit;
-  Tile t;
+  // everything above touches only this CTA's shared memory and TMEM; the expert offsets and the operands may
+  // come from the kernel before
+  pdl_wait();
+  const TileMap tm = read_tile_map(P, lane);
+  const int n_work = tm.total * n_tiles * P.ksplit;
 
   if (warp == 0) {
     // ================================================================= TMA producer (both CTAs)
@@ -337,10 +363,10 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     const uint32_t full0 = (uint32_t)lane0((int)map_to_rank(&sm.full[0], 0u));  // the leader's stage barriers, 8 bytes apart
     const int half_bn = P.bn / 2;
     for (int idx = pair; ok && idx < n_work; idx += n_pairs) {
-      decode_tile(P, sm, idx, n_tiles, t);
-      const int e = lane0(t.e), n0 = t.n0;
+      const Tile t = decode_tile(P, tm, idx, n_tiles);
+      const int n0 = t.n0;
       const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
-      const int a_row = lane0(t.m0) + (int)rank * kBM;
+      const int a_row = t.m0 + (int)rank * kBM;
       int k0 = kb0 * kBK;
       int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
@@ -357,18 +383,18 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], tx_pair);
           tma_load_2d(st_a0, &map_a0, k0, a_row, bar);
           if (P.bmode == B_PAIR) {
-            tma_load_4d(st_b, &map_b, kB, (int)rank, n0, e, bar);
+            tma_load_4d(st_b, &map_b, kB, (int)rank, n0, t.e, bar);
           } else if (P.bmode == B_DUAL) {
             const int nr = n0 + (int)rank * half_bn;
             tma_load_2d(st_a0 + a_bytes, &map_a1, k0, a_row, bar);
-            tma_load_4d(st_b, &map_b, kB, 0, nr, e, bar);
-            tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, e, bar);
+            tma_load_4d(st_b, &map_b, kB, 0, nr, t.e, bar);
+            tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, t.e, bar);
           } else if (P.bmode == B_SINGLE) {
-            tma_load_4d(st_b, &map_b, kB, P.b_sub, n0 + (int)rank * half_bn, e, bar);
+            tma_load_4d(st_b, &map_b, kB, P.b_sub, n0 + (int)rank * half_bn, t.e, bar);
           } else {
             const int nc = n0 + (int)rank * half_bn;
-            tma_load_4d(st_b, &map_b, nc, P.b_sub, kB, e, bar);
-            if (P.bn > 128) tma_load_4d(st_b + (size_t)64 * kBK * 2, &map_b, nc + 64, P.b_sub, kB, e, bar);
+            tma_load_4d(st_b, &map_b, nc, P.b_sub, kB, t.e, bar);
+            if (P.bn > 128) tma_load_4d(st_b + (size_t)64 * kBK * 2, &map_b, nc + 64, P.b_sub, kB, t.e, bar);
           }
         }
         __syncwarp();
@@ -451,7 +477,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     unsigned char* const ebuf = epi_bufs + (warp - 2) * kEpiBuf;
     int tile_i = 0;
     for (int idx = pair; idx < n_work; idx += n_pairs, ++tile_i) {
-      decode_tile(P, sm, idx, n_tiles, t);
+      const Tile t = decode_tile(P, tm, idx, n_tiles);
       const int buf = tile_i & 1;
       if (!mbar_wait(&sm.accum_full[buf], (tile_i >> 1) & 1)) {
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x402u);
@@ -484,15 +510,24 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           }
         }
       } else {
-        for (int c = 32 * cpar; c < P.bn; c += 64) {
-          uint32_t a[32];
-          tc_ld32(tbase + c, a);
-          tc_wait_ld();
-          if (P.epi == EPI_F32) {
-            float* out = (float*)P.out + (size_t)t.ks * P.plane_elems + row0 * P.ld_out + t.n0 + c;
-            store_rows(ebuf, lane, a, out, P.ld_out * 4, rows, (ncols - c) / 4);
-            store_rows(ebuf, lane, a + 16, out + 16, P.ld_out * 4, rows, (ncols - c - 16) / 4);
-          } else {
+        if (P.epi == EPI_F32) {
+          float* out = (float*)P.out + (size_t)t.ks * P.plane_elems + row0 * P.ld_out + t.n0;
+          uint32_t a[2][32];  // the next chunk's columns are fetched while this one's leave
+          if (32 * cpar < P.bn) tc_ld32(tbase + 32 * cpar, a[0]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int c = 32 * cpar + 64 * i;
+            if (c < P.bn) {
+              tc_wait_ld();
+              if (c + 64 < P.bn) tc_ld32(tbase + c + 64, a[(i + 1) & 1]);
+              store_rows128(ebuf, lane, a[i & 1], out + c, P.ld_out * 4, rows, (ncols - c) / 4);
+            }
+          }
+        } else {
+          for (int c = 32 * cpar; c < P.bn; c += 64) {
+            uint32_t a[32];
+            tc_ld32(tbase + c, a);
+            tc_wait_ld();
             store_bf16(ebuf, lane, a, (__nv_bfloat16*)P.out + row0 * P.ld_out + t.n0 + c, P.ld_out * 2, rows, (ncols - c) / 8,
                        P.split ? P.out_off_lo : 0);
           }
