@@ -471,5 +471,40 @@ __device__ __forceinline__ void warp_route_forced(float l0, float l1, int E, int
   }
 }
 
+// Eight sums over a warp, nine shuffles instead of forty: each of the first three exchanges halves the values a lane still
+// carries.  Lane l returns the sum of a[l >> 2] (four neighbouring lanes the same one).
+__device__ __forceinline__ float warp_sum8(float (&a)[8], int lane) {
+#pragma unroll
+  for (int half = 4; half >= 1; half >>= 1) {
+    const bool up = lane & (half * 4);
+#pragma unroll
+    for (int e = 0; e < half; ++e) {
+      const float send = up ? a[e] : a[e + half], keep = up ? a[e + half] : a[e];
+      a[e] = keep + __shfl_xor_sync(0xffffffffu, send, half * 4);
+    }
+  }
+  float v = a[0];
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  return v + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+
+// Grouping of at most 32 (token, choice) pairs by expert, in one warp's registers: lane p < n holds pair p's expert.  pos: the
+// pair's slot (ascending by expert, pairs of one expert in order); first: it is its expert's first pair; rank: number of
+// selected experts below its own.  Returns the number of selected experts.
+__device__ __forceinline__ int warp_group32(int e, int n, int lane, int& pos, int& rank, bool& first) {
+  const unsigned FULL = 0xffffffffu, below = (1u << lane) - 1u;
+  const unsigned same = __match_any_sync(FULL, e);
+  first = lane < n && (same & below) == 0u;
+  const unsigned firsts = __ballot_sync(FULL, first);
+  pos = __popc(same & below), rank = 0;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const bool lower = __shfl_sync(FULL, e, i) < e;
+    pos += lower;
+    rank += lower && ((firsts >> i) & 1u);
+  }
+  return __popc(firsts);
+}
+
 #endif  // __CUDACC__
 }  // namespace cosmoe

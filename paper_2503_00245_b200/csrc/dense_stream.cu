@@ -953,7 +953,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
     // four at a time so that all their loads are in flight together.
     float* part = sm.scratch;  // [warp][16 tokens][16 experts]
     constexpr int XJ = (V == V_MMA_BF16_S || V == V_MMA_F32_S) ? 4 : kXIters;  // features per thread
-    constexpr int TC = 32 / XJ;                                                // tokens per round trip
     __syncthreads();  // the barriers the producer thread initialised are waited on below
     if (warp < kWarps) {
       const int d = P.d, E = P.E;
@@ -965,22 +964,22 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
           wr[j] = e8 == 0 ? wr0[j]
                           : __ldg(reinterpret_cast<const uint4*>(P.w_router +
                                                                  (size_t)min(tid + j * kConsumerThreads, d - 1) * E + e8));
-        for (int t0 = 0; t0 < P.T; t0 += TC) {
-          float xv[TC][XJ];
+        // (the loop over the tokens stays rolled, two at a time: it runs once per launch, and its instructions come from L2)
+#pragma unroll 1
+        for (int t0 = 0; t0 < P.T; t0 += 2) {
+          float xv[2][XJ];
 #pragma unroll
-          for (int tt = 0; tt < TC; ++tt) {
+          for (int tt = 0; tt < 2; ++tt) {
             const size_t rowo = (size_t)min(t0 + tt, P.T - 1) * d;
 #pragma unroll
             for (int j = 0; j < XJ; ++j) {
-              const int i = tid + j * kConsumerThreads;
-              if (i < d)
-                xv[tt][j] = P.x_is_bf16 ? bf16_to_float(((const uint16_t*)xs)[rowo + i]) : ((const float*)xs)[rowo + i];
-              else
-                xv[tt][j] = 0.f;
+              const int i = min(tid + j * kConsumerThreads, d - 1);
+              xv[tt][j] = P.x_is_bf16 ? bf16_to_float(((const uint16_t*)xs)[rowo + i]) : ((const float*)xs)[rowo + i];
+              if (tid + j * kConsumerThreads >= d) xv[tt][j] = 0.f;
             }
           }
 #pragma unroll
-          for (int tt = 0; tt < TC; ++tt) {
+          for (int tt = 0; tt < 2; ++tt) {
             float a[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) a[q] = 0.f;
@@ -991,11 +990,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
 #pragma unroll
               for (int q = 0; q < 8; ++q) a[q] = fmaf(xv[tt][j], w[q], a[q]);
             }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const float v = warp_sum(a[q]);
-              if (lane == 0 && t0 + tt < P.T) part[(warp * 16 + t0 + tt) * 16 + e8 + q] = v;
-            }
+            const float v = warp_sum8(a, lane);
+            if ((lane & 3) == 0 && t0 + tt < P.T) part[(warp * 16 + t0 + tt) * 16 + e8 + (lane >> 2)] = v;
           }
         }
       }
@@ -1006,6 +1002,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
       for (int t = warp; t < P.T; t += kWarps) {
         float l0 = 0.f, l1 = 0.f;
         if (lane < P.E) {
+#pragma unroll
           for (int w = 0; w < kWarps; ++w) l0 += part[(w * 16 + t) * 16 + lane];
           l0 += bias;
         }
@@ -1055,7 +1052,25 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
     }
   }
   if (!fused1) __syncthreads();  // (one token with the router fused: nothing happens between this barrier and the next)
-  if (kAllX && warp == 0 && !fused1 && !given1 && P.mode == 0) {
+  if (kAllX && warp == 0 && P.mode == 0 && n_pairs <= 32) {
+    // routing products -> active experts and their slots (same numbering as moe_permute): lane p works for pair p
+    const int n = n_pairs, e = lane < n ? sm.stage_e[lane] : -1;
+    int pos, rank, bad = lane < n && (e < 0 || e >= P.E);
+    bool first;
+    const int na = warp_group32(e, n, lane, pos, rank, first);
+    if (first && !bad) {
+      const int sl = P.expert_slot ? P.expert_slot[e] : e;
+      bad = sl < 0;
+      sm.act_e[rank] = e, sm.act_off[rank] = pos, sm.act_slot[rank] = sl < 0 ? 0 : sl;
+    }
+    if (lane < n) sm.slot_tok[pos] = lane / P.k, sm.slot_w[pos] = sm.stage_w[lane];
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      sm.act_off[bad ? 0 : na] = bad ? 0 : n;
+      sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: no CTA streams anything
+      if (bad) flag_error(st, MOE_ERR_STATE, 0x300u);
+    }
+  } else if (kAllX && warp == 0 && !fused1 && !given1 && P.mode == 0) {
     // routing products -> active experts and their slots (same numbering as moe_permute): lane e works for
     // experts e and e + 32
     const int n = n_pairs, E = P.E;

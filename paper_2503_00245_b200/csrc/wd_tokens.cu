@@ -366,21 +366,10 @@ __device__ __forceinline__ void route_tokens(const WtParams& P, WtSmem& sm, floa
 #pragma unroll
             for (int e = 0; e < 8; ++e) a[e] = fmaf(xv[t][q], w[e], a[e]);
           }
-          // eight sums over the warp: each exchange halves the values a lane still carries
-#pragma unroll
-          for (int half = 4; half >= 1; half >>= 1) {
-            const bool up = lane & (half * 4);
-#pragma unroll
-            for (int e = 0; e < half; ++e) {
-              const float send = up ? a[e] : a[e + half], keep = up ? a[e + half] : a[e];
-              a[e] = keep + __shfl_xor_sync(0xffffffffu, send, half * 4);
-            }
-          }
-          a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
-          a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+          const float v = warp_sum8(a, lane);
           if ((lane & 3) == 0 && t0 + t < P.T) {
             float* dst = part + (warp * 16 + t0 + t) * 16 + e8 + (lane >> 2);
-            *dst = q0 == 0 ? a[0] : *dst + a[0];
+            *dst = q0 == 0 ? v : *dst + v;
           }
         }
       }
@@ -435,7 +424,26 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
 
   // ---------------------------------------------------------------- routing -> active experts and their slots
   const int n = P.T * P.k;
-  if (warp == 0 && P.mode == 0) {
+  if (warp == 0 && P.mode == 0 && n <= 32) {
+    const int e = lane < n ? (P.w_router ? sm.stage_e[lane] : P.topk_idx[lane]) : -1;
+    const float wt = lane < n ? (P.w_router ? sm.stage_w[lane] : P.topk_w[lane]) : 0.f;
+    int pos, rank, bad = lane < n && (e < 0 || e >= P.E);
+    bool first;
+    const int na = warp_group32(e, n, lane, pos, rank, first);
+    if (first && !bad) {
+      const int sl = P.expert_slot ? P.expert_slot[e] : e;
+      bad = sl < 0;
+      sm.act_e[rank] = e, sm.act_off[rank] = pos, sm.act_slot[rank] = sl < 0 ? 0 : sl;
+    }
+    if (lane < n) sm.slot_tok[pos] = lane / P.k, sm.slot_w[pos] = wt;
+    bad = __any_sync(0xffffffffu, bad);
+    __syncwarp();
+    if (lane == 0) {
+      sm.act_off[bad ? 0 : na] = bad ? 0 : n;
+      sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: nobody streams anything
+      if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
+    }
+  } else if (warp == 0 && P.mode == 0) {
     const unsigned below = (1u << lane) - 1u;
     int bad = 0;
     sm.cursor[lane] = 0, sm.cursor[lane + 32] = 0;
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: nobody streams anything
       if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
     }
-  } else if (tid == 0) {
+  } else if (tid == 0 && P.mode != 0) {
     // the caller's grouping (moe_permute's products)
     int na = 0, bad = 0;
     sm.act_off[0] = 0;
