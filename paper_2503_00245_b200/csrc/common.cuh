@@ -88,6 +88,13 @@ struct WsLayout {
   size_t total;
 };
 WsLayout ws_layout(const moe_config& c, int T);
+// Whether T tokens select seven experts in eight or more (under even routing): some of their weights may then be asked
+// into L2 before the routing is known.
+inline bool mostly_active(const moe_config& c, int T) {
+  double idle = 1.0;
+  for (int t = 0; t < T && idle > 0.125; ++t) idle *= 1.0 - (double)c.top_k / c.n_experts;
+  return idle <= 0.125;
+}
 
 int validate_config(const moe_config* c);
 
@@ -271,6 +278,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src, uint32
           smem_u32(dst_smem)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
+}
+
+// Asks for bytes (16-byte aligned, a multiple of 16) to be brought into L2; fire and forget.
+__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
 // Same, with an L2 eviction-priority hint: evict_first for data that is read exactly once (streamed weights),

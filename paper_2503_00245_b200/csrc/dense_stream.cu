@@ -54,6 +54,8 @@ constexpr float kFixScaleCnt = 4294967296.0f;  // 2^32
 constexpr double kFixInvCnt = 1.0 / 4294967296.0;
 constexpr int kCntBits = 8;
 
+constexpr int kPrefetchBytes = 128 * 1024;  // of each CTA
+
 struct DenseParams {
   int T, k, E, d, f, mode, x_is_bf16, renorm, fused_route;
   const void* x;
@@ -72,6 +74,7 @@ struct DenseParams {
   int stage_bytes, n_stages, xs_bytes;
   int stage_rows;              // hidden units per stage: kRows, or kRowsWide for several tokens at d <= 1024
   int unit_stride;             // bytes between the hidden units of a stage (3 rows, padded for the MMA passes)
+  int prefetch;                // > 0: bytes of its likely share that a CTA asks into L2 while the tokens are routed
   int use_mma;                 // more than one token: every pass goes through consume_pass_mma
   int wpart_ok;                // shared memory holds the [8][d] merge buffer of the unit-owner passes (d <= 1024)
   int acc_copies;              // the CTAs spread their atomics over this many accumulator copies
@@ -785,6 +788,17 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
 #pragma unroll
     for (int j = 0; j < kRJ; ++j)
       wr0[j] = __ldg(reinterpret_cast<const uint4*>(P.w_router + (size_t)min(tid + j * kConsumerThreads, P.d - 1) * P.E));
+  }
+  if (kAllX && P.prefetch > 0 && warp == kProducerWarp - 1) {
+    // Nearly every expert will be selected: the start of the share this CTA would have with all of them is on its way
+    // while the tokens are routed (weights are constants; if an expert is idle the shares shift, and the bytes serve a
+    // neighbour).
+    PassIt lik;
+    pass_split((unsigned)P.E, P.f, lik);
+    const long long row = 3ll * P.d * 2, lo = (long long)lik.u0 * row, n = min((long long)P.prefetch, (long long)(lik.u1 - lik.u0) * row);
+    constexpr int kRun = 8192;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(P.gud) + lo;
+    for (long long o = (long long)lane * kRun; o < n; o += 32 * kRun) prefetch_l2(src + o, (uint32_t)min((long long)kRun, n - o));
   }
   if (tid != kConsumerThreads) asm volatile("griddepcontrol.wait;" ::: "memory");
   // Stacked decode: the layer input is u = h / rms(h) (fp32 h, no learned scale), formed here by every CTA, rounded
@@ -1542,6 +1556,7 @@ int launch_dense_stream(moe_ctx* ctx, int mode, const void* x, int T, const moe_
   if (avail < 2ll * P.stage_bytes) return MOE_ERR_UNSUPPORTED;
   P.n_stages = (int)min((long long)kMaxStages, avail / P.stage_bytes);
   const size_t smem = (size_t)P.n_stages * P.stage_bytes + fixed;
+  P.prefetch = (P.use_mma && P.fused_route && !w->expert_slot && mostly_active(c, T)) ? kPrefetchBytes : 0;
   const int G = ctx->sm_count;
   const int v = !P.use_mma ? (P.wpart_ok ? V_T1 : V_COLS)
                            : (c.d_model <= 1024 ? (P.x_is_bf16 ? V_MMA_BF16_S : V_MMA_F32_S)
