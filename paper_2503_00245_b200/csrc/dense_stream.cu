@@ -869,11 +869,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
 #pragma unroll
             for (int q = 0; q < 8; ++q) a[q] = fmaf(xv[j], w[q], a[q]);
           }
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float t = warp_sum(a[j]);
-            if (lane == 0) sm.rlog[warp][e8 + j] = t;
-          }
+          const float t = warp_sum8(a, lane);
+          if ((lane & 3) == 0) sm.rlog[warp][e8 + (lane >> 2)] = t;
         }
       } else {
         for (int e = 0; e < E; ++e) {

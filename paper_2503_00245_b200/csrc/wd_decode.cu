@@ -145,16 +145,14 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
         for (int j = 0; j < 8; ++j)
           if (e0 + j < E) a[j] = fmaf(sm.x[i], bf16_to_float(__ldg(P.w_router + (size_t)i * E + e0 + j)), a[j]);
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float v = warp_sum(a[j]);
-      if (lane == 0 && e0 + j < E) sm.rlog[warp][e0 + j] = v;
-    }
+    const float v = warp_sum8(a, lane);
+    if ((lane & 3) == 0 && e0 + (lane >> 2) < E) sm.rlog[warp][e0 + (lane >> 2)] = v;
   }
   __syncthreads();
   if (warp == 0) {
     float l0 = 0.f, l1 = 0.f;
     if (lane < E) {
+#pragma unroll
       for (int w = 0; w < kWdWarps; ++w) l0 += sm.rlog[w][lane];
       if (P.b_router) l0 += P.b_router[lane];
     }
@@ -453,17 +451,15 @@ __global__ void __launch_bounds__(kWsThreads, 1) wd_stream_kernel(const WdParams
           for (int j = 0; j < 8; ++j)
             if (e0 + j < E) a[j] = fmaf(sm.x[i], bf16_to_float(__ldg(P.w_router + (size_t)i * E + e0 + j)), a[j]);
       }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float v = warp_sum(a[j]);
-        if (lane == 0 && e0 + j < E) sm.rlog[warp][e0 + j] = v;
-      }
+      const float v = warp_sum8(a, lane);
+      if ((lane & 3) == 0 && e0 + (lane >> 2) < E) sm.rlog[warp][e0 + (lane >> 2)] = v;
     }
   }
   __syncthreads();
   if (warp == 0) {
     float l0 = 0.f, l1 = 0.f;
     if (lane < E) {
+#pragma unroll
       for (int w = 0; w < kWdWarps; ++w) l0 += sm.rlog[w][lane];
       if (P.b_router) l0 += P.b_router[lane];
     }
