@@ -98,6 +98,19 @@ __device__ __forceinline__ float dot8f(const uint4& w, const float* v) {
   return a;
 }
 
+// 16 bytes of weights, asked for here and not where they are used
+__device__ __forceinline__ uint4 ldg_now(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// What a warp keeps of the later products' weights in registers: they depend on the routing only, so they are asked for
+// before the first product and have arrived when a meeting is over; what does not fit is loaded where it is used.
+constexpr int kPf2 = 3;  // product 2: groups of four units, when a unit's pair of rows is one chunk per lane (r <= 128)
+constexpr int kPf3 = 8;  // product 3: chunks of the warp's first segment
+constexpr int kPf4 = 2;  // product 4: rows, when the k rows of r values are one chunk per lane
+
 __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P) {
   extern __shared__ __align__(16) unsigned char wd_smem_raw[];
   WdSmem& sm = *reinterpret_cast<WdSmem*>(wd_smem_raw);
@@ -194,6 +207,34 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
     }
   }
 
+  // ---- the later products' weights, as far as they fit into registers
+  const bool one2 = 2 * rc <= 32, one4 = k * rc <= 32;
+  const int S3 = P.split, seg3 = (fc + S3 - 1) / S3;  // product 3: segments of a row, chunks per segment
+  uint4 w2[kPf2][4], w3[kPf3], w4[kPf4];
+  if (one2) {
+#pragma unroll
+    for (int b = 0; b < kPf2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int u = min(gw + (4 * b + q) * n_warps, k * f - 1), a = u / f, c = u - a * f;
+        w2[b][q] = ldg_now(reinterpret_cast<const uint4*>(P.wd_b + ((size_t)sm.sel_slot[a] * f + c) * 2 * r) + min(lane, 2 * rc - 1));
+      }
+  }
+  {
+    const int item = min(gw, k * r * S3 - 1), row = item / S3, sg = item - row * S3, a = row / r, j = row - a * r;
+    const uint4* wrow = reinterpret_cast<const uint4*>(P.wd_c + ((size_t)sm.sel_slot[a] * r + j) * f);
+    const int c_lo = sg * seg3, c_hi = min(fc, c_lo + seg3);
+#pragma unroll
+    for (int u = 0; u < kPf3; ++u) w3[u] = ldg_now(wrow + max(min(c_lo + lane + 32 * u, c_hi - 1), 0));
+  }
+  if (one4) {
+#pragma unroll
+    for (int n = 0; n < kPf4; ++n) {
+      const int i = min(gw + n * n_warps, d - 1), q = min(lane, k * rc - 1), a = q / rc;
+      w4[n] = ldg_now(reinterpret_cast<const uint4*>(P.wd_d + ((size_t)sm.sel_slot[a] * d + i) * r) + (q - a * rc));
+    }
+  }
+
   // ---------------------------------------------------------------- t = x [gL | uL]: k * 2r rows of d
   for (int row = gw; row < k * 2 * r; row += n_warps) {
     const int a = row / (2 * r), j2 = row - a * 2 * r;
@@ -219,7 +260,32 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
   __syncthreads();
 
   // ---------------------------------------------------------------- h_c: k * f units, rows (gR_c | uR_c) of 2r
-  for (int u0 = gw; u0 < k * f; u0 += 4 * n_warps) {
+  // (four units' gate and up sums are reduced together; lane 4 q < 16 ends up with unit q's gate sum, lane 4 q + 16 with its up)
+  auto finish4 = [&](int u0, float (&g)[4], float (&up)[4]) {
+    float v[8] = {g[0], g[1], g[2], g[3], up[0], up[1], up[2], up[3]};
+    const float s = warp_sum8(v, lane), us = __shfl_down_sync(0xffffffffu, s, 16);
+    const int u = u0 + (lane >> 2) * n_warps;
+    if ((lane & 3) == 0 && lane < 16 && u < k * f) P.h[u] = __fdividef(s, 1.0f + __expf(-s)) * us;
+  };
+  int u0 = gw;
+  if (one2) {
+    const bool live = lane < 2 * rc, part = lane >= rc;
+    const float* src = (part ? sm.tu : sm.tg) + (live ? lane - (part ? rc : 0) : 0) * 8;
+#pragma unroll
+    for (int b = 0; b < kPf2; ++b) {
+      if (u0 < k * f) {
+        float g[4], up[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float v = live ? dot8s(w2[b][q], src + min(u0 + q * n_warps, k * f - 1) / f * r) : 0.f;
+          g[q] = part ? 0.f : v, up[q] = part ? v : 0.f;
+        }
+        finish4(u0, g, up);
+      }
+      u0 += 4 * n_warps;
+    }
+  }
+  for (; u0 < k * f; u0 += 4 * n_warps) {
     float g[4], up[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) g[q] = up[q] = 0.f;
@@ -240,18 +306,13 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
         if (part) up[q] += v; else g[q] += v;
       }
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float gs = warp_sum(g[q]), us = warp_sum(up[q]);
-      const int u = u0 + q * n_warps;
-      if (lane == 0 && u < k * f) P.h[u] = __fdividef(gs, 1.0f + __expf(-gs)) * us;
-    }
+    finish4(u0, g, up);
   }
   if (!meet(st, sm)) return;
 
   // ---------------------------------------------------------------- v = h dL: k * r rows of f, in `split` segments
   {
-    const int S = P.split, seg = ((fc + S - 1) / S);  // chunks per segment
+    const int S = S3, seg = seg3;
     for (int item = gw; item < k * r * S; item += n_warps) {
       const int row = item / S, s = item - row * S;
       const int a = row / r, j = row - a * r;
@@ -259,7 +320,25 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
       const float* hv = P.h + (size_t)a * f;
       const int c_lo = s * seg, c_hi = min(fc, c_lo + seg);
       float acc = 0.f;
-      for (int c0 = c_lo + lane; c0 < c_hi; c0 += 32 * 4) {
+      int c0 = c_lo + lane;
+      if (item == gw) {  // the warp's first segment: its weights are here
+        float4 ha[kPf3], hb[kPf3];
+#pragma unroll
+        for (int u = 0; u < kPf3; ++u) {
+          const int c = max(min(c0 + 32 * u, c_hi - 1), 0);
+          ha[u] = __ldcg(reinterpret_cast<const float4*>(hv) + 2 * c);
+          hb[u] = __ldcg(reinterpret_cast<const float4*>(hv) + 2 * c + 1);
+        }
+#pragma unroll
+        for (int u = 0; u < kPf3; ++u) {
+          if (c0 + 32 * u < c_hi) {
+            const float hh[8] = {ha[u].x, ha[u].y, ha[u].z, ha[u].w, hb[u].x, hb[u].y, hb[u].z, hb[u].w};
+            acc += dot8f(w3[u], hh);
+          }
+        }
+        c0 += 32 * kPf3;
+      }
+      for (; c0 < c_hi; c0 += 32 * 4) {
         uint4 w[4];
         float4 ha[4], hb[4];
 #pragma unroll
@@ -291,13 +370,7 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
 
   // ---------------------------------------------------------------- y_i = sum_a w_a (v_a . dR_a[i]): d outputs
   const bool good = ld_acquire(&st->status) == 0u;
-  for (int i = gw; i < d; i += n_warps) {
-    float acc = 0.f;
-    for (int q = lane; q < k * rc; q += 32) {
-      const int a = q / rc, c = q - a * rc;
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(P.wd_d + ((size_t)sm.sel_slot[a] * d + i) * r) + c);
-      acc = fmaf(sm.sel_w[a], dot8s(w, sm.tg + a * r + c * 8), acc);
-    }
+  auto put = [&](int i, float acc) {
     acc = warp_sum(acc);
     if (lane == 0 && good) {
       if (P.x_is_bf16)
@@ -305,9 +378,25 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
       else
         ((float*)P.y)[i] = acc;
     }
+  };
+  int i = gw;
+  if (one4) {
+    const int q = min(lane, k * rc - 1);
+    const float wa = lane < k * rc ? sm.sel_w[q / rc] : 0.f;  // (chunk q of the k * r values of v)
+#pragma unroll
+    for (int n = 0; n < kPf4; ++n, i += n_warps)
+      if (i < d) put(i, wa * dot8s(w4[n], sm.tg + q * 8));
+  }
+  for (; i < d; i += n_warps) {
+    float acc = 0.f;
+    for (int q = lane; q < k * rc; q += 32) {
+      const int a = q / rc, c = q - a * rc;
+      const uint4 w = __ldg(reinterpret_cast<const uint4*>(P.wd_d + ((size_t)sm.sel_slot[a] * d + i) * r) + c);
+      acc = fmaf(sm.sel_w[a], dot8s(w, sm.tg + a * r + c * 8), acc);
+    }
+    put(i, acc);
   }
 }
-
 
 // =====================================================================================================
 // The same chain for LARGE factors (tens of MB per token: the paper's rank, r = d / 2): bandwidth counts, so the
