@@ -487,7 +487,9 @@ __global__ void __launch_bounds__(kWsThreads, 1) wd_stream_kernel(const WdParams
   WsSmem& sm = *reinterpret_cast<WsSmem*>(ws_smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = P.d, f = P.f, r = P.r, k = P.k, E = P.E;
-  float* const hs = reinterpret_cast<float*>(ws_smem_raw + kWsHeader);  // h of the selected experts, [k][f]
+  // h of the selected experts, [k][2][f / 2]: the first four of every eight values, then the last four, so that lanes reading
+  // eight values each meet no bank conflict
+  float* const hs = reinterpret_cast<float*>(ws_smem_raw + kWsHeader);
   unsigned char* const ring = ws_smem_raw + kWsHeader + (((size_t)k * f * 4 + 127) / 128) * 128;
   DeviceState* const st = P.st;
   pdl_launch_dependents();
@@ -759,8 +761,11 @@ __global__ void __launch_bounds__(kWsThreads, 1) wd_stream_kernel(const WdParams
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int l = l0 + u * kWdThreads, i = l;
-        if (l < n4) reinterpret_cast<float4*>(hs)[i] = v[u];
+        const int l = l0 + u * kWdThreads;
+        if (l < n4) {
+          const int a = l / (f >> 2), i = l - a * (f >> 2);
+          reinterpret_cast<float4*>(hs)[a * (f >> 2) + (i & 1) * fc + (i >> 1)] = v[u];
+        }
       }
     }
   }
@@ -784,7 +789,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) wd_stream_kernel(const WdParams
           float acc = 0.f;
           for (int c = c_lo + lane; c < c_hi; c += 32) {
             const uint4 w = row[c];
-            const float4 ha = reinterpret_cast<const float4*>(hv)[2 * c], hb = reinterpret_cast<const float4*>(hv)[2 * c + 1];
+            const float4 ha = reinterpret_cast<const float4*>(hv)[c], hb = reinterpret_cast<const float4*>(hv)[fc + c];
             const float hh[8] = {ha.x, ha.y, ha.z, ha.w, hb.x, hb.y, hb.z, hb.w};
             acc += dot8f(w, hh);
           }
