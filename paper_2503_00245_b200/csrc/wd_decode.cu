@@ -107,6 +107,7 @@ __device__ __forceinline__ uint4 ldg_now(const uint4* p) {
 
 // What a warp keeps of the later products' weights in registers: they depend on the routing only, so they are asked for
 // before the first product and have arrived when a meeting is over; what does not fit is loaded where it is used.
+constexpr int kPf1 = kWdMaxD / 8 / 32;  // product 1: the warp's first row
 constexpr int kPf2 = 3;  // product 2: groups of four units, when a unit's pair of rows is one chunk per lane (r <= 128)
 constexpr int kPf3 = 8;  // product 3: chunks of the warp's first segment
 constexpr int kPf4 = 2;  // product 4: rows, when the k rows of r values are one chunk per lane
@@ -210,7 +211,14 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
   // ---- the later products' weights, as far as they fit into registers
   const bool one2 = 2 * rc <= 32, one4 = k * rc <= 32;
   const int S3 = P.split, seg3 = (fc + S3 - 1) / S3;  // product 3: segments of a row, chunks per segment
-  uint4 w2[kPf2][4], w3[kPf3], w4[kPf4];
+  uint4 w1[kPf1], w2[kPf2][4], w3[kPf3], w4[kPf4];
+  {  // (product 1's first row goes first)
+    const int row = min(gw, k * 2 * r - 1), a = row / (2 * r), j2 = row - a * 2 * r;
+    const uint4* wrow = reinterpret_cast<const uint4*>(P.wd_a + ((size_t)sm.sel_slot[a] * 2 * r + j2) * d);
+#pragma unroll
+    for (int u = 0; u < kPf1; ++u)
+      if (32 * u < dc) w1[u] = ldg_now(wrow + min(lane + 32 * u, dc - 1));
+  }
   if (one2) {
 #pragma unroll
     for (int b = 0; b < kPf2; ++b)
@@ -240,13 +248,19 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
     const int a = row / (2 * r), j2 = row - a * 2 * r;
     const uint4* wrow = reinterpret_cast<const uint4*>(P.wd_a + ((size_t)sm.sel_slot[a] * 2 * r + j2) * d);
     float acc = 0.f;
-    for (int c0 = lane; c0 < dc; c0 += 32 * 4) {
-      uint4 w[4];
+    if (row == gw) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) w[u] = __ldg(wrow + min(c0 + 32 * u, dc - 1));
+      for (int u = 0; u < kPf1; ++u)
+        if (lane + 32 * u < dc) acc += dot8s(w1[u], sm.x + (lane + 32 * u) * 8);
+    } else {
+      for (int c0 = lane; c0 < dc; c0 += 32 * 4) {
+        uint4 w[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (c0 + 32 * u < dc) acc += dot8s(w[u], sm.x + (c0 + 32 * u) * 8);
+        for (int u = 0; u < 4; ++u) w[u] = __ldg(wrow + min(c0 + 32 * u, dc - 1));
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + 32 * u < dc) acc += dot8s(w[u], sm.x + (c0 + 32 * u) * 8);
+      }
     }
     acc = warp_sum(acc);
     if (lane == 0) P.t[row] = acc;
