@@ -191,23 +191,6 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
 
   const int dc = d >> 3, rc = r >> 3, fc = f >> 3;
 
-  // The selected experts' matrices are known now: every CTA asks for its share of all four to be brought into
-  // L2 (fire and forget), in the order the chain needs them, so that the DRAM transfer runs in the background
-  // of the chain instead of once per product behind a meeting.
-  if (tid < 4 * k) {
-    const int which = tid / k, a = tid - which * k;  // which-major: all experts' wd_a first
-    const size_t per_expert[4] = {(size_t)2 * r * d * 2, (size_t)f * 2 * r * 2, (size_t)r * f * 2, (size_t)d * r * 2};
-    const uint16_t* const base[4] = {P.wd_a, P.wd_b, P.wd_c, P.wd_d};
-    const size_t bytes = per_expert[which];
-    const size_t slice = ((bytes + gridDim.x - 1) / gridDim.x + 15) & ~(size_t)15;
-    const size_t lo = (size_t)blockIdx.x * slice;
-    if (lo < bytes) {
-      const size_t n = bytes - lo < slice ? bytes - lo : slice;  // a multiple of 16: bytes is
-      const unsigned char* src = reinterpret_cast<const unsigned char*>(base[which]) + (size_t)sm.sel_slot[a] * bytes + lo;
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)n) : "memory");
-    }
-  }
-
   // ---- the later products' weights, as far as they fit into registers
   const bool one2 = 2 * rc <= 32, one4 = k * rc <= 32;
   const int S3 = P.split, seg3 = (fc + S3 - 1) / S3;  // product 3: segments of a row, chunks per segment
@@ -241,6 +224,22 @@ __global__ void __launch_bounds__(kWdThreads) wd_decode_kernel(const WdParams P)
       const int i = min(gw + n * n_warps, d - 1), q = min(lane, k * rc - 1), a = q / rc;
       w4[n] = ldg_now(reinterpret_cast<const uint4*>(P.wd_d + ((size_t)sm.sel_slot[a] * d + i) * r) + (q - a * rc));
     }
+  }
+
+  // What does not fit is at least brought into L2: every CTA asks for its share of all four matrices (fire and forget), in
+  // the order the chain needs them, so that the DRAM transfer runs in the background of the chain instead of once per
+  // product behind a meeting.
+  const bool all_here = one2 && one4 && k * f <= 4 * kPf2 * n_warps && d <= kPf4 * n_warps && k * r * S3 <= n_warps &&
+                        seg3 <= 32 * kPf3 && k * 2 * r <= n_warps;
+  if (!all_here && tid < 4 * k) {
+    const int which = tid / k, a = tid - which * k;  // which-major: all experts' wd_a first
+    const size_t bytes = 2 * (which == 0 ? (size_t)2 * r * d : which == 1 ? (size_t)f * 2 * r : which == 2 ? (size_t)r * f : (size_t)d * r);
+    const uint16_t* base = which == 0 ? P.wd_a : which == 1 ? P.wd_b : which == 2 ? P.wd_c : P.wd_d;
+    const size_t slice = ((bytes + gridDim.x - 1) / gridDim.x + 15) & ~(size_t)15;
+    const size_t lo = (size_t)blockIdx.x * slice;
+    if (lo < bytes)  // (a multiple of 16: bytes is)
+      prefetch_l2(reinterpret_cast<const unsigned char*>(base) + (size_t)sm.sel_slot[a] * bytes + lo,
+                  (uint32_t)(bytes - lo < slice ? bytes - lo : slice));
   }
 
   // ---------------------------------------------------------------- t = x [gL | uL]: k * 2r rows of d
