@@ -1,0 +1,105 @@
+"""GPU parity at the sizes where the kernels' splits change: slices and tiles with remainders, more pairs than a warp has
+lanes, expert counts that are no multiple of eight, contractions that are cut into planes."""
+import pytest
+import torch
+
+from oracle import moe_oracle as O
+from synth import workloads as W
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+# Decomposed experts in a decode step carry their intermediates as fp32 (one token) or as three bf16 terms of an fp32 value
+# (several): every product is a sum of at most K = 5632 terms, rounded at 2^-24 each, and its rounding errors add up like a
+# random walk, sqrt(K) * 2^-24 = 4.5e-6 per product at most; four products in a row, of the output's RMS.
+F32_TOL = 4 * 5632 ** 0.5 * 2.0 ** -24
+
+
+def check_prefill(lay, t, host, k):
+    """Element by element: half a unit in the last place of y's type, and six standard deviations of what rounding the
+    hidden activations to bf16 leaves in y.  Rounding changes a value by 2^-9 / sqrt(3) of itself (RMS), y is a sum of
+    f >= 512 such terms of random sign, so an element's standard deviation is that share of its own TOKEN's RMS; fp32 token
+    rows are rounded to bf16 as well, which both products pass on: about twice that in all."""
+    _, ora, y = U.check_layer(lay, t, host, k, tol=1.0)
+    sigma = 2.0 ** -9 / 3 ** 0.5 * (2.0 if t["x"].dtype == torch.float32 else 1.0)
+    widest = max(U.rms(row) for row in ora["y"]) / U.rms(ora["y"])
+    U.assert_close_in_output_type(U.to64(y), ora["y"], rms_tol=6 * sigma * widest, mant_bits=8 if y.dtype == torch.bfloat16 else 24)
+
+
+def shape(d, f, E=8, k=2, r=0, xd="bf16", bias="none"):
+    return W.LayerShape("t", 9, d, f, n_experts=E, top_k=k, wd_rank=r, x_dtype=xd, bias=bias)
+
+
+@pytest.mark.parametrize("sh,T", [
+    (shape(448, 456, r=448, xd="f32"), 2),              # a whole slice of the contraction, and one of eight values beside it
+    (shape(904, 896, r=8, xd="f32"), 3),                # a rank below one unit, a slice of eight values
+    (shape(264, 1000, E=6, k=3, r=232, xd="f32"), 5),   # router as a launch of its own
+    (shape(256, 520, E=1, k=1, r=72, xd="f32"), 16),    # one expert with two groups of eight tokens
+    (shape(256, 512, E=16, k=4, r=40, xd="f32"), 16),   # 64 pairs: grouped in rounds
+    (shape(136, 64, E=64, k=8, r=16, xd="f32"), 9),     # more active experts than CTAs share evenly
+    (shape(2312, 512, r=64, xd="f32"), 4),              # more features than one round of the router holds
+    (shape(2048, 5632, r=1024), 8),
+])
+def test_decomposed_decode_of_several_tokens(sh, T):
+    lay, t, host = U.build(sh, T)
+    U.check_layer(lay, t, host, sh.top_k, tol=F32_TOL if sh.x_dtype == "f32" else U.Y_TOL)
+    # the per-slot form of the same kernel
+    ora = U.oracle_layer(host, sh.top_k)
+    out = lay.expert_ffn(t["x"], torch.from_numpy(ora["offsets"]).cuda(), torch.from_numpy(ora["perm"]).cuda())
+    torch.cuda.synchronize()
+    assert lay.check() == 0
+    U.assert_close_rms(out.cpu().numpy().astype("float64"), ora["out_slots"], tol=F32_TOL, what="out_slots")
+
+
+@pytest.mark.parametrize("sh", [
+    shape(2048, 5632, r=128, xd="f32"),                 # every later weight of a warp in registers
+    shape(2048, 5632, r=136, xd="f32"),                 # product 2's rows longer than a chunk per lane
+    shape(256, 5632, E=4, k=4, r=128, xd="f32"),        # more units per warp than registers hold
+    shape(72, 40, E=5, k=1, r=8, xd="f32"),
+])
+def test_decomposed_decode_of_one_token(sh):
+    lay, t, host = U.build(sh, 1)
+    U.check_layer(lay, t, host, sh.top_k, tol=F32_TOL)
+
+
+@pytest.mark.parametrize("sh,T", [
+    (shape(72, 512, E=2, k=2), 17),                     # one CTA and a remainder of one token; features no multiple of 32
+    (shape(264, 512, E=6, k=3, xd="f32"), 33),
+    (shape(128, 512, E=16, k=1, bias="normal"), 1000),
+    (shape(64, 512, E=64, k=8), 700),                   # two logits per lane
+    (shape(64, 512, E=8, k=4), 2100),                   # more pairs per warp than it keeps in registers
+    (shape(2048, 512, E=32, k=2), 40),                  # W_r too large for shared memory: the plain router
+])
+def test_many_tokens_routed_and_grouped(sh, T):
+    lay, t, host = U.build(sh, T)
+    idx, w, probs = lay.route(t["x"], want_probs=True)
+    torch.cuda.synchronize()
+    R, Wt, S, wo = O.route(host["x"], host["w_router"], host["b_router"], sh.top_k, True)
+    U.check_routing(idx.cpu().numpy(), w.cpu().numpy(), {"logits": R, "topk_idx": S, "topk_w": wo}, sh.top_k)
+    assert abs(probs.cpu().numpy() - Wt).max() <= U.W_TOL
+    for _ in range(2):                                  # (the CTAs' counter is back at zero after a call)
+        check_prefill(lay, t, host, sh.top_k)
+
+
+@pytest.mark.parametrize("sh,T", [
+    (shape(1440, 1280), 100),                           # three or four planes, columns no multiple of a tile
+    (shape(200, 2000, E=2, k=1), 40),                   # a row of d shorter than one round of the combine's loads
+    (shape(1024, 1024, xd="f32"), 300),
+    (shape(512, 2048, r=64), 600),                      # third GEMM cut into planes
+    (shape(512, 2048, r=72, E=4), 129),
+])
+def test_prefill_with_a_cut_contraction(sh, T):
+    lay, t, host = U.build(sh, T)
+    check_prefill(lay, t, host, sh.top_k)
+    idx, w, _ = lay.route(t["x"])
+    offsets, perm, inv = lay.permute(idx)
+    y = lay.combine(lay.expert_ffn(t["x"], offsets, perm), w, inv)
+    assert torch.equal(y, lay.forward(t["x"]))          # the layer and its four calls add the planes in the same order
+    assert lay.check() == 0
+
+
+@pytest.mark.parametrize("T", [8, 16])
+def test_dense_decode_of_several_tokens_with_many_pairs(T):
+    sh = shape(512, 1024, E=16, k=8)                    # 64 and 128 pairs: beyond one per lane; every expert active
+    lay, t, host = U.build(sh, T, path=1)
+    U.check_layer(lay, t, host, sh.top_k)
