@@ -108,7 +108,9 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
 // (two units) and are added up in fp32.
 // The last CTA to finish groups the pairs by expert, a stable counting sort: every warp counts and then scatters a
 // contiguous run of them.  One launch instead of two, and no second walk over the routing by a lone CTA in rounds.
-// (2048 tokens, d 2048, 8 experts: FIXME)
+// Bound by latency: one round trip to x, then a CTA's chain of barriers.  Under ncu, cold, 2048 tokens at d 2048: 12.5 us for 8
+// experts where the staged router and the grouping took 11.4 + 7.4; other expert counts had a router that read W_r through L1
+// a value at a time: a whole layer of 272 tokens, 16 experts at d 344 51.2 -> 36.6 us, 107 tokens, 2 experts at d 352 38.9 -> 27.8.
 constexpr int kRtWarps = 16, kRtTokens = 16, kRtUnit = 32, kRtBatch = 4;
 struct RtShape {
   int e8, row_bytes, part_off, smem;  // experts rounded up to 8; bytes between two experts' rows; partial logits; total
@@ -355,7 +357,7 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
   const XT* xp = (const XT*)x;
   const uint16_t* wr = (const uint16_t*)w->w_router;
   const RtShape sh = rt_shape(c.d_model, c.n_experts);
-  // more than a decode step's tokens, and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 24 experts)
+  // more than a decode step's tokens (16 would be a tile of a single CTA: those take a CTA per token), and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 24 experts)
   if (T > MOE_STREAM_MAX_TOKENS && sh.smem <= 112 * 1024) {
     MOE_TRY(allow_full_smem<route_tile_kernel<XT>>(ctx));
     MOE_CUDA_TRY(launch_pdl(route_tile_kernel<XT>, dim3((T + kRtTokens - 1) / kRtTokens), dim3(kRtWarps * 32), (size_t)sh.smem, s,
