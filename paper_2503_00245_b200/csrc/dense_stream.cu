@@ -960,8 +960,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
     }
   } else if (kAllX && P.fused_route) {
     // several tokens, E a multiple of 8 (Eq. 2, Eq. 3); every CTA routes all tokens.  A thread owns the input
-    // features tid, tid + 256, ...: their router rows are fetched once and serve every token; the tokens go
-    // four at a time so that all their loads are in flight together.
+    // features tid, tid + 256, ...: their router rows are fetched once and serve every token.
     float* part = sm.scratch;  // [warp][16 tokens][16 experts]
     constexpr int XJ = (V == V_MMA_BF16_S || V == V_MMA_F32_S) ? 4 : kXIters;  // features per thread
     __syncthreads();  // the barriers the producer thread initialised are waited on below
