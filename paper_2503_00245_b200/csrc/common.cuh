@@ -363,6 +363,23 @@ __device__ __forceinline__ void mma16(float* c, uint32_t a_lo0, uint32_t a_hi0, 
       : "r"(a_lo0), "r"(a_hi0), "r"(a_lo1), "r"(a_hi1), "r"(b0), "r"(b1));
 }
 
+// the same for 8 values of a row
+__device__ __forceinline__ void mma8(float* c, uint32_t a_lo, uint32_t a_hi, uint32_t b) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a_lo), "r"(a_hi), "r"(b));
+}
+
+// a += b, four values in two instructions
+__device__ __forceinline__ void add4(float* a, const float* b) {
+  asm("{\n\t.reg .b64 a0, a1, b0, b1;\n\t"
+      "mov.b64 a0, {%0, %1};\n\tmov.b64 a1, {%2, %3};\n\tmov.b64 b0, {%4, %5};\n\tmov.b64 b1, {%6, %7};\n\t"
+      "add.rn.f32x2 a0, a0, b0;\n\tadd.rn.f32x2 a1, a1, b1;\n\t"
+      "mov.b64 {%0, %1}, a0;\n\tmov.b64 {%2, %3}, a1;\n\t}"
+      : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3])
+      : "f"(b[0]), "f"(b[1]), "f"(b[2]), "f"(b[3]));
+}
+
 // fp32 -> three bf16 terms, the largest first: each remainder is exact in fp32
 __device__ __forceinline__ void split3(float v, uint16_t* out) {
 #pragma unroll

@@ -100,12 +100,13 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
                     probs ? probs + (size_t)t * E : nullptr);
 }
 
-// Many tokens: the logits of 16 tokens per CTA on the tensor cores (mma.sync m16n8k16: 16 tokens x 8 experts; N is far
+// Many tokens: the logits of 16 tokens per CTA on the tensor cores (mma.sync m16n8k8: 16 tokens x 8 experts; N is far
 // below a tcgen05 tile).  W_r lies transposed in shared memory, [expert][feature], the experts' rows 64 bytes beyond a
 // multiple of 128 apart; the 16 warps split the features in units of 32.  A lane takes 8 consecutive features of a row at a
 // time, of x straight from memory (all of a warp's loads of a round in flight together) and of W_r alike: the order of
-// the contraction inside a unit is free.  fp32 rows go in as three bf16 terms.  Sums stay short in the MMA's accumulators
-// (two units) and are added up in fp32.
+// the contraction inside a unit is free.  fp32 rows go in as three bf16 terms.  An MMA cuts its sums instead of rounding them:
+// eight products in one (m16n8k8), everything else is added in fp32, in pairs.  Relative error of the probabilities against 64
+// bits, 512 bf16 tokens at d 1024: 7.9e-8, as with fp32 multiply-adds (64 products in one accumulator: 10.2e-8).
 // The last CTA to finish groups the pairs by expert, a stable counting sort: every warp counts and then scatters a
 // contiguous run of them.  One launch instead of two, and no second walk over the routing by a lone CTA in rounds.
 // Bound by latency: one round trip to x, then a CTA's chain of barriers.  Under ncu, cold, 2048 tokens at d 2048: 12.5 us for 8
@@ -182,33 +183,35 @@ __global__ void __launch_bounds__(kRtWarps * 32)
         }
       }
     for (int e8 = 0; e8 < sh.e8; e8 += 8) {
-      float s[4] = {0.f, 0.f, 0.f, 0.f};
       const unsigned char* wrow = rt_smem + (e8 + g) * sh.row_bytes + q * 16;
+      float sum[4];
 #pragma unroll
       for (int j0 = 0; j0 < kRtBatch; j0 += 2) {
-        float m[NT][4];
+        float m[8][4];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) m[t][0] = m[t][1] = m[t][2] = m[t][3] = 0.f;
+        for (int j = 0; j < 2; ++j) {
+          const uint4 b = *reinterpret_cast<const uint4*>(wrow + min(u0 + (j0 + j) * kRtWarps, units - 1) * (kRtUnit * 2));
+          const uint4(&r)[2][NT] = a[j0 + j];
 #pragma unroll
-        for (int j = j0; j < j0 + 2; ++j) {
-          const int u = u0 + j * kRtWarps;
-          const uint4 b = *reinterpret_cast<const uint4*>(wrow + min(u, units - 1) * (kRtUnit * 2));
+          for (int i = 0; i < 4; ++i) m[4 * j + i][0] = m[4 * j + i][1] = m[4 * j + i][2] = m[4 * j + i][3] = 0.f;
 #pragma unroll
-          for (int t = 0; t < NT; ++t) {
-            mma16(m[t], a[j][0][t].x, a[j][1][t].x, a[j][0][t].y, a[j][1][t].y, b.x, b.y);
-            mma16(m[t], a[j][0][t].z, a[j][1][t].z, a[j][0][t].w, a[j][1][t].w, b.z, b.w);
+          for (int t = NT - 1; t >= 0; --t) {  // (what the small terms' sums lose is far below the first one's last place)
+            mma8(m[4 * j], r[0][t].x, r[1][t].x, b.x), mma8(m[4 * j + 1], r[0][t].y, r[1][t].y, b.y);
+            mma8(m[4 * j + 2], r[0][t].z, r[1][t].z, b.z), mma8(m[4 * j + 3], r[0][t].w, r[1][t].w, b.w);
           }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int n = 4; n > 0; n >>= 1)
 #pragma unroll
-          for (int t = NT - 1; t >= 0; --t) s[i] += m[t][i];
+          for (int j = 0; j < n; ++j) add4(m[j], m[j + n]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[i] = j0 == 0 ? m[0][i] : sum[i] + m[0][i];
       }
       float* dst = mine + e8;  // D: tokens g and g + 8, experts 2q and 2q + 1
       if (u0 == warp) {
-        dst[0] = s[0], dst[1] = s[1], dst[8 * sh.e8] = s[2], dst[8 * sh.e8 + 1] = s[3];
+        dst[0] = sum[0], dst[1] = sum[1], dst[8 * sh.e8] = sum[2], dst[8 * sh.e8 + 1] = sum[3];
       } else {
-        dst[0] += s[0], dst[1] += s[1], dst[8 * sh.e8] += s[2], dst[8 * sh.e8 + 1] += s[3];
+        dst[0] += sum[0], dst[1] += sum[1], dst[8 * sh.e8] += sum[2], dst[8 * sh.e8 + 1] += sum[3];
       }
     }
   }
@@ -217,18 +220,20 @@ __global__ void __launch_bounds__(kRtWarps * 32)
     const int t = t0 + warp;  // a warp finishes one token
     if (t < T) {
       float l0 = 0.f, l1 = 0.f;
-      const float* p = part + warp * sh.e8 + lane;
-      const int step = kRtTokens * sh.e8;
-      if (lane < E) {
+      auto logit = [&](int e) {  // the warps' shares, in pairs
+        const float* p = part + warp * sh.e8 + e;
+        const int step = kRtTokens * sh.e8;
+        float v[kRtWarps];
 #pragma unroll
-        for (int w = 0; w < kRtWarps; ++w) l0 += p[w * step];
-        if (bias) l0 += bias[lane];
-      }
-      if (lane + 32 < E) {
+        for (int w = 0; w < kRtWarps; ++w) v[w] = p[w * step];
 #pragma unroll
-        for (int w = 0; w < kRtWarps; ++w) l1 += p[w * step + 32];
-        if (bias) l1 += bias[lane + 32];
-      }
+        for (int n = kRtWarps / 2; n > 0; n >>= 1)
+#pragma unroll
+          for (int w = 0; w < n; ++w) v[w] += v[w + n];
+        return bias ? v[0] + bias[e] : v[0];
+      };
+      if (lane < E) l0 = logit(lane);
+      if (lane + 32 < E) l1 = logit(lane + 32);
       warp_route_finish(l0, l1, E, k, renorm, lane, topk_idx + (size_t)t * k, topk_w + (size_t)t * k,
                         probs ? probs + (size_t)t * E : nullptr);
     }

@@ -51,6 +51,7 @@ constexpr int kEpiWarps = 2;  // (12 warps in all: three per SM sub-partition, 1
 constexpr int kWeightWarp = kEpiWarp0 + kEpiWarps;
 constexpr int kVectorWarp = kWeightWarp + 1;
 constexpr int kThreads = (kVectorWarp + 1) * 32;
+static_assert(kThreads == 12 * 32, "the router adds twelve warps' shares");
 constexpr int kTileRows = 16;
 constexpr int kTok = 8;                          // tokens of one expert per pass (N of the MMA)
 constexpr int kTerms = 3;                        // bf16 terms of an fp32 value
@@ -212,9 +213,13 @@ __device__ __forceinline__ uint64_t l2_policy_normal() {
 // All groups of one product by one consumer warp.  The loops stay rolled and serve all products (bf16 token rows meet
 // zeros as their second and third term): a launch runs each of them a few dozen times only, and code that is fetched
 // anew from L2 for every tile costs more than the idle columns.
-// The 8 columns of an MMA are two tokens with four columns each, their three terms and a zero: most experts have one or
-// two of the tokens, and one MMA then does what three (one per term) did; the columns of a token are added by its
-// two lanes.
+// The 8 columns of an MMA are two tokens with four columns each: most experts have one or two of the tokens, and one MMA
+// then does what three (one per term) did; the columns of a token are added by its two lanes.
+// An MMA's sums are cut, not rounded, which pulls every product towards zero by as much as its LARGEST term is long.  So the
+// first term has two columns, eight of an MMA's sixteen k-values in either (the second and third terms have one each), every
+// MMA starts at zero, and all adding up is done in fp32, in pairs.  Relative error of the layer (d 1600, f 4352, r 800, fp32
+// rows) against 64 bits: fp32 multiply-adds 2.7e-7; one column per term and two MMAs in a row 2.9e-7, of which 1.8e-7 is that
+// pull; as it is 2.1e-7.  (Eight products per MMA, m16n8k8, instead of the second column: 2.2e-7 and 4 % slower.)
 __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, const unsigned char* stages,
                                         const unsigned char* vecs, float* parts, Ring& rs, Ring& rv, unsigned& turn, Ring& rp,
                                         int warp, int lane) {
@@ -229,6 +234,8 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
   const int g8 = lane >> 2, q4 = lane & 3;
   const uint32_t a_lane = (uint32_t)g8 * (kBoxK * 2) + q4 * 16;
   const int term = g8 & 3, col = tw * kUnit + q4 * 8;
+  const bool live = term == 0 || term == 3 || nt == kTerms;
+  const uint32_t even = live && term != 3 ? ~0u : 0u, odd = live && term != 0 ? ~0u : 0u;  // of the k-values, in pairs of pairs
   constexpr int kUnitStep = kTeamWarps * kUnit;
   const int n_vecs = sm.n_vecs;
   const bool by_group = teams_by_group(ph);
@@ -259,7 +266,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
           return false;
         }
         const unsigned char* vec = vecs + (team * (uint32_t)kTok + (uint32_t)(rv.slot * sm.vec_toks)) * kTokBytes +
-                                   (term < nt ? term : 0) * (kTermRun * 2) + col * 2;
+                                   (term < nt ? term : 0) * (kTermRun * 2) + col * 2;  // (column 3: the first term again)
         // (no branches below: what lies past the vector's end is fetched and dropped, and the weights that would meet it
         // are those of unit 0, which are finite, or the zeros TMA puts past the end of a row)
         uint32_t a_off[kUnits];
@@ -289,21 +296,22 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
 #pragma unroll
             for (int j = 0; j < kUnits; ++j) {
               b[j] = *reinterpret_cast<const uint4*>(vt + j * (kUnitStep * 2));
-              if (col + j * kUnitStep >= width || term >= nt) b[j] = make_uint4(0u, 0u, 0u, 0u);
+              const bool in = col + j * kUnitStep < width;
+              b[j].x &= in ? even : 0u, b[j].y &= in ? odd : 0u, b[j].z &= in ? even : 0u, b[j].w &= in ? odd : 0u;
             }
-            // Every unit has accumulators of its own, added up in fp32: the MMA's sums are cut, not rounded (one accumulator
-            // over the whole contraction: 1.2e-6 relative error at K = 4352 against 2.6e-7 of fp32 multiply-adds).
-            float m[kUnits][4];
+            float m[2 * kUnits][4];
+#pragma unroll
+            for (int j = 0; j < 2 * kUnits; ++j) m[j][0] = m[j][1] = m[j][2] = m[j][3] = 0.f;
 #pragma unroll
             for (int j = 0; j < kUnits; ++j) {
-              m[j][0] = m[j][1] = m[j][2] = m[j][3] = 0.f;
               mma16(m[j], lo[j].x, hi[j].x, lo[j].y, hi[j].y, b[j].x, b[j].y);
+              mma16(m[kUnits + j], lo[j].z, hi[j].z, lo[j].w, hi[j].w, b[j].z, b[j].w);
             }
 #pragma unroll
-            for (int j = 0; j < kUnits; ++j) mma16(m[j], lo[j].z, hi[j].z, lo[j].w, hi[j].w, b[j].z, b[j].w);
-            float top = 0.f, bot = 0.f;  // rows g8 and g8 + 8: this lane's two columns
+            for (int n = kUnits; n > 0; n >>= 1)
 #pragma unroll
-            for (int j = 0; j < kUnits; ++j) top += m[j][1] + m[j][0], bot += m[j][3] + m[j][2];
+              for (int j = 0; j < n; ++j) add4(m[j], m[j + n]);
+            const float top = m[0][1] + m[0][0], bot = m[0][3] + m[0][2];  // rows g8 and g8 + 8: this lane's two columns
             const float send = (q4 & 1) ? top : bot, keep = (q4 & 1) ? bot : top;
             const float v = keep + __shfl_xor_sync(0xffffffffu, send, 1);
             dst[t0 * kPartTok] = first ? v : dst[t0 * kPartTok] + v;
@@ -382,7 +390,10 @@ __device__ __forceinline__ void route_tokens(const WtParams& P, WtSmem& sm, floa
   for (int t = warp; t < P.T; t += kThreads / 32) {
     float l = 0.f;
     if (lane < P.E) {
-      for (int w = 0; w < kThreads / 32; ++w) l += part[(w * 16 + t) * 16 + lane];
+      float a[kThreads / 64];  // (in pairs: a serial sum of the warps' shares loses more than all that is in front of it)
+#pragma unroll
+      for (int w = 0; w < kThreads / 64; ++w) a[w] = part[(2 * w * 16 + t) * 16 + lane] + part[((2 * w + 1) * 16 + t) * 16 + lane];
+      l = ((a[0] + a[1]) + (a[2] + a[3])) + (a[4] + a[5]);
       if (P.b_router) l += P.b_router[lane];
     }
     warp_route_finish(l, 0.f, P.E, P.k, P.renorm, lane, sm.stage_e + t * P.k, sm.stage_w + t * P.k, nullptr);

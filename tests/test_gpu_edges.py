@@ -103,3 +103,32 @@ def test_dense_decode_of_several_tokens_with_many_pairs(T):
     sh = shape(512, 1024, E=16, k=8)                    # 64 and 128 pairs: beyond one per lane; every expert active
     lay, t, host = U.build(sh, T, path=1)
     U.check_layer(lay, t, host, sh.top_k)
+
+
+def error_against_64_bits(got, want):
+    """Of an output as a whole: its RMS error, and how far it is pulled along the result (both relative)."""
+    err = got - want
+    return (err ** 2).sum() ** 0.5 / (want ** 2).sum() ** 0.5, float((err * want).sum() / (want ** 2).sum())
+
+
+@pytest.mark.parametrize("sh,T", [(shape(1600, 4352, r=800, xd="f32"), 5), (shape(512, 1024, E=16, k=4, r=256, xd="f32"), 7),
+                                  (shape(256, 512, r=32, xd="f32"), 16)])
+def test_decomposed_decode_of_several_tokens_sums_like_fp32(sh, T):
+    """Four products in a row, each a sum in fp32: about ten roundings in pairs or runs, 0.42 * 2^-24 of the value each (RMS), are
+    1.4 * 2^-24 per product; h takes t's error twice, y all of them: 3.5 * 2^-24, so below 2^-22.  Sums that are rounded pull the
+    result nowhere; 2^-23 of it is allowed (sums that a tensor core cuts over 32 products pull by 3 * 2^-24, four of them)."""
+    lay, t, host = U.build(sh, T)
+    rel, ora, y = U.check_layer(lay, t, host, sh.top_k, tol=F32_TOL)
+    rms, pull = error_against_64_bits(U.to64(y), ora["y"])
+    assert rms <= 2.0 ** -22 and abs(pull) <= 2.0 ** -23, (rms, pull)
+
+
+@pytest.mark.parametrize("d,E,k,T", [(1024, 8, 2, 512), (2048, 16, 4, 600), (512, 8, 2, 1000)])
+def test_router_of_many_tokens_sums_like_fp32(d, E, k, T):
+    """bf16 rows: products are exact in fp32, and fp32 multiply-adds with the same number of additions in a row leave
+    1.3 * 2^-24 to 1.6 * 2^-24 of the probabilities (measured: 512 to 2048 features); sums cut over 64 products 1.7 to 2.1."""
+    sh = shape(d, 64, E=E, k=k)
+    lay, t, host = U.build(sh, T)
+    _, _, probs = lay.route(t["x"], want_probs=True)
+    rms, _ = error_against_64_bits(probs.cpu().numpy().astype("float64"), O.route(host["x"], host["w_router"], None, k)[1])
+    assert rms <= (1.5 if E == 8 else 1.8) * 2.0 ** -24, rms / 2.0 ** -24
