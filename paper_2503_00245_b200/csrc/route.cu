@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(kRtWarps * 32)
   pdl_wait();  // x may come from the kernel before
   __syncthreads();
   const int t0 = blockIdx.x * kRtTokens, g = lane >> 2, q = lane & 3;
-  const XT* const row0 = x + (size_t)min(t0 + g, T - 1) * d + q * 8;
-  const XT* const row1 = x + (size_t)min(t0 + g + 8, T - 1) * d + q * 8;
+  const XT* const row0 = x + (size_t)min(t0 + g, T - 1) * d;
+  const XT* const row1 = x + (size_t)min(t0 + g + 8, T - 1) * d;
   float* const mine = part + (warp * kRtTokens + g) * sh.e8 + 2 * q;
   for (int u0 = warp; u0 < units || u0 == warp; u0 += kRtWarps * kRtBatch) {
     uint4 a[kRtBatch][2][NT];
@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(kRtWarps * 32)
     for (int j = 0; j < kRtBatch; ++j)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int c = (u0 + j * kRtWarps) * kRtUnit;
-        const bool in = c + q * 8 < d;  // (what lies past the row: zeros)
+        const int c = (u0 + j * kRtWarps) * kRtUnit + q * 8;
+        const bool in = c < d;  // (what lies past the row: zeros, in place of its first eight values)
         const XT* src = (h ? row1 : row0) + (in ? c : 0);
         if constexpr (NT == 1) {
           a[j][h][0] = *reinterpret_cast<const uint4*>(src);

@@ -81,6 +81,28 @@ def test_many_tokens_routed_and_grouped(sh, T):
         check_prefill(lay, t, host, sh.top_k)
 
 
+@pytest.mark.parametrize("xd", ["bf16", "f32"])
+@pytest.mark.parametrize("d", [8, 16, 24, 40])
+@pytest.mark.parametrize("T", [17, 32])
+def test_rows_shorter_than_a_unit_of_the_router(d, T, xd):
+    """Fewer features than the 32 a group of lanes takes at once (and one more than that): nothing past a row counts, wherever x
+    lies in memory."""
+    sh = shape(d, 64, xd=xd)
+    t = W.make_layer(sh, T, device="cuda")
+    room = torch.full((T * d + 64,), float("nan"), dtype=t["x"].dtype, device="cuda")
+    room[:T * d] = t["x"].reshape(-1)
+    t["x"] = room[:T * d].view(T, d)
+    lay, t, host = U.build(sh, T, tensors=t)
+    idx, w, probs = lay.route(t["x"], want_probs=True)
+    torch.cuda.synchronize()
+    R, Wt, S, wo = O.route(host["x"], host["w_router"], host["b_router"], sh.top_k, True)
+    U.check_routing(idx.cpu().numpy(), w.cpu().numpy(), {"logits": R, "topk_idx": S, "topk_w": wo}, sh.top_k)
+    assert abs(probs.cpu().numpy() - Wt).max() <= U.W_TOL
+    offsets, perm, inv = lay.permute(idx)
+    assert torch.equal(lay.forward(t["x"]), lay.combine(lay.expert_ffn(t["x"], offsets, perm), w, inv))
+    assert lay.check() == 0
+
+
 @pytest.mark.parametrize("sh,T", [
     (shape(1440, 1280), 100),                           # three or four planes, columns no multiple of a tile
     (shape(200, 2000, E=2, k=1), 40),                   # a row of d shorter than one round of the combine's loads
