@@ -190,7 +190,11 @@ int moe_workspace_bytes(const moe_config* cfg, int32_t T, size_t* bytes) {
   int rc = validate_config(cfg);
   if (rc != MOE_OK) return rc;
   if (T < 0) return MOE_ERR_INVALID_ARG;
+  // A caller sizes its scratch once, for the most tokens it will pass, and a call with fewer may need more: decode steps keep
+  // vectors of their own, and up to kKSplitMaxSlots slots come as several planes.  In between the need grows with T.
   *bytes = ws_layout(*cfg, T).total;
+  for (const int fewer : {(int)MOE_STREAM_MAX_TOKENS, kKSplitMaxSlots / cfg->top_k})
+    if (fewer < T) *bytes = std::max(*bytes, ws_layout(*cfg, fewer).total);
   return MOE_OK;
 }
 

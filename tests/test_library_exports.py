@@ -49,6 +49,15 @@ def test_host_only_calls_work_without_a_gpu(lib):
     assert e.value.status == 1
 
 
+@pytest.mark.parametrize("d,f,E,k,r,xd", [(2048, 5632, 8, 2, 128, 1), (1600, 4352, 8, 2, 800, 0), (256, 512, 16, 4, 64, 0), (1024, 2816, 8, 8, 0, 1)])
+def test_scratch_for_many_tokens_is_enough_for_fewer(lib, d, f, E, k, r, xd):
+    """A layer's scratch is sized once, for its largest call; every smaller call must find it large enough."""
+    from paper_2503_00245_b200 import binding as B
+    cfg = B.make_config(d, f, E, k, r, xd)
+    need = [B.moe_workspace_bytes(cfg, T) for T in range(0, 2048 // k + 40)]
+    assert need == sorted(need)
+
+
 def test_no_cpu_fallback_without_a_device():
     import torch
     if torch.cuda.is_available():
