@@ -96,7 +96,14 @@ def _lib():
 
 
 # the current stream's handle, without the Stream object that torch.cuda.current_stream() builds on every call
-_current_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+try:
+    from torch._C import _cuda_getCurrentRawStream as _current_raw_stream, _cuda_getDevice as _current_device
+except ImportError:  # a PyTorch without them (one built without CUDA): the package imports all the same
+    def _current_device():
+        return torch.cuda.current_device()
+
+    def _current_raw_stream(device):
+        return torch.cuda.current_stream(device).cuda_stream
 
 
 def _ptr(t) -> int | None:
