@@ -208,6 +208,8 @@ def moe_combine(ctx, out_slots, topk_w, inv, T, y, stream=None):
 
 
 def moe_layer_forward(ctx, x, T, w: moe_weights, y, topk_idx=None, topk_w=None, ws=None, stream=None):
+    if not isinstance(w, moe_weights):  # (what a typed pointer argument would say)
+        raise C.ArgumentError(f"moe_layer_forward: expected moe_weights, got {type(w).__name__}")
     rc = (_LIB or _lib()).moe_layer_forward(
         ctx, _ptr(x), T, C.addressof(w), _ptr(y), None if topk_idx is None else _ptr(topk_idx),
         None if topk_w is None else _ptr(topk_w), _ptr(ws), ws.nbytes,
