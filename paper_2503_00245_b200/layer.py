@@ -39,6 +39,7 @@ class MoELayer:
         self.d, self.f, self.E, self.k = d_model, d_ff, n_experts, top_k
         self.x_dtype = x_dtype
         self.device = w_router.device
+        self._cuda_index = self.device.index if self.device.type == "cuda" else None
         self.rank = 0 if wd is None else wd[0].shape[1]
         self.cfg = B.make_config(d_model, d_ff, n_experts, top_k, self.rank,
                                  B.MOE_F32 if x_dtype == torch.float32 else B.MOE_BF16, int(renorm), path)
@@ -102,8 +103,10 @@ class MoELayer:
         if T > self.max_tokens:
             self._need(T)
         if y is None:
-            # one token's layer takes about as long as a few calls into PyTorch: y is allocated the cheapest way
-            if x.is_cuda and len(shape) == 2 and shape[1] == self.d and x.dtype == self.x_dtype:
+            # one token's layer takes about as long as a few calls into PyTorch: y is allocated the cheapest way where that
+            # gives the same tensor (a plain one on the layer's device)
+            if (x.get_device() == self._cuda_index and type(x) is torch.Tensor and len(shape) == 2 and shape[1] == self.d
+                    and x.dtype == self.x_dtype):
                 y = torch.empty_like(x)
             else:
                 y = torch.empty((T, self.d), dtype=self.x_dtype, device=self.device)
