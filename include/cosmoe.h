@@ -22,6 +22,10 @@
  *  - One moe_ctx serves one stream at a time: calls on the same ctx from two
  *    streams that overlap on the device race on the ctx's barrier state.
  *  - Weights are read-only for the library and may be shared between ctxs.
+ *  - Kernels that use programmatic dependent launch overlap the end of the kernel in front of them in the stream.  What
+ *    that one writes is read after it has completed, with one exception: decode calls of dense experts, and of one token,
+ *    read w_router earlier.  If the kernel in front lets its successors start early (griddepcontrol.launch_dependents; this
+ *    library's do) it must not write w_router for such a call.
  *  - Shapes: d_model, d_ff and wd_rank multiples of 8; 1 <= top_k <= n_experts <= 64;
  *    top_k <= 8.  Anything else: MOE_ERR_UNSUPPORTED, nothing is read or written.
  *    The streaming path of dense experts also needs d_model <= 2048.

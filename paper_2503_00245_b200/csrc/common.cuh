@@ -280,9 +280,24 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src, uint32
       : "memory");
 }
 
+// 16 bytes that a kernel before may have written, past L1, asked for here and not where they are used
+__device__ __forceinline__ uint4 ldcg_now(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 // Asks for bytes (16-byte aligned, a multiple of 16) to be brought into L2; fire and forget.
 __device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
+// The CTAs of a launch that fills the GPU ask for their shares of the router's matrix, before they wait for the kernel ahead of
+// them: that one may still be writing it, so its VALUES are fetched after the wait, but then they come from L2 (where a later
+// write changes them).  (No division: this stands in front of a decode launch's first load.)
+__device__ __forceinline__ void prefetch_router(const uint16_t* w_router, int d, int E) {
+  const uint32_t bytes = (uint32_t)d * E * 2u, run = bytes > 128u * 256u ? 2048u : 256u, lo = blockIdx.x * run;
+  if (lo < bytes) prefetch_l2(reinterpret_cast<const unsigned char*>(w_router) + lo, min(run, bytes - lo));
 }
 
 // Same, with an L2 eviction-priority hint: evict_first for data that is read exactly once (streamed weights),

@@ -139,27 +139,14 @@ __global__ void __launch_bounds__(kRtWarps * 32)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
   const int units = (d + kRtUnit - 1) / kRtUnit;
-  for (int r = tid; r < units * kRtUnit; r += kRtWarps * 32) {
-    for (int e8 = 0; e8 < sh.e8; e8 += 8) {
-      uint16_t v[8];
-      if (r < d && (E & 7) == 0) {
-        *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(w_router + (size_t)r * E + e8));
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = r < d && e8 + e < E ? __ldg(w_router + (size_t)r * E + e8 + e) : (uint16_t)0;
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) *reinterpret_cast<uint16_t*>(rt_smem + (e8 + e) * sh.row_bytes + r * 2) = v[e];
-    }
-  }
-  pdl_wait();  // x may come from the kernel before
-  __syncthreads();
+  for (uint32_t i = tid * 128u, n = (uint32_t)d * E * 2u; i < n; i += kRtWarps * 32 * 128u)  // (W_r: its lines into L2 ...)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const unsigned char*>(w_router) + i));
+  pdl_wait();  // (... its values, like x, may come from the kernel before)
   const int t0 = blockIdx.x * kRtTokens, g = lane >> 2, q = lane & 3;
   const XT* const row0 = x + (size_t)min(t0 + g, T - 1) * d;
   const XT* const row1 = x + (size_t)min(t0 + g + 8, T - 1) * d;
-  float* const mine = part + (warp * kRtTokens + g) * sh.e8 + 2 * q;
-  for (int u0 = warp; u0 < units || u0 == warp; u0 += kRtWarps * kRtBatch) {
-    uint4 a[kRtBatch][2][NT];
+  uint4 a[kRtBatch][2][NT];
+  auto fetch = [&](int u0) {
 #pragma unroll
     for (int j = 0; j < kRtBatch; ++j)
 #pragma unroll
@@ -168,7 +155,7 @@ __global__ void __launch_bounds__(kRtWarps * 32)
         const bool in = c < d;  // (what lies past the row: zeros, in place of its first eight values)
         const XT* src = (h ? row1 : row0) + (in ? c : 0);
         if constexpr (NT == 1) {
-          a[j][h][0] = *reinterpret_cast<const uint4*>(src);
+          a[j][h][0] = ldcg_now(reinterpret_cast<const uint4*>(src));
           if (!in) a[j][h][0] = make_uint4(0u, 0u, 0u, 0u);
         } else {
           float f[8];
@@ -182,6 +169,35 @@ __global__ void __launch_bounds__(kRtWarps * 32)
                                     tm[4][t] | (uint32_t)tm[5][t] << 16, tm[6][t] | (uint32_t)tm[7][t] << 16);
         }
       }
+  };
+  if (NT == 1) fetch(warp);  // on its way while W_r is laid out (fp32 rows: no registers for that)
+  constexpr int kRowsFly = 4;  // rows of W_r a thread has on their way at a time (d <= 2048: one round trip)
+  for (int e8 = 0; e8 < sh.e8; e8 += 8)
+    for (int r0 = tid; r0 < units * kRtUnit; r0 += kRowsFly * kRtWarps * 32) {
+      uint16_t v[kRowsFly][8];
+#pragma unroll
+      for (int u = 0; u < kRowsFly; ++u) {
+        const int r = r0 + u * kRtWarps * 32;
+        if ((E & 7) == 0) {
+          const uint4 w = ldcg_now(reinterpret_cast<const uint4*>(w_router + (size_t)min(r, d - 1) * E + e8));
+          *reinterpret_cast<uint4*>(v[u]) = r < d ? w : make_uint4(0u, 0u, 0u, 0u);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[u][e] = r < d && e8 + e < E ? __ldcg(w_router + (size_t)r * E + e8 + e) : (uint16_t)0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kRowsFly; ++u) {
+        const int r = r0 + u * kRtWarps * 32;
+        if (r >= units * kRtUnit) break;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) *reinterpret_cast<uint16_t*>(rt_smem + (e8 + e) * sh.row_bytes + r * 2) = v[u][e];
+      }
+    }
+  __syncthreads();
+  float* const mine = part + (warp * kRtTokens + g) * sh.e8 + 2 * q;
+  for (int u0 = warp; u0 < units || u0 == warp; u0 += kRtWarps * kRtBatch) {
+    if (NT != 1 || u0 != warp) fetch(u0);
     for (int e8 = 0; e8 < sh.e8; e8 += 8) {
       const unsigned char* wrow = rt_smem + (e8 + g) * sh.row_bytes + q * 16;
       float sum[4];

@@ -334,25 +334,20 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
 }
 
 // Router (Eq. 2, Eq. 3) of all T tokens by every CTA, E = 8 or 16.  A thread owns the input features tid, tid + 384, ...:
-// their rows of W_r are fetched once (wr0: the first eight experts', before the dependency wait) and serve every token.
+// their rows of W_r are fetched once and serve every token.
 // part: [12 warps][16 tokens][16 experts].
 constexpr int kRouteQ = 6;  // features per thread and round: d <= 2304 in one
 __device__ __forceinline__ void route_fetch(const WtParams& P, int q0, int e8, int tid, uint4* wr) {
 #pragma unroll
   for (int q = 0; q < kRouteQ; ++q)
-    wr[q] = __ldg(reinterpret_cast<const uint4*>(P.w_router + (size_t)min(tid + (q0 + q) * kThreads, P.d - 1) * P.E + e8));
+    wr[q] = ldcg_now(reinterpret_cast<const uint4*>(P.w_router + (size_t)min(tid + (q0 + q) * kThreads, P.d - 1) * P.E + e8));
 }
-__device__ __forceinline__ void route_tokens(const WtParams& P, WtSmem& sm, float* part, const uint4* wr0, int tid) {
+__device__ __forceinline__ void route_tokens(const WtParams& P, WtSmem& sm, float* part, int tid) {
   const int lane = tid & 31, warp = tid >> 5, d = P.d;
   for (int e8 = 0; e8 < P.E; e8 += 8) {
     for (int q0 = 0; q0 * kThreads < d; q0 += kRouteQ) {
       uint4 wr[kRouteQ];
-      if (e8 == 0 && q0 == 0) {
-#pragma unroll
-        for (int q = 0; q < kRouteQ; ++q) wr[q] = wr0[q];
-      } else {
-        route_fetch(P, q0, e8, tid, wr);
-      }
+      route_fetch(P, q0, e8, tid, wr);
 #pragma unroll 1
       for (int t0 = 0; t0 < P.T; t0 += 4) {
         float xv[4][kRouteQ];  // four tokens' features in one round trip
@@ -431,10 +426,9 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
   }
   if (P.mode == 0)
     for (int i = tid; i < P.T * P.y_rows; i += kThreads) yacc[i] = 0.f;
-  uint4 wr0[kRouteQ];  // constants: fetched before the dependency wait
-  if (P.w_router) route_fetch(P, 0, 0, tid, wr0);
+  if (P.w_router && tid == 0) prefetch_router(P.w_router, P.d, P.E);
   pdl_wait();
-  if (P.w_router) route_tokens(P, sm, parts, wr0, tid);
+  if (P.w_router) route_tokens(P, sm, parts, tid);
 
   // ---------------------------------------------------------------- routing -> active experts and their slots
   const int n = P.T * P.k;

@@ -154,3 +154,23 @@ def test_router_of_many_tokens_sums_like_fp32(d, E, k, T):
     _, _, probs = lay.route(t["x"], want_probs=True)
     rms, _ = error_against_64_bits(probs.cpu().numpy().astype("float64"), O.route(host["x"], host["w_router"], None, k)[1])
     assert rms <= (1.5 if E == 8 else 1.8) * 2.0 ** -24, rms / 2.0 ** -24
+
+
+@pytest.mark.parametrize("r,T,k", [(0, 40, 2), (0, 100, 2), (64, 5, 2), (64, 16, 4), (64, 40, 2)])
+def test_router_weights_written_by_the_call_before(r, T, k):
+    """The kernel in front of a layer in the stream may be what writes its w_router, and may let its successor start early (as this
+    library's do): here another layer's output is that matrix.  Nothing of it may be read before it is complete."""
+    writer, tw, _ = U.build(W.WEARABLE, 8)
+    lay, t, _ = U.build(shape(1024, 1024, k=k, r=r), T)
+    matrix = t["w_router"].view(8, 1024)             # [d][E] = [1024][8], as the writer's [T][d]
+    out, want = [], []
+    for step in range(12):
+        xw = W.make_x(W.WEARABLE, 8, device="cuda", step=step)
+        writer.forward(xw, y=matrix)
+        out.append(lay.forward(t["x"]))
+        torch.cuda.synchronize()
+        want.append(lay.forward(t["x"]))
+        torch.cuda.synchronize()
+    assert lay.check() == 0 and writer.check() == 0
+    assert all(torch.equal(a, b) for a, b in zip(out, want))
+    assert not torch.equal(want[0], want[1])         # (the matrix does change)
