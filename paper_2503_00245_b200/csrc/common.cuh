@@ -246,6 +246,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
 }
 
+// The same for a whole warp whose lanes go on to meet in shuffles and votes: all of them give up, or none does.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+
 // Same contract, but polls with the non-blocking test_wait: the waiter is never parked by the hardware.
 // For short waits between warps of one CTA.
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {

@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       int k0 = kb0 * kBK;
       int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        if (it >= NS && !__all_sync(0xffffffffu, mbar_wait(&sm.empty[slot], par))) {
+        if (it >= NS && !mbar_wait_warp(&sm.empty[slot], par)) {
           if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x400u);
           sm.abort = 1;
           ok = false;
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       for (int idx = pair; ok && idx < n_work; idx += n_pairs, ++tile_i) {
         const int buf = tile_i & 1;
         if (tile_i >= 2) {  // the accumulators two tiles back must have left this buffer, in both CTAs
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1))) {
+          if (!mbar_wait_warp(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1)) {
             if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x403u);
             sm.abort = 1;
             break;
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
         const int kb0 = ks * num_kb / P.ksplit, kb1 = (ks + 1) * num_kb / P.ksplit;
         uint32_t acc = 0;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.full[slot], par))) {
+          if (!mbar_wait_warp(&sm.full[slot], par)) {
             if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x401u);
             sm.abort = 1;
             ok = false;
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     for (int idx = pair; idx < n_work; idx += n_pairs, ++tile_i) {
       const Tile t = decode_tile(P, tm, idx, n_tiles);
       const int buf = tile_i & 1;
-      if (!mbar_wait(&sm.accum_full[buf], (tile_i >> 1) & 1)) {
+      if (!mbar_wait_warp(&sm.accum_full[buf], (tile_i >> 1) & 1)) {
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x402u);
         break;
       }

@@ -210,7 +210,8 @@ __device__ __forceinline__ uint64_t l2_policy_normal() {
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-// All groups of one product by one consumer warp.  The loops stay rolled and serve all products (bf16 token rows meet
+// All groups of one product by one consumer warp.  (A lane that gives up a wait leaves the kernel, so none waits for it.)
+// The loops stay rolled and serve all products (bf16 token rows meet
 // zeros as their second and third term): a launch runs each of them a few dozen times only, and code that is fetched
 // anew from L2 for every tile costs more than the idle columns.
 // The 8 columns of an MMA are two tokens with four columns each: most experts have one or two of the tokens, and one MMA
@@ -680,7 +681,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       const Product& pr = P.pr[ph];
       const bool by_group = teams_by_group(ph);
       ok = walk(P, sm, ph, [&](const Group& g) -> bool {
-        if (!mbar_wait(&sm.pfull[rp.slot], rp.par)) {
+        if (!mbar_wait_warp(&sm.pfull[rp.slot], rp.par)) {
           if (lane == 0) give_up(P, sm, 0x640u);
           return false;
         }
