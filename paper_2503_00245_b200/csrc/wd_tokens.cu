@@ -210,7 +210,7 @@ __device__ __forceinline__ uint64_t l2_policy_normal() {
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-// All groups of one product by one consumer warp.  (A lane that gives up a wait leaves the kernel, so none waits for it.)
+// All groups of one product by one consumer warp.  (A lane that gives up a wait says so and leaves the kernel: none waits for it.)
 // The loops stay rolled and serve all products (bf16 token rows meet
 // zeros as their second and third term): a launch runs each of them a few dozen times only, and code that is fetched
 // anew from L2 for every tile costs more than the idle columns.
@@ -243,7 +243,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
   return walk(P, sm, ph, [&](const Group& g) -> bool {
     const int tiles = (g.rows + kTileRows - 1) / kTileRows;
     if (rp.n >= 2 && !mbar_wait(&sm.pfree[rp.slot], rp.par ^ 1u)) {
-      if (lane == 0) give_up(P, sm, 0x612u);
+      give_up(P, sm, 0x612u);
       return false;
     }
     if (by_group && turn++ % kTeams != team) {
@@ -263,7 +263,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
       for (int sub = 0; sub < nsub; ++sub) {
         if (!by_group && turn++ % kTeams != team) continue;
         if (!mbar_wait(&sm.vfull[team][rv.slot], rv.par)) {
-          if (lane == 0) give_up(P, sm, 0x610u);
+          give_up(P, sm, 0x610u);
           return false;
         }
         const unsigned char* vec = vecs + (team * (uint32_t)kTok + (uint32_t)(rv.slot * sm.vec_toks)) * kTokBytes +
@@ -279,7 +279,7 @@ __device__ __forceinline__ bool consume(const WtParams& P, WtSmem& sm, int ph, c
 #pragma unroll 1
         for (int u = 0; u < tiles; ++u) {
           if (!mbar_wait(&sm.full[team][rs.slot], rs.par)) {
-            if (lane == 0) give_up(P, sm, 0x611u);
+            give_up(P, sm, 0x611u);
             return false;
           }
           const unsigned char* st = stages + (team * (uint32_t)P.n_stages + (uint32_t)rs.slot) * kStageBytes;
