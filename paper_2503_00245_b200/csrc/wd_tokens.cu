@@ -70,7 +70,7 @@ constexpr int kTermRun = kWdTermRun;             // values between two terms of 
 constexpr int kVecRun = kTerms * kTermRun;       // values of one token's slice, in memory as in shared memory
 constexpr int kTokBytes = kVecRun * 2;
 constexpr int kMaxStages = 5;                    // of one team
-constexpr int kMaxVecs = 4;
+constexpr int kMaxVecs = 8;
 constexpr int kGroupTiles = 4;                   // tiles of 16 rows of a group
 constexpr int kPartTok = kTileRows;              // floats between two tokens' partial sums
 constexpr int kPartTile = kTok * kPartTok;
@@ -153,30 +153,34 @@ struct Group {
   bool last_use;  // no further token group reads these rows
 };
 
-// Every role walks this list of groups: a pure function of (routing, product, CTA).
-template <class F>
-__device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph, F&& body) {
+// This CTA's rows of a product: [g0, g1) of all active experts' rows in a row, beginning in expert a0 (product 3: of each one's).
+struct Share {
+  int g0, g1, a0;
+};
+__device__ __forceinline__ Share share_of(const WtParams& P, const WtSmem& sm, int ph) {
   const int N = P.pr[ph].rows, na = sm.n_act;
   const long long b = blockIdx.x, G = gridDim.x;
-  const bool split_out = ph == kProducts - 1;
-  constexpr int per = kGroupTiles * kTileRows;
-  int g0, g1, a0 = 0;
-  if (split_out) {
-    g0 = (int)(N * b / G), g1 = (int)(N * (b + 1) / G);
-  } else if ((int)G >= kAlignCtas * na) {
+  if (ph == kProducts - 1) return Share{(int)(N * b / G), (int)(N * (b + 1) / G), 0};
+  if ((int)G >= kAlignCtas * na) {
     // a CTA works for one expert: the first G mod na experts get one CTA more
     const int c = (int)G / na, more = (int)G - c * na, big = more * (c + 1), bi = (int)b;
-    a0 = bi < big ? bi / (c + 1) : more + (bi - big) / c;
+    const int a0 = bi < big ? bi / (c + 1) : more + (bi - big) / c;
     const int jn = bi < big ? bi - a0 * (c + 1) : bi - big - (a0 - more) * c, cn = bi < big ? c + 1 : c;
-    g0 = a0 * N + (int)((long long)N * jn / cn), g1 = a0 * N + (int)((long long)N * (jn + 1) / cn);
-  } else {
-    const long long tot = (long long)na * N;
-    g0 = (int)(tot * b / G), g1 = (int)(tot * (b + 1) / G);
-    a0 = g0 / N;
+    return Share{a0 * N + (int)((long long)N * jn / cn), a0 * N + (int)((long long)N * (jn + 1) / cn), a0};
   }
-  if (g0 >= g1) return true;
-  for (int a = a0; a < na; ++a) {
-    const int lo = split_out ? g0 : max(g0 - a * N, 0), hi = split_out ? g1 : min(g1 - a * N, N);
+  const long long tot = (long long)na * N;
+  const int g0 = (int)(tot * b / G);
+  return Share{g0, (int)(tot * (b + 1) / G), g0 / N};
+}
+// Every role walks this list of groups: a pure function of (routing, product, CTA).
+template <class F>
+__device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph, const Share& my, F&& body) {
+  const int N = P.pr[ph].rows, na = sm.n_act;
+  const bool split_out = ph == kProducts - 1;
+  constexpr int per = kGroupTiles * kTileRows;
+  if (my.g0 >= my.g1) return true;
+  for (int a = my.a0; a < na; ++a) {
+    const int lo = split_out ? my.g0 : max(my.g0 - a * N, 0), hi = split_out ? my.g1 : min(my.g1 - a * N, N);
     if (hi <= lo) break;
     const int groups = (hi - lo + per - 1) / per;
     const int step = ((hi - lo + groups - 1) / groups + kTileRows - 1) / kTileRows * kTileRows;
@@ -186,6 +190,10 @@ __device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph
         if (!body(Group{a, s0, min(kTok, s_hi - s0), r0, min(step, hi - r0), s0 + kTok >= s_hi})) return false;
   }
   return true;
+}
+template <class F>
+__device__ __forceinline__ bool walk(const WtParams& P, const WtSmem& sm, int ph, F&& body) {
+  return walk(P, sm, ph, share_of(P, sm, ph), body);
 }
 
 // The two consumer teams take the slices of the contraction in turn; in product 3, whose groups are one short tile per
@@ -510,34 +518,44 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: nobody streams anything
       if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
     }
-  } else if (tid == 0 && P.mode != 0) {
-    // the caller's grouping (moe_permute's products)
-    int na = 0, bad = 0;
-    sm.act_off[0] = 0;
-    for (int e = 0; e < P.E && !bad; ++e) {
-      const int lo = P.offsets[e], hi = P.offsets[e + 1];
-      if (lo < 0 || hi < lo || hi > n || (hi > lo && lo != sm.act_off[na])) {
-        bad = 1;
-        break;
+  } else if (warp == 0) {
+    // the caller's grouping (moe_permute's products): lane e works for experts e and e + 32
+    int bad = 0, run = 0, na = 0;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int e = lane + 32 * half;
+      const int lo = e < P.E ? P.offsets[e] : 0, hi = e < P.E ? P.offsets[e + 1] : 0;
+      const int c = hi - lo;
+      bad |= lo < 0 || c < 0 || hi > n;
+      int end = bad ? 0 : c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += u;
       }
-      if (hi == lo) continue;
-      for (int s = lo; s < hi; ++s) {
-        const int p = P.perm[s];
-        if (p < 0 || p >= n) {
-          bad = 1;
-          break;
-        }
-        sm.slot_tok[s] = p / P.k;
-        sm.slot_w[s] = 1.0f;
+      const bool any = !bad && c > 0;
+      const int off = run + end - c;
+      bad |= any && lo != off;
+      run += __shfl_sync(0xffffffffu, end, 31);
+      const unsigned m = __ballot_sync(0xffffffffu, any);
+      if (any) {
+        const int a = na + __popc(m & ((1u << lane) - 1u)), sl = P.expert_slot ? P.expert_slot[e] : e;
+        bad |= sl < 0;
+        sm.act_e[a] = e, sm.act_slot[a] = sl < 0 ? 0 : sl, sm.act_off[a] = off;
       }
-      const int sl = P.expert_slot ? P.expert_slot[e] : e;
-      bad |= sl < 0;
-      sm.act_e[na] = e, sm.act_slot[na] = sl < 0 ? 0 : sl;
-      sm.act_off[++na] = hi;
+      na += __popc(m);
     }
-    if (!bad && sm.act_off[na] != n) bad = 1;
-    if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
-    sm.n_act = bad ? 0 : na;
+    for (int s = lane; s < n; s += 32) {
+      const int p = P.perm[s];
+      bad |= p < 0 || p >= n;
+      sm.slot_tok[s] = p / P.k, sm.slot_w[s] = 1.0f;
+    }
+    bad = __any_sync(0xffffffffu, bad || run != n);
+    if (lane == 0) {
+      sm.act_off[bad ? 0 : na] = bad ? 0 : n;
+      sm.n_act = bad ? 0 : na;
+      if (bad) flag_error(st, MOE_ERR_STATE, 0x600u);
+    }
   }
   if (warp == 0) {
     // the vector buffers are cut to the tokens the busiest expert has: with few, more slices are on their way
@@ -606,6 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
     bool ok = true;
 #pragma unroll 1
     for (int ph = 0; ph < last && ok; ++ph) {
+      const Share my = share_of(P, sm, ph);  // (its divisions are done when the meeting is over)
       if (ph > 0) {  // every CTA has stored its outputs of the product before
         int met = 1;
         if (lane == 0) {
@@ -631,7 +650,7 @@ __global__ void __launch_bounds__(kThreads, 1) wd_tokens_kernel(const __grid_con
       const Product& pr = P.pr[ph];
       const int K = pr.K;
       const bool by_group = teams_by_group(ph);
-      ok = walk(P, sm, ph, [&](const Group& g) -> bool {
+      ok = walk(P, sm, ph, my, [&](const Group& g) -> bool {
         // lane = the token whose slices it brings
         const bool mine = lane < g.ns;
         const int s = g.slot0 + min(lane, g.ns - 1);
