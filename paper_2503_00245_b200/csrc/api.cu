@@ -135,6 +135,7 @@ int moe_create(const moe_config* cfg, moe_ctx** out) {
   c->cfg = *cfg;
   c->device = dev;
   c->launches = 0;
+  c->smem_ok = &c->smem_ok_own;
   c->fin_wait_budget = 0;
   c->d_state = nullptr;
   c->h_state = nullptr;

@@ -58,24 +58,30 @@ struct moe_ctx {
   long long* acc;                // device: fixed-point output accumulators of the dense streaming path, kept zero
   size_t acc_elems;              //         between calls by the kernel itself (MOE_STREAM_MAX_TOKENS*top_k*d)
   unsigned long long launches;
+  std::atomic<unsigned>* smem_ok;  // kernels that may use all the shared memory of a CTA, a bit each (allow_full_smem)
+  std::atomic<unsigned> smem_ok_own;
   long long fin_wait_budget;     // cycles the dense streaming kernel's finalisers wait for the arrival counter (0 = default)
 };
 
 namespace cosmoe {
 
-// Lets `Kernel` use all the dynamic shared memory the device offers a CTA: once per kernel and device instead of a
-// driver call in front of every launch.  (The limit only permits; a launch still takes what it asks for.)
+// Lets `Kernel` use all the dynamic shared memory the device offers a CTA: once per kernel and ctx instead of a driver call in
+// front of every launch.  (The limit only permits; a launch still takes what it asks for.  It is an attribute of the function
+// in one CUDA context, as a ctx's memory belongs to one: a device may have several.)
 constexpr int kMaxDevices = 64;
+inline unsigned next_smem_bit() {
+  static std::atomic<unsigned> n{0};
+  return 1u << n.fetch_add(1);
+}
 template <auto Kernel>
 int allow_full_smem(const moe_ctx* ctx) {
-  static std::atomic<bool> done[kMaxDevices];
-  const bool tracked = ctx->device >= 0 && ctx->device < kMaxDevices;
-  if (tracked && done[ctx->device].load(std::memory_order_acquire)) return MOE_OK;
+  static const unsigned bit = next_smem_bit();
+  if (ctx->smem_ok->load(std::memory_order_relaxed) & bit) return MOE_OK;
   cudaFuncAttributes fa{};
   MOE_CUDA_TRY(cudaFuncGetAttributes(&fa, Kernel));
   MOE_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     ctx->max_smem_optin - (int)fa.sharedSizeBytes));
-  if (tracked) done[ctx->device].store(true, std::memory_order_release);
+  ctx->smem_ok->fetch_or(bit, std::memory_order_relaxed);
   return MOE_OK;
 }
 

@@ -1611,6 +1611,7 @@ struct StaticDevice {
   int rc;               // outcome of the one-off set-up
   unsigned char* base;  // device address of g_static_scratch on this GPU
   int sm_count, max_smem_optin;
+  std::atomic<unsigned> smem_ok;  // as of a ctx: the array's address belongs to one CUDA context as well
 };
 StaticDevice g_static_dev[kMaxDevices];
 
@@ -1681,6 +1682,7 @@ extern "C" int moe_layer_forward_static(const moe_config* cfg, const void* x, in
   tmp.d_state = st;
   tmp.h_state = nullptr;
   tmp.acc = acc;
+  tmp.smem_ok = &sd->smem_ok;
   tmp.acc_elems = kStaticAccBytes / sizeof(long long);
   if (!dense_stream_fuses_route(tmp.cfg, T)) {
     rc = launch_route(&tmp, x, T, w, topk_idx, topk_w, nullptr, s);
