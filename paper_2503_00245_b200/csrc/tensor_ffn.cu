@@ -156,7 +156,24 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t* v) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// A load's registers may be read behind the wait only; going through it ties every use and copy of them to that place.
+__device__ __forceinline__ void tc_wait_ld(uint32_t* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+      : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+        "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+        "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+        "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+      :
+      : "memory");
+}
+__device__ __forceinline__ void tc_wait_ld(uint32_t* a, uint32_t* v) {  // two loads, one wait
+  tc_wait_ld(a);
+  asm volatile(""
+      : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+        "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+        "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+        "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]));
+}
 
 // Shared-memory operand descriptor (128-byte swizzle).  K-major tiles: rows of 128 bytes, 8-row groups 1024
 // bytes apart (stride byte offset), the leading offset is not used.  N-major tiles: 64 columns (128 bytes) per
@@ -497,7 +514,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           uint32_t g[32], u[32];
           tc_ld32(tbase + c, g);
           tc_ld32(tbase + P.bn + c, u);
-          tc_wait_ld();
+          tc_wait_ld(g, u);
           const int pieces = (ncols - c) / 8;  // of 16 bytes
           uint32_t o[16];
           if (P.epi == EPI_SWIGLU) {
@@ -520,7 +537,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           for (int i = 0; i < 4; ++i) {
             const int c = 32 * cpar + 64 * i;
             if (c < P.bn) {
-              tc_wait_ld();
+              tc_wait_ld(a[i & 1]);
               if (c + 64 < P.bn) tc_ld32(tbase + c + 64, a[(i + 1) & 1]);
               store_rows128(ebuf, lane, a[i & 1], out + c, P.ld_out * 4, rows, (ncols - c) / 4);
             }
@@ -529,7 +546,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           for (int c = 32 * cpar; c < P.bn; c += 64) {
             uint32_t a[32];
             tc_ld32(tbase + c, a);
-            tc_wait_ld();
+            tc_wait_ld(a);
             store_bf16(ebuf, lane, a, (__nv_bfloat16*)P.out + row0 * P.ld_out + t.n0 + c, P.ld_out * 2, rows, (ncols - c) / 8,
                        P.split ? P.out_off_lo : 0);
           }
