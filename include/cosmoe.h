@@ -20,7 +20,8 @@
  *    bounded wait, an index out of range) set a device status word that
  *    moe_check() reads; the output of that call is then undefined.
  *  - One moe_ctx serves one stream at a time: calls on the same ctx from two
- *    streams that overlap on the device race on the ctx's barrier state.
+ *    streams that overlap on the device race on the ctx's state (arrival counters, sums, the
+ *    grouping of a prefill).
  *  - Weights are read-only for the library and may be shared between ctxs.
  *  - Kernels that use programmatic dependent launch overlap the end of the kernel in front of them in the stream.  What
  *    that one writes is read after it has completed, with one exception: decode calls of dense experts, and of one token,
@@ -157,7 +158,8 @@ int moe_fp8_dequantize_rows(const void* codes, const float* scales, int64_t rows
 /* Router logits, softmax over experts (Eq. 2), top-k (Eq. 3), gate weights.
  * x dev [T][d] (cfg.x_dtype).  topk_idx dev [T][k] int32: descending weight, equal
  * weights to the lower expert index.  topk_w dev [T][k] fp32.  probs dev [T][E] fp32
- * or NULL.  fp32 arithmetic.  T >= 0 (T == 0 is a no-op).                          */
+ * or NULL.  fp32 sums of exact products (fp32 x bf16; above
+ * MOE_STREAM_MAX_TOKENS tokens on the tensor cores, whose sums of eight products are cut, not rounded).  T >= 0 (T == 0 is a no-op).                          */
 int moe_route(moe_ctx* ctx, const void* x, int32_t T, const moe_weights* w, int32_t* topk_idx, float* topk_w,
               float* probs, void* stream);
 

@@ -1080,7 +1080,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_stream_kernel(const DensePa
       sm.n_act = bad ? 0 : na;  // every CTA takes the same decision from the same data: no CTA streams anything
       if (bad) flag_error(st, MOE_ERR_STATE, 0x300u);
     }
-  } else if (kAllX && warp == 0 && !fused1 && !given1 && P.mode == 0) {
+  } else if (kAllX && warp == 0 && P.mode == 0) {
     // routing products -> active experts and their slots (same numbering as moe_permute): lane e works for
     // experts e and e + 32
     const int n = n_pairs, E = P.E;

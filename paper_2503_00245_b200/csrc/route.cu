@@ -378,7 +378,7 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
   const XT* xp = (const XT*)x;
   const uint16_t* wr = (const uint16_t*)w->w_router;
   const RtShape sh = rt_shape(c.d_model, c.n_experts);
-  // more than a decode step's tokens (16 would be a tile of a single CTA: those take a CTA per token), and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 24 experts)
+  // more than a decode step's tokens (16 would be a tile of a single CTA: those take a CTA per token), and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 16 experts)
   if (T > MOE_STREAM_MAX_TOKENS && sh.smem <= 112 * 1024) {
     MOE_TRY(allow_full_smem<route_tile_kernel<XT>>(ctx));
     MOE_CUDA_TRY(launch_pdl(route_tile_kernel<XT>, dim3((T + kRtTokens - 1) / kRtTokens), dim3(kRtWarps * 32), (size_t)sh.smem, s,

@@ -207,7 +207,6 @@ struct SmemGG {
   uint64_t accum_full[2];        // own: all MMAs of the tile in accumulator buffer b have completed
   uint64_t accum_empty[2];       // leader's: the epilogue warps of both CTAs have read buffer b out of TMEM
   uint32_t tmem_base;
-  int abort;
 };
 
 struct Tile {
@@ -330,7 +329,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   const uint32_t b_bytes = b_rows * kBK * 2;
   const uint32_t stage_bytes = n_a * a_bytes + 128u * kBK * 2u;
   unsigned char* stages = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* const epi_bufs = stages + (size_t)P.n_stages * stage_bytes;  // 2 KB per epilogue warp
+  unsigned char* const epi_bufs = stages + (size_t)P.n_stages * stage_bytes;  // kEpiBuf per epilogue warp
   SmemGG& sm = *reinterpret_cast<SmemGG*>(epi_bufs + kEpiWarps * kEpiBuf);
   const int tid = threadIdx.x, lane = tid & 31, warp = lane0(tid >> 5);
   const int NS = P.n_stages;
@@ -349,7 +348,6 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       mbar_init(&sm.accum_full[b], 1);
       mbar_init(&sm.accum_empty[b], 2 * kEpiWarps);
     }
-    sm.abort = 0;
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a0) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
     fence_mbar_init();
@@ -391,7 +389,6 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
         if (it >= NS && !mbar_wait_warp(&sm.empty[slot], par)) {
           if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x400u);
-          sm.abort = 1;
           ok = false;
           break;
         }
@@ -447,7 +444,6 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
         if (tile_i >= 2) {  // the accumulators two tiles back must have left this buffer, in both CTAs
           if (!mbar_wait_warp(&sm.accum_empty[buf], ((tile_i >> 1) - 1) & 1)) {
             if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x403u);
-            sm.abort = 1;
             break;
           }
           tc_fence_after();
@@ -459,7 +455,6 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait_warp(&sm.full[slot], par)) {
             if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x401u);
-            sm.abort = 1;
             ok = false;
             break;
           }

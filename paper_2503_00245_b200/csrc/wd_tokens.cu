@@ -15,7 +15,8 @@
 // fp32 value (8 + 8 + 8 significand bits), each with accumulators of its own, so t, h and v carry fp32 precision as
 // in the one-token kernels; bf16 token rows are one exact term.
 //
-// Rows of (active expert x product) are dealt to the CTAs (one per SM) evenly, row by row; in product 3 the CTAs split
+// Rows of (active expert x product) are dealt to the CTAs (one per SM) evenly, row by row, while there are many active experts;
+// with eight CTAs or more for each a CTA works for one of them (kAlignCtas); in product 3 the CTAs split
 // the output columns instead, each summing all experts itself, so every value has one writer and a fixed order of
 // summation: no atomics, results bit-identical from call to call.  Between the products the CTAs meet at an arrival
 // counter that runs over launches, with a bounded wait.
@@ -33,7 +34,7 @@
 //                          contraction inside a unit is free;
 //   2 epilogue warps       add the 8 warps' partial sums in order, SiLU * mul, split into terms, store.
 // Measured on B200, d 1600, f 4352, r 800, 8 experts, 2 active, T = 5, two layers (about 170 MB of factors each, 26 us at
-// the copy bandwidth): 133 us.  The kernel before it (fp32 multiply-adds, one warp for vectors, barriers and epilogues, a
+// the copy bandwidth): 134 to 139 us, by GPU.  The kernel before it (fp32 multiply-adds, one warp for vectors, barriers and epilogues, a
 // router launch of 10 us) took 430 to 470.  What a layer's 66 us go to: three meetings and the refill behind them (about 15), the
 // router (4), the products at 4 to 5 TB/s.
 #include <cuda.h>
