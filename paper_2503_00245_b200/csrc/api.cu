@@ -46,7 +46,11 @@ WsLayout ws_layout(const moe_config& c, int T) {
   L.vec_a = take(wd_stream ? n * 2 * rs * 6 : 0);
   L.vec_b = take(wd_stream ? n * fs * 6 : 0);
   L.vec_c = take(wd_stream ? n * std::max(rs * 6, (size_t)c.wd_rank * 8 * 4) : 0);
-  L.xperm = take(tensor_ok ? n * (size_t)c.d_model * 2 : 0);
+  L.pos = take(n * 4);
+  // by slot; or, dense experts, T rows per expert while that is not more than kScatterBytesMax (rounded so that fewer tokens
+  // never need more)
+  const size_t room = c.wd_rank == 0 ? std::min((size_t)c.n_experts * T * c.d_model * 2, kScatterBytesMax) : 0;
+  L.xperm = take(tensor_ok ? std::max(n * (size_t)c.d_model * 2, room) : 0);
   L.hidden = take(tensor_ok ? n * (size_t)c.d_ff * 2 : 0);
   const size_t rp = ((size_t)c.wd_rank + 63) / 64 * 64;            // the rank rounded up to the tensor path's K step
   L.mid_a = take(tensor_ok ? n * 4 * rp * 2 : 0);  // t_g, t_u as hi + lo bf16 pairs
@@ -305,6 +309,20 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   int32_t* perm = (int32_t*)(wsb + L.perm);
   int32_t* inv = (int32_t*)(wsb + L.inv);
   float* out_slots = (float*)(wsb + L.out_slots);
+  if (w->expert_slot) return MOE_ERR_UNSUPPORTED;  // the tensor path reads experts in place (slot == expert)
+  if (prefill_scatters(ctx->cfg, T) && route_tile_applies(ctx->cfg, T)) {
+    const Scatter sc{wsb + L.xperm, (int32_t*)(wsb + L.pos)};
+    MOE_TRY(launch_route(ctx, x, T, w, idx, wt, nullptr, s, nullptr, &sc));
+    const PrefillRows rows{wsb + L.xperm, ctx->d_state->route_count, idx, sc.pos, inv, nullptr};
+    int planes = 1;
+    rc = launch_dense_prefill(ctx, T, w, rows, wsb + L.hidden, out_slots, nullptr, &planes, s);
+    if (rc != MOE_OK) {  // (the router has counted, and nobody will clear the counts)
+      (void)cudaMemsetAsync(ctx->d_state->route_count, 0, sizeof(ctx->d_state->route_count), s);
+      (void)cudaGetLastError();
+      return rc;
+    }
+    return launch_combine(ctx, out_slots, wt, inv, T, y, planes, s);
+  }
   const Grouping grp{offsets, perm, inv};
   rc = launch_route(ctx, x, T, w, idx, wt, nullptr, s, &grp);
   if (rc != MOE_OK) return rc;

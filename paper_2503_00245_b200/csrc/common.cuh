@@ -43,7 +43,11 @@ struct DeviceState {
   unsigned int tail_bias;
   // router of many tokens: CTAs that have stored their tokens' routing; the last one sets it back
   unsigned int route_done;
-  unsigned int pad3[18];
+  // prefill: CTAs of the expert kernel that have finished (the last one clears this line and the two below)
+  unsigned int ffn_exit;
+  unsigned int pad3[17];
+  unsigned int route_count[MOE_MAX_EXPERTS];  // tokens that the router has placed with each expert
+  unsigned int ffn_done[MOE_MAX_EXPERTS];     // warps that have stored their part of a tile of the expert's hidden activations
 };
 
 }  // namespace cosmoe
@@ -89,6 +93,7 @@ int allow_full_smem(const moe_ctx* ctx) {
 struct WsLayout {
   size_t topk_idx, topk_w, offsets, perm, inv;  // routing products when the caller does not ask for them
   size_t vec_x, vec_a, vec_b, vec_c;            // vectors between the products of the weight-decomposed streaming path
+  size_t pos;                                   // places of the (token, choice) pairs among their expert's
   size_t xperm, hidden, mid_a, mid_b;           // bf16 operands of the tensor path
   size_t out_slots;                             // fp32 [T*k][d]
   size_t total;
@@ -109,9 +114,16 @@ int validate_config(const moe_config* c);
 struct Grouping {
   int32_t *offsets, *perm, *inv;
 };
-// With `grp` the pairs are grouped as well.
+// Where the router of many tokens places the rows of x, rounded to bf16, grouped by expert: T rows of room per expert, in the
+// order in which the CTAs come; pos: each pair's place among its expert's rows.
+struct Scatter {
+  void* rows;
+  int32_t* pos;
+};
+bool route_tile_applies(const moe_config& c, int T);
+// With `grp` the pairs are grouped as well; with `sc` the rows are placed, their numbers in ctx's route_count.
 int launch_route(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt, float* probs,
-                 cudaStream_t s, const Grouping* grp = nullptr);
+                 cudaStream_t s, const Grouping* grp = nullptr, const Scatter* sc = nullptr);
 int launch_permute(moe_ctx* ctx, const int32_t* idx, int T, int32_t* offsets, int32_t* perm, int32_t* inv,
                    cudaStream_t s);
 // out_slots may come as `planes` partial sums, one [T*k][d] plane after the other (summed in order).
@@ -163,6 +175,19 @@ int launch_fp8_dequant(const void* codes, const float* scales, long long rows, i
 // of box_inner x box_rows of one sub-row, rows box_inner values apart in shared memory (csrc/tensor_ffn.cu).
 int make_map_rows(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
                   int box_rows);
+// Prefill of dense experts (csrc/dense_prefill.cu).  The rows of x, bf16: placed by the router (counts set), or grouped by slot.
+struct PrefillRows {
+  const void* x;
+  const unsigned* counts;
+  const int32_t *topk_idx, *pos;
+  int32_t* inv;
+  const int32_t* offsets;
+};
+constexpr size_t kScatterBytesMax = (size_t)256 << 20;  // room for the rows placed by the router, at most
+bool prefill_scatters(const moe_config& c, int T);
+// planes: room for the partial sums of a cut contraction when the caller wants one sum (out_planes null)
+int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,
+                         float* planes, int* out_planes, cudaStream_t s);
 // Tensor-core (prefill) path: out_slots from x gathered by perm.
 int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, const int32_t* offsets,
                       const int32_t* perm, char* ws, const WsLayout& L, float* out_slots, int* out_planes,
@@ -352,6 +377,9 @@ __device__ __forceinline__ unsigned long long atom_add_acq_rel64(unsigned long l
   unsigned long long old;
   asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
   return old;
+}
+__device__ __forceinline__ void red_add_release(unsigned* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
   unsigned old;

@@ -131,13 +131,15 @@ template <typename XT>
 __global__ void __launch_bounds__(kRtWarps * 32)
     route_tile_kernel(const XT* __restrict__ x, const uint16_t* __restrict__ w_router, const float* __restrict__ bias, int T,
                       int d, int E, int k, int renorm, int32_t* topk_idx, float* __restrict__ topk_w,
-                      float* __restrict__ probs, Grouping grp, DeviceState* st) {
+                      float* __restrict__ probs, Grouping grp, Scatter sc, DeviceState* st) {
   constexpr int NT = sizeof(XT) == 4 ? 3 : 1;  // bf16 terms of a value
   extern __shared__ __align__(128) unsigned char rt_smem[];
   const RtShape sh = rt_shape(d, E);
   float* const part = reinterpret_cast<float*>(rt_smem + sh.part_off);  // [warp][token][expert]
+  __shared__ int s_last, s_base[MOE_MAX_EXPERTS + 1], s_count[MOE_MAX_EXPERTS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
+  if (tid < MOE_MAX_EXPERTS) s_count[tid] = 0;
   const int units = (d + kRtUnit - 1) / kRtUnit;
   for (uint32_t i = tid * 128u, n = (uint32_t)d * E * 2u; i < n; i += kRtWarps * 32 * 128u)  // (W_r: its lines into L2 ...)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const unsigned char*>(w_router) + i));
@@ -232,6 +234,7 @@ __global__ void __launch_bounds__(kRtWarps * 32)
     }
   }
   __syncthreads();
+  int my_e = 0, my_pos = 0;  // (lane j: the token's j-th choice)
   {
     const int t = t0 + warp;  // a warp finishes one token
     if (t < T) {
@@ -250,13 +253,52 @@ __global__ void __launch_bounds__(kRtWarps * 32)
       };
       if (lane < E) l0 = logit(lane);
       if (lane + 32 < E) l1 = logit(lane + 32);
-      warp_route_finish(l0, l1, E, k, renorm, lane, topk_idx + (size_t)t * k, topk_w + (size_t)t * k,
-                        probs ? probs + (size_t)t * E : nullptr);
+      int e;
+      float wt;
+      unsigned long long selected;
+      warp_route_top(l0, l1, E, k, renorm, lane, probs ? probs + (size_t)t * E : nullptr, e, wt, selected);
+      if (lane < k) {
+        topk_idx[(size_t)t * k + lane] = e, topk_w[(size_t)t * k + lane] = wt;
+        if (sc.rows) my_e = e, my_pos = atomicAdd(&s_count[e], 1);
+      }
     }
+  }
+  if (sc.rows) {
+    // ---- the CTA takes places for its tokens and copies their rows there
+    const int t = min(t0 + warp, T - 1), chunks = d / 8;
+    const XT* const row = x + (size_t)t * d;
+    constexpr int kFly = sizeof(XT) == 4 ? 4 : 8;
+    float f[kFly][8];
+    auto get = [&](int c0) {
+#pragma unroll
+      for (int u = 0; u < kFly; ++u)
+        if (c0 + 32 * u < chunks) load_x8<XT>(row + (c0 + 32 * u) * 8, f[u]);
+    };
+    get(lane);
+    __syncthreads();
+    if (tid < E && s_count[tid] > 0) s_base[tid] = (int)atomicAdd(&st->route_count[tid], (unsigned)s_count[tid]);
+    __syncthreads();
+    if (t0 + warp >= T) return;
+    if (lane < k) {
+      my_pos += s_base[my_e];
+      sc.pos[(size_t)t * k + lane] = my_pos;
+    }
+    for (int c0 = lane; __any_sync(0xffffffffu, c0 < chunks); c0 += 32 * kFly) {
+      if (c0 != lane) get(c0);
+      for (int j = 0; j < k; ++j) {
+        const size_t r = (size_t)__shfl_sync(0xffffffffu, my_e, j) * T + __shfl_sync(0xffffffffu, my_pos, j);
+        uint4* const dst = reinterpret_cast<uint4*>(sc.rows) + r * chunks;
+#pragma unroll
+        for (int u = 0; u < kFly; ++u)
+          if (c0 + 32 * u < chunks)
+            dst[c0 + 32 * u] = make_uint4(pack_bf16x2(f[u][0], f[u][1]), pack_bf16x2(f[u][2], f[u][3]), pack_bf16x2(f[u][4], f[u][5]),
+                                          pack_bf16x2(f[u][6], f[u][7]));
+      }
+    }
+    return;
   }
   if (!grp.perm) return;
   // ---- the last CTA groups the pairs
-  __shared__ int s_last, s_base[MOE_MAX_EXPERTS + 1];
   __syncthreads();
   if (tid == 0) {
     // (release: the CTA's routing, ordered before this thread by the barrier; acquire: the other CTAs')
@@ -371,19 +413,24 @@ __global__ void __launch_bounds__(kRouteWarps * 32)
                     probs ? probs + (size_t)t * E : nullptr);
 }
 
+// more than a decode step's tokens (16 would be a tile of a single CTA: those take a CTA per token), and W_r fits into shared
+// memory (two CTAs' share of an SM: d = 2048 up to 16 experts)
+bool route_tile_applies(const moe_config& c, int T) {
+  return T > MOE_STREAM_MAX_TOKENS && rt_shape(c.d_model, c.n_experts).smem <= 112 * 1024;
+}
+
 template <typename XT>
 static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt,
-                          float* probs, cudaStream_t s, const Grouping* grp) {
+                          float* probs, cudaStream_t s, const Grouping* grp, const Scatter* sc) {
   const moe_config& c = ctx->cfg;
   const XT* xp = (const XT*)x;
   const uint16_t* wr = (const uint16_t*)w->w_router;
   const RtShape sh = rt_shape(c.d_model, c.n_experts);
-  // more than a decode step's tokens (16 would be a tile of a single CTA: those take a CTA per token), and W_r fits into shared memory (two CTAs' share of an SM: d = 2048 up to 16 experts)
-  if (T > MOE_STREAM_MAX_TOKENS && sh.smem <= 112 * 1024) {
+  if (route_tile_applies(c, T)) {
     MOE_TRY(allow_full_smem<route_tile_kernel<XT>>(ctx));
     MOE_CUDA_TRY(launch_pdl(route_tile_kernel<XT>, dim3((T + kRtTokens - 1) / kRtTokens), dim3(kRtWarps * 32), (size_t)sh.smem, s,
                             xp, wr, w->b_router, T, c.d_model, c.n_experts, c.top_k, c.renorm, idx, wt, probs,
-                            grp ? *grp : Grouping{nullptr, nullptr, nullptr}, ctx->d_state));
+                            grp ? *grp : Grouping{nullptr, nullptr, nullptr}, sc ? *sc : Scatter{nullptr, nullptr}, ctx->d_state));
     ctx->launches++;
     return MOE_OK;
   }
@@ -407,9 +454,9 @@ static int launch_route_t(moe_ctx* ctx, const void* x, int T, const moe_weights*
 }
 
 int launch_route(moe_ctx* ctx, const void* x, int T, const moe_weights* w, int32_t* idx, float* wt, float* probs,
-                 cudaStream_t s, const Grouping* grp) {
-  if (ctx->cfg.x_dtype == MOE_F32) return launch_route_t<float>(ctx, x, T, w, idx, wt, probs, s, grp);
-  return launch_route_t<__nv_bfloat16>(ctx, x, T, w, idx, wt, probs, s, grp);
+                 cudaStream_t s, const Grouping* grp, const Scatter* sc) {
+  if (ctx->cfg.x_dtype == MOE_F32) return launch_route_t<float>(ctx, x, T, w, idx, wt, probs, s, grp, sc);
+  return launch_route_t<__nv_bfloat16>(ctx, x, T, w, idx, wt, probs, s, grp, sc);
 }
 
 // ------------------------------------------------------------------------------------ grouping

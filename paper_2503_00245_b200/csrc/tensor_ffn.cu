@@ -1,11 +1,9 @@
-// Tensor-core (prefill) path of the expert FFN: grouped GEMMs on the 5th-generation tensor cores.
+// Prefill of weight-decomposed experts: grouped GEMMs on the 5th-generation tensor cores (dense experts: csrc/dense_prefill.cu).
 //
 // Tokens are grouped by expert (moe_permute), their rows gathered into a bf16 operand, and every expert's
 // FFN becomes dense contractions  C[m, n] = sum_k A[m, k] * B_e[n, k]  over that expert's rows:
 //
-//   dense experts  (1) H = silu(X Wg) * (X Wu)   A = gathered x,  B = gate / up rows of gud   -> bf16 hidden
-//                  (2) O = H Wd                  A = H,           B = down rows of gud (N-major) -> fp32 slots
-//   Eq. 1 factors  (1) T = X [gL | uL]   (2) H = silu(Tg gR) * (Tu uR)   (3) V = H dL   (4) O = V dR
+//   (1) T = X [gL | uL]   (2) H = silu(Tg gR) * (Tu uR)   (3) V = H dL   (4) O = V dR
 //
 // Two CTAs on neighbouring SMs (a cluster of 2) compute one tile of 256 rows x up to 256 columns with
 // tcgen05.mma.cta_group::2: each CTA stages its own 128 rows of A and HALF of the tile's B rows, the tensor
@@ -25,22 +23,13 @@
 // Ragged groups: a tile may read rows of the next expert (or zeros past the end); they are never stored.
 // K and N tails are zero-filled by TMA.  All waits are bounded; an expired wait sets the ctx's status word.
 // No copy in this file uses cluster multicast: every CTA fetches what it needs with its own loads.
-#include <cuda.h>
-
-#include <algorithm>
-
-#include "common.cuh"
+#include "tcgen.cuh"
 
 namespace cosmoe {
 
 namespace {
 
-constexpr int kBM = 128;  // rows per CTA and tile (TMEM lanes)
-constexpr int kBK = 64;   // K elements per stage (128 bytes of bf16 = one swizzle row)
-constexpr int kEpiWarps = 8;  // two per quarter of the TMEM lanes, splitting the columns
 constexpr int kThreadsGG = (2 + kEpiWarps) * 32;
-constexpr int kTmemCols = 512;  // two accumulator buffers of 256 columns
-constexpr int kAccCols = 256;
 constexpr int kMaxStagesGG = 6;
 constexpr int kEpiBuf = 4096;
 constexpr int kPairRows = 2 * kBM;  // rows of a pair's tile
@@ -50,8 +39,7 @@ enum Epi { EPI_SWIGLU = 0, EPI_BF16_PAIR = 1, EPI_BF16 = 2, EPI_F32 = 3 };
 enum BMode {
   B_PAIR = 0,    // interleaved matrix, columns [0, bn) = sub-row 0 (rank 0 loads them), [bn, 2 bn) = sub-row 1 (rank 1)
   B_DUAL = 1,    // the same columns, but sub-row 1 meets a second A operand: two MMAs of N = bn, each rank loads half of both
-  B_SINGLE = 2,  // one sub-row, K-major: rank r loads rows [n0 + r bn/2, n0 + (r+1) bn/2)
-  B_NMAJOR = 3   // one sub-row stored [k][n] (the down rows of gud): rank r loads its bn/2 columns in 64-column boxes
+  B_SINGLE = 2   // one sub-row: rank r loads rows [n0 + r bn/2, n0 + (r+1) bn/2)
 };
 
 struct GGParams {
@@ -63,7 +51,6 @@ struct GGParams {
                  // not exist), so that a consumer may read the padded width
   int bn;        // output columns per tile (per sub-row in B_PAIR / B_DUAL: <= 128; else <= 256)
   int bmode;
-  int b_sub;     // sub-row of the interleaved matrix that B_SINGLE / B_NMAJOR tiles read
   int k_wrap;    // > 0: the B operand's k coordinate wraps at k_wrap (A = [hi | lo] halves of a split operand)
   int split;     // bf16 epilogues also store the rounding remainder: value = hi + lo, lo at column offset out_off_lo
   int epi;
@@ -76,130 +63,6 @@ struct GGParams {
   int n_stages;
   DeviceState* st;
 };
-
-// ---- PTX wrappers ------------------------------------------------------------------------------------
-// Tiled loads whose completion may be counted on a barrier of the other CTA of the pair (cta_group::2); the
-// data always lands in the issuing CTA's own shared memory.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1, uint32_t bar_cluster) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-      "[%4];" ::"r"(smem_u32(dst)),
-      "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint32_t bar_cluster) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-      "%5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar_cluster)
-      : "memory");
-}
-// One lane of a converged warp.  The loops that issue loads and MMAs are run by the whole warp, with loop bounds and
-// coordinates taken from lane 0, and only the issuing itself is one lane's: the operands of these instructions live in
-// registers that a warp shares, and inside a branch that one lane takes every operand of every instruction has to be
-// moved there first -- about 100 cycles for each load and MMA.
-// (A K step of the phone-shape GEMM: 720 -> 630 cycles, of which the tensor pipe needs 512; the layer 365 -> 349 us.)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ int lane0(int v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// address of the same shared-memory object in CTA `rank` of this cluster
-__device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(smem_ptr)), "r"(rank));
-  return r;
-}
-// (Release at CTA scope: what the arrival hands over are tensor-memory columns, ordered by tcgen05.wait::ld and the tcgen05
-// fence.  A release at cluster scope also waits for the warp's stores to memory, about a microsecond per tile.)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// The barrier at this shared-memory offset gets one arrival IN BOTH CTAs of the pair when every MMA this thread
-// has issued so far has completed.  (A multicast of barrier arrivals, not of data: no copy in this file is multicast.)
-__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-                   smem_u32(bar)),
-               "h"((unsigned short)3)
-               : "memory");
-}
-// `acc` == 0: the product overwrites the accumulator; otherwise it is added.
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr)
-      : "memory");
-}
-// A load's registers may be read behind the wait only; going through it ties every use and copy of them to that place.
-__device__ __forceinline__ void tc_wait_ld(uint32_t* v) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-      : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-        "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-        "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-        "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
-      :
-      : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld(uint32_t* a, uint32_t* v) {  // two loads, one wait
-  tc_wait_ld(a);
-  asm volatile(""
-      : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-        "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-        "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-        "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]));
-}
-
-// Shared-memory operand descriptor (128-byte swizzle).  K-major tiles: rows of 128 bytes, 8-row groups 1024
-// bytes apart (stride byte offset), the leading offset is not used.  N-major tiles: 64 columns (128 bytes) per
-// k-row, 8-k-row groups 1024 bytes apart (stride), 64-column blocks `lbo` bytes apart (leading).
-// The start address sits in the low 14 bits (in units of 16 bytes), so stepping through a stage or through the
-// ring is an addition to the low word.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3ffffu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3fffu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3fffu) << 32;
-  d |= 1ull << 46;  // descriptor version of this architecture
-  d |= 2ull << 61;  // 128-byte swizzle
-  return d;
-}
-// Instruction descriptor: bf16 x bf16 -> fp32, A K-major, B K- or N-major, M = 256 over the pair, N = n.
-__device__ __forceinline__ uint32_t instr_desc(int n, bool b_nmajor) {
-  uint32_t d = 0;
-  d |= 1u << 4;   // accumulator format: fp32
-  d |= 1u << 7;   // A: bf16
-  d |= 1u << 10;  // B: bf16
-  d |= (b_nmajor ? 1u : 0u) << 16;
-  d |= (uint32_t)(n >> 3) << 17;
-  d |= (uint32_t)(kPairRows >> 4) << 24;
-  return d;
-}
 
 struct SmemGG {
   uint64_t full[kMaxStagesGG];   // leader's: both CTAs' operands of the stage have landed
@@ -379,6 +242,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     const uint32_t tx_pair = 2u * (n_a * a_bytes + b_bytes);  // bytes both CTAs bring in per stage
     const uint32_t full0 = (uint32_t)lane0((int)map_to_rank(&sm.full[0], 0u));  // the leader's stage barriers, 8 bytes apart
     const int half_bn = P.bn / 2;
+    const uint32_t st0 = (uint32_t)lane0((int)smem_u32(stages));
     for (int idx = pair; ok && idx < n_work; idx += n_pairs) {
       const Tile t = decode_tile(P, tm, idx, n_tiles);
       const int n0 = t.n0;
@@ -392,8 +256,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           ok = false;
           break;
         }
-        unsigned char* st_a0 = stages + (size_t)slot * stage_bytes;
-        unsigned char* st_b = st_a0 + n_a * a_bytes;
+        const uint32_t st_a0 = st0 + slot * stage_bytes, st_b = st_a0 + n_a * a_bytes;
         const uint32_t bar = full0 + 8u * slot;
         if (elect_one()) {
           if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], tx_pair);
@@ -404,13 +267,9 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
             const int nr = n0 + (int)rank * half_bn;
             tma_load_2d(st_a0 + a_bytes, &map_a1, k0, a_row, bar);
             tma_load_4d(st_b, &map_b, kB, 0, nr, t.e, bar);
-            tma_load_4d(st_b + (size_t)half_bn * kBK * 2, &map_b, kB, 1, nr, t.e, bar);
-          } else if (P.bmode == B_SINGLE) {
-            tma_load_4d(st_b, &map_b, kB, P.b_sub, n0 + (int)rank * half_bn, t.e, bar);
+            tma_load_4d(st_b + (uint32_t)half_bn * kBK * 2, &map_b, kB, 1, nr, t.e, bar);
           } else {
-            const int nc = n0 + (int)rank * half_bn;
-            tma_load_4d(st_b, &map_b, nc, P.b_sub, kB, t.e, bar);
-            if (P.bn > 128) tma_load_4d(st_b + (size_t)64 * kBK * 2, &map_b, nc + 64, P.b_sub, kB, t.e, bar);
+            tma_load_4d(st_b, &map_b, kB, 0, n0 + (int)rank * half_bn, t.e, bar);
           }
         }
         __syncwarp();
@@ -427,13 +286,10 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
     if (rank == 0) {
       // One warp feeds the tensor cores of both SMs, so its instruction stream is kept short: the ring position
       // is a counter, not a division, and the operand descriptors are a constant high word plus a low word that
-      // steps through the stage (K-major operands: 32 bytes per 16 k-values; N-major: 16 k-rows of 128 bytes).
+      // steps through the stage (32 bytes per 16 k-values).
       const int n_mma = P.bmode == B_PAIR ? 2 * P.bn : P.bn;
-      const uint32_t idesc = instr_desc(n_mma, P.bmode == B_NMAJOR);
+      const uint32_t idesc = instr_desc(n_mma, false);
       const uint64_t hi_k = smem_desc(0, 16, 1024) & 0xffffffff00000000ull;
-      const uint64_t hi_b = (P.bmode == B_NMAJOR ? smem_desc(0, 64 * kBK * 2, 1024) : smem_desc(0, 16, 1024)) & 0xffffffff00000000ull;
-      const uint32_t lo_b_lbo = (P.bmode == B_NMAJOR ? (uint32_t)(64 * kBK * 2 >> 4) : 1u) << 16;
-      const uint32_t b_step = P.bmode == B_NMAJOR ? (2048u >> 4) : (32u >> 4);
       const uint32_t stage0 = (uint32_t)lane0((int)(smem_u32(stages) >> 4)), stage_step = stage_bytes >> 4;
       const uint32_t b_off = (n_a * a_bytes) >> 4, a1_off = a_bytes >> 4, b1_off = ((uint32_t)(P.bn / 2) * kBK * 2) >> 4;
       uint32_t slot = 0, par = 0, st_lo = stage0;
@@ -460,7 +316,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           }
           tc_fence_after();
           const uint64_t da = hi_k | (uint64_t)(st_lo | (1u << 16));
-          const uint64_t db = hi_b | (uint64_t)((st_lo + b_off) | lo_b_lbo);
+          const uint64_t db = hi_k | (uint64_t)((st_lo + b_off) | (1u << 16));
           if (elect_one()) {
             if (P.bmode == B_DUAL) {
               const uint64_t da1 = da + a1_off, db1 = db + b1_off;
@@ -471,7 +327,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
               }
             } else {
 #pragma unroll
-              for (uint32_t kk = 0; kk < kBK / 16; ++kk) tc_mma_bf16(d_tmem, da + 2u * kk, db + b_step * kk, idesc, acc | kk);
+              for (uint32_t kk = 0; kk < kBK / 16; ++kk) tc_mma_bf16(d_tmem, da + 2u * kk, db + 2u * kk, idesc, acc | kk);
             }
             tc_commit_pair(&sm.empty[slot]);  // both CTAs' producers may refill the stage once these MMAs have read it
             if (kb + 1 == kb1) tc_commit_pair(&sm.accum_full[buf]);
@@ -564,87 +420,6 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   }
 }
 
-// ---- host: tensor maps --------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      (void)cudaGetLastError();
-      return nullptr;
-    }
-    fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
-// rank-2 map over a row-major bf16 matrix [rows][ld], columns [0, cols): box 64 x 128
-int make_map_a(CUtensorMap* m, const void* base, long long rows, long long cols, long long ld) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return MOE_ERR_CUDA;
-  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  const cuuint32_t box[2] = {kBK, kBM};
-  const cuuint32_t es[2] = {1, 1};
-  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
-}
-// rank-4 map over an interleaved matrix [S][rows][nsub][inner]: coordinates (inner, sub, row, slot)
-int make_map_b(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
-               int box_rows, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return MOE_ERR_CUDA;
-  const cuuint64_t dims[4] = {(cuuint64_t)inner, (cuuint64_t)nsub, (cuuint64_t)rows, (cuuint64_t)slots};
-  const cuuint64_t strides[3] = {(cuuint64_t)inner * 2, (cuuint64_t)inner * nsub * 2,
-                                 (cuuint64_t)inner * nsub * rows * 2};
-  const cuuint32_t box[4] = {(cuuint32_t)box_inner, 1, (cuuint32_t)box_rows, 1};
-  const cuuint32_t es[4] = {1, 1, 1, 1};
-  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
-}
-
-void pair_launch_config(cudaLaunchConfig_t& lc, cudaLaunchAttribute* attr, int ctas, size_t smem, cudaStream_t s) {
-  lc = cudaLaunchConfig_t{};
-  lc.gridDim = dim3(ctas), lc.blockDim = dim3(kThreadsGG), lc.dynamicSmemBytes = smem, lc.stream = s;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2, attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = attr, lc.numAttrs = 2;
-}
-
-// Pairs of CTAs the device can hold at once (one CTA per SM; a pair sits on two SMs of one cluster).
-// Every launch of the kernel takes more than half of an SM's shared memory, so the number does not depend on the
-// launch: the driver is asked once per device (the query costs more than a launch).
-int max_pairs(const moe_ctx* ctx, size_t smem) {
-  static std::atomic<int> known[kMaxDevices];
-  const bool tracked = ctx->device >= 0 && ctx->device < kMaxDevices;
-  if (tracked && known[ctx->device].load(std::memory_order_relaxed) > 0)
-    return known[ctx->device].load(std::memory_order_relaxed);
-  cudaLaunchConfig_t lc;
-  cudaLaunchAttribute attr[2];
-  pair_launch_config(lc, attr, ctx->sm_count & ~1, smem, nullptr);
-  lc.numAttrs = 1;  // the cluster shape alone decides the occupancy
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, grouped_gemm_kernel, &lc) != cudaSuccess || n < 1) {
-    (void)cudaGetLastError();
-    n = ctx->sm_count / 2;
-  }
-  n = std::max(1, std::min(n, ctx->sm_count / 2));
-  if (tracked) known[ctx->device].store(n, std::memory_order_relaxed);
-  return n;
-}
-
 int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b, GGParams P,
               int n_slots, cudaStream_t s) {
   const moe_config& c = ctx->cfg;
@@ -659,10 +434,10 @@ int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const 
   if ((long long)smem > ctx->max_smem_optin) return MOE_ERR_UNSUPPORTED;
   MOE_TRY(allow_full_smem<grouped_gemm_kernel>(ctx));
   const long long m_tiles = (n_slots + kPairRows - 1) / kPairRows + c.n_experts;  // upper bound
-  const int pairs = (int)std::min<long long>(m_tiles * n_tiles * P.ksplit, max_pairs(ctx, smem));
+  const int pairs = (int)std::min<long long>(m_tiles * n_tiles * P.ksplit, max_pairs<grouped_gemm_kernel>(ctx, kThreadsGG, smem));
   cudaLaunchConfig_t lc;
   cudaLaunchAttribute attr[2];
-  pair_launch_config(lc, attr, 2 * pairs, smem, s);
+  pair_launch_config(lc, attr, 2 * pairs, kThreadsGG, smem, s);
   MOE_CUDA_TRY(cudaLaunchKernelEx(&lc, grouped_gemm_kernel, a0, a1, b, P));
   ctx->launches++;
   return MOE_OK;
@@ -714,34 +489,8 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   GGParams P{};
   P.offsets = offsets;
   if (r == 0) {
-    // (1) hidden = silu(X Wg) * (X Wu): the tile's 128 gate rows come in through one CTA, its 128 up rows through the other
-    if ((rc = make_map_a(&ma, xperm, n_slots, d, d)) != MOE_OK) return rc;
-    if ((rc = make_map_b(&mb, w->gud, d, 3, f, E, kBK, 128)) != MOE_OK) return rc;
-    P.K = d, P.n_total = f, P.bn = 128, P.bmode = B_PAIR, P.b_sub = 0, P.epi = EPI_SWIGLU;
-    P.out = hidden, P.ld_out = f, P.out_off2 = 0;
-    if ((rc = launch_gg(ctx, ma, ma, mb, P, n_slots, s)) != MOE_OK) return rc;
-    // (2) out_slots = hidden Wd   (B = down rows of gud: [k = hidden unit][n = model column], n contiguous)
-    if ((rc = make_map_a(&ma, hidden, n_slots, f, f)) != MOE_OK) return rc;
-    if ((rc = make_map_b(&mb, w->gud, d, 3, f, E, 64, kBK)) != MOE_OK) return rc;
-    P.K = f, P.n_total = d, P.bn = pick_bn(d, 256, 128), P.bmode = B_NMAJOR, P.b_sub = 2;
-    P.epi = EPI_F32, P.out = out_slots, P.ld_out = d, P.out_off2 = 0;
-    if (n_slots <= kKSplitMaxSlots) {
-      // short prefill: too few tiles for the SMs, and every tile streams a long run of weights.  Cut the contraction so
-      // that every pair streams a part, each part into its own plane; the caller sums the planes, or they are summed
-      // here (in the same order: the layer and its four calls give the same bits).
-      const long long tiles = (long long)row_tiles(n_slots, E) * ((d + P.bn - 1) / P.bn);
-      const int ks = pick_ksplit(tiles, (f + kBK - 1) / kBK, ctx->sm_count / 2, kKSplitMax);
-      if (ks > 1) {
-        P.ksplit = ks, P.plane_elems = (long long)n_slots * d;
-        if (!out_planes) {
-          P.out = ws + L.out_slots;
-          if ((rc = launch_gg(ctx, ma, ma, mb, P, n_slots, s)) != MOE_OK) return rc;
-          return launch_sum_planes(ctx, (const float*)P.out, P.plane_elems, ks, out_slots, s);
-        }
-        *out_planes = ks;
-      }
-    }
-    return launch_gg(ctx, ma, ma, mb, P, n_slots, s);
+    const PrefillRows rows{xperm, nullptr, nullptr, nullptr, nullptr, offsets};
+    return launch_dense_prefill(ctx, T, w, rows, hidden, out_slots, (float*)(ws + L.out_slots), out_planes, s);
   }
   // The rank-r intermediates t and v are kept as hi + lo pairs of bf16 (value = hi + lo): the GEMMs that
   // consume them run over K = 2 * rp with the weight slices repeated, so the intermediates carry ~16 mantissa
@@ -758,21 +507,21 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   P.bn = pick_bn(r, 128);
   while (P.bn > 64 && 2 * m_tiles * ((r + P.bn - 1) / P.bn) <= pairs) P.bn /= 2;  // a small rank leaves pairs idle: narrower tiles
   if ((rc = make_map_b(&mb, w->wd_a, d, 2, r, E, kBK, P.bn)) != MOE_OK) return rc;
-  P.K = d, P.n_total = r, P.bmode = B_PAIR, P.b_sub = 0, P.epi = EPI_BF16_PAIR;
+  P.K = d, P.n_total = r, P.bmode = B_PAIR, P.epi = EPI_BF16_PAIR;
   P.k_wrap = 0, P.split = 1, P.out = mid_a, P.ld_out = 2 * tw, P.out_off2 = tw, P.out_off_lo = rp, P.n_store = rp;
   if ((rc = launch_gg(ctx, ma, ma, mb, P, n_slots, s)) != MOE_OK) return rc;
   // (2) hidden = silu(Tg gR) * (Tu uR): two A operands, each CTA brings half of the gate and half of the up rows
   if ((rc = make_map_a(&ma, mid_a, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
   if ((rc = make_map_a(&ma1, (const __nv_bfloat16*)mid_a + tw, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
   if ((rc = make_map_b(&mb, w->wd_b, r, 2, f, E, kBK, 64)) != MOE_OK) return rc;
-  P.K = tw, P.n_total = f, P.bn = 128, P.bmode = B_DUAL, P.b_sub = 0, P.epi = EPI_SWIGLU;
+  P.K = tw, P.n_total = f, P.bn = 128, P.bmode = B_DUAL, P.epi = EPI_SWIGLU;
   P.k_wrap = rp, P.split = 0, P.out = hidden, P.ld_out = f, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
   if ((rc = launch_gg(ctx, ma, ma1, mb, P, n_slots, s)) != MOE_OK) return rc;
   // (3) V = hidden dL
   if ((rc = make_map_a(&ma, hidden, n_slots, f, f)) != MOE_OK) return rc;
   P.bn = pick_bn(r, 256);
   if ((rc = make_map_b(&mb, w->wd_c, f, 1, r, E, kBK, P.bn / 2)) != MOE_OK) return rc;
-  P.K = f, P.n_total = r, P.bmode = B_SINGLE, P.b_sub = 0, P.epi = EPI_BF16;
+  P.K = f, P.n_total = r, P.bmode = B_SINGLE, P.epi = EPI_BF16;
   P.k_wrap = 0, P.split = 1, P.out = mid_b, P.ld_out = tw, P.out_off2 = 0, P.out_off_lo = rp, P.n_store = rp;
   // few tiles of a long contraction: cut into parts whose fp32 sums (in the gathered rows' place, which are not needed any
   // more) are added, in order, and split by a kernel of their own.  r 128, 2048 tokens: 20 tiles on 74 pairs, 37 us.
@@ -790,7 +539,7 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   if ((rc = make_map_a(&ma, mid_b, n_slots, tw, tw)) != MOE_OK) return rc;
   P.bn = pick_bn(d, 256);
   if ((rc = make_map_b(&mb, w->wd_d, r, 1, d, E, kBK, P.bn / 2)) != MOE_OK) return rc;
-  P.K = tw, P.n_total = d, P.bmode = B_SINGLE, P.b_sub = 0, P.epi = EPI_F32;
+  P.K = tw, P.n_total = d, P.bmode = B_SINGLE, P.epi = EPI_F32;
   P.k_wrap = rp, P.split = 0, P.out = out_slots, P.ld_out = d, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
   return launch_gg(ctx, ma, ma, mb, P, n_slots, s);
 }

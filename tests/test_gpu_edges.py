@@ -120,6 +120,30 @@ def test_prefill_with_a_cut_contraction(sh, T):
     assert lay.check() == 0
 
 
+@pytest.mark.parametrize("sh,T", [
+    (shape(72, 512, E=2, k=2), 17),                     # few tiles: some pairs of CTAs start with the second product
+    (shape(264, 520, E=33, k=8, xd="f32"), 31),         # a second expert per lane; experts with fewer tokens than a tile's 32
+    (shape(136, 5632, E=1, k=1), 257),                  # two token tiles, uneven
+    (shape(1024, 520, E=4, k=4), 129),                  # more than 128 columns: one accumulator buffer, then two again
+    (shape(2056, 512, bias="normal"), 200),             # features beyond a tile of 256, uneven load
+    (shape(512, 512, E=64, k=2), 4100),                 # room for every token at every expert would be too much: grouped by slot
+    (shape(512, 512, E=64, k=2, r=64), 4100),
+    (shape(264, 520, E=33, k=8, r=40, xd="f32"), 31),
+    (shape(512, 1024, E=4, k=4, r=128, bias="normal"), 300),
+])
+def test_prefill_tiles_and_the_rows_places(sh, T):
+    lay, t, host = U.build(sh, T)
+    check_prefill(lay, t, host, sh.top_k)
+    idx, w, _ = lay.route(t["x"])
+    offsets, perm, inv = lay.permute(idx)
+    y = lay.combine(lay.expert_ffn(t["x"], offsets, perm), w, inv)
+    for _ in range(3):                                  # the rows' places differ from call to call, an element's value does not
+        assert torch.equal(y, lay.forward(t["x"]))
+    fewer = t["x"][:max(17, T // 3)].contiguous()
+    assert torch.equal(lay.forward(fewer), lay.forward(fewer))
+    assert lay.check() == 0
+
+
 @pytest.mark.parametrize("T", [8, 16])
 def test_dense_decode_of_several_tokens_with_many_pairs(T):
     sh = shape(512, 1024, E=16, k=8)                    # 64 and 128 pairs: beyond one per lane; every expert active
