@@ -574,7 +574,10 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
       double worst = std::max(load(q1, q), std::min(r1, r) > 0 ? load(q1 + 1, q + 1) : 0.0);
       if (r > r1) worst = std::max(worst, load(q1, q + 1));
       if (r1 > r) worst = std::max(worst, load(q1 + 1, q));
-      worst += (ks - 1) * 8.0 * n_slots * d / 3800.0;  // (a further plane of partial sums, written and read)
+      worst = std::max(worst, (q1 + (r1 > 0)) * c1 + c2);  // (the last experts' second product starts when all of phase 1 is done)
+      // a further plane of partial sums, written and read, in the epilogue and in the combine (wearable, 512 tokens: one plane 56.9
+      // us, two 52.8, four 54.7; paper, 333 tokens: 74.7, 69.6, 74.8)
+      worst += (ks - 1) * 16.0 * n_slots * d / 3800.0;
       if (hb1 == 0 || worst < 0.98 * best) best = worst, hb1 = h1, ks2 = ks;
     }
   }
