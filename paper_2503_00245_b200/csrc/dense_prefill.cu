@@ -18,8 +18,8 @@
 // Why so: with the tokens on the M side, an expert's last 256-row tile cost what a full one does, and 128 weight rows were loaded
 // for every 128 token rows.  Here a K step of a pair is 48 KB per CTA for 2 x 256 features x 256 tokens instead of 64 KB, an
 // expert's last tile costs what its tokens cost, and the tiles of (2) fill what the last round of (1) leaves idle.
-// What bounds it: with 256 tokens per expert and more, the tensor cores (a K step of phase 1 with 224 columns: 560 ns against 510
-// at the sampled clock) and the special-function unit, which the epilogue's exponentials and reciprocals keep busy for 2 us per
+// What bounds it: with 256 tokens per expert and more, the tensor cores (a tile of phase 1 with 224 columns and 32 K steps takes 17
+// us, 28.7 k cycles of them) and the special-function unit, which the epilogue's exponentials and reciprocals keep busy for 2 us per
 // tile, in the open when a tile takes all 512 columns; with fewer, HBM and the round trip of 1.5 us through the ring.
 // Before (five launches, tokens on the M side) and now, whole layer: d 1024, f 2816, 512 tokens 57 -> 52.7 us; d 1440, f 3840,
 // 333 tokens 90 -> 70; d 2048, f 5632, 2048 tokens 300-340 -> 262-267.
