@@ -47,9 +47,9 @@ WsLayout ws_layout(const moe_config& c, int T) {
   L.vec_b = take(wd_stream ? n * fs * 6 : 0);
   L.vec_c = take(wd_stream ? n * std::max(rs * 6, (size_t)c.wd_rank * 8 * 4) : 0);
   L.pos = take(n * 4);
-  // by slot; or, dense experts, T rows per expert while that is not more than kScatterBytesMax (rounded so that fewer tokens
+  // by slot; or T rows per expert while that is not more than kScatterBytesMax (rounded so that fewer tokens
   // never need more)
-  const size_t room = c.wd_rank == 0 ? std::min((size_t)c.n_experts * T * c.d_model * 2, kScatterBytesMax) : 0;
+  const size_t room = std::min((size_t)c.n_experts * T * c.d_model * 2, kScatterBytesMax);
   L.xperm = take(tensor_ok ? std::max(n * (size_t)c.d_model * 2, room) : 0);
   L.hidden = take(tensor_ok ? n * (size_t)c.d_ff * 2 : 0);
   const size_t rp = ((size_t)c.wd_rank + 63) / 64 * 64;            // the rank rounded up to the tensor path's K step
@@ -266,7 +266,11 @@ int moe_expert_ffn(moe_ctx* ctx, const void* x, int32_t T, const moe_weights* w,
     return launch_wd_tokens(ctx, 1, x, T, w, nullptr, nullptr, expert_offsets, perm, nullptr, out_slots, (char*)ws, L,
                              s);
   }
-  return launch_tensor_ffn(ctx, x, T, w, expert_offsets, perm, (char*)ws, L, out_slots, nullptr, s);
+  if (w->expert_slot) return MOE_ERR_UNSUPPORTED;  // the tensor path reads experts in place (slot == expert)
+  char* const xperm = (char*)ws + L.xperm;
+  MOE_TRY(launch_gather_rows(ctx, x, perm, T * ctx->cfg.top_k, xperm, s));
+  return launch_prefill_ffn(ctx, T, w, PrefillRows{xperm, nullptr, nullptr, nullptr, nullptr, expert_offsets}, (char*)ws, L, out_slots,
+                            nullptr, s);
 }
 
 int moe_combine(moe_ctx* ctx, const float* out_slots, const float* topk_w, const int32_t* inv, int32_t T, void* y,
@@ -315,7 +319,7 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
     MOE_TRY(launch_route(ctx, x, T, w, idx, wt, nullptr, s, nullptr, &sc));
     const PrefillRows rows{wsb + L.xperm, ctx->d_state->route_count, idx, sc.pos, inv, nullptr};
     int planes = 1;
-    rc = launch_dense_prefill(ctx, T, w, rows, wsb + L.hidden, out_slots, nullptr, &planes, s);
+    rc = launch_prefill_ffn(ctx, T, w, rows, wsb, L, out_slots, &planes, s);
     if (rc != MOE_OK) {  // (the router has counted, and nobody will clear the counts)
       (void)cudaMemsetAsync(ctx->d_state->route_count, 0, sizeof(ctx->d_state->route_count), s);
       (void)cudaGetLastError();
@@ -327,7 +331,8 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   rc = launch_route(ctx, x, T, w, idx, wt, nullptr, s, &grp);
   if (rc != MOE_OK) return rc;
   int planes = 1;
-  rc = launch_tensor_ffn(ctx, x, T, w, offsets, perm, wsb, L, out_slots, &planes, s);
+  MOE_TRY(launch_gather_rows(ctx, x, perm, T * ctx->cfg.top_k, wsb + L.xperm, s));
+  rc = launch_prefill_ffn(ctx, T, w, PrefillRows{wsb + L.xperm, nullptr, nullptr, nullptr, nullptr, offsets}, wsb, L, out_slots, &planes, s);
   if (rc != MOE_OK) return rc;
   return launch_combine(ctx, out_slots, wt, inv, T, y, planes, s);
 }

@@ -188,10 +188,9 @@ bool prefill_scatters(const moe_config& c, int T);
 // planes: room for the partial sums of a cut contraction when the caller wants one sum (out_planes null)
 int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,
                          float* planes, int* out_planes, cudaStream_t s);
-// Tensor-core (prefill) path: out_slots from x gathered by perm.
-int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, const int32_t* offsets,
-                      const int32_t* perm, char* ws, const WsLayout& L, float* out_slots, int* out_planes,
-                      cudaStream_t s);
+// Tensor-core (prefill) path (decomposed experts: csrc/tensor_ffn.cu): out_slots from the grouped rows.
+int launch_prefill_ffn(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, char* ws, const WsLayout& L,
+                       float* out_slots, int* out_planes, cudaStream_t s);
 
 // ------------------------------------------------------------------ device side
 #ifdef __CUDACC__

@@ -127,15 +127,6 @@ __device__ __forceinline__ TokTile decode_tile(const DPPhase& H, int cap, int w_
   return t;
 }
 
-// (One reciprocal for two values' denominators would save a quarter of the special-function instructions, whose rate bounds the
-// epilogue; but a value would then depend on its neighbour, which is another token.)
-__device__ __forceinline__ float silu_mul(float g, float u) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-  return g * r * u;
-}
-
 // 16 tokens (registers) x 32 features (lanes) as bf16 to rows of tokens, through 1 KB of shared memory: two tokens of the lane's
 // feature at a time ...
 __device__ __forceinline__ void put_tokens(unsigned char* ebuf, int lane, int j, float v0, float v1) {
@@ -535,8 +526,10 @@ double hbm_cycles(int na, int hb, double tiles_per_weight) { return na * hb * 12
 
 }  // namespace
 
+// (Decomposed experts with few pairs: the four GEMMs' prefix sums over the counts cost what the gather's launch does.  384 pairs at d
+// 440, r 216: 55.6 us placed, 53.2 grouped and gathered; 1488 at d 648, r 104: 49.2 and 51.5; 4096 at d 2048, r 128: 102.8 and 109.5.)
 bool prefill_scatters(const moe_config& c, int T) {
-  return c.wd_rank == 0 && (size_t)c.n_experts * T * c.d_model * 2 <= kScatterBytesMax;
+  return (size_t)c.n_experts * T * c.d_model * 2 <= kScatterBytesMax && (c.wd_rank == 0 || T * c.top_k >= 1024);
 }
 
 int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,

@@ -163,6 +163,15 @@ __device__ __forceinline__ uint32_t instr_desc(int n, bool a_mmajor) {
   return d;
 }
 
+// (One reciprocal for two values' denominators would save a quarter of the special-function instructions, whose rate bounds the
+// epilogue; but a value would then depend on its neighbour, which is another token.)
+__device__ __forceinline__ float silu_mul(float g, float u) {
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * -1.4426950408889634f));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+  return g * r * u;
+}
+
 // ---- host: tensor maps --------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

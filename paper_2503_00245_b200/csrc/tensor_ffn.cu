@@ -43,7 +43,13 @@ enum BMode {
 };
 
 struct GGParams {
-  const int32_t* offsets;  // [E+1] slot ranges per expert
+  const unsigned* counts;  // [E] tokens of each expert, or null: ...
+  const int32_t* offsets;  // ... [E+1] slot ranges
+  int cap;                 // > 0: the rows of A are grouped at [e * cap ...] and not by slot
+  const int32_t *topk_idx, *pos;  // with inv: the (token, choice) pairs' experts and places among their expert's tokens ...
+  int32_t* inv;                   // ... from which their slots are worked out, by this launch
+  int n_pairs_tk;
+  int clear;                      // the last CTA clears the counts
   int E;
   int K;         // contraction length
   int n_total;   // output columns (per sub-row in B_PAIR / B_DUAL)
@@ -74,6 +80,7 @@ struct SmemGG {
 
 struct Tile {
   int e, m0, m_end, n0, ks;
+  int a0;  // first row of A
 };
 
 // The experts' slot ranges and tiles, spread over a warp's lanes (lane l: experts l and l + 32).  Every warp keeps its own:
@@ -85,9 +92,21 @@ struct TileMap {
 };
 __device__ __forceinline__ TileMap read_tile_map(const GGParams& P, int lane) {
   TileMap m;
-  const int e0 = min(lane, P.E), e1 = min(lane + 32, P.E);
-  m.lo0 = P.offsets[e0], m.hi0 = P.offsets[min(e0 + 1, P.E)];
-  m.lo1 = P.offsets[e1], m.hi1 = P.offsets[min(e1 + 1, P.E)];
+  if (P.counts) {
+    const int n0 = lane < P.E ? (int)__ldcg(P.counts + lane) : 0, n1 = lane + 32 < P.E ? (int)__ldcg(P.counts + lane + 32) : 0;
+    m.hi0 = n0, m.hi1 = n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v0 = __shfl_up_sync(0xffffffffu, m.hi0, o), v1 = __shfl_up_sync(0xffffffffu, m.hi1, o);
+      if (lane >= o) m.hi0 += v0, m.hi1 += v1;
+    }
+    m.hi1 += __shfl_sync(0xffffffffu, m.hi0, 31);
+    m.lo0 = m.hi0 - n0, m.lo1 = m.hi1 - n1;
+  } else {
+    const int e0 = min(lane, P.E), e1 = min(lane + 32, P.E);
+    m.lo0 = P.offsets[e0], m.hi0 = P.offsets[min(e0 + 1, P.E)];
+    m.lo1 = P.offsets[e1], m.hi1 = P.offsets[min(e1 + 1, P.E)];
+  }
   m.p0 = (max(m.hi0 - m.lo0, 0) + kPairRows - 1) / kPairRows;
   m.p1 = (max(m.hi1 - m.lo1, 0) + kPairRows - 1) / kPairRows;
 #pragma unroll
@@ -118,10 +137,10 @@ __device__ __forceinline__ Tile decode_tile(const GGParams& P, const TileMap& m,
   t.e = e;
   t.m0 = (e < 32 ? lo0 : lo1) + (mt - before) * kPairRows;
   t.m_end = e < 32 ? hi0 : hi1;
+  t.a0 = P.cap > 0 ? e * P.cap + (mt - before) * kPairRows : t.m0;
   return t;
 }
 
-__device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
 
 // 64 bytes of each of 32 rows from a warp's registers (lane = row) to memory, through 2 KB of shared memory: a store of
 // the accumulator layout as it is touches 32 lines with 16 bytes each; this one writes 8 rows' 64 bytes per instruction.
@@ -247,7 +266,7 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
       const Tile t = decode_tile(P, tm, idx, n_tiles);
       const int n0 = t.n0;
       const int kb0 = t.ks * num_kb / P.ksplit, kb1 = (t.ks + 1) * num_kb / P.ksplit;
-      const int a_row = t.m0 + (int)rank * kBM;
+      const int a_row = t.a0 + (int)rank * kBM;
       int k0 = kb0 * kBK;
       int kB = P.k_wrap > 0 ? k0 % P.k_wrap : k0;
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
@@ -338,6 +357,12 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
           if (++slot == (uint32_t)NS) slot = 0, par ^= 1u, st_lo = stage0;
         }
       }
+    } else if (P.inv) {  // slots of the (token, choice) pairs, for the combine
+      for (int p0 = pair * 32; p0 < P.n_pairs_tk; p0 += n_pairs * 32) {
+        const int p = min(p0 + lane, P.n_pairs_tk - 1), e = P.topk_idx[p];
+        const int a = __shfl_sync(0xffffffffu, tm.lo0, e & 31), b = __shfl_sync(0xffffffffu, tm.lo1, e & 31);
+        P.inv[p] = (e < 32 ? a : b) + P.pos[p];
+      }
     }
   } else {
     // ================================================================= epilogue (warps 2..9, both CTAs)
@@ -418,6 +443,15 @@ __global__ void __launch_bounds__(kThreadsGG, 1)
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
   }
+  if (P.clear && warp == 0) {  // the last CTA leaves the counts as the next call's router expects them
+    unsigned old = 0;
+    if (lane == 0) old = atom_add_acq_rel(&P.st->ffn_exit, 1u);
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (old == gridDim.x - 1u) {
+      for (int e = lane; e < MOE_MAX_EXPERTS; e += 32) P.st->route_count[e] = 0u;
+      if (lane == 0) P.st->ffn_exit = 0u;
+    }
+  }
 }
 
 int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b, GGParams P,
@@ -473,25 +507,20 @@ int make_map_rows(CUtensorMap* m, const void* base, long long inner, int nsub, l
   return make_map_b(m, base, inner, nsub, rows, slots, box_inner, box_rows, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, const int32_t* offsets,
-                      const int32_t* perm, char* ws, const WsLayout& L, float* out_slots, int* out_planes,
-                      cudaStream_t s) {
+int launch_prefill_ffn(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, char* ws, const WsLayout& L,
+                       float* out_slots, int* out_planes, cudaStream_t s) {
   const moe_config& c = ctx->cfg;
   if (w->expert_slot) return MOE_ERR_UNSUPPORTED;  // the tensor path reads experts in place (slot == expert)
   const int d = c.d_model, f = c.d_ff, r = c.wd_rank, E = c.n_experts;
   const int n_slots = T * c.top_k;
   if (out_planes) *out_planes = 1;
+  if (r == 0) return launch_dense_prefill(ctx, T, w, rows, ws + L.hidden, out_slots, (float*)(ws + L.out_slots), out_planes, s);
   void* xperm = ws + L.xperm;
   void* hidden = ws + L.hidden;
-  int rc = launch_gather_rows(ctx, x, perm, n_slots, xperm, s);
-  if (rc != MOE_OK) return rc;
+  int rc;
   CUtensorMap ma, ma1, mb;
   GGParams P{};
-  P.offsets = offsets;
-  if (r == 0) {
-    const PrefillRows rows{xperm, nullptr, nullptr, nullptr, nullptr, offsets};
-    return launch_dense_prefill(ctx, T, w, rows, hidden, out_slots, (float*)(ws + L.out_slots), out_planes, s);
-  }
+  P.counts = rows.counts, P.offsets = rows.offsets;
   // The rank-r intermediates t and v are kept as hi + lo pairs of bf16 (value = hi + lo): the GEMMs that
   // consume them run over K = 2 * rp with the weight slices repeated, so the intermediates carry ~16 mantissa
   // bits and the chain's only bf16 roundings are those of the dense path (hidden activations, output).
@@ -502,14 +531,16 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   void* mid_a = ws + L.mid_a;  // [n_slots][2*tw]: t_g (hi | lo) | t_u (hi | lo)
   void* mid_b = ws + L.mid_b;  // [n_slots][tw]:   v (hi | lo)
   // (1) T = X [gL | uL]
-  if ((rc = make_map_a(&ma, xperm, n_slots, d, d)) != MOE_OK) return rc;
+  if ((rc = make_map_a(&ma, rows.x, rows.counts ? (long long)E * T : n_slots, d, d)) != MOE_OK) return rc;
   const int pairs = ctx->sm_count / 2, m_tiles = row_tiles(n_slots, E);
   P.bn = pick_bn(r, 128);
   while (P.bn > 64 && 2 * m_tiles * ((r + P.bn - 1) / P.bn) <= pairs) P.bn /= 2;  // a small rank leaves pairs idle: narrower tiles
   if ((rc = make_map_b(&mb, w->wd_a, d, 2, r, E, kBK, P.bn)) != MOE_OK) return rc;
   P.K = d, P.n_total = r, P.bmode = B_PAIR, P.epi = EPI_BF16_PAIR;
   P.k_wrap = 0, P.split = 1, P.out = mid_a, P.ld_out = 2 * tw, P.out_off2 = tw, P.out_off_lo = rp, P.n_store = rp;
+  if (rows.counts) P.cap = T, P.topk_idx = rows.topk_idx, P.pos = rows.pos, P.inv = rows.inv, P.n_pairs_tk = n_slots;
   if ((rc = launch_gg(ctx, ma, ma, mb, P, n_slots, s)) != MOE_OK) return rc;
+  P.cap = 0, P.inv = nullptr;
   // (2) hidden = silu(Tg gR) * (Tu uR): two A operands, each CTA brings half of the gate and half of the up rows
   if ((rc = make_map_a(&ma, mid_a, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
   if ((rc = make_map_a(&ma1, (const __nv_bfloat16*)mid_a + tw, n_slots, tw, 2 * tw)) != MOE_OK) return rc;
@@ -541,6 +572,7 @@ int launch_tensor_ffn(moe_ctx* ctx, const void* x, int T, const moe_weights* w, 
   if ((rc = make_map_b(&mb, w->wd_d, r, 1, d, E, kBK, P.bn / 2)) != MOE_OK) return rc;
   P.K = tw, P.n_total = d, P.bmode = B_SINGLE, P.epi = EPI_F32;
   P.k_wrap = rp, P.split = 0, P.out = out_slots, P.ld_out = d, P.out_off2 = 0, P.out_off_lo = 0, P.n_store = 0;
+  P.clear = rows.counts != nullptr;
   return launch_gg(ctx, ma, ma, mb, P, n_slots, s);
 }
 
