@@ -23,6 +23,11 @@
  *    streams that overlap on the device race on the ctx's state (arrival counters, sums, the
  *    grouping of a prefill).
  *  - Weights are read-only for the library and may be shared between ctxs.
+ *  - Calls of different ctxs may run beside each other on different streams.  A prefill call ends with whatever part of the GPU it
+ *    finds.  A decode call of dense experts, or of one token with decomposed experts, is a CTA per SM that wait for one another:
+ *    it may run beside anything that ends by itself, prefill calls and cooperative launches included, but two such decode calls
+ *    (or one and another kernel of that kind) must not overlap: each could hold SMs that the other one's missing CTAs
+ *    need until both give up with MOE_ERR_TIMEOUT.  Put them on one stream, or order them with events.
  *  - Kernels that use programmatic dependent launch overlap the end of the kernel in front of them in the stream.  What
  *    that one writes is read after it has completed, with one exception: decode calls of dense experts, and of one token,
  *    read w_router earlier.  If the kernel in front lets its successors start early (griddepcontrol.launch_dependents; this

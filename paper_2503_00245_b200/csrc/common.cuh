@@ -45,7 +45,8 @@ struct DeviceState {
   unsigned int route_done;
   // prefill: CTAs of the expert kernel that have finished (the last one clears this line and the two below)
   unsigned int ffn_exit;
-  unsigned int pad3[17];
+  unsigned int ffn_next;  // prefill of dense experts: next tile that no pair of CTAs has taken yet
+  unsigned int pad3[16];
   unsigned int route_count[MOE_MAX_EXPERTS];  // tokens that the router has placed with each expert
   unsigned int ffn_done[MOE_MAX_EXPERTS];     // warps that have stored their part of a tile of the expert's hidden activations
 };

@@ -10,10 +10,13 @@
 //   warp 0     loads weights, 64-wide K slices, into a ring of shared-memory slots;
 //   warp 2     loads the K step's tokens (both CTAs' copies complete on a barrier of the leader's);
 //   warp 1     in the leader, one elected lane issues the MMAs for the pair;
-//   warp 3     writes down where the (token, choice) pairs went;
+//   warp 3     in the leader, takes the pair's tiles; in the other CTA, writes down where the (token, choice) pairs went;
 //   warps 4-19 epilogue: one tensor-memory lane = one feature per thread.
-// Tiles of (1), then of (2), are numbered through and dealt out in turn.  A tile of (2) waits for its expert's tiles of (1) at a
-// counter; there is no barrier over the grid and no second launch.
+// Tiles of (1), then of (2), are numbered through, and a pair takes the next number from a counter when it is about to run out of
+// loads.  A tile of (2) waits for its expert's tiles of (1) at a counter of theirs; there is no barrier over the grid and no second
+// launch.  Because the numbers are taken in order and by pairs that run, a wait is always for tiles that a running pair has in
+// hand, and those of (1) wait for nobody: the launch ends however few of its CTAs find room at a time, beside whatever else the
+// GPU runs.  (With the tiles dealt out by block number it did not: a pair without an SM held tiles that others waited for.)
 //
 // Why so: with the tokens on the M side, an expert's last 256-row tile cost what a full one does, and 128 weight rows were loaded
 // for every 128 token rows.  Here a K step of a pair is 48 KB per CTA for 2 x 256 features x 256 tokens instead of 64 KB, an
@@ -38,6 +41,8 @@ constexpr int kEpiWarpsDP = 16;  // four per quarter of the tensor-memory lanes
 constexpr int kThreadsDP = (4 + kEpiWarpsDP) * 32;
 constexpr int kSteps = 16;  // K steps in the ring at most (a power of two)
 constexpr int kEpiBytesDP = kEpiWarpsDP * 1024;
+constexpr int kAhead = 4;   // K steps in front of a tile's end at which the next tile is taken: a microsecond or two
+constexpr int kQueue = 4;   // tiles on their way to the roles (a power of two)
 
 struct DPPhase {
   int K, num_kb;    // contraction length, its K steps
@@ -77,6 +82,11 @@ struct SmemDP {
   uint64_t empty[kSteps];   // own: the MMAs have finished reading this CTA's operands of the K step
   uint64_t accum_full[2];        // own: all MMAs of the tile have completed
   uint64_t accum_empty[2];       // leader's: columns [256 b, 256 b + 256) have been read out of both CTAs' tensor memory
+  uint64_t tile_full[kQueue];    // own: the pair's next tile is there
+  uint64_t tile_empty[kQueue];   // leader's: all roles of both CTAs have read it (the epilogue, which comes last, arrives)
+  uint64_t tile_ask;             // leader's: the loads of the tokens of the tile in hand are about to end
+  int first_no;
+  int4 tile[kQueue][2];
   TokenMap map;
   uint32_t tmem_base;
 };
@@ -177,6 +187,7 @@ struct RingPos {
 struct Room {
   int free, oldest;
 };
+// steps1: the pair's K steps of phase 1, as far as they are known.
 __device__ __forceinline__ bool make_room(SmemDP& sm, Room& r, int step, int need, int steps1) {
   while (r.free < need || step - r.oldest >= kSteps) {
     if (!mbar_wait_warp(&sm.empty[r.oldest & (kSteps - 1)], (r.oldest / kSteps) & 1)) return false;
@@ -185,6 +196,17 @@ __device__ __forceinline__ bool make_room(SmemDP& sm, Room& r, int step, int nee
   }
   r.free -= need;
   return true;
+}
+
+// The pair's tiles after the first go to both CTAs as a whole, so that no role but one works them out.  idx >= the number of
+// tiles: there is none.  By one thread of the leader.
+__device__ __forceinline__ void hand_out(SmemDP& sm, int b, int idx, const TokTile& t) {
+#pragma unroll
+  for (uint32_t r = 0; r < 2; ++r) {
+    const uint32_t dst = map_to_rank(&sm.tile[b][0], r), bar = map_to_rank(&sm.tile_full[b], r);
+    st_async4(dst, make_int4(idx, t.e, t.s0, t.x0), bar);
+    st_async4(dst + 16, make_int4(t.toks | t.n << 16, t.f0, t.ks, t.tiles), bar);
+  }
 }
 
 __global__ void __launch_bounds__(kThreadsDP, 1)
@@ -202,7 +224,13 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
   const uint32_t rank = (uint32_t)lane0((int)cluster_ctarank());
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
-  pdl_launch_dependents();
+  // The pair's first number is taken in front of the dependency wait, and lies there when the counts are known.  That is safe
+  // because this kernel does not let its successors start early: they find the counter set back.  (Started early, they would
+  // only hold places: letting them in at the start of the launch costs a microsecond, d 1024, f 2816, 512 tokens 51.7 and 50.5 us.)
+  cluster_arrive();
+  int first_no = 0;
+  const bool takes = rank == 0 && tid == 3 * 32;
+  if (takes) first_no = (int)atomicAdd(&P.st->ffn_next, 1u);
   if (tid == 0) {
     for (int i = 0; i < kSteps; ++i) {
       mbar_init(&sm.full[i], 2);
@@ -212,6 +240,12 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
       mbar_init(&sm.accum_full[b], 1);
       mbar_init(&sm.accum_empty[b], 2 * kEpiWarpsDP);
     }
+    for (int i = 0; i < kQueue; ++i) {
+      mbar_init(&sm.tile_full[i], 1);
+      mbar_init(&sm.tile_empty[i], 2 * kEpiWarpsDP);
+      mbar_arrive_expect_tx(&sm.tile_full[i], 32);
+    }
+    mbar_init(&sm.tile_ask, 1);
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w1) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x1) : "memory");
     fence_mbar_init();
@@ -224,6 +258,8 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  cluster_wait();  // (the other CTA has started: its shared memory may be written)
+  if (takes) sm.first_no = first_no, st_cluster(map_to_rank(&sm.first_no, 1u), (uint32_t)first_no);
   __syncthreads();
   __syncwarp();
   cluster_sync_all();
@@ -234,7 +270,7 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
   // the same number of tokens, and from the counts behind it.  The first pass only brings in the code of the second, which
   // stands in front of the first loads.
   TokTile t{};
-  int total = 0, widest = 0, n_work1 = 0, n_work = 0;
+  int total = 0, widest = 0, n_work1 = 0, n_work = 0, idx = lane0(sm.first_no);
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     const int e1 = lane + 32;
@@ -252,31 +288,43 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
     token_map(sm.map, lane, P.w_max, n0, n1, total, widest);
     n_work1 = total * P.ph[0].per_tok, n_work = n_work1 + total * P.ph[1].per_tok;
     t.e = -1;
-    if (pair < n_work) {  // (with few tiles a pair's first one may be of phase 2)
-      const int ph = pair >= n_work1;
-      t = decode_tile(P.ph[ph], ph ? 0 : P.cap, P.w_max, sm.map, lane, pair - (ph ? n_work1 : 0));
+    if (idx < n_work) {  // (with few tiles a pair's first one may be of phase 2)
+      const int ph = idx >= n_work1;
+      t = decode_tile(P.ph[ph], ph ? 0 : P.cap, P.w_max, sm.map, lane, idx - (ph ? n_work1 : 0));
     }
   }
-  const int steps1 = pair < n_work1 ? (n_work1 - pair + n_pairs - 1) / n_pairs * P.ph[0].num_kb : 0;  // this pair's K steps of phase 1
   // accumulators: two buffers of 256 columns, or, for two matrices and more than 128 tokens, a single one of 512
   const bool two = widest <= 128;
   const uint32_t acc1 = two ? 128u : 256u;  // the up products' columns behind the gate's
-  auto tile_at = [&](int idx) {
-    const int ph = idx >= n_work1;
-    return decode_tile(P.ph[ph], ph ? 0 : P.cap, P.w_max, sm.map, lane, idx - (ph ? n_work1 : 0));
+  // the pair's seq-th tile to idx and t (the first one is there); false: there is none
+  auto next_tile = [&](int seq) {
+    if (seq > 0) {
+      const int b = (seq - 1) & (kQueue - 1);
+      if (!mbar_wait_warp(&sm.tile_full[b], ((seq - 1) / kQueue) & 1)) {
+        if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x416u);
+        return false;
+      }
+      const int4 u = sm.tile[b][0], v = sm.tile[b][1];
+      if (tid == 0) mbar_arrive_expect_tx(&sm.tile_full[b], 32);  // (for the tile kQueue further on)
+      idx = lane0(u.x);
+      t.e = lane0(u.y), t.s0 = lane0(u.z), t.x0 = lane0(u.w);
+      t.toks = lane0(v.x) & 0xffff, t.n = lane0(v.x) >> 16, t.f0 = lane0(v.y), t.ks = lane0(v.z), t.tiles = lane0(v.w);
+    }
+    return idx < n_work;
   };
 
   if (warp == 0) {
     // ================================================================= weights (both CTAs)
     RingPos at{0, 0};
     Room room{NS, 0};
-    bool ok = true, first = true;
-    for (int idx = pair; ok && idx < n_work; idx += n_pairs, first = false) {
-      if (!first) t = tile_at(idx);
+    int steps1 = 0x7fffffff;
+    bool ok = true;
+    for (int seq = 0; ok && next_tile(seq); ++seq) {
       const int ph = idx >= n_work1;
       const DPPhase& H = P.ph[ph];
-      const int kb1 = (t.ks + 1) * H.num_kb / H.ksplit, f = t.f0 + (int)rank * H.hb;
-      for (int kb = t.ks * H.num_kb / H.ksplit; kb < kb1; ++kb) {
+      if (ph) steps1 = min(steps1, at.step);
+      const int kb0 = t.ks * H.num_kb / H.ksplit, kb1 = (t.ks + 1) * H.num_kb / H.ksplit, f = t.f0 + (int)rank * H.hb;
+      for (int kb = kb0; kb < kb1; ++kb) {
         if (!(ok = make_room(sm, room, at.step, 3 - ph, steps1))) {
           if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x410u);
           break;
@@ -297,11 +345,12 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
     // ================================================================= tokens (both CTAs)
     RingPos at{0, 0};
     Room room{NS, 0};
-    bool ok = true, first = true;
-    for (int idx = pair; ok && idx < n_work; idx += n_pairs, first = false) {
-      if (!first) t = tile_at(idx);
+    int steps1 = 0x7fffffff;
+    bool ok = true;
+    for (int seq = 0; ok && next_tile(seq); ++seq) {
       const int ph = idx >= n_work1;
       const DPPhase& H = P.ph[ph];
+      if (ph) steps1 = min(steps1, at.step);
       if (ph == 1) {  // the expert's hidden activations: all of its tiles of phase 1 have been stored
         const unsigned want = (unsigned)(t.tiles * P.ph[0].per_tok * 2 * kEpiWarpsDP);
         const long long c0 = clock64();
@@ -315,8 +364,10 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
       }
       const int boxes = (t.n / 2 + P.tb - 1) / P.tb, box_bytes = P.tb * kBK * 2;
       const int row = (ph ? t.s0 : t.x0) + (int)rank * (t.n / 2);
-      const int kb1 = (t.ks + 1) * H.num_kb / H.ksplit;
-      for (int kb = t.ks * H.num_kb / H.ksplit; kb < kb1; ++kb) {
+      const int kb0 = t.ks * H.num_kb / H.ksplit, kb1 = (t.ks + 1) * H.num_kb / H.ksplit, ask = max(kb0, kb1 - kAhead);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        // (here and not where the weights are loaded: a pair that waits for hidden activations takes no further tiles meanwhile)
+        if (kb == ask && rank == 0 && lane == 0) mbar_arrive(&sm.tile_ask);
         if (!(ok = make_room(sm, room, at.step, 3 - ph, steps1))) {
           if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x415u);
           break;
@@ -347,8 +398,8 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
       const uint32_t lbo_k = 1u << 16, lbo_m = (uint32_t)(64 * kBK * 2 >> 4) << 16;
       const uint32_t slot0 = st0 >> 4, slot_step = slot_bytes >> 4;
       RingPos at{0, 0};
-      int tile_i = 0, used0 = 0, used1 = 0;  // tiles that have gone through either half of the accumulators
-      bool ok = true, first = true;
+      int used0 = 0, used1 = 0;  // tiles that have gone through either half of the accumulators
+      bool ok = true;
       auto operands = [&]() {  // of the ring's current K step
         if (mbar_wait_warp(&sm.full[at.step & (kSteps - 1)], (at.step / kSteps) & 1)) {
           tc_fence_after();
@@ -366,11 +417,10 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x413u);
         return false;
       };
-      for (int idx = pair; ok && idx < n_work; idx += n_pairs, ++tile_i, first = false) {
-        if (!first) t = tile_at(idx);
+      for (int seq = 0; ok && next_tile(seq); ++seq) {
         const int ph = idx >= n_work1;
         const DPPhase& H = P.ph[ph];
-        const int buf = ph == 0 && !two ? 0 : tile_i & 1;
+        const int buf = ph == 0 && !two ? 0 : seq & 1;
         const bool both = ph == 0 && !two;
         if (!(ok = drained(buf, buf ? used1 : used0) && (!both || drained(1, used1)))) break;
         const uint32_t idesc = instr_desc(t.n, ph == 1), d_tmem = tmem + (uint32_t)(buf * kAccCols);
@@ -412,31 +462,54 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
       }
     }
   } else if (warp == 3) {
-    // ================================================================= slots of the (token, choice) pairs, for the combine
-    if (P.counts) {
+    if (rank == 0) {
+      // =============================================================== takes the pair's tiles
+      // Every pair takes one number that is past the last tile, so the launch takes n_work + n_pairs of them; who has the
+      // highest sets the counter back.
+      if (lane == 0 && idx == n_work + n_pairs - 1) atomicExch(&P.st->ffn_next, 0u);
+      for (int q = 0; idx < n_work; ++q) {
+        const int b = q & (kQueue - 1);
+        if (!mbar_wait_warp(&sm.tile_ask, q & 1) || (q >= kQueue && !mbar_wait_warp(&sm.tile_empty[b], (q / kQueue - 1) & 1))) {
+          if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x417u);
+          break;
+        }
+        if (lane == 0) idx = (int)atomicAdd(&P.st->ffn_next, 1u);
+        idx = lane0(idx);
+        if (idx < n_work) {
+          const int ph = idx >= n_work1;
+          t = decode_tile(P.ph[ph], ph ? 0 : P.cap, P.w_max, sm.map, lane, idx - (ph ? n_work1 : 0));
+        }
+        if (lane == 0) {
+          hand_out(sm, b, idx, t);
+          if (idx == n_work + n_pairs - 1) atomicExch(&P.st->ffn_next, 0u);
+        }
+      }
+    } else if (P.counts) {
+      // =============================================================== slots of the (token, choice) pairs, for the combine
       __syncwarp();
-      for (int p = blockIdx.x * 32 + lane; p < P.n_pairs_tk; p += gridDim.x * 32) {
+      for (int p = pair * 32 + lane; p < P.n_pairs_tk; p += n_pairs * 32) {
         const int e = P.topk_idx[p];
         P.inv[p] = sm.map.lo[e >> 5][e & 31] + P.pos[p];
       }
     }
   } else {
-    // ================================================================= epilogue (warps 4..11, both CTAs)
+    // ================================================================= epilogue (warps 4..19, both CTAs)
     const int q = warp & 3, part = (warp - 4) >> 2;  // quarter of the lanes it may read; every fourth 16-column chunk
     const uint32_t acce_bar[2] = {map_to_rank(&sm.accum_empty[0], 0u), map_to_rank(&sm.accum_empty[1], 0u)};
     unsigned char* const ebuf = epi_bufs + (warp - 4) * (kEpiBytesDP / kEpiWarpsDP);
-    int tile_i = 0, seen0 = 0, seen1 = 0;
-    bool first = true;
-    for (int idx = pair; idx < n_work; idx += n_pairs, ++tile_i, first = false) {
-      if (!first) t = tile_at(idx);
+    const uint32_t tile_bar = map_to_rank(&sm.tile_empty[0], 0u);
+    int seen0 = 0, seen1 = 0;
+    for (int seq = 0; next_tile(seq); ++seq) {
       const int ph = idx >= n_work1;
       const bool both = ph == 0 && !two;
-      const int buf = both ? 0 : tile_i & 1, hb = P.ph[ph].hb, m_total = P.ph[ph].m_total;
+      const int buf = both ? 0 : seq & 1, hb = P.ph[ph].hb, m_total = P.ph[ph].m_total;
       if (!mbar_wait_warp(&sm.accum_full[buf], (buf ? seen1 : seen0) & 1)) {
         if (lane == 0) flag_error(P.st, MOE_ERR_TIMEOUT, 0x412u);
         break;
       }
       if (buf) ++seen1; else ++seen0;
+      // (the tile is in the lanes' registers; the producers and the issuer have had it before any of the tile's products)
+      if (lane == 0 && seq > 0) mbar_arrive_cluster(tile_bar + 8u * (uint32_t)((seq - 1) & (kQueue - 1)));
       tc_fence_after();
       const int fb = t.f0 + (int)rank * hb + 32 * q;              // this warp's first feature,
       const int feats = min(min(hb - 32 * q, 32), m_total - fb);  // how many it has (a multiple of 8; <= 0: none)
