@@ -613,38 +613,42 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   DPParams P{};
   P.counts = rows.counts, P.offsets = rows.offsets, P.E = E, P.T = T, P.n_pairs_tk = n_slots, P.cap = rows.counts ? T : 0;
   P.topk_idx = rows.topk_idx, P.pos = rows.pos, P.inv = rows.inv;
-  P.w_max = std::min(256, (m + m / 4 + 16 + 31) / 32 * 32);  // an expert's tokens mostly in one tile, no more room than that
-  P.tb = std::max(16, P.w_max / 4);
+  P.tb = m + m / 4 + 16 <= 192 ? 32 : 64;  // (32 rows: less read past an expert's tokens; 64: fewer loads to issue)
   P.likely = m, P.st = ctx->d_state;
   P.hidden = (__nv_bfloat16*)hidden, P.plane_elems = (long long)n_slots * d;
   // how the work is cut: the fewest cycles for the pair with the most, tiles of both phases being dealt out in turn
   const size_t fixed = kEpiBytesDP + sizeof(SmemDP) + 1024 + 128;  // (an MMA reads 128 rows of weights, whatever hb is: the
                                                                    // epilogue's buffers are long enough behind the last slot)
-  const auto slot_rows = [&](int h1, int h2) { return std::max(std::max(h1, h2), (P.w_max / 2 + P.tb - 1) / P.tb * P.tb); };
-  const auto ring_slots = [&](int h1, int h2) { return (int)((ctx->max_smem_optin - fixed) / ((size_t)slot_rows(h1, h2) * kBK * 2)); };
-  const int nt = token_tiles_expected(n_slots, E, P.w_max), n = std::min(P.w_max, (n_slots / nt + 31) / 32 * 32);
-  const double tpw = (double)nt / active;
+  const auto ring_slots = [&](int h) { return (int)((ctx->max_smem_optin - fixed) / ((size_t)h * kBK * 2)); };
   const int kb1 = (d + kBK - 1) / kBK, kb2 = (f + kBK - 1) / kBK;
   int hb1 = 0, ks2 = 1;
   const int hb2 = d > 128 ? 128 : 64;
   double best = 0;
-  for (int h1 = 128; h1 >= 32; h1 -= 8) {
-    const int n1 = nt * ((f + 2 * h1 - 1) / (2 * h1)), ns = ring_slots(h1, hb2);
-    // (a pair whose loads take longer than its neighbours' gets more of HBM: half of that term)
-    const double c1 = kb1 * (step_cycles(2, h1, n, ns / 3) + 0.5 * hbm_cycles(2, h1, tpw)) + (n > 128 ? 4000 : 1500);
-    for (int ks = 1; ks <= (n_slots <= kKSplitMaxSlots ? std::min(kKSplitMax, kb2) : 1); ++ks) {
-      const int n2 = nt * ((d + 2 * hb2 - 1) / (2 * hb2)) * ks;
-      const double c2 = (kb2 + ks - 1) / ks * (step_cycles(1, hb2, n, ns / 2) + 0.5 * hbm_cycles(1, hb2, tpw)) + 1500;
-      const int q1 = n1 / pairs_all, r1 = n1 % pairs_all, q = (n1 + n2) / pairs_all, r = (n1 + n2) % pairs_all;
-      const auto load = [&](int a, int all) { return a * c1 + (all - a) * c2; };
-      double worst = std::max(load(q1, q), std::min(r1, r) > 0 ? load(q1 + 1, q + 1) : 0.0);
-      if (r > r1) worst = std::max(worst, load(q1, q + 1));
-      if (r1 > r) worst = std::max(worst, load(q1 + 1, q));
-      worst = std::max(worst, (q1 + (r1 > 0)) * c1 + c2);  // (the last experts' second product starts when all of phase 1 is done)
-      // a further plane of partial sums, written and read, in the epilogue and in the combine (wearable, 512 tokens: one plane 56.9
-      // us, two 52.8, four 54.7; paper, 333 tokens: 74.7, 69.6, 74.8)
-      worst += (ks - 1) * 16.0 * n_slots * d / 3800.0;
-      if (hb1 == 0 || worst < 0.98 * best) best = worst, hb1 = h1, ks2 = ks;
+  // Tiles of up to 256 tokens: an expert with more than its share needs no further pass over its weights (512 tokens, d 1024, f 2816,
+  // all at the same two of 8 experts: tiles as wide as an even share, 192, 45.6 us, 256 41.7; 1000 tokens, d 2048, f 5632, 2 of 16:
+  // 133.9, 122.9).  Up to 128 where the contractions are short and the epilogue of a wide tile, in the open, weighs more (1900
+  // tokens, d 304, f 904, 2 experts: 256 30.2 us, 128 27.4).
+  for (const int w_max : {256, 128}) {
+    const int nt = token_tiles_expected(n_slots, E, w_max), n = std::min(w_max, (n_slots / nt + 31) / 32 * 32), ns = ring_slots(128);
+    const double tpw = (double)nt / active;
+    for (int h1 = 128; h1 >= 32; h1 -= 8) {
+      const int n1 = nt * ((f + 2 * h1 - 1) / (2 * h1));
+      // (a pair whose loads take longer than its neighbours' gets more of HBM: half of that term)
+      const double c1 = kb1 * (step_cycles(2, h1, n, ns / 3) + 0.5 * hbm_cycles(2, h1, tpw)) + (n > 128 ? 4000 : 1500);
+      for (int ks = 1; ks <= (n_slots <= kKSplitMaxSlots ? std::min(kKSplitMax, kb2) : 1); ++ks) {
+        const int n2 = nt * ((d + 2 * hb2 - 1) / (2 * hb2)) * ks;
+        const double c2 = (kb2 + ks - 1) / ks * (step_cycles(1, hb2, n, ns / 2) + 0.5 * hbm_cycles(1, hb2, tpw)) + 1500;
+        const int q1 = n1 / pairs_all, r1 = n1 % pairs_all, q = (n1 + n2) / pairs_all, r = (n1 + n2) % pairs_all;
+        const auto load = [&](int a, int all) { return a * c1 + (all - a) * c2; };
+        double worst = std::max(load(q1, q), std::min(r1, r) > 0 ? load(q1 + 1, q + 1) : 0.0);
+        if (r > r1) worst = std::max(worst, load(q1, q + 1));
+        if (r1 > r) worst = std::max(worst, load(q1 + 1, q));
+        worst = std::max(worst, (q1 + (r1 > 0)) * c1 + c2);  // (the last experts' second product starts when all of phase 1 is done)
+        // a further plane of partial sums, written and read, in the epilogue and in the combine (wearable, 512 tokens: one plane 56.9
+        // us, two 52.8, four 54.7; paper, 333 tokens: 74.7, 69.6, 74.8)
+        worst += (ks - 1) * 16.0 * n_slots * d / 3800.0;
+        if (hb1 == 0 || worst < 0.98 * best) best = worst, hb1 = h1, ks2 = ks, P.w_max = w_max;
+      }
     }
   }
   P.ph[0] = DPPhase{d, kb1, f, hb1, 1, (f + 2 * hb1 - 1) / (2 * hb1)};
@@ -656,8 +660,8 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   MOE_TRY(make_map_a(&x1, rows.x, P.cap ? (long long)E * T : n_slots, d, d, P.tb));
   MOE_TRY(make_map_b(&w2, w->gud, d, 3, f, E, 64, kBK));
   MOE_TRY(make_map_a(&x2, hidden, n_slots, f, f, P.tb));
-  P.slot_bytes = slot_rows(hb1, hb2) * kBK * 2;
-  P.n_slots = ring_slots(hb1, hb2);
+  P.slot_bytes = 128 * kBK * 2;
+  P.n_slots = ring_slots(128);
   if (P.n_slots < 6) return MOE_ERR_UNSUPPORTED;
   const size_t smem = (size_t)P.n_slots * P.slot_bytes + fixed;
   MOE_TRY(allow_full_smem<dense_prefill_kernel>(ctx));

@@ -144,6 +144,28 @@ def test_prefill_tiles_and_the_rows_places(sh, T):
     assert lay.check() == 0
 
 
+@pytest.mark.parametrize("sh,T,bias,spread", [
+    (shape(264, 520, E=16, k=2), 600, 30.0, 1),         # every token at the same two experts: tiles far wider than an even share
+    (shape(264, 520, E=16, k=2), 600, 30.0, 8),         # ... and the others' few tokens beside them
+    (shape(1024, 1032, E=8, k=2, xd="f32"), 257, 30.0, 1),  # two tiles of 160 columns
+    (shape(136, 512, E=64, k=1), 1100, 30.0, 8),
+    (shape(304, 904, E=2, k=1), 1900, 0.0, 1),          # short contractions: tiles of at most 128 columns
+])
+def test_prefill_of_unevenly_routed_tokens(sh, T, bias, spread):
+    """The first experts' logits are `bias` higher, all logits `spread` times as wide as usual (in w_router, a power of two, so that
+    the rows keep the one scale that check_prefill's bound is derived for)."""
+    t = W.make_layer(sh, T, device="cuda")
+    t["b_router"] = torch.zeros(sh.n_experts, device="cuda")
+    t["b_router"][:sh.top_k] = bias
+    t["w_router"] *= spread
+    lay, t, host = U.build(sh, T, tensors=t)
+    check_prefill(lay, t, host, sh.top_k)
+    idx, w, _ = lay.route(t["x"])
+    offsets, perm, inv = lay.permute(idx)
+    assert torch.equal(lay.combine(lay.expert_ffn(t["x"], offsets, perm), w, inv), lay.forward(t["x"]))
+    assert lay.check() == 0
+
+
 @pytest.mark.parametrize("T", [8, 16])
 def test_dense_decode_of_several_tokens_with_many_pairs(T):
     sh = shape(512, 1024, E=16, k=8)                    # 64 and 128 pairs: beyond one per lane; every expert active
