@@ -175,8 +175,14 @@ __device__ __forceinline__ uint32_t instr_desc(int n, bool a_mmajor) {
   return d;
 }
 
-// (One reciprocal for two values' denominators would save a quarter of the special-function instructions, whose rate bounds the
-// epilogue; but a value would then depend on its neighbour, which is another token.)
+// silu(g) u = g u / (1 + e^-g), with e^-g = 2^(-g log2(e)): one power of two and one reciprocal on the special-function unit, whose
+// rate bounds the epilogue.  The PTX manual gives their relative errors, 2^-22 and 2^-23.  The exponent is rounded to fp32 (its
+// factor too), 1.25 2^-24 of itself, which is |g| 1.25 2^-24 of e^-g; the sum and the two products round at 2^-24.  With
+// p = e^-g / (1 + e^-g), at most 1: the relative error is at most p (|g| 1.25 2^-24 + 2^-22) + 5 2^-24.  Below g = -87 the
+// reciprocal would be smaller than 2^-126 and is zero, as is the result then: |g| 2^-126 is lost.  The bf16 that the value is
+// stored as is 2^-9 wide.
+// (One reciprocal for two values' denominators would save a quarter of these instructions; but a value would then depend on its
+// neighbour, which is another token.)
 __device__ __forceinline__ float silu_mul(float g, float u) {
   float e, r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * -1.4426950408889634f));
