@@ -125,7 +125,11 @@ int moe_device_sm_count(void);
 int moe_create(const moe_config* cfg, moe_ctx** out);
 int moe_destroy(moe_ctx* ctx);
 int moe_check(moe_ctx* ctx, void* stream);
-/* Scratch the hot calls need for T tokens (upper bound over all calls and paths). */
+/* Scratch the hot calls need for T tokens (upper bound over all calls and paths, and over calls with fewer tokens).  A prefill
+ * takes, per (token, choice) pair, 2 f bytes for hidden activations, 4 d for outputs (16 d up to 2048 pairs) and 24 r for
+ * decomposed experts' intermediates; its rows take 2 d per pair, or, where the router places them as it goes, 2 d per token and
+ * EXPERT, at most 256 MB: more than 16 tokens, experts (rounded up to 8) x about 2 d + 1100 bytes within 112 KB (d = 2048: 16
+ * experts), and, for decomposed experts, 1024 pairs or more.  (d 2048, 8 experts, 2048 tokens: 67 MB.)                                              */
 int moe_workspace_bytes(const moe_config* cfg, int32_t T, size_t* bytes);
 /* Diagnostics, for testing the time-out path without hanging or faulting anything.  Not for production use.
  * moe_set_finaliser_wait: how many SM clock cycles the finalising CTAs of the dense streaming kernel wait for

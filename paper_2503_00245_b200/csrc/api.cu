@@ -47,9 +47,9 @@ WsLayout ws_layout(const moe_config& c, int T) {
   L.vec_b = take(wd_stream ? n * fs * 6 : 0);
   L.vec_c = take(wd_stream ? n * std::max(rs * 6, (size_t)c.wd_rank * 8 * 4) : 0);
   L.pos = take(n * 4);
-  // by slot; or T rows per expert while that is not more than kScatterBytesMax (rounded so that fewer tokens
-  // never need more)
-  const size_t room = std::min((size_t)c.n_experts * T * c.d_model * 2, kScatterBytesMax);
+  // by slot; or, where the router places the rows, room for every token at every expert (for the call of up to T tokens that
+  // needs most: fewer never need more)
+  const size_t room = (size_t)c.n_experts * prefill_placed_tokens(c, T) * c.d_model * 2;
   L.xperm = take(tensor_ok ? std::max(n * (size_t)c.d_model * 2, room) : 0);
   L.hidden = take(tensor_ok ? n * (size_t)c.d_ff * 2 : 0);
   const size_t rp = ((size_t)c.wd_rank + 63) / 64 * 64;            // the rank rounded up to the tensor path's K step
@@ -314,7 +314,7 @@ int moe_layer_forward(moe_ctx* ctx, const void* x, int32_t T, const moe_weights*
   int32_t* inv = (int32_t*)(wsb + L.inv);
   float* out_slots = (float*)(wsb + L.out_slots);
   if (w->expert_slot) return MOE_ERR_UNSUPPORTED;  // the tensor path reads experts in place (slot == expert)
-  if (prefill_scatters(ctx->cfg, T) && route_tile_applies(ctx->cfg, T)) {
+  if (prefill_placed_tokens(ctx->cfg, T) == T) {
     const Scatter sc{wsb + L.xperm, (int32_t*)(wsb + L.pos)};
     MOE_TRY(launch_route(ctx, x, T, w, idx, wt, nullptr, s, nullptr, &sc));
     const PrefillRows rows{wsb + L.xperm, ctx->d_state->route_count, idx, sc.pos, inv, nullptr};

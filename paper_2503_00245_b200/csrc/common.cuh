@@ -185,7 +185,8 @@ struct PrefillRows {
   const int32_t* offsets;
 };
 constexpr size_t kScatterBytesMax = (size_t)256 << 20;  // room for the rows placed by the router, at most
-bool prefill_scatters(const moe_config& c, int T);
+// The most tokens, up to T, of a prefill call whose rows the router places (0: none).
+int prefill_placed_tokens(const moe_config& c, int T);
 // planes: room for the partial sums of a cut contraction when the caller wants one sum (out_planes null)
 int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,
                          float* planes, int* out_planes, cudaStream_t s);

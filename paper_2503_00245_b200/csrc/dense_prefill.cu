@@ -601,8 +601,9 @@ double hbm_cycles(int na, int hb, double tiles_per_weight) { return na * hb * 12
 
 // (Decomposed experts with few pairs: the four GEMMs' prefix sums over the counts cost what the gather's launch does.  384 pairs at d
 // 440, r 216: 55.6 us placed, 53.2 grouped and gathered; 1488 at d 648, r 104: 49.2 and 51.5; 4096 at d 2048, r 128: 102.8 and 109.5.)
-bool prefill_scatters(const moe_config& c, int T) {
-  return (size_t)c.n_experts * T * c.d_model * 2 <= kScatterBytesMax && (c.wd_rank == 0 || T * c.top_k >= 1024);
+int prefill_placed_tokens(const moe_config& c, int T) {
+  const int t = (int)std::min<size_t>(T, kScatterBytesMax / ((size_t)c.n_experts * c.d_model * 2));
+  return route_tile_applies(c, t) && (c.wd_rank == 0 || (long long)t * c.top_k >= 1024) ? t : 0;
 }
 
 int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,
