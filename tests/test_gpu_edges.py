@@ -166,6 +166,54 @@ def test_prefill_of_unevenly_routed_tokens(sh, T, bias, spread):
     assert lay.check() == 0
 
 
+@pytest.mark.parametrize("sh,T,bias", [
+    (shape(264, 520, E=33, k=8, r=40, xd="f32"), 200, 0.0),  # a second expert per lane, rows placed by the router
+    (shape(136, 512, E=64, k=8, r=64), 300, 0.0),
+    (shape(136, 512, E=64, k=8, r=64), 300, 30.0),           # ... most experts without a token
+    (shape(264, 520, E=33, k=8), 200, 30.0),
+])
+def test_prefill_of_many_experts_and_then_of_fewer_tokens(sh, T, bias):
+    t = W.make_layer(sh, T, device="cuda")
+    t["b_router"] = torch.zeros(sh.n_experts, device="cuda")
+    t["b_router"][-sh.top_k:] = bias
+    lay, t, host = U.build(sh, T, tensors=t)
+    check_prefill(lay, t, host, sh.top_k)
+    for n in (T, 150, 129, 17):                         # (decomposed experts: placed from 1024 pairs, 128 tokens, on)
+        x = t["x"][:n].contiguous()
+        idx, w, _ = lay.route(x)
+        offsets, perm, inv = lay.permute(idx)
+        y = lay.combine(lay.expert_ffn(x, offsets, perm), w, inv)
+        assert torch.equal(y, lay.forward(x)), n
+    assert lay.check() == 0
+
+
+@pytest.mark.parametrize("r", [0, 64])
+def test_captured_prefill_follows_its_inputs(r):
+    """One graph of two calls, replayed on other rows in the same buffer: routing, places, tile counts and sums are those of the new
+    rows, and the counters are where the next call wants them."""
+    sh = shape(512, 1024, r=r, bias="normal")
+    lay, t, host = U.build(sh, 600)
+    x, others = t["x"].clone(), [t["x"], t["x"].flip(0).contiguous(), (t["x"] * 0.5).roll(3, 1).contiguous(), t["x"]]
+    others[1][::3] = others[1][0]                       # a third of the tokens share their experts
+    want = [lay.forward(v) for v in others]
+    y = torch.empty_like(x)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lay.forward(x, y=y)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            lay.forward(x, y=y)
+            z = lay.forward(x)
+        for v, ref in zip(others, want):
+            x.copy_(v), y.zero_(), z.zero_()
+            graph.replay()
+            stream.synchronize()
+            assert torch.equal(y, ref) and torch.equal(z, ref)
+    assert lay.check() == 0
+    assert torch.equal(lay.forward(others[2]), want[2])
+
+
 @pytest.mark.parametrize("T", [8, 16])
 def test_dense_decode_of_several_tokens_with_many_pairs(T):
     sh = shape(512, 1024, E=16, k=8)                    # 64 and 128 pairs: beyond one per lane; every expert active
