@@ -43,9 +43,11 @@ struct DeviceState {
   unsigned int tail_bias;
   // router of many tokens: CTAs that have stored their tokens' routing; the last one sets it back
   unsigned int route_done;
-  // prefill: CTAs of the expert kernel that have finished (the last one clears this line and the two below)
+  // prefill: CTAs of the expert kernel that have finished (the last one clears this word and the two lines below)
   unsigned int ffn_exit;
-  unsigned int ffn_next;  // prefill of dense experts: next tile that no pair of CTAs has taken yet
+  // prefill of dense experts: next tile that no pair of CTAs has taken yet (who takes the launch's last number sets it back; after a
+  // wait that ran out moe_check does)
+  unsigned int ffn_next;
   unsigned int pad3[16];
   unsigned int route_count[MOE_MAX_EXPERTS];  // tokens that the router has placed with each expert
   unsigned int ffn_done[MOE_MAX_EXPERTS];     // warps that have stored their part of a tile of the expert's hidden activations
@@ -176,7 +178,7 @@ int launch_fp8_dequant(const void* codes, const float* scales, long long rows, i
 // of box_inner x box_rows of one sub-row, rows box_inner values apart in shared memory (csrc/tensor_ffn.cu).
 int make_map_rows(CUtensorMap* m, const void* base, long long inner, int nsub, long long rows, int slots, int box_inner,
                   int box_rows);
-// Prefill of dense experts (csrc/dense_prefill.cu).  The rows of x, bf16: placed by the router (counts set), or grouped by slot.
+// The rows of x of a prefill, bf16: placed by the router (counts set), or grouped by slot.
 struct PrefillRows {
   const void* x;
   const unsigned* counts;
@@ -187,7 +189,8 @@ struct PrefillRows {
 constexpr size_t kScatterBytesMax = (size_t)256 << 20;  // room for the rows placed by the router, at most
 // The most tokens, up to T, of a prefill call whose rows the router places (0: none).
 int prefill_placed_tokens(const moe_config& c, int T);
-// planes: room for the partial sums of a cut contraction when the caller wants one sum (out_planes null)
+// Prefill of dense experts (csrc/dense_prefill.cu).  planes: room for the partial sums of a cut contraction when the caller wants one
+// sum (out_planes null)
 int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const PrefillRows& rows, void* hidden, float* out_slots,
                          float* planes, int* out_planes, cudaStream_t s);
 // Tensor-core (prefill) path (decomposed experts: csrc/tensor_ffn.cu): out_slots from the grouped rows.
@@ -447,8 +450,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-
-__device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
 
 // fp32 -> unsigned key with the same order (-0 counts as +0; NaN is not ordered), and back
 __device__ __forceinline__ unsigned f32_key(float v) {

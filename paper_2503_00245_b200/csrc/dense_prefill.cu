@@ -55,7 +55,7 @@ struct DPPhase {
 struct DPParams {
   const unsigned* counts;  // [E] tokens of each expert, or null: ...
   const int32_t* offsets;  // ... [E+1] slot ranges
-  int E, T, n_pairs_tk;    // experts, tokens, (token, choice) pairs
+  int E, n_pairs_tk;       // experts, (token, choice) pairs
   int cap;                 // > 0: the rows of x are grouped at [e * cap ...] and not by slot
   const int32_t *topk_idx, *pos;  // with counts: the pairs' experts and places among their expert's tokens ...
   int32_t* inv;                   // ... from which their slots are worked out
@@ -64,7 +64,7 @@ struct DPParams {
   __nv_bfloat16* hidden;
   float* out;
   long long plane_elems;
-  int n_slots, slot_bytes;  // the ring: slots of one operand's K step each
+  int ring_slots, slot_bytes;  // the ring: slots of one operand's K step each
   int likely;  // tokens per expert under even routing
   DeviceState* st;
 };
@@ -217,10 +217,10 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
   // the ring's slots are identical in both CTAs, because the MMA addresses the pair's operands by one shared-memory offset
   const uint32_t a1_bytes = (uint32_t)P.ph[0].hb * kBK * 2, a2_bytes = (uint32_t)P.ph[1].hb * kBK * 2;
   unsigned char* slots = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* const epi_bufs = slots + (size_t)P.n_slots * P.slot_bytes;
+  unsigned char* const epi_bufs = slots + (size_t)P.ring_slots * P.slot_bytes;
   SmemDP& sm = *reinterpret_cast<SmemDP*>(epi_bufs + kEpiBytesDP);
   const int tid = threadIdx.x, lane = tid & 31, warp = lane0(tid >> 5);
-  const int NS = P.n_slots;
+  const int NS = P.ring_slots;
   const uint32_t rank = (uint32_t)lane0((int)cluster_ctarank());
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
@@ -599,8 +599,10 @@ double hbm_cycles(int na, int hb, double tiles_per_weight) { return na * hb * 12
 
 }  // namespace
 
-// (Decomposed experts with few pairs: the four GEMMs' prefix sums over the counts cost what the gather's launch does.  384 pairs at d
-// 440, r 216: 55.6 us placed, 53.2 grouped and gathered; 1488 at d 648, r 104: 49.2 and 51.5; 4096 at d 2048, r 128: 102.8 and 109.5.)
+// Decomposed experts with few pairs gain too little by it for E / k times the scratch.  Grouped and gathered -> placed, graph of 20
+// calls, us: d 2048, r 128, 8 experts, 512 pairs 57.4 -> 57.5, 768 60.2 -> 60.2, 1024 62.9 -> 62.4, 2048 77.8 -> 77.0, 4096 101.8 -> 97.4;
+// d 440, r 216: 384 45.6 -> 44.8, 1024 50.9 -> 49.4, 4096 63.9 -> 59.2; d 512, r 64, 16 experts: 512 40.8 -> 40.3, 1024 42.9 -> 41.3,
+// 4096 53.9 -> 48.6.
 int prefill_placed_tokens(const moe_config& c, int T) {
   const int t = (int)std::min<size_t>(T, kScatterBytesMax / ((size_t)c.n_experts * c.d_model * 2));
   return route_tile_applies(c, t) && (c.wd_rank == 0 || (long long)t * c.top_k >= 1024) ? t : 0;
@@ -612,7 +614,7 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   const int d = c.d_model, f = c.d_ff, E = c.n_experts, n_slots = T * c.top_k, pairs_all = ctx->sm_count / 2;
   const int active = std::min(E, n_slots), m = std::max(1, n_slots / E);
   DPParams P{};
-  P.counts = rows.counts, P.offsets = rows.offsets, P.E = E, P.T = T, P.n_pairs_tk = n_slots, P.cap = rows.counts ? T : 0;
+  P.counts = rows.counts, P.offsets = rows.offsets, P.E = E, P.n_pairs_tk = n_slots, P.cap = rows.counts ? T : 0;
   P.topk_idx = rows.topk_idx, P.pos = rows.pos, P.inv = rows.inv;
   P.tb = m + m / 4 + 16 <= 192 ? 32 : 64;  // (32 rows: less read past an expert's tokens; 64: fewer loads to issue)
   P.likely = m, P.st = ctx->d_state;
@@ -624,6 +626,7 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   const int kb1 = (d + kBK - 1) / kBK, kb2 = (f + kBK - 1) / kBK;
   int hb1 = 0, ks2 = 1;
   const int hb2 = d > 128 ? 128 : 64;
+  int last_nt = 0;
   double best = 0;
   // Tiles of up to 256 tokens: an expert with more than its share needs no further pass over its weights (512 tokens, d 1024, f 2816,
   // all at the same two of 8 experts: tiles as wide as an even share, 192, 45.6 us, 256 41.7; 1000 tokens, d 2048, f 5632, 2 of 16:
@@ -631,6 +634,8 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   // tokens, d 304, f 904, 2 experts: 256 30.2 us, 128 27.4).
   for (const int w_max : {256, 128}) {
     const int nt = token_tiles_expected(n_slots, E, w_max), n = std::min(w_max, (n_slots / nt + 31) / 32 * 32), ns = ring_slots(128);
+    if (nt == last_nt) break;  // (an even share fits into either: the same tiles)
+    last_nt = nt;
     const double tpw = (double)nt / active;
     for (int h1 = 128; h1 >= 32; h1 -= 8) {
       const int n1 = nt * ((f + 2 * h1 - 1) / (2 * h1));
@@ -662,9 +667,9 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   MOE_TRY(make_map_b(&w2, w->gud, d, 3, f, E, 64, kBK));
   MOE_TRY(make_map_a(&x2, hidden, n_slots, f, f, P.tb));
   P.slot_bytes = 128 * kBK * 2;
-  P.n_slots = ring_slots(128);
-  if (P.n_slots < 6) return MOE_ERR_UNSUPPORTED;
-  const size_t smem = (size_t)P.n_slots * P.slot_bytes + fixed;
+  P.ring_slots = ring_slots(128);
+  if (P.ring_slots < 6) return MOE_ERR_UNSUPPORTED;
+  const size_t smem = (size_t)P.ring_slots * P.slot_bytes + fixed;
   MOE_TRY(allow_full_smem<dense_prefill_kernel>(ctx));
   const long long most = ((long long)(n_slots + P.w_max - 1) / P.w_max + E) * (P.ph[0].per_tok + P.ph[1].per_tok);
   const int pairs = (int)std::min<long long>(most, max_pairs<dense_prefill_kernel>(ctx, kThreadsDP, smem));

@@ -478,9 +478,9 @@ int launch_gg(moe_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const 
 }
 
 // Output columns per tile: the largest of 64, 128, ... `cap` that is not mostly padding.
-int pick_bn(int n_total, int cap, int floor_bn = 64) {
+int pick_bn(int n_total, int cap) {
   int bn = cap;
-  while (bn > floor_bn && bn / 2 >= n_total) bn /= 2;
+  while (bn > 64 && bn / 2 >= n_total) bn /= 2;
   return bn;
 }
 
