@@ -197,6 +197,7 @@ def test_captured_prefill_follows_its_inputs(r):
     others[1][::3] = others[1][0]                       # a third of the tokens share their experts
     want = [lay.forward(v) for v in others]
     y = torch.empty_like(x)
+    torch.cuda.synchronize()                            # (a context serves one stream at a time)
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
         lay.forward(x, y=y)
