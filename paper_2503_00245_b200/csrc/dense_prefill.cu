@@ -24,10 +24,10 @@
 // What bounds it: with 256 tokens per expert and more, the tensor cores (a tile of phase 1 with 224 columns and 32 K steps takes 17
 // us, 28.7 k cycles of them) and the special-function unit, which the epilogue's exponentials and reciprocals keep busy for 2 us per
 // tile, in the open when a tile takes all 512 columns; with fewer, HBM and the round trip of 1.5 us through the ring.
-// Before (five launches, tokens on the M side) and now, whole layer: d 1024, f 2816, 512 tokens 57 -> 52.7 us; d 1440, f 3840,
-// 333 tokens 90 -> 70; d 2048, f 5632, 2048 tokens 300-340 -> 262-267.
-// Tried: weights asked into L2 ahead of their loads, from the router's launch or from here (0 to -1 us for 30 MB, +2 for 90);
-// the first K steps loaded in front of the dependency wait (-0.5 us); eight epilogue warps that keep a tile's gate sums in 128
+// Before (five launches, tokens on the M side) and now, whole layer, graphs of 20 calls on one GPU: d 1024, f 2816, 512 tokens 53.6 ->
+// 51.1 us; d 1440, f 3840, 333 tokens 81.2 -> 66.7; d 2048, f 5632, 2048 tokens 296 -> 256 (for seconds on end, under the power cap, 301).
+// Tried: weights asked into L2 ahead of their loads, from the router's launch or from here (less than 1 us for 30 MB, 2 lost for 92);
+// the first K steps loaded in front of the dependency wait (about half a us); eight epilogue warps that keep a tile's gate sums in 128
 // registers, to free half of the accumulators early (registers spill to L2: +100 us).
 // All waits are bounded; an expired wait sets the ctx's status word.  Every CTA fetches what it needs with its own loads (no
 // multicast).
@@ -466,7 +466,14 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
       // =============================================================== takes the pair's tiles
       // Every pair takes one number that is past the last tile, so the launch takes n_work + n_pairs of them; who has the
       // highest sets the counter back.
-      if (lane == 0 && idx == n_work + n_pairs - 1) atomicExch(&P.st->ffn_next, 0u);
+      // (The fence: it is zero before this CTA ends, so before any successor starts.)
+      auto set_back = [&]() {
+        if (idx == n_work + n_pairs - 1) {
+          atomicExch(&P.st->ffn_next, 0u);
+          __threadfence();
+        }
+      };
+      if (lane == 0) set_back();
       for (int q = 0; idx < n_work; ++q) {
         const int b = q & (kQueue - 1);
         if (!mbar_wait_warp(&sm.tile_ask, q & 1) || (q >= kQueue && !mbar_wait_warp(&sm.tile_empty[b], (q / kQueue - 1) & 1))) {
@@ -481,7 +488,7 @@ __global__ void __launch_bounds__(kThreadsDP, 1)
         }
         if (lane == 0) {
           hand_out(sm, b, idx, t);
-          if (idx == n_work + n_pairs - 1) atomicExch(&P.st->ffn_next, 0u);
+          set_back();
         }
       }
     } else if (P.counts) {
