@@ -249,7 +249,8 @@ PROFILE_OF = {
     "wearable-decode-T1": "dense_stream_kernel_wearable_decode_T1.md",
     "wearable-decode-T8": "dense_stream_kernel_wearable_decode_T8.md",
     "phone-decode-T1": "dense_stream_kernel_phone_decode_T1.md",
-    "phone-prefill-T2048": "grouped_gemm_kernel_phone_prefill_T2048.md",
+    "wearable-prefill-T512": "dense_prefill_kernel_wearable_prefill_T512.md",
+    "phone-prefill-T2048": "dense_prefill_kernel_phone_prefill_T2048.md",
     "phone-wd128-decode-T1": "wd_decode_kernel_phone_wd128_decode_T1.md",
     "phone-wd1024-decode-T1": "wd_stream_kernel_phone_wd1024_decode_T1.md",
 }
