@@ -1483,6 +1483,8 @@ int launch_variant(const moe_ctx* ctx, const DenseParams& P, int grid, size_t sm
   MOE_TRY(allow_full_smem<dense_stream_kernel<V>>(ctx));
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(grid), lc.blockDim = dim3(kThreads), lc.dynamicSmemBytes = smem, lc.stream = s;
+  // (The CTAs wait for one another, and the launch is not cooperative: that costs 2.8 us a layer, d 256 f 512, one token 7.4 -> 10.2.  So
+  // the header says which launches may not overlap with it.)
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
