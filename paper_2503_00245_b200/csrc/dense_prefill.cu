@@ -627,8 +627,8 @@ int launch_dense_prefill(moe_ctx* ctx, int T, const moe_weights* w, const Prefil
   P.likely = m, P.st = ctx->d_state;
   P.hidden = (__nv_bfloat16*)hidden, P.plane_elems = (long long)n_slots * d;
   // how the work is cut: the fewest cycles for the pair with the most, tiles of both phases being dealt out in turn
-  const size_t fixed = kEpiBytesDP + sizeof(SmemDP) + 1024 + 128;  // (an MMA reads 128 rows of weights, whatever hb is: the
-                                                                   // epilogue's buffers are long enough behind the last slot)
+  // (a slot has 128 rows: an MMA reads as many of the weights, whatever hb is, and half of a tile's tokens are no more)
+  const size_t fixed = kEpiBytesDP + sizeof(SmemDP) + 1024 + 128;
   const auto ring_slots = [&](int h) { return (int)((ctx->max_smem_optin - fixed) / ((size_t)h * kBK * 2)); };
   const int kb1 = (d + kBK - 1) / kBK, kb2 = (f + kBK - 1) / kBK;
   int hb1 = 0, ks2 = 1;
